@@ -348,7 +348,7 @@ struct tt_ctx {
     unsigned graph_launches = 0;       // library kernels one replay runs
     bool ranks_stale = false;          // h->r lags the device after replays
     int cap1 = 0, cap2 = 0;            // rank caps of the two bonds
-    DevBuf dyn_buf, dyn_part;          // size block (ints) and product partials
+    DevBuf dyn_buf, dyn_part, dyn_tc;  // size block (ints), product partials, digit-product scratch
     int* dyn = nullptr;
     int* h_dyn = nullptr;              // pinned mirror, refreshed by every replay
     double* h_dyn_dec = nullptr;       // pinned decisions of the two bonds (8 doubles)
@@ -400,7 +400,7 @@ struct tt_ctx {
                           &partials, &bwd, &f_sigma_a, &f_sigma_s, &f_cv, &f_T, &f_Estar, &f_E,
                           &thbar, &red, &ang_buf, &src_x, &src_th, &src_ph, &src_q,
                           &split_fac, &sp_F, &sp_tmp[0], &sp_tmp[1], &f_fw, &usr_x, &usr_th, &usr_ph,
-                          &sk_Y, &sk_Q, &sk_G, &sk_lam, &sk_Vt, &sk_Vs, &xch, &dyn_buf, &dyn_part, &ydots,
+                          &sk_Y, &sk_Q, &sk_G, &sk_lam, &sk_Vt, &sk_Vs, &xch, &dyn_buf, &dyn_part, &dyn_tc, &ydots,
                           &ts_Qa, &ts_Qb, &ts_Y, &ts_R, &ts_J, &ts_lam, &ts_Vt, &ts_U, &ts_M};
         for (DevBuf* b : bufs) b->release();
         for (auto& ax : inflow)
@@ -535,7 +535,7 @@ tt_status eig_orthonormalise(tt_ctx* h, long m, int l, const double* Y, DevBuf& 
     TT_TRY(h->sk_lam.ensure((size_t)l, s));
     TT_TRY(h->sk_Vt.ensure((size_t)l * l, s));
     TT_TRY(h->sk_Vs.ensure((size_t)l * l, s));
-    TT_TRY(gram(s, (int)m, l, Y, l, h->sk_G.p, l, h->partials));
+    TT_TRY(gram(s, (int)m, l, Y, l, h->sk_G.p, l, h->partials, h->d_int + HI_STATUS));
     // Y^T Y is positive semidefinite: the handle's eigensolver for such matrices
     if (h->eig_method == TT_EIG_ONE_SIDED)
         TT_TRY(syev_psd(s, l, h->sk_G.p, l, h->sk_lam.p, h->sk_Vt.p, l, h->eig, h->d_int + HI_STATUS,
@@ -551,7 +551,8 @@ tt_status eig_orthonormalise(tt_ctx* h, long m, int l, const double* Y, DevBuf& 
     if (k == 0) return TT_OK;
     scale_rows(s, k, l, h->sk_Vt.p, l, h->sk_lam.p, 2, h->sk_Vs.p, l);  // rows v_j / sqrt(lambda_j)
     TT_TRY(Q.ensure((size_t)m * k, s));
-    TT_TRY(dgemm(s, false, true, (int)m, k, l, 1.0, Y, l, h->sk_Vs.p, l, 0.0, Q.p, k));
+    TT_TRY(dgemm_sk(s, false, true, (int)m, k, l, 1.0, Y, l, h->sk_Vs.p, l, Q.p, k,
+                    h->partials, h->d_int + HI_STATUS));
     return TT_OK;
 }
 
@@ -594,15 +595,15 @@ tt_status round_randomized(tt_ctx* h, DevBuf* src, const int* R, DevBuf* dst, in
         PhaseScope ps(h, TT_PH_GRAM_RIGHT, fl, 0.0);
         TT_TRY(h->sk_W[d - 2].ensure((size_t)R[d - 1] * l[d - 1], s));
         TT_TRY(dgemm_sk(s, false, true, R[d - 1], l[d - 1], n[d - 1], 1.0, src[d - 1].p, n[d - 1],
-                        h->sk_sub[d - 1].p, n[d - 1], h->sk_W[d - 2].p, l[d - 1], h->partials));
+                        h->sk_sub[d - 1].p, n[d - 1], h->sk_W[d - 2].p, l[d - 1], h->partials, h->d_int + HI_STATUS));
         for (int c = d - 2; c >= 1; --c) {
             // T = G_c W_c (R_c n_c x l_{c+1}); W_{c-1} = T (R_c x n_c l_{c+1}) Omega_c^T
             TT_TRY(h->bwd.ensure((size_t)R[c] * n[c] * l[c + 1], s));
-            TT_TRY(dgemm(s, false, false, R[c] * n[c], l[c + 1], R[c + 1], 1.0, src[c].p, R[c + 1],
-                         h->sk_W[c].p, l[c + 1], 0.0, h->bwd.p, l[c + 1]));
+            TT_TRY(dgemm_sk(s, false, false, R[c] * n[c], l[c + 1], R[c + 1], 1.0, src[c].p, R[c + 1],
+                         h->sk_W[c].p, l[c + 1], h->bwd.p, l[c + 1], h->partials, h->d_int + HI_STATUS));
             TT_TRY(h->sk_W[c - 1].ensure((size_t)R[c] * l[c], s));
             TT_TRY(dgemm_sk(s, false, true, R[c], l[c], n[c] * l[c + 1], 1.0, h->bwd.p, (long)n[c] * l[c + 1],
-                            h->sk_sub[c].p, (long)n[c] * l[c + 1], h->sk_W[c - 1].p, l[c], h->partials));
+                            h->sk_sub[c].p, (long)n[c] * l[c + 1], h->sk_W[c - 1].p, l[c], h->partials, h->d_int + HI_STATUS));
         }
     }
     rr[0] = 1;
@@ -615,7 +616,8 @@ tt_status round_randomized(tt_ctx* h, DevBuf* src, const int* R, DevBuf* dst, in
         TT_TRY(h->sk_Y.ensure((size_t)m * lb, s));
         {
             PhaseScope ps(h, TT_PH_GRAM_LEFT, 2.0 * m * (double)Rk * lb + 2.0 * m * (double)lb * lb, 0.0);
-            TT_TRY(dgemm(s, false, false, (int)m, lb, Rk, 1.0, A, Rk, h->sk_W[b].p, lb, 0.0, h->sk_Y.p, lb));
+            TT_TRY(dgemm_sk(s, false, false, (int)m, lb, Rk, 1.0, A, Rk, h->sk_W[b].p, lb, h->sk_Y.p, lb,
+                            h->partials, h->d_int + HI_STATUS));
         }
         int k1 = 0, k2 = 0;
         {
@@ -641,9 +643,9 @@ tt_status round_randomized(tt_ctx* h, DevBuf* src, const int* R, DevBuf* dst, in
             // M_upd = Q^T A (rk x Rk), then the next core M_upd x_1 G_{b+1}
             TT_TRY(h->Mupd.ensure((size_t)rk * Rk, s));
             TT_TRY(dgemm_sk(s, true, false, rk, Rk, (int)m, 1.0, dst[b].p, rk, A, Rk, h->Mupd.p, Rk,
-                            h->partials));
+                            h->partials, h->d_int + HI_STATUS));
             TT_TRY(dgemm_sk(s, false, false, rk, (int)ncols, Rk, 1.0, h->Mupd.p, Rk, src[b + 1].p, ncols,
-                            next, ncols, h->partials));
+                            next, ncols, h->partials, h->d_int + HI_STATUS));
         }
         rr[b + 1] = rk;
         A = next;
@@ -673,12 +675,13 @@ tt_status orth_qr3(tt_ctx* h, long m, int l, const double* Y, DevBuf** Q, int* k
     TT_TRY(h->sk_lam.ensure((size_t)l, s));
     TT_TRY(h->sk_Vt.ensure((size_t)l * l, s));
     TT_TRY(h->sk_Vs.ensure((size_t)l * l, s));
-    TT_TRY(gram(s, (int)m, l, Y, l, h->sk_G.p, l, h->partials));
+    TT_TRY(gram(s, (int)m, l, Y, l, h->sk_G.p, l, h->partials, h->d_int + HI_STATUS));
     TT_TRY(syev(s, l, h->sk_G.p, l, h->sk_lam.p, h->sk_Vt.p, l, h->eig, h->d_int + HI_STATUS,
                 h->d_int + next_sweep_slot(h), h->max_sweeps));
     shifted_scale_rows(s, l, h->sk_Vt.p, l, h->sk_lam.p, h->sk_Vs.p, l);
     TT_TRY(h->ts_Qa.ensure((size_t)m * l, s));
-    TT_TRY(dgemm(s, false, true, (int)m, l, l, 1.0, Y, l, h->sk_Vs.p, l, 0.0, h->ts_Qa.p, l));
+    TT_TRY(dgemm_sk(s, false, true, (int)m, l, l, 1.0, Y, l, h->sk_Vs.p, l, h->ts_Qa.p, l,
+                    h->partials, h->d_int + HI_STATUS));
     int k2 = 0, k3 = 0;
     TT_TRY(eig_orthonormalise(h, m, l, h->ts_Qa.p, h->ts_Qb, &k2));
     if (k2 == 0) {
@@ -730,13 +733,13 @@ tt_status round_ttsvd(tt_ctx* h, DevBuf* src, const int* R, DevBuf* dst, int* rr
             if (q == 0) return zero_tt(h, dst, rr);
             TT_TRY(h->ts_R.ensure((size_t)q * rows, s));
             TT_TRY(dgemm_sk(s, true, false, q, rows, (int)ncols, 1.0, Q->p, q, h->ts_Y.p, rows, h->ts_R.p, rows,
-                            h->partials));
+                            h->partials, h->d_int + HI_STATUS));
             TT_TRY(h->ts_core[k].ensure((size_t)q * ncols, s));
             transpose(s, ncols, q, Q->p, q, h->ts_core[k].p, ncols);
             const long prow = (long)Rb[k - 1] * n[k - 1];
             TT_TRY(h->ts_core[k - 1].ensure((size_t)prow * q, s));
-            TT_TRY(dgemm(s, false, true, (int)prow, q, rows, 1.0, src[k - 1].p, rows, h->ts_R.p, rows, 0.0,
-                         h->ts_core[k - 1].p, q));
+            TT_TRY(dgemm_sk(s, false, true, (int)prow, q, rows, 1.0, src[k - 1].p, rows, h->ts_R.p, rows, h->ts_core[k - 1].p, q,
+                            h->partials, h->d_int + HI_STATUS));
             Rb[k] = q;
         }
     }
@@ -758,7 +761,8 @@ tt_status round_ttsvd(tt_ctx* h, DevBuf* src, const int* R, DevBuf* dst, int* rr
             TT_TRY(orth_qr3(h, m, l, A, &Q, &q));
             if (q == 0) return zero_tt(h, dst, rr);
             TT_TRY(h->ts_R.ensure((size_t)q * l, s));
-            TT_TRY(dgemm_sk(s, true, false, q, l, (int)m, 1.0, Q->p, q, A, l, h->ts_R.p, l, h->partials));
+            TT_TRY(dgemm_sk(s, true, false, q, l, (int)m, 1.0, Q->p, q, A, l, h->ts_R.p, l,
+                            h->partials, h->d_int + HI_STATUS));
         }
         const int p = q + l, pm = std::min(q, l);
         {
@@ -799,7 +803,8 @@ tt_status round_ttsvd(tt_ctx* h, DevBuf* src, const int* R, DevBuf* dst, int* rr
             jw_split(s, rk, q, l, h->ts_lam.p, h->d_dbl + HD_JWC, h->ts_Vt.p, p, h->ts_U.p, h->ts_M.p);
             // A' = Q U_r
             TT_TRY(dst[k].ensure((size_t)m * rk, s));
-            TT_TRY(dgemm(s, false, true, (int)m, rk, q, 1.0, Q->p, q, h->ts_U.p, q, 0.0, dst[k].p, rk));
+            TT_TRY(dgemm_sk(s, false, true, (int)m, rk, q, 1.0, Q->p, q, h->ts_U.p, q, dst[k].p, rk,
+                            h->partials, h->d_int + HI_STATUS));
             // next core = S_r V_r^T x_1 (right-orthonormal core k+1)
             if (k == d - 2) {
                 TT_TRY(dst[d - 1].ensure((size_t)rk * ncols, s));
@@ -810,7 +815,7 @@ tt_status round_ttsvd(tt_ctx* h, DevBuf* src, const int* R, DevBuf* dst, int* rr
                 tmp_idx ^= 1;
             }
             TT_TRY(dgemm_sk(s, false, false, rk, (int)ncols, l, 1.0, h->ts_M.p, l, h->ts_core[k + 1].p, ncols,
-                            next, ncols, h->partials));
+                            next, ncols, h->partials, h->d_int + HI_STATUS));
         }
         rr[k + 1] = rk;
         A = next;
@@ -867,7 +872,7 @@ tt_status round_cores(tt_ctx* h, DevBuf* src, const int* R, DevBuf* dst, int* rr
         const int Rl = R[d - 1];
         TT_TRY(h->GB[d - 2].ensure((size_t)Rl * Rl, s));
         TT_TRY(dgemm_sk(s, false, true, Rl, Rl, n[d - 1], 1.0, src[d - 1].p, n[d - 1], src[d - 1].p,
-                        n[d - 1], h->GB[d - 2].p, Rl, h->partials));
+                        n[d - 1], h->GB[d - 2].p, Rl, h->partials, h->d_int + HI_STATUS));
         for (int k = d - 3; k >= 0; --k) {
             const int Ra = R[k + 1], nn = n[k + 1], Rb = R[k + 2];
             TT_TRY(h->bwd.ensure((size_t)Ra * nn * Rb, s));
@@ -881,10 +886,10 @@ tt_status round_cores(tt_ctx* h, DevBuf* src, const int* R, DevBuf* dst, int* rr
                 TT_TRY(slgemm_nt(s, Ra, Ra, nn * Rb, h->bwd.p, (long)nn * Rb, src[k + 1].p,
                                  (long)nn * Rb, h->GB[k].p, Ra, h->slscratch, h->d_int + HI_STATUS));
             } else {
-                TT_TRY(dgemm(s, false, false, Ra * nn, Rb, Rb, 1.0, src[k + 1].p, Rb, h->GB[k + 1].p,
-                             Rb, 0.0, h->bwd.p, Rb));
+                TT_TRY(dgemm_sk(s, false, false, Ra * nn, Rb, Rb, 1.0, src[k + 1].p, Rb, h->GB[k + 1].p,
+                             Rb, h->bwd.p, Rb, h->partials, h->d_int + HI_STATUS));
                 TT_TRY(dgemm_sk(s, false, true, Ra, Ra, nn * Rb, 1.0, h->bwd.p, (long)nn * Rb,
-                                src[k + 1].p, (long)nn * Rb, h->GB[k].p, Ra, h->partials));
+                                src[k + 1].p, (long)nn * Rb, h->GB[k].p, Ra, h->partials, h->d_int + HI_STATUS));
             }
         }
     }
@@ -937,7 +942,7 @@ tt_status round_cores(tt_ctx* h, DevBuf* src, const int* R, DevBuf* dst, int* rr
                               reinterpret_cast<int*>(h->erowA.p)));
             }
             else
-                TT_TRY(gram(s, (int)m, Rk, A, Rk, h->GA.p, Rk, h->partials));
+                TT_TRY(gram(s, (int)m, Rk, A, Rk, h->GA.p, Rk, h->partials, h->d_int + HI_STATUS));
             // a spatial shard holds some rows of the spatial core: its left
             // Gram is the sum of the shards' partial Grams
             if (k == 0 && h->shard.on) TT_TRY(shard_exchange(h, TT_XCHG_SUM, h->GA.p, (size_t)Rk * Rk));
@@ -948,8 +953,10 @@ tt_status round_cores(tt_ctx* h, DevBuf* src, const int* R, DevBuf* dst, int* rr
             const double* Wk = h->VtB[k].p;
             TT_TRY(h->T1.ensure((size_t)Rk * kB, s));
             TT_TRY(h->K.ensure((size_t)kB * kB, s));
-            TT_TRY(dgemm_sk(s, false, true, Rk, kB, Rk, 1.0, h->GA.p, Rk, Wk, Rk, h->T1.p, kB, h->partials));
-            TT_TRY(dgemm_sk(s, false, false, kB, kB, Rk, 1.0, Wk, Rk, h->T1.p, kB, h->K.p, kB, h->partials));
+            TT_TRY(dgemm_sk(s, false, true, Rk, kB, Rk, 1.0, h->GA.p, Rk, Wk, Rk, h->T1.p, kB,
+                            h->partials, h->d_int + HI_STATUS));
+            TT_TRY(dgemm_sk(s, false, false, kB, kB, Rk, 1.0, Wk, Rk, h->T1.p, kB, h->K.p, kB,
+                            h->partials, h->d_int + HI_STATUS));
         }
         TT_TRY(h->lamK.ensure((size_t)kB, s));
         TT_TRY(h->VtK.ensure((size_t)kB * kB, s));
@@ -988,13 +995,13 @@ tt_status round_cores(tt_ctx* h, DevBuf* src, const int* R, DevBuf* dst, int* rr
             scale_rows(s, rk, kB, h->VtK.p, kB, h->lamK.p, 2, h->Vts.p, kB);
             TT_TRY(h->PAt.ensure((size_t)rk * Rk, s));
             TT_TRY(dgemm_sk(s, false, false, rk, Rk, kB, 1.0, h->Vts.p, kB, h->VtB[k].p, Rk, h->PAt.p, Rk,
-                            h->partials));
+                            h->partials, h->d_int + HI_STATUS));
             // M_upd = P_A^T G_A = A'^T A  (rk x Rk): B'^T = A'^T A B^T, the orthogonal
             // projection of A B^T onto span(A'); equals App. A.2's (V_B S_B^{-1} V~ S~)^T
             // on the retained eigenspace of G_B without forming S_B^{-1}
             TT_TRY(h->Mupd.ensure((size_t)rk * Rk, s));
             TT_TRY(dgemm_sk(s, false, false, rk, Rk, Rk, 1.0, h->PAt.p, Rk, h->GA.p, Rk, h->Mupd.p, Rk,
-                            h->partials));
+                            h->partials, h->d_int + HI_STATUS));
         }
         if (h->cur_rec && h->rec_proj && k < 2) {
             tt_ctx::StepRec* rc = h->cur_rec;
@@ -1012,7 +1019,8 @@ tt_status round_cores(tt_ctx* h, DevBuf* src, const int* R, DevBuf* dst, int* rr
                 TT_TRY(slgemm_nt(s, m, rk, Rk, A, Rk, h->PAt.p, Rk, dst[k].p, rk, h->slscratch,
                                  h->d_int + HI_STATUS, &h->partials, reinterpret_cast<const int*>(h->erowA.p)));
             else
-                TT_TRY(dgemm(s, false, true, (int)m, rk, Rk, 1.0, A, Rk, h->PAt.p, Rk, 0.0, dst[k].p, rk));
+                TT_TRY(dgemm_sk(s, false, true, (int)m, rk, Rk, 1.0, A, Rk, h->PAt.p, Rk, dst[k].p, rk,
+                                h->partials, h->d_int + HI_STATUS));
         }
         // next core = M_upd x_1 G_{k+1}
         double* next;
@@ -1028,7 +1036,7 @@ tt_status round_cores(tt_ctx* h, DevBuf* src, const int* R, DevBuf* dst, int* rr
             PhaseScope ps(h, TT_PH_UPDATE, 2.0 * rk * (double)Rk * ncols,
                           8.0 * ((double)Rk * ncols + (double)rk * ncols));
             TT_TRY(dgemm_sk(s, false, false, rk, (int)ncols, Rk, 1.0, h->Mupd.p, Rk, src[k + 1].p, ncols,
-                            next, ncols, h->partials));
+                            next, ncols, h->partials, h->d_int + HI_STATUS));
         }
         rr[k + 1] = rk;
         A = next;
@@ -1130,8 +1138,8 @@ tt_status split_contract(tt_ctx* h, const double* U, int P, double* out) {
             dst = h->sp_tmp[ti].p;
             ti ^= 1;
         }
-        TT_TRY(dgemm(s, false, zt, (int)rows, (int)cols, h->r[k + 1], 1.0, h->core[k].p, h->r[k + 1], Z,
-                     zt ? h->r[k + 1] : cols, 0.0, dst, cols));
+        TT_TRY(dgemm_sk(s, false, zt, (int)rows, (int)cols, h->r[k + 1], 1.0, h->core[k].p, h->r[k + 1], Z,
+                     zt ? h->r[k + 1] : cols, dst, cols, h->partials, h->d_int + HI_STATUS));
         Z = dst;
         zt = false;
         cols *= h->n[k];
@@ -1452,18 +1460,24 @@ tt_status graph_step_body(tt_ctx* h) {
                           h->ydots.p, Sources(), dd);
     // rounding (App. A.2, one-sided Gram truncation): backward sweep
     fill(s, h->d_dbl + HD_DELTA2, 1, -1.0);
-    TT_TRY(dgemm_dyn(s, false, true, desc + 0, G2, G2, np, 1.0, h->gcore[2].p, h->gcore[2].p, h->GB[1].p, P, PC, 1));
-    TT_TRY(dgemm_dyn(s, false, false, desc + 8, G1 * nt, G2, G2, 1.0, h->gcore[1].p, h->GB[1].p, h->bwd.p, P, PC, 0));
-    TT_TRY(dgemm_dyn(s, false, true, desc + 16, G1, G1, nt * G2, 1.0, h->bwd.p, h->gcore[1].p, h->GB[0].p, P, PC, 1));
+    TT_TRY(dgemm_dyn(s, false, true, desc + 0, G2, G2, np, 1.0, h->gcore[2].p, h->gcore[2].p, h->GB[1].p, P, PC, 1, h->dyn_tc,
+                     h->d_int + HI_STATUS));
+    TT_TRY(dgemm_dyn(s, false, false, desc + 8, G1 * nt, G2, G2, 1.0, h->gcore[1].p, h->GB[1].p, h->bwd.p, P, PC, 1, h->dyn_tc,
+                     h->d_int + HI_STATUS));
+    TT_TRY(dgemm_dyn(s, false, true, desc + 16, G1, G1, nt * G2, 1.0, h->bwd.p, h->gcore[1].p, h->GB[0].p, P, PC, 1, h->dyn_tc,
+                     h->d_int + HI_STATUS));
     TT_TRY(pchol_dyn(s, dd + DYN_G1, G1, h->GB[0].p, h->VtB[0].p, h->Wc.p, h->lamB[0].p, h->eig,
                      h->d_int + HI_STATUS, dd + DYN_KB0));
     TT_TRY(pchol_dyn(s, dd + DYN_G2, G2, h->GB[1].p, h->VtB[1].p, h->Wc.p, h->lamB[1].p, h->eig,
                      h->d_int + HI_STATUS, dd + DYN_KB1));
     plan(1);
     // bond 0: G_A, K = W G_A W^T, eig(K), decision
-    TT_TRY(dgemm_dyn(s, true, false, desc + 24, G1, G1, (int)nc, 1.0, h->gcore[0].p, h->gcore[0].p, h->GA.p, P, PC, 2));
-    TT_TRY(dgemm_dyn(s, false, true, desc + 32, G1, G1, G1, 1.0, h->GA.p, h->VtB[0].p, h->T1.p, P, PC, 1));
-    TT_TRY(dgemm_dyn(s, false, false, desc + 40, G1, G1, G1, 1.0, h->VtB[0].p, h->T1.p, h->K.p, P, PC, 1));
+    TT_TRY(dgemm_dyn(s, true, false, desc + 24, G1, G1, (int)nc, 1.0, h->gcore[0].p, h->gcore[0].p, h->GA.p, P, PC, 2, h->dyn_tc,
+                     h->d_int + HI_STATUS));
+    TT_TRY(dgemm_dyn(s, false, true, desc + 32, G1, G1, G1, 1.0, h->GA.p, h->VtB[0].p, h->T1.p, P, PC, 1, h->dyn_tc,
+                     h->d_int + HI_STATUS));
+    TT_TRY(dgemm_dyn(s, false, false, desc + 40, G1, G1, G1, 1.0, h->VtB[0].p, h->T1.p, h->K.p, P, PC, 1, h->dyn_tc,
+                     h->d_int + HI_STATUS));
     TT_TRY((h->eig_method == TT_EIG_ONE_SIDED ? syev_psd_dyn : syev_dyn)(
         s, dd + DYN_KB0, G1, h->K.p, h->lamK.p, h->VtK.p, h->eig, h->d_int + HI_STATUS, dd + DYN_SWEEPS,
         h->max_sweeps));
@@ -1472,14 +1486,21 @@ tt_status graph_step_body(tt_ctx* h) {
     plan(2);
     // bond 0 update: P_A^T, M_upd, X' = X* P_A, next core = M_upd x_1 Theta*
     scale_rows_dyn(s, desc + 48, (long)c1 * G1, h->VtK.p, h->lamK.p, 2, h->Vts.p);
-    TT_TRY(dgemm_dyn(s, false, false, desc + 56, c1, G1, G1, 1.0, h->Vts.p, h->VtB[0].p, h->PAt.p, P, PC, 1));
-    TT_TRY(dgemm_dyn(s, false, false, desc + 64, c1, G1, G1, 1.0, h->PAt.p, h->GA.p, h->Mupd.p, P, PC, 1));
-    TT_TRY(dgemm_dyn(s, false, true, desc + 72, (int)nc, c1, G1, 1.0, h->gcore[0].p, h->PAt.p, h->core[0].p, P, PC, 0));
-    TT_TRY(dgemm_dyn(s, false, false, desc + 80, c1, nt * G2, G1, 1.0, h->Mupd.p, h->gcore[1].p, h->tmp[0].p, P, PC, 1));
+    TT_TRY(dgemm_dyn(s, false, false, desc + 56, c1, G1, G1, 1.0, h->Vts.p, h->VtB[0].p, h->PAt.p, P, PC, 1, h->dyn_tc,
+                     h->d_int + HI_STATUS));
+    TT_TRY(dgemm_dyn(s, false, false, desc + 64, c1, G1, G1, 1.0, h->PAt.p, h->GA.p, h->Mupd.p, P, PC, 1, h->dyn_tc,
+                     h->d_int + HI_STATUS));
+    TT_TRY(dgemm_dyn(s, false, true, desc + 72, (int)nc, c1, G1, 1.0, h->gcore[0].p, h->PAt.p, h->core[0].p, P, PC, 1, h->dyn_tc,
+                     h->d_int + HI_STATUS));
+    TT_TRY(dgemm_dyn(s, false, false, desc + 80, c1, nt * G2, G1, 1.0, h->Mupd.p, h->gcore[1].p, h->tmp[0].p, P, PC, 1, h->dyn_tc,
+                     h->d_int + HI_STATUS));
     // bond 1 on the next core (replicated rows r0 n_theta)
-    TT_TRY(dgemm_dyn(s, true, false, desc + 88, G2, G2, c1 * nt, 1.0, h->tmp[0].p, h->tmp[0].p, h->GA.p, P, PC, 2));
-    TT_TRY(dgemm_dyn(s, false, true, desc + 96, G2, G2, G2, 1.0, h->GA.p, h->VtB[1].p, h->T1.p, P, PC, 1));
-    TT_TRY(dgemm_dyn(s, false, false, desc + 104, G2, G2, G2, 1.0, h->VtB[1].p, h->T1.p, h->K.p, P, PC, 1));
+    TT_TRY(dgemm_dyn(s, true, false, desc + 88, G2, G2, c1 * nt, 1.0, h->tmp[0].p, h->tmp[0].p, h->GA.p, P, PC, 2, h->dyn_tc,
+                     h->d_int + HI_STATUS));
+    TT_TRY(dgemm_dyn(s, false, true, desc + 96, G2, G2, G2, 1.0, h->GA.p, h->VtB[1].p, h->T1.p, P, PC, 1, h->dyn_tc,
+                     h->d_int + HI_STATUS));
+    TT_TRY(dgemm_dyn(s, false, false, desc + 104, G2, G2, G2, 1.0, h->VtB[1].p, h->T1.p, h->K.p, P, PC, 1, h->dyn_tc,
+                     h->d_int + HI_STATUS));
     TT_TRY((h->eig_method == TT_EIG_ONE_SIDED ? syev_psd_dyn : syev_dyn)(
         s, dd + DYN_KB1, G2, h->K.p, h->lamK.p, h->VtK.p, h->eig, h->d_int + HI_STATUS, dd + DYN_SWEEPS + 1,
         h->max_sweeps));
@@ -1487,10 +1508,14 @@ tt_status graph_step_body(tt_ctx* h) {
                             dd + DYN_DEC1, dec_d + 4);
     plan(3);
     scale_rows_dyn(s, desc + 112, (long)c2 * G2, h->VtK.p, h->lamK.p, 2, h->Vts.p);
-    TT_TRY(dgemm_dyn(s, false, false, desc + 120, c2, G2, G2, 1.0, h->Vts.p, h->VtB[1].p, h->PAt.p, P, PC, 1));
-    TT_TRY(dgemm_dyn(s, false, false, desc + 128, c2, G2, G2, 1.0, h->PAt.p, h->GA.p, h->Mupd.p, P, PC, 1));
-    TT_TRY(dgemm_dyn(s, false, true, desc + 136, c1 * nt, c2, G2, 1.0, h->tmp[0].p, h->PAt.p, h->core[1].p, P, PC, 0));
-    TT_TRY(dgemm_dyn(s, false, false, desc + 144, c2, np, G2, 1.0, h->Mupd.p, h->gcore[2].p, h->core[2].p, P, PC, 1));
+    TT_TRY(dgemm_dyn(s, false, false, desc + 120, c2, G2, G2, 1.0, h->Vts.p, h->VtB[1].p, h->PAt.p, P, PC, 1, h->dyn_tc,
+                     h->d_int + HI_STATUS));
+    TT_TRY(dgemm_dyn(s, false, false, desc + 128, c2, G2, G2, 1.0, h->PAt.p, h->GA.p, h->Mupd.p, P, PC, 1, h->dyn_tc,
+                     h->d_int + HI_STATUS));
+    TT_TRY(dgemm_dyn(s, false, true, desc + 136, c1 * nt, c2, G2, 1.0, h->tmp[0].p, h->PAt.p, h->core[1].p, P, PC, 1, h->dyn_tc,
+                     h->d_int + HI_STATUS));
+    TT_TRY(dgemm_dyn(s, false, false, desc + 144, c2, np, G2, 1.0, h->Mupd.p, h->gcore[2].p, h->core[2].p, P, PC, 1, h->dyn_tc,
+                     h->d_int + HI_STATUS));
     // energy-conserving temperature update (Sec. 3.2) from the rounded TT
     plain_thbar(s, h->ang, c1, c2, h->core[1].p, h->core[2].p, h->thbar.p, dd);
     energy_rows(s, nc, c1, h->core[0].p, c1, h->thbar.p, h->fields.c, nullptr, h->f_Estar.p, h->f_cv.p,
@@ -1513,14 +1538,20 @@ tt_status graph_reserve(tt_ctx* h) {
     const long Gm = std::max(G1, G2);
     // partials of the captured split products: the largest need over the
     // (mode, M, N, K) capacities of graph_step_body's products
-    size_t part = 1;
+    size_t part = 1, tcs = 1;
     {
         const int c[][4] = {{1, (int)G2, (int)G2, (int)np},       {1, (int)G1, (int)G1, (int)(nt * G2)},
                             {2, (int)G1, (int)G1, (int)nc},       {1, (int)G1, (int)G1, (int)G1},
                             {1, (int)c1, (int)G1, (int)G1},       {1, (int)c1, (int)(nt * G2), (int)G1},
                             {2, (int)G2, (int)G2, (int)(c1 * nt)}, {1, (int)G2, (int)G2, (int)G2},
-                            {1, (int)c2, (int)G2, (int)G2},       {1, (int)c2, (int)np, (int)G2}};
-        for (const auto& q : c) part = std::max(part, dyn_partials_need(q[0], q[1], q[2], q[3]));
+                            {1, (int)c2, (int)G2, (int)G2},       {1, (int)c2, (int)np, (int)G2},
+                            {1, (int)(G1 * nt), (int)G2, (int)G2}, {1, (int)nc, (int)c1, (int)G1},
+                            {1, (int)(c1 * nt), (int)c2, (int)G2}};
+        for (const auto& q : c) {
+            part = std::max(part, dyn_partials_need(q[0], q[1], q[2], q[3]));
+            if (tc8_wanted(q[1], q[2], q[3]))
+                tcs = std::max(tcs, tc8_scratch_doubles(q[1], q[2], q[3], q[0] == 2));
+        }
     }
     struct Need {
         DevBuf* b;
@@ -1537,6 +1568,7 @@ tt_status graph_reserve(tt_ctx* h) {
         {&h->eig.lam_unsorted, Gm}, {&h->eig.abc, 3 * (Gm + 1)}, {&h->eig.cs, Gm + 1},
         {&h->eig.psd, 3 * Gm + 2},
         {&h->dyn_part, (long)part},
+        {&h->dyn_tc, (long)tcs},
     };
     for (auto& x : need) TT_TRY(x.b->ensure((size_t)std::max<long>(x.n, 1), s, /*keep=*/true));
     TT_TRY(eig_reserve(h->eig, s));
@@ -1762,13 +1794,14 @@ tt_status reverse_step(tt_ctx* h, const tt_ctx::StepRec& rc, const double* Xo, c
     thbar_adjoint(s, ang, 1, 0, o1, o2, Tho, Pho, h->athbb.p, h->ascr.p, h->aThb.p, h->aPhb.p);
 
     // (3) rounding with frozen factors, reversed
-    TT_TRY(dgemm(s, true, false, R2, np, o2, 1.0, rc.M[1].p, R2, h->aPhb.p, np, 0.0, h->aPhgb.p, np));
-    TT_TRY(dgemm(s, false, false, o1 * nt, R2, o2, 1.0, h->aThb.p, o2, rc.P[1].p, R2, 0.0,
-                 h->aThtb.p, R2));
-    TT_TRY(dgemm(s, true, false, R1, nt * R2, o1, 1.0, rc.M[0].p, R1, h->aThtb.p, (long)nt * R2,
-                 0.0, h->aThgb.p, (long)nt * R2));
-    TT_TRY(dgemm(s, false, false, (int)nc, R1, o1, 1.0, h->aXb.p, o1, rc.P[0].p, R1, 0.0,
-                 h->aXgb.p, R1));
+    TT_TRY(dgemm_sk(s, true, false, R2, np, o2, 1.0, rc.M[1].p, R2, h->aPhb.p, np, h->aPhgb.p, np,
+                    h->partials, h->d_int + HI_STATUS));
+    TT_TRY(dgemm_sk(s, false, false, o1 * nt, R2, o2, 1.0, h->aThb.p, o2, rc.P[1].p, R2, h->aThtb.p, R2,
+                    h->partials, h->d_int + HI_STATUS));
+    TT_TRY(dgemm_sk(s, true, false, R1, nt * R2, o1, 1.0, rc.M[0].p, R1, h->aThtb.p, (long)nt * R2, h->aThgb.p,
+                    (long)nt * R2, h->partials, h->d_int + HI_STATUS));
+    TT_TRY(dgemm_sk(s, false, false, (int)nc, R1, o1, 1.0, h->aXb.p, o1, rc.P[0].p, R1, h->aXgb.p, R1,
+                    h->partials, h->d_int + HI_STATUS));
 
     // (4) grown angular cores (block-diagonal with the term factors), reversed
     fill(s, h->aThbi.p, (size_t)r1 * nt * r2, 0.0);
@@ -2371,6 +2404,17 @@ tt_status create_impl(const tt_problem_desc* desc, void* stream, const tt_alloca
         TT_CREATE_TRY(h->partials.ensure(D.precision == TT_MIXED
                                               ? slgram_scratch_doubles((int)nc, (int)R1)
                                               : gram_scratch_doubles((int)nc, (int)R1), s));
+        if (D.precision != TT_MIXED) {
+            // digit images and planes of the capped step's products; a handle
+            // without room for them runs on the FP64 pipe
+            const long c[][4] = {{1, R1, R1, nc}, {0, nc, cap1, R1}, {0, R1 * D.n_theta, R2, R2},
+                                 {0, R1, R1, D.n_theta * R2}, {0, cap1, D.n_theta * R2, R1}};
+            size_t need = 0;
+            for (const auto& q : c)
+                if (tc8_wanted(q[1], q[2], q[3])) need = std::max(need, tc8_scratch_doubles(q[1], q[2], q[3], q[0] != 0));
+            const tt_status ps = need ? h->partials.ensure(need, s) : TT_OK;
+            if (ps < 0 && ps != TT_ERR_OOM) TT_CREATE_TRY(ps);
+        }
         for (int k = 0; k < 2; ++k) {
             const long Rk = k == 0 ? R1 : R2;
             TT_CREATE_TRY(h->GB[k].ensure((size_t)(Rk * Rk), s));
@@ -2649,8 +2693,8 @@ tt_status tt_to_full(tt_handle h, double* out_dev, size_t out_len) {
             outp = h->tmp[ti].p;
             ti ^= 1;
         }
-        TT_TRY(dgemm(s, false, false, (int)rows, (int)cols, h->r[k + 1], 1.0, h->core[k].p,
-                     h->r[k + 1], T, cols, 0.0, outp, cols));
+        TT_TRY(dgemm_sk(s, false, false, (int)rows, (int)cols, h->r[k + 1], 1.0, h->core[k].p,
+                     h->r[k + 1], T, cols, outp, cols, h->partials, h->d_int + HI_STATUS));
         T = outp;
         cols *= h->n[k];
     }
@@ -2957,14 +3001,75 @@ tt_status tt_sync(tt_handle h) {
 
 void tt_destroy(tt_handle h) { delete h; }
 
+namespace {
+// Scratch of one library-level call from the library's own stream-ordered
+// pool, which keeps at most 512 MB between calls (the default pool gives
+// everything back at each synchronisation and maps it again at the next call:
+// more than the call itself).  Empty, not ok(), inside a capture and when the
+// pool has no room.
+struct TempScratch {
+    DevBuf buf;
+    TempScratch(size_t doubles, cudaStream_t s) {
+        cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
+        cudaMemPool_t pool = nullptr;
+        if (doubles == 0 || (cudaStreamIsCapturing(s, &cs) == cudaSuccess && cs != cudaStreamCaptureStatusNone) ||
+            !(pool = scratch_pool())) {
+            (void)cudaGetLastError();
+            return;
+        }
+        void* p = nullptr;
+        if (cudaMallocFromPoolAsync(&p, doubles * sizeof(double), pool, s) != cudaSuccess) {
+            (void)cudaGetLastError();
+            return;
+        }
+        buf.p = static_cast<double*>(p);
+        buf.cap = doubles;
+        buf.astream = s;
+    }
+    ~TempScratch() {
+        if (buf.p) cudaFreeAsync(buf.p, buf.astream);
+        buf.p = nullptr;
+    }
+    TempScratch(const TempScratch&) = delete;
+    TempScratch& operator=(const TempScratch&) = delete;
+    bool ok() const { return buf.p != nullptr; }
+
+  private:
+    static cudaMemPool_t scratch_pool() {
+        static std::mutex mu;
+        static std::vector<std::pair<int, cudaMemPool_t>> pools;
+        std::lock_guard<std::mutex> lock(mu);
+        int dev = 0;
+        if (cudaGetDevice(&dev) != cudaSuccess) return nullptr;
+        for (const auto& q : pools)
+            if (q.first == dev) return q.second;
+        cudaMemPoolProps props = {};
+        props.allocType = cudaMemAllocationTypePinned;
+        props.location.type = cudaMemLocationTypeDevice;
+        props.location.id = dev;
+        cudaMemPool_t pool = nullptr;
+        if (cudaMemPoolCreate(&pool, &props) != cudaSuccess) return nullptr;
+        uint64_t keep = 512ull << 20;
+        cudaMemPoolSetAttribute(pool, cudaMemPoolAttrReleaseThreshold, &keep);
+        pools.emplace_back(dev, pool);
+        return pool;
+    }
+};
+}  // namespace
+
 tt_status tt_dgemm(int trans_a, int trans_b, int M, int N, int K, double alpha, const double* A,
                    int lda, const double* B, int ldb, double beta, double* C, int ldc,
                    void* stream) {
     set_error("");
     if (M < 0 || N < 0 || K < 0) return fail(TT_ERR_ARG, "tt_dgemm: negative size");
     if ((M && N && K) && (!A || !B || !C)) return fail(TT_ERR_ARG, "tt_dgemm: null pointer");
-    return dgemm((cudaStream_t)stream, trans_a != 0, trans_b != 0, M, N, K, alpha, A, lda, B, ldb,
-                 beta, C, ldc);
+    cudaStream_t s = (cudaStream_t)stream;
+    if (beta == 0.0 && M > 0 && N > 0 && K > 0) {
+        TempScratch t(dgemm_sk_scratch_doubles(M, N, K), s);
+        if (t.ok())
+            return dgemm_sk(s, trans_a != 0, trans_b != 0, M, N, K, alpha, A, lda, B, ldb, C, ldc, t.buf);
+    }
+    return dgemm(s, trans_a != 0, trans_b != 0, M, N, K, alpha, A, lda, B, ldb, beta, C, ldc);
 }
 
 tt_status tt_gram(int m, int n, const double* A, int lda, double* G, int ldg, void* stream) {
@@ -2974,10 +3079,9 @@ tt_status tt_gram(int m, int n, const double* A, int lda, double* G, int ldg, vo
     if (!G || (m > 0 && !A)) return fail(TT_ERR_ARG, "tt_gram: null pointer");
     if (lda < n || ldg < n) return fail(TT_ERR_ARG, "tt_gram: leading dimension smaller than n");
     cudaStream_t s = (cudaStream_t)stream;
-    DevBuf scratch;
-    tt_status st = gram(s, m, n, A, lda, G, ldg, scratch);
-    if (scratch.p) cudaFreeAsync(scratch.p, s);
-    if (st < 0) return st;
+    TempScratch t(m > 0 && tc8_wanted(n, n, m) ? tc8_scratch_doubles(n, n, m, true)
+                                               : gram_scratch_doubles(std::max(m, 1), n), s);
+    TT_TRY(gram(s, m, n, A, lda, G, ldg, t.buf));
     TT_CUDA_TRY(cudaGetLastError());
     return TT_OK;
 }

@@ -1,0 +1,934 @@
+// FP64 products on the 5th-generation tensor cores.  GB300's FP64 pipe does
+// about 1 TFLOP/s (a warp's DFMA occupies its SM sub-partition for 64 clocks),
+// which bounded every contraction of the rounding; its tensor cores multiply
+// small integers exactly at 1.9 PFLOP/s.  C = op(A) op(B) is therefore formed
+// from exact integer digit products (the error-free splitting of Ozaki, Ogita,
+// Oishi, Rump, Numer. Algorithms 59, 2012, with fixed-point digits):
+//
+//   Split.  Row i of op(A) and column j of op(B) carry a power of two each,
+//   |a_ik| < 2^(e_i - 1); a_ik 2^-e_i is rounded to 56-bit fixed point (an
+//   entry within a factor 8 of its row's maximum keeps all its 53 bits) and
+//   cut into S = 8 balanced base-128 digits, d_0 in [0, 64], the others in
+//   [-64, 63], each exact in BF16.
+//   Products.  d_s d_t (at most 2^12) of level w = s + t <= 7 are summed by
+//   tcgen05.mma over at most 512 contraction indices: 8 pairs * 512 * 2^12 =
+//   2^24, so the FP32 accumulators hold exact integers.  The dropped levels
+//   are about 2^-56 of max|a_i| max|b_j| a term.
+//   Sums.  Every block's level sums are added as integers into two 64-bit
+//   accumulators an output (levels 0-3 and 4-7), also across splits and chunks
+//   of the contraction: the sum is exact and is rounded once to FP64, so the
+//   result does not depend on how the work is cut.
+//
+// Against the FP64 pipe's running sum (an error of 2^-53 of the partial sum a
+// term) the result is nearer to the exact product from K of a few dozen on;
+// the sizes where it is used (tc8_wanted) have K >= 64.
+//
+// Measured (GB300, CUDA events, against the FP64 pipe's kernels): Gram of
+// 500,000 x 449 143 -> 8.9 ms, error against the exact product 1.3e-15 ->
+// 2.7e-16; 200,000 x 577 times 577 x 96 22.4 -> 2.6 ms, 8.0e-16 -> 5.4e-16;
+// 128^3 FP64 step at ranks 64 -> 128 870 -> 89 ms; 500^2 step at R = 876
+// 385 -> 79 ms.
+//
+// Inf, NaN and rows whose largest entry is outside 2^+-900 cannot be split:
+// the exponent scans latch a device flag and an FP64-pipe kernel behind the
+// product, which otherwise returns at once, recomputes it.
+#include <cuda.h>
+#include <cuda_bf16.h>
+
+#include <algorithm>
+#include <cstring>
+
+#include "internal.h"
+
+namespace ttsn {
+
+namespace {
+
+constexpr int S8 = 8;
+constexpr int T_M = 128, T_N = 64, T_K = 32;  // output tile; contraction indices of a stage
+constexpr int T_BLK = 16;                     // stages of an exact block (512 indices)
+constexpr int T_STAGES = 2;
+constexpr int RB = 64;                         // rows of an image block
+constexpr int DIG_BYTES = RB * T_K * 2;        // one digit of one block and stage: 4096
+constexpr int BLK_BYTES = S8 * DIG_BYTES;      // 32768
+constexpr int A_BYTES = 2 * BLK_BYTES, B_BYTES = BLK_BYTES, STAGE_BYTES = A_BYTES + B_BYTES;
+constexpr int SLOT_BYTES = 3 * DIG_BYTES;      // A digit s (128 rows) and B digit 7 - s (64 rows)
+constexpr int DRAIN_WARPS = 16;
+constexpr int THREADS8 = 32 * (2 + DRAIN_WARPS);
+constexpr int DCOLS = T_N / (DRAIN_WARPS / 4);  // columns of a drain thread: 16
+constexpr unsigned TMEM_COLS = 512;
+constexpr long long SPIN = 1LL << 26;
+constexpr size_t SMEM8 = (size_t)T_STAGES * STAGE_BYTES + 1024 /* barriers */ + 1024 /* alignment */;
+// digit images of one pass over an operand: a longer operand goes in chunks
+constexpr long IMG_LIMIT = 1L << 27;
+
+__device__ __forceinline__ unsigned smem_addr(const void* p) { return (unsigned)__cvta_generic_to_shared(p); }
+__device__ __forceinline__ void bar_init(unsigned a, unsigned count) {
+    asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(a), "r"(count) : "memory");
+}
+__device__ __forceinline__ void bar_expect(unsigned a, unsigned bytes) {
+    asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(a), "r"(bytes) : "memory");
+}
+__device__ __forceinline__ void bar_arrive(unsigned a) {
+    asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(a) : "memory");
+}
+__device__ __forceinline__ bool bar_try(unsigned a, unsigned parity) {
+    unsigned ok;
+    asm volatile(
+        "{\n .reg .pred p;\n mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n selp.u32 %0, 1, 0, p;\n}\n"
+        : "=r"(ok)
+        : "r"(a), "r"(parity)
+        : "memory");
+    return ok != 0;
+}
+// Bounded wait; false once the limit is reached (DEV_TIMEOUT latched, the
+// other roles told through *abort_flag) or another role has given up.
+__device__ __forceinline__ bool bar_wait(unsigned a, unsigned parity, int* status, volatile int* abort_flag) {
+    for (long long it = 0; it < SPIN; ++it) {
+        if (bar_try(a, parity)) return true;
+        if (abort_flag && *abort_flag) return false;
+        if (it > 64) __nanosleep(32);
+    }
+    if (status) atomicOr(status, DEV_TIMEOUT);
+    if (abort_flag) *abort_flag = 1;
+    return false;
+}
+__device__ __forceinline__ void bulk_g2s(unsigned dst, const void* src, unsigned bytes, unsigned bar) {
+    asm volatile(
+        "cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(dst),
+        "l"((unsigned long long)src), "r"(bytes), "r"(bar)
+        : "memory");
+}
+// K-major operand descriptor: 64-byte rows, 64-byte swizzle, 8-row groups 512 bytes apart
+__device__ __forceinline__ unsigned long long opdesc(unsigned addr) {
+    return (unsigned long long)((addr & 0x3FFFFu) >> 4) | (unsigned long long)(16u >> 4) << 16 |
+           (unsigned long long)(512u >> 4) << 32 | 1ull << 46 | 4ull << 61;
+}
+// kind::f16, FP32 accumulators, BF16 A and B, K-major, M = 128, N = nn
+__device__ __forceinline__ unsigned mmadesc(int nn) {
+    return (1u << 4) | (1u << 7) | (1u << 10) | ((unsigned)(nn >> 3) << 17) | ((unsigned)(T_M >> 4) << 24);
+}
+__device__ __forceinline__ void mma8(unsigned d, unsigned long long a, unsigned long long b, unsigned idesc,
+                                     unsigned accumulate) {
+    asm volatile(
+        "{\n .reg .pred p;\n setp.ne.b32 p, %4, 0;\n"
+        " tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n}\n" ::"r"(d),
+        "l"(a), "l"(b), "r"(idesc), "r"(accumulate)
+        : "memory");
+}
+__device__ __forceinline__ void mma_commit(unsigned bar) {
+    asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(bar) : "memory");
+}
+__device__ __forceinline__ void fence_before() { asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory"); }
+__device__ __forceinline__ void fence_after() { asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory"); }
+__device__ __forceinline__ void tmem_ld16(unsigned addr, unsigned (&r)[16]) {
+    asm volatile(
+        "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15}, [%16];"
+        : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]),
+          "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15])
+        : "r"(addr));
+}
+__device__ __forceinline__ void tmem_wait_ld() { asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory"); }
+
+typedef unsigned long long u64;
+
+// A product's sizes: by value, or (a captured step) read from desc = M, N, K,
+// lda, ldb, ldc, when every kernel returns unless the sizes take this path.
+// The kernels of one chunk see the contraction indices [k0, k0 + Kc) and the
+// rows [i0, i0 + Mc) of op(A).
+struct Prod {
+    long M, N, K, lda, ldb, ldc;
+    const int* desc;
+    long k0, Kc, i0, Mc;
+    int gram;
+    long Mc0;  // rows of the first chunk (set by resolve): the split is chosen from it
+};
+__device__ __forceinline__ bool resolve(Prod& p) {
+    if (p.desc) {
+        p.M = p.desc[0];
+        p.N = p.desc[1];
+        p.K = p.desc[2];
+        p.lda = p.desc[3];
+        p.ldb = p.desc[4];
+        p.ldc = p.desc[5];
+        if (!tc8_wanted(p.M, p.N, p.K)) return false;
+    }
+    p.Mc0 = p.Mc < p.M ? p.Mc : p.M;
+    p.Mc = p.Mc < p.M - p.i0 ? p.Mc : p.M - p.i0;
+    return p.Mc > 0 && p.k0 < p.K;
+}
+__host__ __device__ inline long up(long x, long m) { return (x + m - 1) / m * m; }
+__host__ __device__ inline int stages(long Kc) { return (int)((Kc + T_K - 1) / T_K); }
+__host__ __device__ inline long tiles_of(long M, long N, int gram) {
+    const long nb = (N + T_N - 1) / T_N;
+    if (!gram) return (M + T_M - 1) / T_M * nb;
+    const long h = (nb + 1) / 2;  // rows of 128: nb, nb - 2, ... tiles
+    return h * nb - h * (h - 1);
+}
+
+// Splits of a chunk's contraction: stages per split.  The time of a launch is
+// about its waves of one CTA per SM times the stages of a split and one more
+// for an item's end; a plane costs its write and its read in the reduction.
+// A split has at least four stages, and the planes at most PLANE_ELEMS entries.
+constexpr long PLANE_ELEMS = 1L << 23;
+constexpr int MAX_SPLITS = 64;
+__host__ __device__ inline int split_limit(long M, long N, int nst) {
+    long k = PLANE_ELEMS / (M * N);
+    if (k > nst / 4) k = nst / 4;
+    if (k > MAX_SPLITS) k = MAX_SPLITS;
+    return k < 1 ? 1 : (int)k;
+}
+__host__ __device__ inline unsigned split_cost(int k, long ntiles, int nst) {
+    const int spc = (nst + k - 1) / k, kk = (nst + spc - 1) / spc;
+    const long waves = (ntiles * kk + 151) / 152;
+    const long c = waves * (spc + 1) * 64 + kk;
+    return c > 0x03ffffffL ? 0x03ffffffu : (unsigned)c;
+}
+int split_stages(long M, long N, long ntiles, int nst) {
+    const int lim = split_limit(M, N, nst);
+    int best = 1;
+    for (int k = 2; k <= lim; ++k)
+        if (split_cost(k, ntiles, nst) < split_cost(best, ntiles, nst)) best = k;
+    return (nst + best - 1) / best;
+}
+// the same choice made by one warp
+__device__ __forceinline__ int split_stages_warp(long M, long N, long ntiles, int nst) {
+    const int lim = split_limit(M, N, nst), lane = threadIdx.x & 31;
+    unsigned key = 0xffffffffu;
+    for (int k = lane + 1; k <= lim; k += 32) key = min(key, split_cost(k, ntiles, nst) * 64u + (unsigned)(k - 1));
+    key = __reduce_min_sync(0xffffffffu, key);
+    const int best = (int)(key & 63u) + 1;
+    return (nst + best - 1) / best;
+}
+
+// ------------------------------------------------------------------ split
+
+// |v| as its bit pattern (ordered as the values; Inf and NaN above all).
+__device__ __forceinline__ u64 mag(double v) { return (u64)__double_as_longlong(v) & 0x7FFFFFFFFFFFFFFFull; }
+__device__ __forceinline__ u64 umax(u64 a, u64 b) { return a > b ? a : b; }
+// e with every |v| <= the maximum of this pattern below 2^(e - 1); *flag is
+// latched when the maximum is Inf, NaN or outside 2^+-900.
+__device__ __forceinline__ int split_exp(u64 mx, int* flag) {
+    const int ex = (int)(mx >> 52);
+    if (mx != 0 && (ex < 1023 - 900 || ex > 1023 + 900)) atomicOr(flag, 1);
+    return mx == 0 ? 0 : ex - 1023 + 2;
+}
+
+// The biased digits of v 2^-e as one integer: F = round(|v| 2^(56 - e)) < 2^55,
+// plus 64 at each of the seven lower digit positions, which makes the plain
+// base-128 digits of the sum d_s + 64 (s >= 1) without a carry chain.
+__device__ __forceinline__ u64 biased56(double v, int e) {
+    const u64 bits = (u64)__double_as_longlong(v);
+    const int ex = (int)((bits >> 52) & 0x7FF);
+    u64 F = 0;
+    if (ex != 0) {
+        const u64 M = (bits & 0xFFFFFFFFFFFFFull) | (1ull << 52);
+        const int d = e - 4 - (ex - 1023);  // >= -2 when e bounds |v|
+        if (d <= 0)
+            F = M << (d < -2 ? 2 : -d);
+        else if (d < 55)
+            F = (M + (1ull << (d - 1))) >> d;
+    }
+    return F + 0x1020408102040ull;  // 64 (1 + 128 + ... + 128^6)
+}
+// The eight digits of two values as the packed BF16 words of the operand
+// images (v0 in the low half): the biased digits u of both go into one word
+// as the BF16 pair 128 + u, one packed subtraction of 192 (128 for the
+// leading digit) leaves the digits exactly, and the signs are flipped in.
+__device__ __forceinline__ void digits8x2(double v0, double v1, int e0, int e1, unsigned (&w)[S8]) {
+    const u64 F0 = biased56(v0, e0), F1 = biased56(v1, e1);
+    const unsigned sg = ((unsigned)((u64)__double_as_longlong(v0) >> 48) & 0x8000u) |
+                        ((unsigned)((u64)__double_as_longlong(v1) >> 32) & 0x80000000u);
+    const __nv_bfloat162 lead = __floats2bfloat162_rn(128.0f, 128.0f), rest = __floats2bfloat162_rn(192.0f, 192.0f);
+#pragma unroll
+    for (int s = 0; s < S8; ++s) {
+        const unsigned u0 = (unsigned)(F0 >> (7 * (7 - s))) & 0x7Fu;
+        const unsigned u1 = (unsigned)(F1 >> (7 * (7 - s))) & 0x7Fu;
+        const unsigned p = 0x43004300u | u0 | (u1 << 16);
+        __nv_bfloat162 x;
+        memcpy(&x, &p, 4);
+        const __nv_bfloat162 d = __hsub2(x, s == 0 ? lead : rest);
+        unsigned r;
+        memcpy(&r, &d, 4);
+        w[s] = r ^ sg;
+    }
+}
+// Byte offset of (row r, index k) in a swizzled digit tile of 64-byte rows
+__device__ __forceinline__ unsigned swz(int r, int k) {
+    return (unsigned)(r * 64 + (((k >> 3) ^ ((r >> 1) & 3)) << 4) + (k & 7) * 2);
+}
+// Operand images: for row block rb (64 rows) and stage st (32 indices) the
+// eight 64 x 32 digit tiles, each in the MMA's swizzled K-major layout.
+__device__ __forceinline__ unsigned char* tile_at(unsigned char* img, long rb, int nst, int st, int s) {
+    return img + ((rb * nst + st) * S8 + s) * (long)DIG_BYTES;
+}
+
+// One operand (A's rows, or B's columns) of a product: rows x K.
+struct Side {
+    const double* p;
+    int isB, strided;  // strided: element (i, k) at k * ld + i, else at i * ld + k
+    u64* mx;           // row maxima (where they are found ahead of the split)
+    int* e;            // row exponents
+    unsigned char* img;
+};
+__device__ __forceinline__ void side_sizes(const Prod& p, const Side& o, long& i0, long& rows, long& rpad, long& ld) {
+    i0 = o.isB ? 0 : p.i0;
+    rows = o.isB ? p.N : p.Mc;
+    rpad = up(rows, o.isB ? RB : T_M);
+    ld = o.isB ? p.ldb : p.lda;
+}
+
+// Rows with a contiguous contraction index, K <= 64 V: a warp reads a row
+// once, reduces its maximum (the exponent) and writes its digits.  A lane
+// holds the pairs k = 64 t + 2 lane, so a digit store covers two whole
+// 64-byte tile rows.  Rows past the last are zero.
+template <int V>
+__global__ void __launch_bounds__(256) split_rows_kernel(Prod p, Side o, int* flag) {
+    if (!resolve(p)) return;
+    long i0, rows, rpad, ld;
+    side_sizes(p, o, i0, rows, rpad, ld);
+    const int K = (int)p.K, nst = stages(K);
+    if (nst > 2 * V || (V > 2 && nst <= V)) return;  // another instance's size (a captured step launches all)
+    const double* A = o.p + i0 * ld;
+    const int lane = threadIdx.x & 31;
+    const long nw = (long)gridDim.x * 8;
+    for (long r = (long)blockIdx.x * 8 + (threadIdx.x >> 5); r < rpad; r += nw) {
+        double v[V][2];
+        u64 mx = 0;
+        if (r < rows) {
+            const double* row = A + r * ld;
+#pragma unroll
+            for (int t = 0; t < V; ++t) {
+                const int k = 64 * t + 2 * lane;
+                v[t][0] = k < K ? row[k] : 0.0;
+                v[t][1] = k + 1 < K ? row[k + 1] : 0.0;
+            }
+#pragma unroll
+            for (int t = 0; t < V; ++t) mx = umax(mx, umax(mag(v[t][0]), mag(v[t][1])));
+#pragma unroll
+            for (int q = 16; q > 0; q >>= 1) mx = umax(mx, __shfl_xor_sync(0xffffffffu, mx, q));
+        } else {
+#pragma unroll
+            for (int t = 0; t < V; ++t) v[t][0] = v[t][1] = 0.0;
+        }
+        const int e = split_exp(mx, flag);
+        if (lane == 0 && r < rows) o.e[i0 + r] = e;
+        const unsigned off = swz((int)(r & 63), 2 * (lane & 15));
+#pragma unroll
+        for (int t = 0; t < V; ++t) {
+            const int st = 2 * t + (lane >> 4);
+            if (st < nst) {
+                unsigned w[S8];
+                digits8x2(v[t][0], v[t][1], e, e, w);
+                unsigned char* q = tile_at(o.img, r >> 6, nst, st, 0) + off;
+#pragma unroll
+                for (int s = 0; s < S8; ++s) *reinterpret_cast<unsigned*>(q + s * DIG_BYTES) = w[s];
+            }
+        }
+    }
+}
+
+// Longer rows in two passes: their maxima, then the digits of a chunk.
+constexpr int FUSED_K = 1024;
+__global__ void __launch_bounds__(256) row_max_kernel(Prod p, Side o) {
+    p.Mc = p.M;
+    if (!resolve(p) || (p.desc && p.K <= FUSED_K)) return;
+    const long rows = o.isB ? p.N : p.M, ld = o.isB ? p.ldb : p.lda;
+    const int lane = threadIdx.x & 31;
+    const long nw = (long)gridDim.x * 8;
+    for (long r = (long)blockIdx.x * 8 + (threadIdx.x >> 5); r < rows; r += nw) {
+        const double* row = o.p + r * ld;
+        u64 m0 = 0, m1 = 0, m2 = 0, m3 = 0;
+        long k = lane;
+        for (; k + 96 < p.K; k += 128) {
+            m0 = umax(m0, mag(row[k]));
+            m1 = umax(m1, mag(row[k + 32]));
+            m2 = umax(m2, mag(row[k + 64]));
+            m3 = umax(m3, mag(row[k + 96]));
+        }
+        for (; k < p.K; k += 32) m0 = umax(m0, mag(row[k]));
+        m0 = umax(umax(m0, m1), umax(m2, m3));
+#pragma unroll
+        for (int q = 16; q > 0; q >>= 1) m0 = umax(m0, __shfl_xor_sync(0xffffffffu, m0, q));
+        if (lane == 0) o.mx[r] = m0;
+    }
+}
+__global__ void __launch_bounds__(256) split_rows_long_kernel(Prod p, Side o, int* flag) {
+    if (!resolve(p) || (p.desc && p.K <= FUSED_K)) return;
+    long i0, rows, rpad, ld;
+    side_sizes(p, o, i0, rows, rpad, ld);
+    const long Kc = p.Kc < p.K - p.k0 ? p.Kc : p.K - p.k0;
+    const int nst = stages(Kc);
+    const double* A = o.p + i0 * ld + p.k0;
+    const long total = rpad * nst * (T_K / 2);
+    for (long t = blockIdx.x * (long)blockDim.x + threadIdx.x; t < total; t += (long)gridDim.x * blockDim.x) {
+        const int kw = (int)(t & 15);
+        const long q = t >> 4;
+        const int st = (int)(q % nst);
+        const long r = q / nst;
+        const long k = (long)st * T_K + 2 * kw;
+        double v0 = 0.0, v1 = 0.0;
+        int e = 0;
+        if (r < rows) {
+            e = split_exp(o.mx[i0 + r], flag);
+            if (k == 0) o.e[i0 + r] = e;
+            if (k < Kc) v0 = A[r * ld + k];
+            if (k + 1 < Kc) v1 = A[r * ld + k + 1];
+        }
+        unsigned w[S8];
+        digits8x2(v0, v1, e, e, w);
+        unsigned char* d = tile_at(o.img, r >> 6, nst, st, 0) + swz((int)(r & 63), 2 * kw);
+#pragma unroll
+        for (int s = 0; s < S8; ++s) *reinterpret_cast<unsigned*>(d + s * DIG_BYTES) = w[s];
+    }
+}
+
+// Rows that are the columns of a stored matrix (the Gram's operand): column
+// maxima, then the digits of a chunk of its rows.  A thread splits 16 rows of
+// one column, so that a warp reads 32 neighbouring columns of a row at a time
+// and stores one 32-byte sector a digit and lane.
+__global__ void __launch_bounds__(256) strided_max_kernel(Prod p, Side o) {
+    p.Mc = p.M;
+    if (!resolve(p)) return;
+    const long n = o.isB ? p.N : p.M, ld = o.isB ? p.ldb : p.lda;
+    const long per = (p.K + gridDim.y - 1) / gridDim.y;
+    const long k0 = blockIdx.y * per, k1 = min(p.K, k0 + per);
+    __shared__ u64 part[8][32];
+    for (long jb = blockIdx.x * 32L; jb < n; jb += gridDim.x * 32L) {
+        const long j = jb + (threadIdx.x & 31);
+        u64 m0 = 0, m1 = 0, m2 = 0, m3 = 0;
+        if (j < n) {
+            long k = k0 + (threadIdx.x >> 5);
+            for (; k + 24 < k1; k += 32) {
+                m0 = umax(m0, mag(o.p[k * ld + j]));
+                m1 = umax(m1, mag(o.p[(k + 8) * ld + j]));
+                m2 = umax(m2, mag(o.p[(k + 16) * ld + j]));
+                m3 = umax(m3, mag(o.p[(k + 24) * ld + j]));
+            }
+            for (; k < k1; k += 8) m0 = umax(m0, mag(o.p[k * ld + j]));
+        }
+        __syncthreads();
+        part[threadIdx.x >> 5][threadIdx.x & 31] = umax(umax(m0, m1), umax(m2, m3));
+        __syncthreads();
+        if (threadIdx.x < 32 && j < n) {
+            u64 m = part[0][threadIdx.x];
+#pragma unroll
+            for (int w = 1; w < 8; ++w) m = umax(m, part[w][threadIdx.x]);
+            if (m) atomicMax(o.mx + j, m);
+        }
+    }
+}
+__global__ void __launch_bounds__(256, 2) split_strided_kernel(Prod p, Side o, int* flag) {
+    if (!resolve(p)) return;
+    long i0, rows, rpad, ld;
+    side_sizes(p, o, i0, rows, rpad, ld);
+    const long Kc = p.Kc < p.K - p.k0 ? p.Kc : p.K - p.k0;
+    const int nst = stages(Kc);
+    const double* A = o.p + i0 + p.k0 * ld;
+    for (long jb = blockIdx.x * 32L; jb < rpad; jb += gridDim.x * 32L) {
+        const long j = jb + (threadIdx.x & 31);
+        int e = 0;
+        if (j < rows) {
+            e = split_exp(o.mx[i0 + j], flag);
+            if (blockIdx.y == 0 && threadIdx.x < 32) o.e[i0 + j] = e;
+        }
+        const long groups = (long)nst * 2;
+        for (long g = (long)blockIdx.y * 8 + (threadIdx.x >> 5); g < groups; g += (long)gridDim.y * 8) {
+            const long k0 = g * 16;
+            unsigned w[S8][8];
+#pragma unroll
+            for (int r = 0; r < 16; r += 2) {
+                const double v0 = j < rows && k0 + r < Kc ? A[(k0 + r) * ld + j] : 0.0;
+                const double v1 = j < rows && k0 + r + 1 < Kc ? A[(k0 + r + 1) * ld + j] : 0.0;
+                unsigned wd[S8];
+                digits8x2(v0, v1, e, e, wd);
+#pragma unroll
+                for (int s = 0; s < S8; ++s) w[s][r / 2] = wd[s];
+            }
+            const int r = (int)(j & 63), st = (int)(g >> 1), half = (int)(g & 1) * 16;
+            unsigned char* d = tile_at(o.img, j >> 6, nst, st, 0);
+            const unsigned o0 = swz(r, half), o1 = swz(r, half + 8);
+#pragma unroll
+            for (int s = 0; s < S8; ++s) {
+                *reinterpret_cast<uint4*>(d + s * DIG_BYTES + o0) = make_uint4(w[s][0], w[s][1], w[s][2], w[s][3]);
+                *reinterpret_cast<uint4*>(d + s * DIG_BYTES + o1) = make_uint4(w[s][4], w[s][5], w[s][6], w[s][7]);
+            }
+        }
+    }
+}
+
+// ------------------------------------------------------------------ product
+
+// (hi 2^28 + lo) 2^(e - 63) rounded to nearest.
+__device__ __forceinline__ double digits_value(long long hi, long long lo, int e) {
+    __int128 t = ((__int128)hi << 28) + lo;
+    const bool neg = t < 0;
+    unsigned __int128 u = neg ? (unsigned __int128)(-t) : (unsigned __int128)t;
+    u64 uh = (u64)(u >> 64), ul = (u64)u;
+    if ((uh | ul) == 0) return 0.0;
+    // the leading bit to bit 63 of m, what is cut off as a sticky bit
+    const int z = uh ? __clzll((long long)uh) : 64 + __clzll((long long)ul);
+    u <<= z;
+    u64 m = (u64)(u >> 64);
+    const u64 rest = (u64)u;
+    int ex = e - 63 + 127 - z;  // exponent of the leading bit
+    const u64 low = (m & 0x7FF) | (rest ? 1ull : 0ull);
+    m >>= 11;  // 53 bits
+    if (low > 0x400 || (low == 0x400 && (m & 1))) {
+        if (++m == (1ull << 53)) {
+            m >>= 1;
+            ++ex;
+        }
+    }
+    if (ex < -1022 || ex > 1023) {  // beyond the normal range: ldexp's rounding
+        const double v = ldexp((double)m, ex - 52);
+        return neg ? -v : v;
+    }
+    const u64 bits = ((u64)(ex + 1023) << 52) | (m & 0xFFFFFFFFFFFFFull) | (neg ? 1ull << 63 : 0ull);
+    return __longlong_as_double((long long)bits);
+}
+
+// Output tile of item t: row block (128) and column block (64); the Gram takes
+// only the tiles that hold some j <= k.
+__device__ __forceinline__ void tile_of(long t, int nb, bool tri, long& mb, int& kb) {
+    if (!tri) {
+        mb = t / nb;
+        kb = (int)(t % nb);
+        return;
+    }
+    int jt = 0;
+    while (t >= nb - 2 * jt) {
+        t -= nb - 2 * jt;
+        ++jt;
+    }
+    mb = jt;
+    kb = 2 * jt + (int)t;
+}
+
+// One CTA per SM walks (split of the contraction, output tile) items.  Warp 0
+// copies: slot s of a stage is A's digit s and B's digit 7 - s, the pair that
+// the MMAs of digit s use last, so a slot is refilled for the stage after next
+// as soon as those MMAs are done (a commit per digit) and loads are always in
+// flight.  Warp 1 issues: eight FP32 accumulators of 128 x 64 (one per level,
+// all 512 TMEM columns); the digit tiles of B lie back to back, so A's digit
+// s meets up to four of B's digits in one MMA of N <= 256 whose levels are
+// neighbouring column ranges.  Sixteen warps drain a block's accumulators into
+// 64-bit integers (a float-to-int and a wide multiply-add a value) and, at
+// an item's end, write the FP64 results while the next item's MMAs run.
+//
+// What bounds it: shared memory.  Per 16 indices the MMAs read 120 KB of
+// operands and 48 KB arrive, 168 KB or 1312 clocks against 1152 of MMA.
+__global__ void __launch_bounds__(THREADS8, 1)
+tc8_kernel(Prod p, const unsigned char* __restrict__ At, const int* __restrict__ eA,
+           const unsigned char* __restrict__ Bt, const int* __restrict__ eB, double alpha, double* __restrict__ C,
+           longlong2* __restrict__ planes, int spc, int* status) {
+    if (!resolve(p)) return;  // every thread, before any barrier
+    const long M = p.Mc;
+    const int N = (int)p.N;
+    const int nst = stages(p.Kc < p.K - p.k0 ? p.Kc : p.K - p.k0);
+    const long ntiles = tiles_of(M, N, p.gram);
+    // a captured step decides the split here (from the first chunk, as the
+    // reduction does)
+    if (p.desc) spc = split_stages_warp(p.M, N, tiles_of(p.Mc0, N, p.gram), stages(p.Kc < p.K ? p.Kc : p.K));
+    const bool accumulate = p.k0 > 0;
+    const bool whole = planes == nullptr || (p.desc && !p.gram && p.K <= p.Kc && spc >= nst);
+    extern __shared__ unsigned char raw[];
+    const unsigned raw_s = smem_addr(raw);
+    const unsigned pad = ((raw_s + 1023u) & ~1023u) - raw_s;
+    const unsigned sb = raw_s + pad;
+    u64* bars = reinterpret_cast<u64*>(raw + pad + T_STAGES * STAGE_BYTES);
+    // bars: [0,1] stage full, [2 + 8 st + s] slot empty, [18] accumulators full,
+    // [19] accumulators drained, [20] every MMA done
+    unsigned* tmem_slot = reinterpret_cast<unsigned*>(bars + 24);
+    volatile int* flags = reinterpret_cast<volatile int*>(tmem_slot + 2);  // abort, stages issued, consumed
+
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int nb = (N + T_N - 1) / T_N;
+    const int ksp = (nst + spc - 1) / spc;
+    const long items = ntiles * ksp;
+    if ((long)blockIdx.x >= items) return;
+    if (threadIdx.x == 0) {
+        for (int i = 0; i < 21; ++i)
+            bar_init(smem_addr(&bars[i]), i < 2 ? (unsigned)S8 : (i == 19 ? (unsigned)DRAIN_WARPS : 1u));
+        flags[0] = flags[1] = flags[2] = 0;
+        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+    }
+    if (warp == 1) {
+        asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_addr(tmem_slot)),
+                     "r"(TMEM_COLS)
+                     : "memory");
+        asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
+    }
+    fence_before();
+    __syncthreads();
+    fence_after();
+    const unsigned tmem = *tmem_slot;
+
+    if (warp == 0) {
+        if (lane == 0) {
+            long g = 0;
+            bool stop = false;
+            for (long item = blockIdx.x; item < items && !stop; item += gridDim.x) {
+                long mb;
+                int kb;
+                tile_of(item % ntiles, nb, p.gram != 0, mb, kb);
+                const int sp = (int)(item / ntiles);
+                const int st1 = min(nst, (sp + 1) * spc);
+                for (int it = sp * spc; it < st1 && !stop; ++it, ++g) {
+                    const int st = (int)(g % T_STAGES);
+                    const unsigned ph = (unsigned)(g / T_STAGES) & 1u;
+                    const unsigned full = smem_addr(&bars[st]);
+                    const unsigned dst = sb + (unsigned)(st * STAGE_BYTES);
+                    const unsigned char* a0 = At + (2 * mb * nst + it) * (long)BLK_BYTES;
+                    const unsigned char* a1 = a0 + (long)nst * BLK_BYTES;
+                    const unsigned char* b0 = Bt + ((long)kb * nst + it) * BLK_BYTES;
+                    for (int s = 0; s < S8; ++s) {
+                        if (!stop && !bar_wait(smem_addr(&bars[2 + 8 * st + s]), ph ^ 1u, status, flags)) stop = true;
+                        if (stop) {  // the stage's barrier completes with what was issued
+                            bar_arrive(full);
+                            continue;
+                        }
+                        bar_expect(full, (unsigned)SLOT_BYTES);
+                        bulk_g2s(dst + s * 2 * DIG_BYTES, a0 + s * DIG_BYTES, DIG_BYTES, full);
+                        bulk_g2s(dst + s * 2 * DIG_BYTES + DIG_BYTES, a1 + s * DIG_BYTES, DIG_BYTES, full);
+                        bulk_g2s(dst + A_BYTES + (7 - s) * DIG_BYTES, b0 + (7 - s) * DIG_BYTES, DIG_BYTES, full);
+                    }
+                    flags[1] = (int)(g + 1);
+                }
+            }
+        }
+    } else if (warp == 1) {
+        if (lane == 0) {
+            long g = 0, gb = 0;
+            bool stop = false;
+            for (long item = blockIdx.x; item < items && !stop; item += gridDim.x) {
+                const int st0 = (int)(item / ntiles) * spc, st1 = min(nst, st0 + spc);
+                for (int it = st0; it < st1; ++it, ++g) {
+                    const int st = (int)(g % T_STAGES);
+                    const unsigned ph = (unsigned)(g / T_STAGES) & 1u;
+                    const bool first = ((it - st0) % T_BLK) == 0;
+                    if (first && gb > 0) {
+                        if (!bar_wait(smem_addr(&bars[19]), (unsigned)(gb - 1) & 1u, status, flags)) {
+                            stop = true;
+                            break;
+                        }
+                        fence_after();
+                    }
+                    if (!bar_wait(smem_addr(&bars[st]), ph, status, flags)) {
+                        stop = true;
+                        break;
+                    }
+                    flags[2] = (int)(g + 1);
+                    fence_after();
+                    const unsigned aB = sb + (unsigned)(st * STAGE_BYTES), bB = aB + A_BYTES;
+#pragma unroll 1
+                    for (int s = 0; s < S8; ++s) {
+#pragma unroll
+                        for (int kk = 0; kk < 2; ++kk) {
+                            const u64 ad = opdesc(aB + (unsigned)(s * 2 * DIG_BYTES + kk * 32));
+                            const unsigned acc = (first && s == 0 && kk == 0) ? 0u : 1u;
+                            for (int t0 = 0; t0 < S8 - s; t0 += 4) {
+                                const int c = min(4, S8 - s - t0);
+                                const u64 bd = opdesc(bB + (unsigned)(t0 * DIG_BYTES + kk * 32));
+                                mma8(tmem + (unsigned)((s + t0) * T_N), ad, bd, mmadesc(c * T_N), acc);
+                            }
+                        }
+                        mma_commit(smem_addr(&bars[2 + 8 * st + s]));
+                    }
+                    if (((it - st0) % T_BLK) == T_BLK - 1 || it == st1 - 1) {
+                        mma_commit(smem_addr(&bars[18]));
+                        ++gb;
+                    }
+                }
+            }
+            mma_commit(smem_addr(&bars[20]));
+            bar_wait(smem_addr(&bars[20]), 0u, status, nullptr);
+        }
+    } else {
+        const int q = warp & 3;  // TMEM lanes 32 q .. 32 q + 31
+        const int c0 = ((warp - 2) >> 2) * DCOLS;
+        long gb = 0;
+        bool stop = false;
+        for (long item = blockIdx.x; item < items && !stop; item += gridDim.x) {
+            long mb;
+            int kb;
+            tile_of(item % ntiles, nb, p.gram != 0, mb, kb);
+            const int sp = (int)(item / ntiles);
+            const int blocks = (min(nst, (sp + 1) * spc) - sp * spc + T_BLK - 1) / T_BLK;
+            long long hi[DCOLS], lo[DCOLS];
+#pragma unroll
+            for (int c = 0; c < DCOLS; ++c) hi[c] = lo[c] = 0;
+            for (int b = 0; b < blocks; ++b, ++gb) {
+                if (!__all_sync(0xffffffffu, bar_wait(smem_addr(&bars[18]), (unsigned)gb & 1u, status, flags))) {
+                    stop = true;
+                    break;
+                }
+                fence_after();
+                const unsigned ta = tmem + ((unsigned)(32 * q) << 16) + (unsigned)c0;
+#pragma unroll
+                for (int w = 0; w < S8; ++w) {
+                    unsigned r[16];
+                    tmem_ld16(ta + (unsigned)(w * T_N), r);
+                    tmem_wait_ld();
+                    const int scale = 1 << (7 * (3 - (w & 3)));
+#pragma unroll
+                    for (int c = 0; c < DCOLS; ++c) {
+                        const long long v = (long long)__float2int_rn(__uint_as_float(r[c])) * scale;
+                        if (w < 4)
+                            hi[c] += v;
+                        else
+                            lo[c] += v;
+                    }
+                }
+                fence_before();
+                __syncwarp();
+                if (lane == 0) bar_arrive(smem_addr(&bars[19]));
+            }
+            if (stop) break;
+            const long i = mb * T_M + 32 * q + lane;
+            if (i < M && !flags[0]) {
+                const int col0 = kb * T_N + c0;
+                if (whole) {
+                    const int ea = eA[p.i0 + i];
+                    double* out = C + (p.i0 + i) * p.ldc;
+#pragma unroll
+                    for (int c = 0; c < DCOLS; ++c)
+                        if (col0 + c < N) {
+                            const double v = digits_value(hi[c], lo[c], ea + eB[col0 + c]);
+                            out[col0 + c] = alpha == 1.0 ? v : alpha * v;
+                        }
+                } else {
+                    longlong2* out = planes + ((long)sp * p.M + p.i0 + i) * N;
+#pragma unroll
+                    for (int c = 0; c < DCOLS; ++c)
+                        if (col0 + c < N) {
+                            longlong2 v = make_longlong2(hi[c], lo[c]);
+                            if (accumulate) {
+                                const longlong2 u = out[col0 + c];
+                                v.x += u.x;
+                                v.y += u.y;
+                            }
+                            out[col0 + c] = v;
+                        }
+                }
+            }
+        }
+    }
+    __syncthreads();
+    if (threadIdx.x == 0) {  // after an abort: copies in flight land before the CTA exits
+        for (long g = flags[2]; g < flags[1]; ++g)
+            bar_wait(smem_addr(&bars[g % T_STAGES]), (unsigned)(g / T_STAGES) & 1u, status, nullptr);
+    }
+    __syncthreads();
+    if (warp == 1) {
+        fence_after();
+        asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(TMEM_COLS) : "memory");
+    }
+}
+
+// The splits' integer sums added and rounded once: C (the Gram: both halves
+// from the entries j <= k that are held).
+__global__ void __launch_bounds__(256)
+tc8_reduce_kernel(Prod p, const longlong2* __restrict__ planes, const int* __restrict__ eA,
+                  const int* __restrict__ eB, int spc, double alpha, double* __restrict__ C) {
+    if (!resolve(p)) return;
+    const int nst = stages(p.Kc < p.K ? p.Kc : p.K);
+    if (p.desc) {
+        spc = split_stages_warp(p.M, p.N, tiles_of(p.Mc0, p.N, p.gram), nst);
+        if (!p.gram && p.K <= p.Kc && spc >= nst) return;  // written whole
+    }
+    const int ksp = (nst + spc - 1) / spc;
+    const long total = p.M * p.N;
+    for (long t = blockIdx.x * (long)blockDim.x + threadIdx.x; t < total; t += (long)gridDim.x * blockDim.x) {
+        const long i = t / p.N, j = t % p.N;
+        const long src = p.gram && j < i ? j * p.N + i : t;
+        longlong2 v = planes[src];
+        for (int z = 1; z < ksp; ++z) {
+            const longlong2 u = planes[z * total + src];
+            v.x += u.x;
+            v.y += u.y;
+        }
+        const double x = digits_value(v.x, v.y, eA[i] + eB[j]);
+        C[i * p.ldc + j] = alpha == 1.0 ? x : alpha * x;
+    }
+}
+
+// The product on the FP64 FMA pipe, only where the split latched *flag.
+constexpr int FB = 16;
+__global__ void __launch_bounds__(FB * FB)
+fallback_kernel(const int* __restrict__ flag, Prod p, int ta, int tb, double alpha, const double* __restrict__ A,
+                const double* __restrict__ B, double* __restrict__ C) {
+    if (*flag == 0) return;
+    p.Mc = p.M;
+    if (!resolve(p)) return;
+    const long ai = ta ? 1 : p.lda, ak = ta ? p.lda : 1, bj = tb ? p.ldb : 1, bk = tb ? 1 : p.ldb;
+    __shared__ double As[FB][FB + 1], Bs[FB][FB + 1];
+    const int ty = threadIdx.x / FB, tx = threadIdx.x % FB;
+    const long nb = (p.N + FB - 1) / FB, tiles = (p.M + FB - 1) / FB * nb;
+    for (long t = blockIdx.x; t < tiles; t += gridDim.x) {
+        const long i = t / nb * FB + ty, j0 = t % nb * FB, j = j0 + tx;
+        double acc = 0.0;
+        for (long k0 = 0; k0 < p.K; k0 += FB) {
+            As[ty][tx] = i < p.M && k0 + tx < p.K ? A[i * ai + (k0 + tx) * ak] : 0.0;
+            Bs[ty][tx] = j0 + ty < p.N && k0 + tx < p.K ? B[(j0 + ty) * bj + (k0 + tx) * bk] : 0.0;
+            __syncthreads();
+            const int kn = (int)min((long)FB, p.K - k0);
+            for (int k = 0; k < kn; ++k) acc = fma(As[ty][k], Bs[tx][k], acc);
+            __syncthreads();
+        }
+        if (i < p.M && j < p.N) C[i * p.ldc + j] = alpha * acc;
+    }
+}
+
+unsigned blocks_for(long work, long cap) { return (unsigned)std::max<long>(1, std::min<long>(work, cap)); }
+
+// Chunks and scratch of a product of at most these sizes.
+struct Plan {
+    long Kc, Mc;
+    bool planes;                         // several splits or chunks of K possible
+    size_t head, imgA, imgB, part;       // bytes: flag, maxima and exponents; images; planes
+    size_t bytes() const { return head + imgA + imgB + part; }
+};
+Plan make_plan(long M, long N, long K, bool gram) {
+    Plan p;
+    const long Np = up(N, gram ? T_M : RB);
+    // images of about IMG_LIMIT bytes each: a long contraction is cut along K
+    // (for an operand of up to 1024 rows), a tall A along its rows
+    const long wide = std::max(up(std::min(M, 1024L), T_M), Np);
+    const long kmax = std::max(16384L, IMG_LIMIT / (2 * S8 * wide) / (T_K * T_BLK) * (T_K * T_BLK));
+    p.Kc = K <= kmax ? K : up((K + (K + kmax - 1) / kmax - 1) / ((K + kmax - 1) / kmax), T_K * T_BLK);
+    const long nst = stages(p.Kc);
+    p.Mc = gram ? M : std::min(M, std::max((long)T_M, IMG_LIMIT / (2L * S8 * nst * T_K) / T_M * T_M));
+    p.planes = gram || p.Kc < K || split_limit(M, N, (int)nst) > 1;
+    p.head = (size_t)up(256 + 8 * (M + N) + 4 * (M + N) + 64, 1024);
+    p.imgB = (size_t)(Np * nst * T_K * 2 * S8);
+    p.imgA = gram ? 0 : (size_t)(up(p.Mc, T_M) * nst * T_K * 2 * S8);
+    p.part = p.planes ? 16 * (size_t)std::max(M * N, std::min(M * N * MAX_SPLITS, PLANE_ELEMS)) : 0;
+    return p;
+}
+
+// desc: a captured product of sizes up to M, N, K (then lda, ldb, ldc are the
+// descriptor's).
+tt_status run(cudaStream_t s, bool ta, bool tb, long M, long N, long K, double alpha, const double* A, long lda,
+              const double* B, long ldb, double* C, long ldc, DevBuf& scratch, int* status_dev, bool gram,
+              const int* desc) {
+    const Plan q = make_plan(M, N, K, gram);
+    // slack to bring the base to a 1024-byte boundary (a pool may give 256)
+    TT_TRY(scratch.ensure((q.bytes() + 1024 + 7) / 8, s));
+    unsigned char* base = reinterpret_cast<unsigned char*>(((uintptr_t)scratch.p + 1023) & ~(uintptr_t)1023);
+    int* flag = reinterpret_cast<int*>(base);
+    u64* mx = reinterpret_cast<u64*>(base + 256);
+    int* ex = reinterpret_cast<int*>(mx + M + N);
+    Side a{A, 0, ta ? 1 : 0, mx, ex, base + q.head + q.imgB};
+    Side b{B, 1, tb ? 0 : 1, mx + M, ex + M, base + q.head};
+    if (gram) a = Side{A, 0, 1, mx, ex, base + q.head};
+    longlong2* planes = q.planes ? reinterpret_cast<longlong2*>(base + q.head + q.imgA + q.imgB) : nullptr;
+    const int* eB = gram ? ex : b.e;
+    Prod p{M, N, K, lda, ldb, ldc, desc, 0, q.Kc, 0, q.Mc, gram ? 1 : 0, q.Mc};
+    int dev = 0, sms = 152;
+    TT_CUDA_TRY(cudaGetDevice(&dev));
+    TT_CUDA_TRY(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
+    TT_TRY(ensure_max_dynamic_smem((const void*)tc8_kernel));
+    // the flag and, where atomics find them, the maxima start at zero
+    TT_CUDA_TRY(cudaMemsetAsync(flag, 0, 256 + (a.strided || b.strided ? 8 * (size_t)(M + N) : 0), s));
+    const bool fusable = K <= FUSED_K;  // a captured step launches both forms when K may be longer
+    auto maxima = [&](const Side& o) {
+        const long rows = o.isB ? N : M;
+        if (o.strided) {
+            note_launch();
+            strided_max_kernel<<<dim3(blocks_for((rows + 31) / 32, 4096), blocks_for(K / 256, 512)), 256, 0, s>>>(p, o);
+        } else if (!fusable) {
+            note_launch();
+            row_max_kernel<<<blocks_for((rows + 7) / 8, 152L * 64), 256, 0, s>>>(p, o);
+        }
+    };
+    auto split = [&](const Side& o) {
+        const long rows = o.isB ? N : std::min(q.Mc, M - p.i0), rpad = up(rows, T_M);
+        const int nst = stages(q.Kc);
+        if (o.strided) {
+            note_launch();
+            split_strided_kernel<<<dim3(blocks_for((rpad + 31) / 32, 4096), blocks_for(((long)nst * 2 + 7) / 8, 2048)),
+                                   256, 0, s>>>(p, o, flag);
+            return;
+        }
+        if (!fusable) {
+            note_launch();
+            split_rows_long_kernel<<<blocks_for((rpad * nst * 16 + 255) / 256, 152L * 64), 256, 0, s>>>(p, o, flag);
+            if (!desc) return;
+        }
+        const unsigned grid = blocks_for((rpad + 7) / 8, 152L * 64);
+        const int need = std::min(nst, FUSED_K / T_K);
+        // by value one instance, the smallest that holds the row; a captured
+        // product launches each that a size up to its capacity may need
+        if (desc ? true : need <= 4) {
+            note_launch();
+            split_rows_kernel<2><<<grid, 256, 0, s>>>(p, o, flag);
+        }
+        if (need > 4 && (desc || need <= 8)) {
+            note_launch();
+            split_rows_kernel<4><<<grid, 256, 0, s>>>(p, o, flag);
+        }
+        if (need > 8 && (desc || need <= 16)) {
+            note_launch();
+            split_rows_kernel<8><<<grid, 256, 0, s>>>(p, o, flag);
+        }
+        if (need > 16) {
+            note_launch();
+            split_rows_kernel<16><<<grid, 256, 0, s>>>(p, o, flag);
+        }
+    };
+    const int nst0 = stages(q.Kc);
+    const int spc = split_stages(M, N, tiles_of(q.Mc, N, gram), nst0);
+    const bool direct = !desc && !gram && q.Kc >= K && spc >= nst0;
+    maxima(a);
+    if (!gram) maxima(b);
+    for (p.k0 = 0; p.k0 < K; p.k0 += q.Kc) {
+        if (!gram) {
+            p.i0 = 0;
+            p.Mc = M;
+            split(b);
+        }
+        for (p.i0 = 0; p.i0 < M; p.i0 += q.Mc) {
+            p.Mc = q.Mc;
+            split(a);
+            const long items = tiles_of(std::min(q.Mc, M - p.i0), N, gram) * ((nst0 + spc - 1) / spc);
+            note_launch();
+            tc8_kernel<<<desc ? sms : (int)std::min<long>(items, sms), THREADS8, SMEM8, s>>>(
+                p, a.img, a.e, b.img, eB, alpha, C, direct ? nullptr : planes, spc, status_dev);
+            TT_CUDA_TRY(cudaGetLastError());
+        }
+    }
+    p.k0 = p.i0 = 0;
+    p.Mc = q.Mc;
+    if (!direct) {
+        note_launch();
+        tc8_reduce_kernel<<<blocks_for((M * N + 255) / 256, 152L * 16), 256, 0, s>>>(p, planes, a.e, eB, spc, alpha, C);
+    }
+    note_launch();
+    fallback_kernel<<<152 * 4, FB * FB, 0, s>>>(flag, p, ta ? 1 : 0, tb ? 1 : 0, alpha, A, B, C);
+    TT_CUDA_TRY(cudaGetLastError());
+    return TT_OK;
+}
+
+}  // namespace
+
+size_t tc8_scratch_doubles(long M, long N, long K, bool gram) {
+    return (make_plan(M, N, K, gram).bytes() + 1024 + 7) / 8;
+}
+
+tt_status tc8_gemm(cudaStream_t s, bool ta, bool tb, long M, long N, long K, double alpha, const double* A, long lda,
+                   const double* B, long ldb, double* C, long ldc, DevBuf& scratch, int* status_dev) {
+    return run(s, ta, tb, M, N, K, alpha, A, lda, B, ldb, C, ldc, scratch, status_dev, false, nullptr);
+}
+
+tt_status tc8_gram(cudaStream_t s, long m, long n, const double* A, long lda, double* G, long ldg, DevBuf& scratch,
+                   int* status_dev) {
+    return run(s, true, false, n, n, m, 1.0, A, lda, A, lda, G, ldg, scratch, status_dev, true, nullptr);
+}
+
+tt_status tc8_dyn(cudaStream_t s, bool ta, bool tb, const int* desc, long Mcap, long Ncap, long Kcap, double alpha,
+                  const double* A, const double* B, double* C, DevBuf& scratch, int* status_dev, bool gram) {
+    return run(s, ta, tb, Mcap, Ncap, Kcap, alpha, A, 0, B, 0, C, 0, scratch, status_dev, gram, desc);
+}
+
+}  // namespace ttsn

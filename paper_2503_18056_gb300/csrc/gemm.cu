@@ -157,8 +157,9 @@ template <bool TA, bool TB>
 __global__ void __launch_bounds__(THREADS, 4)
 dgemm_dyn_kernel(const int* __restrict__ desc, double alpha, const double* __restrict__ A,
                  const double* __restrict__ B, double* __restrict__ C, double* __restrict__ P, int mode,
-                 long resident) {
+                 long resident, int tc) {
     const int M = desc[0], N = desc[1], K = desc[2];
+    if (tc && tc8_wanted(M, N, K)) return;  // formed from digit products (tc8_dyn)
     const long lda = desc[3], ldb = desc[4], ldc = desc[5];
     const int TM = (M + BM - 1) / BM, TN = (N + BN - 1) / BN;
     int tm, tn, z = 0;
@@ -206,8 +207,9 @@ dgemm_dyn_kernel(const int* __restrict__ desc, double alpha, const double* __res
 
 // mode 1 partials -> C (nothing to do when the rule gave one split)
 __global__ void splitk_reduce_dyn_kernel(const int* __restrict__ desc, const double* __restrict__ P,
-                                         double alpha, double* C) {
+                                         double alpha, double* C, int tc) {
     const int M = desc[0], N = desc[1], K = desc[2];
+    if (tc && tc8_wanted(M, N, K)) return;
     const long ldc = desc[5];
     int ks = 1, kchunk = K;
     sk_split(M, N, K, &ks, &kchunk);
@@ -223,8 +225,9 @@ __global__ void splitk_reduce_dyn_kernel(const int* __restrict__ desc, const dou
 
 // mode 2 partials -> the symmetric G (leading dimension desc[5])
 __global__ void gram_reduce_dyn_kernel(const int* __restrict__ desc, const double* __restrict__ P,
-                                       long resident, double* G) {
+                                       long resident, double* G, int tc) {
     const int n = desc[0], m = desc[2];
+    if (tc && tc8_wanted(n, n, m)) return;
     const long ldg = desc[5];
     const int ks = gram_split_rule(m, n, resident);
     const long total = (long)n * n;
@@ -491,9 +494,20 @@ tt_status dgemm(cudaStream_t s, bool ta, bool tb, int M, int N, int K, double al
                        strideC, batch, 1, K, 0, 0);
 }
 
+size_t dgemm_sk_scratch_doubles(int M, int N, int K) {
+    if (tc8_wanted(M, N, K)) return tc8_scratch_doubles(M, N, K, false);
+    int ks = 1, kchunk = K;
+    sk_split(M, N, K, &ks, &kchunk);
+    return ks > 1 ? (size_t)ks * M * N : 0;
+}
+
 tt_status dgemm_sk(cudaStream_t s, bool ta, bool tb, int M, int N, int K, double alpha,
                    const double* A, long lda, const double* B, long ldb, double* C, long ldc,
-                   DevBuf& scratch) {
+                   DevBuf& scratch, int* status_dev) {
+    if (tc8_wanted(M, N, K)) {
+        const tt_status st = tc8_gemm(s, ta, tb, M, N, K, alpha, A, lda, B, ldb, C, ldc, scratch, status_dev);
+        if (st != TT_ERR_OOM) return st;  // without room for the digits: the FP64 pipe
+    }
     int ks = 1, kchunk = K;
     sk_split(M, N, K, &ks, &kchunk);
     if (ks == 1 || M <= 0 || N <= 0)
@@ -635,8 +649,11 @@ size_t dyn_partials_need(int mode, int Mcap, int Ncap, int Kcap) {
 }
 
 tt_status dgemm_dyn(cudaStream_t s, bool ta, bool tb, const int* desc, int Mcap, int Ncap, int Kcap,
-                    double alpha, const double* A, const double* B, double* C, double* P, size_t pcap, int mode) {
+                    double alpha, const double* A, const double* B, double* C, double* P, size_t pcap, int mode,
+                    DevBuf& tcbuf, int* status_dev) {
     if (Mcap <= 0 || Ncap <= 0) return TT_OK;
+    const int tc = mode != 0 && tc8_wanted(Mcap, Ncap, Kcap) ? 1 : 0;
+    if (tc) TT_TRY(tc8_dyn(s, ta, tb, desc, Mcap, Ncap, Kcap, alpha, A, B, C, tcbuf, status_dev, mode == 2));
     if (dyn_partials_need(mode, Mcap, Ncap, Kcap) > pcap) {
         set_error("dgemm: the partials buffer of a captured product is smaller than its split needs");
         return TT_ERR_TOO_LARGE;
@@ -657,19 +674,19 @@ tt_status dgemm_dyn(cudaStream_t s, bool ta, bool tb, const int* desc, int Mcap,
     }
     note_launch();
     if (ta && tb)
-        dgemm_dyn_kernel<true, true><<<grid, THREADS, 0, s>>>(desc, alpha, A, B, C, P, mode, resident);
+        dgemm_dyn_kernel<true, true><<<grid, THREADS, 0, s>>>(desc, alpha, A, B, C, P, mode, resident, tc);
     else if (ta)
-        dgemm_dyn_kernel<true, false><<<grid, THREADS, 0, s>>>(desc, alpha, A, B, C, P, mode, resident);
+        dgemm_dyn_kernel<true, false><<<grid, THREADS, 0, s>>>(desc, alpha, A, B, C, P, mode, resident, tc);
     else if (tb)
-        dgemm_dyn_kernel<false, true><<<grid, THREADS, 0, s>>>(desc, alpha, A, B, C, P, mode, resident);
+        dgemm_dyn_kernel<false, true><<<grid, THREADS, 0, s>>>(desc, alpha, A, B, C, P, mode, resident, tc);
     else
-        dgemm_dyn_kernel<false, false><<<grid, THREADS, 0, s>>>(desc, alpha, A, B, C, P, mode, resident);
+        dgemm_dyn_kernel<false, false><<<grid, THREADS, 0, s>>>(desc, alpha, A, B, C, P, mode, resident, tc);
     if (mode == 1) {
         note_launch();
-        splitk_reduce_dyn_kernel<<<grid_for((long)Mcap * Ncap), 256, 0, s>>>(desc, P, alpha, C);
+        splitk_reduce_dyn_kernel<<<grid_for((long)Mcap * Ncap), 256, 0, s>>>(desc, P, alpha, C, tc);
     } else if (mode == 2) {
         note_launch();
-        gram_reduce_dyn_kernel<<<grid_for((long)Mcap * Ncap), 256, 0, s>>>(desc, P, resident, C);
+        gram_reduce_dyn_kernel<<<grid_for((long)Mcap * Ncap), 256, 0, s>>>(desc, P, resident, C, tc);
     }
     TT_CUDA_TRY(cudaGetLastError());
     return TT_OK;
@@ -683,8 +700,12 @@ void scale_rows_dyn(cudaStream_t s, const int* desc, long total_cap, const doubl
 }
 
 tt_status gram(cudaStream_t s, int m, int n, const double* A, long lda, double* G, long ldg,
-               DevBuf& partials) {
+               DevBuf& partials, int* status_dev) {
     if (n <= 0) return TT_OK;
+    if (tc8_wanted(n, n, m)) {
+        const tt_status st = tc8_gram(s, m, n, A, lda, G, ldg, partials, status_dev);
+        if (st != TT_ERR_OOM) return st;
+    }
     const size_t need = gram_scratch_doubles(std::max(m, 1), n);
     TT_TRY(partials.ensure(need, s));
     return gram_with_scratch(s, m, n, A, lda, G, ldg, partials.p, partials.cap);

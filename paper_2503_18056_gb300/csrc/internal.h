@@ -80,7 +80,10 @@ tt_status dgemm(cudaStream_t s, bool ta, bool tb, int M, int N, int K, double al
 // long; otherwise the plain dgemm.
 tt_status dgemm_sk(cudaStream_t s, bool ta, bool tb, int M, int N, int K, double alpha,
                    const double* A, long lda, const double* B, long ldb, double* C, long ldc,
-                   DevBuf& scratch);
+                   DevBuf& scratch, int* status_dev = nullptr);
+
+// Scratch that a dgemm_sk of these sizes uses (0: none).
+size_t dgemm_sk_scratch_doubles(int M, int N, int K);
 
 // Autotuned split table (gemm.cu): buckets of floor(log2 tiles) < 8 and
 // floor(log2 K) < 22; autotune measures and installs it, autotune_install
@@ -104,8 +107,10 @@ constexpr int GRAM_MULTI_SPLITS = 64;
 // (row split by gram_split_rule, partials in P).  The same bits as the host
 // path for the same sizes.  P holds pcap doubles, at least
 // dyn_partials_need(mode, Mcap, Ncap, Kcap) (checked: TT_ERR_TOO_LARGE).
+// tcbuf: scratch of tc8_dyn, reserved ahead of the capture.
 tt_status dgemm_dyn(cudaStream_t s, bool ta, bool tb, const int* desc, int Mcap, int Ncap, int Kcap,
-                    double alpha, const double* A, const double* B, double* C, double* P, size_t pcap, int mode);
+                    double alpha, const double* A, const double* B, double* C, double* P, size_t pcap, int mode,
+                    DevBuf& tcbuf, int* status_dev);
 size_t dyn_partials_need(int mode, int Mcap, int Ncap, int Kcap);
 long gram_resident();
 // scale_rows with rows, cols, ldi, ldo = desc[0..3] (rows * cols <= total_cap)
@@ -115,7 +120,7 @@ void scale_rows_dyn(cudaStream_t s, const int* desc, long total_cap, const doubl
 // G = A^T A (A: m x n row-major, lda); split over rows with fixed-order reduction.
 // `partials` is scratch grown as needed (ksplit * n * n doubles).
 tt_status gram(cudaStream_t s, int m, int n, const double* A, long lda, double* G, long ldg,
-               DevBuf& partials);
+               DevBuf& partials, int* status_dev = nullptr);
 // The same with caller-provided scratch of `scratch_doubles` entries (no allocation).
 tt_status gram_with_scratch(cudaStream_t s, int m, int n, const double* A, long lda, double* G,
                             long ldg, double* scratch, size_t scratch_doubles);
@@ -149,6 +154,28 @@ tt_status tcgram(cudaStream_t s, int m, int n, const double* A, long lda, double
 tt_status slgemm_nt(cudaStream_t s, long M, int N, int K, const double* A, long lda, const double* B,
                     long ldb, double* C, long ldc, DevBuf& scratch, int* status_dev = nullptr,
                     DevBuf* planes = nullptr, const int* erowA = nullptr);
+
+// ---------------------------------------------------------------- FP64 products on tensor cores (digits.cu)
+// C = alpha op(A) op(B) and G = A^T A (A m x n) from exact integer digit
+// products: every sum exact, one rounding an entry (the header of digits.cu).
+// tc8_wanted is the rule by which dgemm_sk, gram and their captured forms
+// take it, from the sizes alone.  Below 16M terms (32 us of the FP64 pipe)
+// the five or six launches cost more than they save; a contraction under 64
+// would not be rounded less often than the FP64 sum it replaces; the 64-bit
+// sums hold 2^26 indices.
+__host__ __device__ inline bool tc8_wanted(long M, long N, long K) {
+    return K >= 64 && K <= (1L << 26) && M >= 32 && N >= 16 && N <= (1L << 20) && M * N <= (1L << 40) &&
+           (N <= 16384 || K <= 16384) && M * N >= (16000000L + K - 1) / K;
+}
+size_t tc8_scratch_doubles(long M, long N, long K, bool gram);
+tt_status tc8_gemm(cudaStream_t s, bool ta, bool tb, long M, long N, long K, double alpha, const double* A, long lda,
+                   const double* B, long ldb, double* C, long ldc, DevBuf& scratch, int* status_dev);
+tt_status tc8_gram(cudaStream_t s, long m, long n, const double* A, long lda, double* G, long ldg, DevBuf& scratch,
+                   int* status_dev);
+// The captured form: sizes from desc (as dgemm_dyn's), at most the capacities;
+// does nothing for sizes that tc8_wanted leaves to the FP64 pipe.
+tt_status tc8_dyn(cudaStream_t s, bool ta, bool tb, const int* desc, long Mcap, long Ncap, long Kcap, double alpha,
+                  const double* A, const double* B, double* C, DevBuf& scratch, int* status_dev, bool gram);
 
 // Row scaling: out[i][j] = in[i][j] * f(v[i]) for i < rows, j < cols, where
 // mode 0: v, 1: sqrt(v), 2: 1/sqrt(v), 3: 1/v.  out may alias in.

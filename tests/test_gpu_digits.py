@@ -1,0 +1,132 @@
+"""FP64 products from exact integer digit products (csrc/digits.cu): the sizes
+where tiles, stages, blocks and chunks end, strides, scales, and what cannot
+be split."""
+import ctypes
+
+import numpy as np
+import pytest
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def ttsn():
+    import torch
+
+    assert torch.cuda.is_available()
+    import paper_2503_18056_gb300 as m
+
+    return m
+
+
+def _call(ttsn, A, B, ta, tb, alpha=1.0, pad=0):
+    """tt_dgemm with leading dimensions `pad` wider than the matrices."""
+    import torch
+
+    from paper_2503_18056_gb300 import _native
+
+    def dev(X):
+        P = torch.full((X.shape[0], X.shape[1] + pad), float("nan"), dtype=torch.float64, device="cuda")
+        P[:, : X.shape[1]] = torch.as_tensor(X)
+        return P
+
+    M, K = A.shape[::-1] if ta else A.shape
+    N = B.shape[0] if tb else B.shape[1]
+    a, b = dev(A), dev(B)
+    c = torch.full((M, N + pad), -7.0, dtype=torch.float64, device="cuda")
+    st = _native.lib.tt_dgemm(int(ta), int(tb), M, N, K, alpha, ctypes.c_void_p(a.data_ptr()), a.shape[1],
+                              ctypes.c_void_p(b.data_ptr()), b.shape[1], 0.0, ctypes.c_void_p(c.data_ptr()),
+                              c.shape[1], ctypes.c_void_p(torch.cuda.current_stream().cuda_stream))
+    assert st == 0
+    torch.cuda.synchronize()
+    assert bool((c[:, N:] == -7.0).all())
+    return c[:, :N].cpu().numpy()
+
+
+# (M, N, K): one past and one short of the 128 x 64 tile, the 32-index stage,
+# the 512-index block, the row forms' 64 / 128 / 256 / 512 / 1024 entries, and
+# a contraction long enough for several splits
+SIZES = [(500, 500, 64), (129, 1999, 65), (1023, 63, 257), (127, 257, 513), (511, 33, 1024), (385, 65, 1025),
+         (32, 16, 40001), (2003, 17, 601)]
+
+
+@pytest.mark.parametrize("M,N,K", SIZES)
+@pytest.mark.parametrize("ta,tb", [(False, False), (True, False), (False, True), (True, True)])
+def test_integer_products_are_exact(ttsn, M, N, K, ta, tb):
+    # entries of 18 bits: every sum is an integer below 2^53, so the FP64
+    # product is exact too and any lost digit, row or index shows
+    rng = np.random.default_rng(M + N + K)
+    A = rng.integers(-(1 << 17), 1 << 17, (K, M) if ta else (M, K)).astype(float)
+    B = rng.integers(-(1 << 17), 1 << 17, (N, K) if tb else (K, N)).astype(float)
+    ref = (A.T if ta else A).astype(np.int64) @ (B.T if tb else B).astype(np.int64)
+    assert np.array_equal(_call(ttsn, A, B, ta, tb, pad=3), ref.astype(float))
+
+
+@pytest.mark.parametrize("M,N,K", SIZES)
+@pytest.mark.parametrize("grade", [0, 8])
+def test_split_error_is_within_its_bound(ttsn, M, N, K, grade):
+    """Rows graded over 8 decades along and across the contraction.  A term
+    loses the levels s + t >= 8 (at most 7.1 * 2^12 * 128^-10 of 2^(e_i + e_j),
+    which is at most 16 max|a_i| max|b_j|) and the 56-bit rounding of both
+    factors (2 * 2^-57 of 4 max|a_i| max|b_j|): together under 2^-51; the FP64
+    reference is off by K eps sum |a||b| at most."""
+    rng = np.random.default_rng(K)
+    A, B = rng.standard_normal((M, K)), rng.standard_normal((N, K))
+    if grade:
+        A *= 10.0 ** (-grade * rng.random(K))[None, :] * 10.0 ** (grade * rng.random(M))[:, None]
+        B *= 10.0 ** (-grade * rng.random(N))[:, None]
+    ref = A @ B.T
+    got = _call(ttsn, A, B, False, True, alpha=1.0)
+    bound = K * 2.0 ** -51 * np.abs(A).max(1)[:, None] * np.abs(B).max(1)[None, :] \
+        + (K + 1) * np.finfo(float).eps * (np.abs(A) @ np.abs(B).T)
+    assert np.all(np.abs(got - ref) <= bound)
+    # alpha scales the rounded result once more
+    scaled = _call(ttsn, A, B, False, True, alpha=-0.75)
+    assert np.array_equal(scaled, -0.75 * got)
+
+
+@pytest.mark.parametrize("m,n", [(1025, 130), (40001, 33), (9001, 129), (140000, 65), (20000, 449)])
+def test_gram_integer_products_are_exact_and_symmetric(ttsn, m, n):
+    import torch
+
+    rng = np.random.default_rng(m)
+    A = rng.integers(-(1 << 16), 1 << 16, (m, n)).astype(float)
+    G = ttsn.gram(torch.as_tensor(A, device="cuda")).cpu().numpy()
+    ref = A.astype(np.int64).T @ A.astype(np.int64)
+    assert np.array_equal(G, ref.astype(float)) and np.array_equal(G, G.T)
+
+
+def test_inf_nan_and_extreme_scales_take_the_fp64_pipe(ttsn):
+    rng = np.random.default_rng(0)
+    A, B = rng.standard_normal((300, 260)), rng.standard_normal((260, 310))
+    for a, b in ((np.inf, 1.0), (1.0, np.nan), (-np.inf, np.inf)):
+        X, Y = A.copy(), B.copy()
+        X[5, 7] *= a
+        Y[11, 9] *= b
+        with np.errstate(all="ignore"):
+            ref = X @ Y
+        got = _call(ttsn, X, Y, False, False)
+        assert np.array_equal(np.isnan(got), np.isnan(ref)) and np.array_equal(np.isinf(got), np.isinf(ref))
+        fine = np.isfinite(ref)
+        assert np.abs(got[fine] - ref[fine]).max() <= 1e-13 * np.abs(ref[fine]).max() * np.sqrt(260)
+    for sa, sb in ((1e-290, 1e280), (1e-310, 1e300), (0.0, 1.0)):
+        ref = (sa * A) @ (sb * B)
+        got = _call(ttsn, sa * A, sb * B, False, False)
+        assert np.abs(got - ref).max() <= 1e-13 * max(np.abs(ref).max(), 1e-300) * np.sqrt(260)
+
+
+def test_captured_steps_above_the_digit_sizes_equal_host_steps(ttsn):
+    """A grid whose grown-core products take the digit form: a captured step
+    decides it from the device's sizes and gives the host-driven bits."""
+    import torch
+
+    import workloads
+
+    p = workloads.problem("small_2d", n=(96, 90), n_theta=16, n_phi=32, eps=1e-6, bc=1)
+    p["max_rank"] = 24
+    a, b = ttsn.TTSN.from_problem(p), ttsn.TTSN.from_problem(p)
+    b.set_graph(True)
+    for _ in range(5):
+        assert a.step()["ranks"] == b.step()["ranks"]
+    assert 96 * 90 * (5 * a.ranks()[1] + 1) ** 2 > 16e6
+    assert torch.equal(a.full(), b.full())
