@@ -69,18 +69,21 @@ struct AllocScope {
 };
 
 // ---------------------------------------------------------------- GEMM (gemm.cu)
-// C = alpha op(A) op(B) + beta C, row-major FP64 on mma.m8n8k4.
-// batch > 1: A, B, C advance by strideA/B/C per batch entry.
+// C = alpha op(A) op(B) + beta C, row-major FP64 on mma.m8n8k4 (no scratch, so
+// the contraction is not split over CTAs).
 tt_status dgemm(cudaStream_t s, bool ta, bool tb, int M, int N, int K, double alpha,
                 const double* A, long lda, const double* B, long ldb, double beta, double* C,
-                long ldc, int batch = 1, long strideA = 0, long strideB = 0, long strideC = 0);
+                long ldc);
 
-// beta = 0 GEMM that splits K over CTAs (fixed-order reduction through
-// scratch) when the M x N tile grid alone would leave most SMs idle and K is
-// long; otherwise the plain dgemm.
+// beta = 0 product: from digits (digits.cu) where tc8_wanted, else on the FP64
+// pipe with K split over CTAs by prod_split's rule.  counters (nullable):
+// SPLIT_ITEMS ints that are zero between products of one stream; without
+// them the arrival counters lie in scratch and cost a memset.
+constexpr long SPLIT_ITEMS = 4096;  // (tile, split) items of a split product, at most
+constexpr size_t SPLIT_DOUBLES = (256 + 1) * SPLIT_ITEMS;  // and its scratch
 tt_status dgemm_sk(cudaStream_t s, bool ta, bool tb, int M, int N, int K, double alpha,
                    const double* A, long lda, const double* B, long ldb, double* C, long ldc,
-                   DevBuf& scratch, int* status_dev = nullptr);
+                   DevBuf& scratch, int* status_dev = nullptr, int* counters = nullptr);
 
 // Scratch that a dgemm_sk of these sizes uses (0: none).
 size_t dgemm_sk_scratch_doubles(int M, int N, int K);
@@ -93,42 +96,30 @@ tt_status autotune(cudaStream_t s, int* table_out);
 tt_status autotune_install(const int* table, int n);
 void autotune_read(int* table);
 
-// The split rules of dgemm_sk (split of K) and of the Gram (split of the
-// rows, from the number of resident CTAs), shared by host and device.
-__host__ __device__ void sk_split(int M, int N, int K, int* ks_out, int* kchunk_out);
-__host__ __device__ int gram_split_rule(int m, int n, long resident);
-// splits of a large Gram dealt in many waves (gram_split_rule)
-constexpr int GRAM_MULTI_SPLITS = 64;
-
 // Products of a captured step, their sizes read from device memory: desc =
 // M, N, K, lda, ldb, ldc (Gram: n, n, m, lda, lda, ldg with A m x n), caps
-// bound every size the step can reach.  mode 0: plain product into C; 1:
-// dgemm_sk (split of K by sk_split, partials in P); 2: the Gram G = A^T A
-// (row split by gram_split_rule, partials in P).  The same bits as the host
-// path for the same sizes.  P holds pcap doubles, at least
-// dyn_partials_need(mode, Mcap, Ncap, Kcap) (checked: TT_ERR_TOO_LARGE).
-// tcbuf: scratch of tc8_dyn, reserved ahead of the capture.
+// bound every size the step can reach.  mode 1: dgemm_sk; 2: the Gram
+// G = A^T A.  The same split rules from the same sizes, so the same bits as
+// the host path.  P holds pcap doubles, at least dyn_partials_need (checked:
+// TT_ERR_TOO_LARGE); tcbuf: scratch of tc8_dyn, reserved ahead of the capture;
+// counters as in dgemm_sk.
 tt_status dgemm_dyn(cudaStream_t s, bool ta, bool tb, const int* desc, int Mcap, int Ncap, int Kcap,
                     double alpha, const double* A, const double* B, double* C, double* P, size_t pcap, int mode,
-                    DevBuf& tcbuf, int* status_dev);
+                    DevBuf& tcbuf, int* status_dev, int* counters);
 size_t dyn_partials_need(int mode, int Mcap, int Ncap, int Kcap);
-long gram_resident();
 // scale_rows with rows, cols, ldi, ldo = desc[0..3] (rows * cols <= total_cap)
 void scale_rows_dyn(cudaStream_t s, const int* desc, long total_cap, const double* in, const double* v, int mode,
                     double* out);
 
-// G = A^T A (A: m x n row-major, lda); split over rows with fixed-order reduction.
-// `partials` is scratch grown as needed (ksplit * n * n doubles).
+// G = A^T A (A: m x n row-major, lda), as dgemm_sk: from digits or on the FP64
+// pipe split over rows.  partials is scratch grown as needed.
 tt_status gram(cudaStream_t s, int m, int n, const double* A, long lda, double* G, long ldg,
-               DevBuf& partials, int* status_dev = nullptr);
-// The same with caller-provided scratch of `scratch_doubles` entries (no allocation).
-tt_status gram_with_scratch(cudaStream_t s, int m, int n, const double* A, long lda, double* G,
-                            long ldg, double* scratch, size_t scratch_doubles);
+               DevBuf& partials, int* status_dev = nullptr, int* counters = nullptr);
 size_t gram_scratch_doubles(int m, int n);
-// The same Gram with a fixed scratch: the split-K factor is reduced so the
-// partials fit in scratch_doubles (needs scratch_doubles >= n * n).
+// The FP64-pipe Gram in a fixed scratch: fewer splits where the partials would
+// not fit in scratch_doubles.
 tt_status gram_fixed_scratch(cudaStream_t s, int m, int n, const double* A, long lda, double* G,
-                             long ldg, double* scratch, size_t scratch_doubles);
+                             long ldg, double* scratch, size_t scratch_doubles, int* counters = nullptr);
 // Measured FP64 tensor-pipe throughput (TFLOP/s).
 tt_status bench_fp64_mma(cudaStream_t s, double* tflops);
 // Measured BF16 mma.sync (m16n8k16, FP32 accumulate) throughput (TFLOP/s).

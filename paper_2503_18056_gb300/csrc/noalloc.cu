@@ -19,7 +19,8 @@
 // stream capture starts.  All calls share the one array: calls that overlap on
 // the GPU (different streams, or different host threads on one device) race on
 // it and must be serialised by the caller.  Nothing in the array needs clearing
-// between calls: every entry a call reads is written earlier in the same call.
+// between calls: a call clears its arrival counters (a memset ahead of the
+// kernel) and writes every partial that it reads.
 #include <mutex>
 
 #include "internal.h"
