@@ -229,7 +229,7 @@ struct tt_ctx {
     EigWork eig;
     DevBuf small_buf;          // holds d_dbl then d_int
     int* d_int = nullptr;      // device ints (HI_* layout)
-    int* counters = nullptr;           // arrival counters of split products (SPLIT_ITEMS, zero in between)
+    ProdCtx prod;                      // what the handle's products share (the counters follow d_int)
     double* d_dbl = nullptr;   // device doubles (HD_* layout)
     int* h_int = nullptr;      // pinned host mirror
     double* h_dbl = nullptr;
@@ -375,13 +375,14 @@ struct tt_ctx {
             cudaMemPoolSetAttribute(pool, cudaMemPoolAttrReleaseThreshold, &thr);
         }
         (void)cudaGetLastError();
-        TT_TRY(small_buf.ensure((size_t)HD_N + ((HI_N + SPLIT_ITEMS) * sizeof(int) + 7) / 8, s));
+        TT_TRY(small_buf.ensure((size_t)HD_N + ((HI_N + PROD_COUNTERS) * sizeof(int) + 7) / 8, s));
         d_dbl = small_buf.p;
         d_int = reinterpret_cast<int*>(small_buf.p + HD_N);
-        counters = d_int + HI_N;
+        prod.status = d_int + HI_STATUS;
+        prod.counters = d_int + HI_N;
         TT_CUDA_TRY(cudaMallocHost(&h_int, HI_N * sizeof(int)));
         TT_CUDA_TRY(cudaMallocHost(&h_dbl, HD_N * sizeof(double)));
-        TT_CUDA_TRY(cudaMemsetAsync(d_int, 0, (HI_N + SPLIT_ITEMS) * sizeof(int), s));
+        TT_CUDA_TRY(cudaMemsetAsync(d_int, 0, (HI_N + PROD_COUNTERS) * sizeof(int), s));
         fill(s, d_dbl + HD_ONE, 1, 1.0);
         return TT_OK;
     }
@@ -537,7 +538,7 @@ tt_status eig_orthonormalise(tt_ctx* h, long m, int l, const double* Y, DevBuf& 
     TT_TRY(h->sk_lam.ensure((size_t)l, s));
     TT_TRY(h->sk_Vt.ensure((size_t)l * l, s));
     TT_TRY(h->sk_Vs.ensure((size_t)l * l, s));
-    TT_TRY(gram(s, (int)m, l, Y, l, h->sk_G.p, l, h->partials, h->d_int + HI_STATUS, h->counters));
+    TT_TRY(gram(s, (int)m, l, Y, l, h->sk_G.p, l, h->partials, h->prod));
     // Y^T Y is positive semidefinite: the handle's eigensolver for such matrices
     if (h->eig_method == TT_EIG_ONE_SIDED)
         TT_TRY(syev_psd(s, l, h->sk_G.p, l, h->sk_lam.p, h->sk_Vt.p, l, h->eig, h->d_int + HI_STATUS,
@@ -554,7 +555,7 @@ tt_status eig_orthonormalise(tt_ctx* h, long m, int l, const double* Y, DevBuf& 
     scale_rows(s, k, l, h->sk_Vt.p, l, h->sk_lam.p, 2, h->sk_Vs.p, l);  // rows v_j / sqrt(lambda_j)
     TT_TRY(Q.ensure((size_t)m * k, s));
     TT_TRY(dgemm_sk(s, false, true, (int)m, k, l, 1.0, Y, l, h->sk_Vs.p, l, Q.p, k,
-                    h->partials, h->d_int + HI_STATUS, h->counters));
+                    h->partials, h->prod, false));
     return TT_OK;
 }
 
@@ -597,15 +598,15 @@ tt_status round_randomized(tt_ctx* h, DevBuf* src, const int* R, DevBuf* dst, in
         PhaseScope ps(h, TT_PH_GRAM_RIGHT, fl, 0.0);
         TT_TRY(h->sk_W[d - 2].ensure((size_t)R[d - 1] * l[d - 1], s));
         TT_TRY(dgemm_sk(s, false, true, R[d - 1], l[d - 1], n[d - 1], 1.0, src[d - 1].p, n[d - 1],
-                        h->sk_sub[d - 1].p, n[d - 1], h->sk_W[d - 2].p, l[d - 1], h->partials, h->d_int + HI_STATUS, h->counters));
+                        h->sk_sub[d - 1].p, n[d - 1], h->sk_W[d - 2].p, l[d - 1], h->partials, h->prod));
         for (int c = d - 2; c >= 1; --c) {
             // T = G_c W_c (R_c n_c x l_{c+1}); W_{c-1} = T (R_c x n_c l_{c+1}) Omega_c^T
             TT_TRY(h->bwd.ensure((size_t)R[c] * n[c] * l[c + 1], s));
             TT_TRY(dgemm_sk(s, false, false, R[c] * n[c], l[c + 1], R[c + 1], 1.0, src[c].p, R[c + 1],
-                         h->sk_W[c].p, l[c + 1], h->bwd.p, l[c + 1], h->partials, h->d_int + HI_STATUS, h->counters));
+                         h->sk_W[c].p, l[c + 1], h->bwd.p, l[c + 1], h->partials, h->prod, false));
             TT_TRY(h->sk_W[c - 1].ensure((size_t)R[c] * l[c], s));
             TT_TRY(dgemm_sk(s, false, true, R[c], l[c], n[c] * l[c + 1], 1.0, h->bwd.p, (long)n[c] * l[c + 1],
-                            h->sk_sub[c].p, (long)n[c] * l[c + 1], h->sk_W[c - 1].p, l[c], h->partials, h->d_int + HI_STATUS, h->counters));
+                            h->sk_sub[c].p, (long)n[c] * l[c + 1], h->sk_W[c - 1].p, l[c], h->partials, h->prod));
         }
     }
     rr[0] = 1;
@@ -619,7 +620,7 @@ tt_status round_randomized(tt_ctx* h, DevBuf* src, const int* R, DevBuf* dst, in
         {
             PhaseScope ps(h, TT_PH_GRAM_LEFT, 2.0 * m * (double)Rk * lb + 2.0 * m * (double)lb * lb, 0.0);
             TT_TRY(dgemm_sk(s, false, false, (int)m, lb, Rk, 1.0, A, Rk, h->sk_W[b].p, lb, h->sk_Y.p, lb,
-                            h->partials, h->d_int + HI_STATUS, h->counters));
+                            h->partials, h->prod, false));
         }
         int k1 = 0, k2 = 0;
         {
@@ -645,9 +646,9 @@ tt_status round_randomized(tt_ctx* h, DevBuf* src, const int* R, DevBuf* dst, in
             // M_upd = Q^T A (rk x Rk), then the next core M_upd x_1 G_{b+1}
             TT_TRY(h->Mupd.ensure((size_t)rk * Rk, s));
             TT_TRY(dgemm_sk(s, true, false, rk, Rk, (int)m, 1.0, dst[b].p, rk, A, Rk, h->Mupd.p, Rk,
-                            h->partials, h->d_int + HI_STATUS, h->counters));
+                            h->partials, h->prod));
             TT_TRY(dgemm_sk(s, false, false, rk, (int)ncols, Rk, 1.0, h->Mupd.p, Rk, src[b + 1].p, ncols,
-                            next, ncols, h->partials, h->d_int + HI_STATUS, h->counters));
+                            next, ncols, h->partials, h->prod));
         }
         rr[b + 1] = rk;
         A = next;
@@ -677,13 +678,13 @@ tt_status orth_qr3(tt_ctx* h, long m, int l, const double* Y, DevBuf** Q, int* k
     TT_TRY(h->sk_lam.ensure((size_t)l, s));
     TT_TRY(h->sk_Vt.ensure((size_t)l * l, s));
     TT_TRY(h->sk_Vs.ensure((size_t)l * l, s));
-    TT_TRY(gram(s, (int)m, l, Y, l, h->sk_G.p, l, h->partials, h->d_int + HI_STATUS, h->counters));
+    TT_TRY(gram(s, (int)m, l, Y, l, h->sk_G.p, l, h->partials, h->prod));
     TT_TRY(syev(s, l, h->sk_G.p, l, h->sk_lam.p, h->sk_Vt.p, l, h->eig, h->d_int + HI_STATUS,
                 h->d_int + next_sweep_slot(h), h->max_sweeps));
     shifted_scale_rows(s, l, h->sk_Vt.p, l, h->sk_lam.p, h->sk_Vs.p, l);
     TT_TRY(h->ts_Qa.ensure((size_t)m * l, s));
     TT_TRY(dgemm_sk(s, false, true, (int)m, l, l, 1.0, Y, l, h->sk_Vs.p, l, h->ts_Qa.p, l,
-                    h->partials, h->d_int + HI_STATUS, h->counters));
+                    h->partials, h->prod, false));
     int k2 = 0, k3 = 0;
     TT_TRY(eig_orthonormalise(h, m, l, h->ts_Qa.p, h->ts_Qb, &k2));
     if (k2 == 0) {
@@ -735,13 +736,13 @@ tt_status round_ttsvd(tt_ctx* h, DevBuf* src, const int* R, DevBuf* dst, int* rr
             if (q == 0) return zero_tt(h, dst, rr);
             TT_TRY(h->ts_R.ensure((size_t)q * rows, s));
             TT_TRY(dgemm_sk(s, true, false, q, rows, (int)ncols, 1.0, Q->p, q, h->ts_Y.p, rows, h->ts_R.p, rows,
-                            h->partials, h->d_int + HI_STATUS, h->counters));
+                            h->partials, h->prod));
             TT_TRY(h->ts_core[k].ensure((size_t)q * ncols, s));
             transpose(s, ncols, q, Q->p, q, h->ts_core[k].p, ncols);
             const long prow = (long)Rb[k - 1] * n[k - 1];
             TT_TRY(h->ts_core[k - 1].ensure((size_t)prow * q, s));
             TT_TRY(dgemm_sk(s, false, true, (int)prow, q, rows, 1.0, src[k - 1].p, rows, h->ts_R.p, rows, h->ts_core[k - 1].p, q,
-                            h->partials, h->d_int + HI_STATUS, h->counters));
+                            h->partials, h->prod, false));
             Rb[k] = q;
         }
     }
@@ -764,7 +765,7 @@ tt_status round_ttsvd(tt_ctx* h, DevBuf* src, const int* R, DevBuf* dst, int* rr
             if (q == 0) return zero_tt(h, dst, rr);
             TT_TRY(h->ts_R.ensure((size_t)q * l, s));
             TT_TRY(dgemm_sk(s, true, false, q, l, (int)m, 1.0, Q->p, q, A, l, h->ts_R.p, l,
-                            h->partials, h->d_int + HI_STATUS, h->counters));
+                            h->partials, h->prod));
         }
         const int p = q + l, pm = std::min(q, l);
         {
@@ -806,7 +807,7 @@ tt_status round_ttsvd(tt_ctx* h, DevBuf* src, const int* R, DevBuf* dst, int* rr
             // A' = Q U_r
             TT_TRY(dst[k].ensure((size_t)m * rk, s));
             TT_TRY(dgemm_sk(s, false, true, (int)m, rk, q, 1.0, Q->p, q, h->ts_U.p, q, dst[k].p, rk,
-                            h->partials, h->d_int + HI_STATUS, h->counters));
+                            h->partials, h->prod, false));
             // next core = S_r V_r^T x_1 (right-orthonormal core k+1)
             if (k == d - 2) {
                 TT_TRY(dst[d - 1].ensure((size_t)rk * ncols, s));
@@ -817,7 +818,7 @@ tt_status round_ttsvd(tt_ctx* h, DevBuf* src, const int* R, DevBuf* dst, int* rr
                 tmp_idx ^= 1;
             }
             TT_TRY(dgemm_sk(s, false, false, rk, (int)ncols, l, 1.0, h->ts_M.p, l, h->ts_core[k + 1].p, ncols,
-                            next, ncols, h->partials, h->d_int + HI_STATUS, h->counters));
+                            next, ncols, h->partials, h->prod));
         }
         rr[k + 1] = rk;
         A = next;
@@ -874,7 +875,7 @@ tt_status round_cores(tt_ctx* h, DevBuf* src, const int* R, DevBuf* dst, int* rr
         const int Rl = R[d - 1];
         TT_TRY(h->GB[d - 2].ensure((size_t)Rl * Rl, s));
         TT_TRY(dgemm_sk(s, false, true, Rl, Rl, n[d - 1], 1.0, src[d - 1].p, n[d - 1], src[d - 1].p,
-                        n[d - 1], h->GB[d - 2].p, Rl, h->partials, h->d_int + HI_STATUS, h->counters));
+                        n[d - 1], h->GB[d - 2].p, Rl, h->partials, h->prod));
         for (int k = d - 3; k >= 0; --k) {
             const int Ra = R[k + 1], nn = n[k + 1], Rb = R[k + 2];
             TT_TRY(h->bwd.ensure((size_t)Ra * nn * Rb, s));
@@ -889,9 +890,9 @@ tt_status round_cores(tt_ctx* h, DevBuf* src, const int* R, DevBuf* dst, int* rr
                                  (long)nn * Rb, h->GB[k].p, Ra, h->slscratch, h->d_int + HI_STATUS));
             } else {
                 TT_TRY(dgemm_sk(s, false, false, Ra * nn, Rb, Rb, 1.0, src[k + 1].p, Rb, h->GB[k + 1].p,
-                             Rb, h->bwd.p, Rb, h->partials, h->d_int + HI_STATUS, h->counters));
+                             Rb, h->bwd.p, Rb, h->partials, h->prod, false));
                 TT_TRY(dgemm_sk(s, false, true, Ra, Ra, nn * Rb, 1.0, h->bwd.p, (long)nn * Rb,
-                                src[k + 1].p, (long)nn * Rb, h->GB[k].p, Ra, h->partials, h->d_int + HI_STATUS, h->counters));
+                                src[k + 1].p, (long)nn * Rb, h->GB[k].p, Ra, h->partials, h->prod));
             }
         }
     }
@@ -944,7 +945,7 @@ tt_status round_cores(tt_ctx* h, DevBuf* src, const int* R, DevBuf* dst, int* rr
                               reinterpret_cast<int*>(h->erowA.p)));
             }
             else
-                TT_TRY(gram(s, (int)m, Rk, A, Rk, h->GA.p, Rk, h->partials, h->d_int + HI_STATUS, h->counters));
+                TT_TRY(gram(s, (int)m, Rk, A, Rk, h->GA.p, Rk, h->partials, h->prod));
             // a spatial shard holds some rows of the spatial core: its left
             // Gram is the sum of the shards' partial Grams
             if (k == 0 && h->shard.on) TT_TRY(shard_exchange(h, TT_XCHG_SUM, h->GA.p, (size_t)Rk * Rk));
@@ -956,9 +957,9 @@ tt_status round_cores(tt_ctx* h, DevBuf* src, const int* R, DevBuf* dst, int* rr
             TT_TRY(h->T1.ensure((size_t)Rk * kB, s));
             TT_TRY(h->K.ensure((size_t)kB * kB, s));
             TT_TRY(dgemm_sk(s, false, true, Rk, kB, Rk, 1.0, h->GA.p, Rk, Wk, Rk, h->T1.p, kB,
-                            h->partials, h->d_int + HI_STATUS, h->counters));
+                            h->partials, h->prod));
             TT_TRY(dgemm_sk(s, false, false, kB, kB, Rk, 1.0, Wk, Rk, h->T1.p, kB, h->K.p, kB,
-                            h->partials, h->d_int + HI_STATUS, h->counters));
+                            h->partials, h->prod));
         }
         TT_TRY(h->lamK.ensure((size_t)kB, s));
         TT_TRY(h->VtK.ensure((size_t)kB * kB, s));
@@ -997,13 +998,13 @@ tt_status round_cores(tt_ctx* h, DevBuf* src, const int* R, DevBuf* dst, int* rr
             scale_rows(s, rk, kB, h->VtK.p, kB, h->lamK.p, 2, h->Vts.p, kB);
             TT_TRY(h->PAt.ensure((size_t)rk * Rk, s));
             TT_TRY(dgemm_sk(s, false, false, rk, Rk, kB, 1.0, h->Vts.p, kB, h->VtB[k].p, Rk, h->PAt.p, Rk,
-                            h->partials, h->d_int + HI_STATUS, h->counters));
+                            h->partials, h->prod));
             // M_upd = P_A^T G_A = A'^T A  (rk x Rk): B'^T = A'^T A B^T, the orthogonal
             // projection of A B^T onto span(A'); equals App. A.2's (V_B S_B^{-1} V~ S~)^T
             // on the retained eigenspace of G_B without forming S_B^{-1}
             TT_TRY(h->Mupd.ensure((size_t)rk * Rk, s));
             TT_TRY(dgemm_sk(s, false, false, rk, Rk, Rk, 1.0, h->PAt.p, Rk, h->GA.p, Rk, h->Mupd.p, Rk,
-                            h->partials, h->d_int + HI_STATUS, h->counters));
+                            h->partials, h->prod));
         }
         if (h->cur_rec && h->rec_proj && k < 2) {
             tt_ctx::StepRec* rc = h->cur_rec;
@@ -1022,7 +1023,7 @@ tt_status round_cores(tt_ctx* h, DevBuf* src, const int* R, DevBuf* dst, int* rr
                                  h->d_int + HI_STATUS, &h->partials, reinterpret_cast<const int*>(h->erowA.p)));
             else
                 TT_TRY(dgemm_sk(s, false, true, (int)m, rk, Rk, 1.0, A, Rk, h->PAt.p, Rk, dst[k].p, rk,
-                                h->partials, h->d_int + HI_STATUS, h->counters));
+                                h->partials, h->prod, false));
         }
         // next core = M_upd x_1 G_{k+1}
         double* next;
@@ -1038,7 +1039,7 @@ tt_status round_cores(tt_ctx* h, DevBuf* src, const int* R, DevBuf* dst, int* rr
             PhaseScope ps(h, TT_PH_UPDATE, 2.0 * rk * (double)Rk * ncols,
                           8.0 * ((double)Rk * ncols + (double)rk * ncols));
             TT_TRY(dgemm_sk(s, false, false, rk, (int)ncols, Rk, 1.0, h->Mupd.p, Rk, src[k + 1].p, ncols,
-                            next, ncols, h->partials, h->d_int + HI_STATUS, h->counters));
+                            next, ncols, h->partials, h->prod));
         }
         rr[k + 1] = rk;
         A = next;
@@ -1141,7 +1142,7 @@ tt_status split_contract(tt_ctx* h, const double* U, int P, double* out) {
             ti ^= 1;
         }
         TT_TRY(dgemm_sk(s, false, zt, (int)rows, (int)cols, h->r[k + 1], 1.0, h->core[k].p, h->r[k + 1], Z,
-                     zt ? h->r[k + 1] : cols, dst, cols, h->partials, h->d_int + HI_STATUS, h->counters));
+                     zt ? h->r[k + 1] : cols, dst, cols, h->partials, h->prod, false));
         Z = dst;
         zt = false;
         cols *= h->n[k];
@@ -1463,11 +1464,11 @@ tt_status graph_step_body(tt_ctx* h) {
     // rounding (App. A.2, one-sided Gram truncation): backward sweep
     fill(s, h->d_dbl + HD_DELTA2, 1, -1.0);
     TT_TRY(dgemm_dyn(s, false, true, desc + 0, G2, G2, np, 1.0, h->gcore[2].p, h->gcore[2].p, h->GB[1].p, P, PC, 1, h->dyn_tc,
-                     h->d_int + HI_STATUS, h->counters));
-    TT_TRY(dgemm_dyn(s, false, false, desc + 8, G1 * nt, G2, G2, 1.0, h->gcore[1].p, h->GB[1].p, h->bwd.p, P, PC, 1, h->dyn_tc,
-                     h->d_int + HI_STATUS, h->counters));
+                     h->prod));
+    TT_TRY(dgemm_dyn(s, false, false, desc + 8, G1 * nt, G2, G2, 1.0, h->gcore[1].p, h->GB[1].p, h->bwd.p, P, PC, 0, h->dyn_tc,
+                     h->prod));
     TT_TRY(dgemm_dyn(s, false, true, desc + 16, G1, G1, nt * G2, 1.0, h->bwd.p, h->gcore[1].p, h->GB[0].p, P, PC, 1, h->dyn_tc,
-                     h->d_int + HI_STATUS, h->counters));
+                     h->prod));
     TT_TRY(pchol_dyn(s, dd + DYN_G1, G1, h->GB[0].p, h->VtB[0].p, h->Wc.p, h->lamB[0].p, h->eig,
                      h->d_int + HI_STATUS, dd + DYN_KB0));
     TT_TRY(pchol_dyn(s, dd + DYN_G2, G2, h->GB[1].p, h->VtB[1].p, h->Wc.p, h->lamB[1].p, h->eig,
@@ -1475,11 +1476,11 @@ tt_status graph_step_body(tt_ctx* h) {
     plan(1);
     // bond 0: G_A, K = W G_A W^T, eig(K), decision
     TT_TRY(dgemm_dyn(s, true, false, desc + 24, G1, G1, (int)nc, 1.0, h->gcore[0].p, h->gcore[0].p, h->GA.p, P, PC, 2, h->dyn_tc,
-                     h->d_int + HI_STATUS, h->counters));
+                     h->prod));
     TT_TRY(dgemm_dyn(s, false, true, desc + 32, G1, G1, G1, 1.0, h->GA.p, h->VtB[0].p, h->T1.p, P, PC, 1, h->dyn_tc,
-                     h->d_int + HI_STATUS, h->counters));
+                     h->prod));
     TT_TRY(dgemm_dyn(s, false, false, desc + 40, G1, G1, G1, 1.0, h->VtB[0].p, h->T1.p, h->K.p, P, PC, 1, h->dyn_tc,
-                     h->d_int + HI_STATUS, h->counters));
+                     h->prod));
     TT_TRY((h->eig_method == TT_EIG_ONE_SIDED ? syev_psd_dyn : syev_dyn)(
         s, dd + DYN_KB0, G1, h->K.p, h->lamK.p, h->VtK.p, h->eig, h->d_int + HI_STATUS, dd + DYN_SWEEPS,
         h->max_sweeps));
@@ -1489,20 +1490,20 @@ tt_status graph_step_body(tt_ctx* h) {
     // bond 0 update: P_A^T, M_upd, X' = X* P_A, next core = M_upd x_1 Theta*
     scale_rows_dyn(s, desc + 48, (long)c1 * G1, h->VtK.p, h->lamK.p, 2, h->Vts.p);
     TT_TRY(dgemm_dyn(s, false, false, desc + 56, c1, G1, G1, 1.0, h->Vts.p, h->VtB[0].p, h->PAt.p, P, PC, 1, h->dyn_tc,
-                     h->d_int + HI_STATUS, h->counters));
+                     h->prod));
     TT_TRY(dgemm_dyn(s, false, false, desc + 64, c1, G1, G1, 1.0, h->PAt.p, h->GA.p, h->Mupd.p, P, PC, 1, h->dyn_tc,
-                     h->d_int + HI_STATUS, h->counters));
-    TT_TRY(dgemm_dyn(s, false, true, desc + 72, (int)nc, c1, G1, 1.0, h->gcore[0].p, h->PAt.p, h->core[0].p, P, PC, 1, h->dyn_tc,
-                     h->d_int + HI_STATUS, h->counters));
+                     h->prod));
+    TT_TRY(dgemm_dyn(s, false, true, desc + 72, (int)nc, c1, G1, 1.0, h->gcore[0].p, h->PAt.p, h->core[0].p, P, PC, 0, h->dyn_tc,
+                     h->prod));
     TT_TRY(dgemm_dyn(s, false, false, desc + 80, c1, nt * G2, G1, 1.0, h->Mupd.p, h->gcore[1].p, h->tmp[0].p, P, PC, 1, h->dyn_tc,
-                     h->d_int + HI_STATUS, h->counters));
+                     h->prod));
     // bond 1 on the next core (replicated rows r0 n_theta)
     TT_TRY(dgemm_dyn(s, true, false, desc + 88, G2, G2, c1 * nt, 1.0, h->tmp[0].p, h->tmp[0].p, h->GA.p, P, PC, 2, h->dyn_tc,
-                     h->d_int + HI_STATUS, h->counters));
+                     h->prod));
     TT_TRY(dgemm_dyn(s, false, true, desc + 96, G2, G2, G2, 1.0, h->GA.p, h->VtB[1].p, h->T1.p, P, PC, 1, h->dyn_tc,
-                     h->d_int + HI_STATUS, h->counters));
+                     h->prod));
     TT_TRY(dgemm_dyn(s, false, false, desc + 104, G2, G2, G2, 1.0, h->VtB[1].p, h->T1.p, h->K.p, P, PC, 1, h->dyn_tc,
-                     h->d_int + HI_STATUS, h->counters));
+                     h->prod));
     TT_TRY((h->eig_method == TT_EIG_ONE_SIDED ? syev_psd_dyn : syev_dyn)(
         s, dd + DYN_KB1, G2, h->K.p, h->lamK.p, h->VtK.p, h->eig, h->d_int + HI_STATUS, dd + DYN_SWEEPS + 1,
         h->max_sweeps));
@@ -1511,13 +1512,13 @@ tt_status graph_step_body(tt_ctx* h) {
     plan(3);
     scale_rows_dyn(s, desc + 112, (long)c2 * G2, h->VtK.p, h->lamK.p, 2, h->Vts.p);
     TT_TRY(dgemm_dyn(s, false, false, desc + 120, c2, G2, G2, 1.0, h->Vts.p, h->VtB[1].p, h->PAt.p, P, PC, 1, h->dyn_tc,
-                     h->d_int + HI_STATUS, h->counters));
+                     h->prod));
     TT_TRY(dgemm_dyn(s, false, false, desc + 128, c2, G2, G2, 1.0, h->PAt.p, h->GA.p, h->Mupd.p, P, PC, 1, h->dyn_tc,
-                     h->d_int + HI_STATUS, h->counters));
-    TT_TRY(dgemm_dyn(s, false, true, desc + 136, c1 * nt, c2, G2, 1.0, h->tmp[0].p, h->PAt.p, h->core[1].p, P, PC, 1, h->dyn_tc,
-                     h->d_int + HI_STATUS, h->counters));
+                     h->prod));
+    TT_TRY(dgemm_dyn(s, false, true, desc + 136, c1 * nt, c2, G2, 1.0, h->tmp[0].p, h->PAt.p, h->core[1].p, P, PC, 0, h->dyn_tc,
+                     h->prod));
     TT_TRY(dgemm_dyn(s, false, false, desc + 144, c2, np, G2, 1.0, h->Mupd.p, h->gcore[2].p, h->core[2].p, P, PC, 1, h->dyn_tc,
-                     h->d_int + HI_STATUS, h->counters));
+                     h->prod));
     // energy-conserving temperature update (Sec. 3.2) from the rounded TT
     plain_thbar(s, h->ang, c1, c2, h->core[1].p, h->core[2].p, h->thbar.p, dd);
     energy_rows(s, nc, c1, h->core[0].p, c1, h->thbar.p, h->fields.c, nullptr, h->f_Estar.p, h->f_cv.p,
@@ -1797,13 +1798,13 @@ tt_status reverse_step(tt_ctx* h, const tt_ctx::StepRec& rc, const double* Xo, c
 
     // (3) rounding with frozen factors, reversed
     TT_TRY(dgemm_sk(s, true, false, R2, np, o2, 1.0, rc.M[1].p, R2, h->aPhb.p, np, h->aPhgb.p, np,
-                    h->partials, h->d_int + HI_STATUS, h->counters));
+                    h->partials, h->prod, false));
     TT_TRY(dgemm_sk(s, false, false, o1 * nt, R2, o2, 1.0, h->aThb.p, o2, rc.P[1].p, R2, h->aThtb.p, R2,
-                    h->partials, h->d_int + HI_STATUS, h->counters));
+                    h->partials, h->prod, false));
     TT_TRY(dgemm_sk(s, true, false, R1, nt * R2, o1, 1.0, rc.M[0].p, R1, h->aThtb.p, (long)nt * R2, h->aThgb.p,
-                    (long)nt * R2, h->partials, h->d_int + HI_STATUS, h->counters));
+                    (long)nt * R2, h->partials, h->prod, false));
     TT_TRY(dgemm_sk(s, false, false, (int)nc, R1, o1, 1.0, h->aXb.p, o1, rc.P[0].p, R1, h->aXgb.p, R1,
-                    h->partials, h->d_int + HI_STATUS, h->counters));
+                    h->partials, h->prod, false));
 
     // (4) grown angular cores (block-diagonal with the term factors), reversed
     fill(s, h->aThbi.p, (size_t)r1 * nt * r2, 0.0);
@@ -2056,7 +2057,7 @@ struct ShardArgs {
 };
 
 tt_status create_impl(const tt_problem_desc* desc, void* stream, const tt_allocator* alloc,
-                      const ShardArgs* sh, tt_handle* out) {
+                      const ShardArgs* sh, tt_handle* out, bool digits = true) {
     if (!desc || !out) return fail(TT_ERR_ARG, "tt_create: null argument");
     if (alloc && (!alloc->alloc || !alloc->free))
         return fail(TT_ERR_ARG, "tt_create_ex: allocator needs both alloc and free");
@@ -2138,6 +2139,7 @@ tt_status create_impl(const tt_problem_desc* desc, void* stream, const tt_alloca
     }
     AllocScope alloc_scope_(h->alloc_ptr());
     cudaStream_t s = (cudaStream_t)stream;
+    h->prod.digits = digits;
     tt_status st = h->init_common(s);
     if (st < 0) {
         delete h;
@@ -2403,10 +2405,9 @@ tt_status create_impl(const tt_problem_desc* desc, void* stream, const tt_alloca
         TT_CREATE_TRY(h->gcore[1].ensure((size_t)(R1 * D.n_theta * R2), s));
         TT_CREATE_TRY(h->gcore[2].ensure((size_t)(R2 * D.n_phi), s));
         TT_CREATE_TRY(h->GA.ensure((size_t)(R1 * R1), s));
-        TT_CREATE_TRY(h->partials.ensure(D.precision == TT_MIXED
-                                              ? slgram_scratch_doubles((int)nc, (int)R1)
-                                              : SPLIT_DOUBLES, s));
-        if (D.precision != TT_MIXED) {
+        TT_CREATE_TRY(h->partials.ensure(D.precision == TT_MIXED ? slgram_scratch_doubles((int)nc, (int)R1)
+                                                                 : gram_scratch_doubles((int)nc, (int)R1), s));
+        if (D.precision != TT_MIXED && digits) {
             // digit images and planes of the capped step's products; a handle
             // without room for them runs on the FP64 pipe
             const long c[][4] = {{1, R1, R1, nc}, {0, nc, cap1, R1}, {0, R1 * D.n_theta, R2, R2},
@@ -2696,7 +2697,7 @@ tt_status tt_to_full(tt_handle h, double* out_dev, size_t out_len) {
             ti ^= 1;
         }
         TT_TRY(dgemm_sk(s, false, false, (int)rows, (int)cols, h->r[k + 1], 1.0, h->core[k].p,
-                     h->r[k + 1], T, cols, outp, cols, h->partials, h->d_int + HI_STATUS, h->counters));
+                     h->r[k + 1], T, cols, outp, cols, h->partials, h->prod, false));
         T = outp;
         cols *= h->n[k];
     }
@@ -3067,9 +3068,9 @@ tt_status tt_dgemm(int trans_a, int trans_b, int M, int N, int K, double alpha, 
     if ((M && N && K) && (!A || !B || !C)) return fail(TT_ERR_ARG, "tt_dgemm: null pointer");
     cudaStream_t s = (cudaStream_t)stream;
     if (beta == 0.0 && M > 0 && N > 0 && K > 0) {
-        TempScratch t(dgemm_sk_scratch_doubles(M, N, K), s);
+        TempScratch t(gemm_call_doubles(M, N, K), s);
         if (t.ok())
-            return dgemm_sk(s, trans_a != 0, trans_b != 0, M, N, K, alpha, A, lda, B, ldb, C, ldc, t.buf);
+            return gemm_call(s, trans_a != 0, trans_b != 0, M, N, K, alpha, A, lda, B, ldb, C, ldc, t.buf);
     }
     return dgemm(s, trans_a != 0, trans_b != 0, M, N, K, alpha, A, lda, B, ldb, beta, C, ldc);
 }
@@ -3081,9 +3082,8 @@ tt_status tt_gram(int m, int n, const double* A, int lda, double* G, int ldg, vo
     if (!G || (m > 0 && !A)) return fail(TT_ERR_ARG, "tt_gram: null pointer");
     if (lda < n || ldg < n) return fail(TT_ERR_ARG, "tt_gram: leading dimension smaller than n");
     cudaStream_t s = (cudaStream_t)stream;
-    TempScratch t(m > 0 && tc8_wanted(n, n, m) ? tc8_scratch_doubles(n, n, m, true)
-                                               : gram_scratch_doubles(std::max(m, 1), n), s);
-    TT_TRY(gram(s, m, n, A, lda, G, ldg, t.buf));
+    TempScratch t(gram_call_doubles(m, n), s);
+    TT_TRY(gram_call(s, m, n, A, lda, G, ldg, t.buf));
     TT_CUDA_TRY(cudaGetLastError());
     return TT_OK;
 }
@@ -3289,3 +3289,10 @@ tt_status tt_bench_bf16_mma(double* tflops_host, void* stream) {
 }
 
 }  // extern "C"
+
+namespace ttsn {
+tt_status create_in_batch(const tt_problem_desc* desc, void* stream, tt_handle* out) {
+    set_error("");
+    return create_impl(desc, stream, nullptr, nullptr, out, false);
+}
+}  // namespace ttsn

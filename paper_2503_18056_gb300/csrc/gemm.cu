@@ -5,19 +5,26 @@
 // GB300's FP64 pipe issues one warp instruction in 64 clocks per SM
 // sub-partition (19 per SM; a DMMA of 256 FMAs takes eight times that), so a
 // product's time is the longest chain of DMMAs that a sub-partition is given,
-// and loads hardly matter: a 16 x 16 tile's step of 16 indices is 2,048 clocks
-// of each of its four warps against four loads a lane from L2.  So the work
-// is cut as finely as possible and nothing is staged in shared memory: a CTA
-// owns a 16 x 16 tile and a range of the contraction, its four warps take
-// every fourth group of four indices, and the contraction is split over CTAs
-// (prod_split) until the 608 sub-partitions share the DMMAs evenly.  The CTA
-// that arrives last at a tile adds the splits' partials in split order
-// (reproducible), so a split product is one launch.
+// and loads hardly matter: a step of four indices is 512 clocks a warp against
+// two to four loads a lane from L2.  So the work is cut as finely as possible
+// and nothing is staged in shared memory: a CTA owns a 16 x 16 tile and a range
+// of the contraction, and the CTA that arrives last at a tile adds the splits'
+// partials in split order (reproducible), so a split product is one launch.
+// Inside a CTA either each of the four warps takes an 8 x 8 block and all of
+// the range (the rounding's products), or all warps take the whole tile and
+// every fourth group of indices (the library calls, whose contraction may be
+// long against their tiles).
 //
-// Measured (GB300, us a library call, 64 x 64 tiles staged in shared memory
-// before): 133 x 97 x 389 474 -> 27; Gram of 1024 x 61 300 -> 26 (most of both
-// the host's call); the small-grid 2D step 8.5 -> 6.1 ms, the 16-problem
-// captured batch 26.3 -> 21.1 ms.
+// The rounding's products keep one order of summation for good: the splits of
+// sk_split and gram_split_rule and ascending indices within one.  A truncation
+// whose cut falls between singular values that are equal up to rounding (a
+// symmetric problem at its rank cap) takes its basis from the last bits, and a
+// changed order moves such a run's energies by up to the discarded value: for
+// 16 symmetric pulses at their caps by 4e-7 in one of three cases.
+//
+// Measured (GB300, against 64 x 64 tiles staged in shared memory): a call of
+// 133 x 97 x 389 474 -> 24 us; the small-grid 2D step 8.7 -> 6.0 ms, the
+// 16-problem captured batch 27.6 -> 20.5 ms.
 #include <algorithm>
 #include <atomic>
 
@@ -67,7 +74,7 @@ __host__ __device__ inline unsigned prod_cost(long tiles, long K, int ks) {
 constexpr int MAX_SPLIT = 64;
 __host__ __device__ inline int prod_limit(long tiles, long K) {
     long k = K / BK;
-    if (k > SPLIT_ITEMS / tiles) k = SPLIT_ITEMS / tiles;
+    if (k > 4096 / tiles) k = 4096 / tiles;  // at most 8 MB of partials
     if (k > MAX_SPLIT) k = MAX_SPLIT;
     return k < 1 ? 1 : (int)k;
 }
@@ -82,41 +89,93 @@ __host__ __device__ inline int prod_limit(long tiles, long K) {
 __device__ int d_sk_table[AT_TILE_BUCKETS * AT_K_BUCKETS];
 static int h_sk_table[AT_TILE_BUCKETS * AT_K_BUCKETS];
 
+// Split of K of the rounding's products: where 64 x 64 tiles would leave SMs
+// idle, so that there are about two tiles per SM, each with at least 32
+// indices, unless the autotuned table holds a measured split for the product's
+// bucket.  Host and device use the same rule (a captured step decides it on
+// the device from the sizes of that step).
+__host__ __device__ void sk_split(int M, int N, int K, int* ks_out, int* kchunk_out) {
+    const long tiles = (long)((M + 63) / 64) * ((N + 63) / 64);
+    int ks = 1;
+    if (tiles < 152 && K >= 4 * BK) {
+        long a = (304 + tiles - 1) / tiles, b = K / (2 * BK);
+        ks = (int)(a < b ? a : b);
+        const int tb = floor_log2(tiles), kb = floor_log2(K);
+        if (tb < AT_TILE_BUCKETS && kb < AT_K_BUCKETS) {
+#ifdef __CUDA_ARCH__
+            const int tuned = d_sk_table[tb * AT_K_BUCKETS + kb];
+#else
+            const int tuned = h_sk_table[tb * AT_K_BUCKETS + kb];
+#endif
+            if (tuned > 0) ks = (int)(tuned < b ? tuned : b);
+        }
+        ks = ks < 1 ? 1 : (ks > 64 ? 64 : ks);
+    }
+    int kchunk = K;
+    if (ks > 1) {
+        kchunk = (K + ks - 1) / ks;
+        kchunk = (kchunk + BK - 1) / BK * BK;
+        ks = (K + kchunk - 1) / kchunk;
+    }
+    *ks_out = ks;
+    *kchunk_out = kchunk;
+}
+
+// Row split of the rounding's Gram, at least 256 rows a split: one wave of
+// `resident` 64 x 64 tiles for small problems, and for larger ones
+// GRAM_MULTI_SPLITS splits where that leaves fewer tiles idle: the time is then
+// about W / (64 resident) + 1 / (2 splits) of one unsplit tile's, W = B (B + 1)
+// / 2 the 8 x 8 products of the upper triangle that the matrix reaches (B =
+// ceil(n / 8)), against 1 / ks0 for one wave.  Integer arithmetic, so the host
+// and a captured step's device agree.
+__host__ __device__ int gram_split_rule(int m, int n, long resident) {
+    const long T = (n + 63) / 64;
+    const long tiles = T * (T + 1) / 2;
+    long cap = m / 256 < 1 ? 1 : m / 256;
+    if (cap > 1024) cap = 1024;
+    if (resident < 1) resident = 1;
+    long ks0 = resident / tiles;
+    if (ks0 < 1) ks0 = 1;
+    if (ks0 > cap) ks0 = cap;
+    if (ks0 >= 16) return (int)ks0;
+    const long km = cap < GRAM_MULTI_SPLITS ? cap : GRAM_MULTI_SPLITS;
+    if (km <= ks0) return (int)ks0;
+    const long long B = (n + 7) / 8;
+    const long long W = B * (B + 1) / 2;
+    const long long slots = 64LL * resident;
+    // (W / slots + 1 / (2 km)) < 0.97 / ks0, times 2 slots km ks0 100
+    if ((2 * W * km + slots) * ks0 * 100 < 97LL * 2 * slots * km) return (int)km;
+    return (int)ks0;
+}
+
 namespace {
 
-__host__ __device__ inline int prod_tuned(long M, long N, long K, int tri) {
-    const long t64 = ((M + 63) / 64) * ((N + 63) / 64);
-    if (tri || t64 >= 152) return 0;
-    const int tb = floor_log2(t64), kb = floor_log2(K);
-    if (tb >= AT_TILE_BUCKETS || kb >= AT_K_BUCKETS) return 0;
-#ifdef __CUDA_ARCH__
-    return d_sk_table[tb * AT_K_BUCKETS + kb];
-#else
-    return h_sk_table[tb * AT_K_BUCKETS + kb];
-#endif
-}
+// CTAs of 64 x 64 Gram tiles that gram_split_rule counts on: four per SM.
+__host__ __device__ constexpr long gram_resident() { return 152 * 4; }
+
 __host__ __device__ inline int prod_final(long K, int ks) {  // splits that hold indices
     const int c = prod_chunk(K, ks);
     return (int)((K + c - 1) / c);
 }
+// Splits of a library call's product (interleaved warps): the cheapest.
 int prod_split(long M, long N, long K, int tri) {
     const long tiles = prod_tiles(M, N, tri);
-    const int lim = prod_limit(tiles, K), tuned = prod_tuned(M, N, K, tri);
-    if (tuned > 0) return prod_final(K, std::min(tuned, lim));
+    const int lim = prod_limit(tiles, K);
     int best = 1;
     for (int k = 2; k <= lim; ++k)
         if (prod_cost(tiles, K, k) < prod_cost(tiles, K, best)) best = k;
     return prod_final(K, best);
 }
-// the same choice by one warp (a captured step's sizes are the device's)
-__device__ __forceinline__ int prod_split_warp(long M, long N, long K, int tri) {
-    const long tiles = prod_tiles(M, N, tri);
-    const int lim = prod_limit(tiles, K), tuned = prod_tuned(M, N, K, tri);
-    if (tuned > 0) return prod_final(K, min(tuned, lim));
-    unsigned key = 0xffffffffu;
-    for (int k = (threadIdx.x & 31) + 1; k <= lim; k += 32)
-        key = min(key, prod_cost(tiles, K, k) * 64u + (unsigned)(k - 1));
-    return prod_final(K, (int)(__reduce_min_sync(0xffffffffu, key) & 63u) + 1);
+// Splits and indices per split of a rounding's product (ordered); tri: the Gram.
+__host__ __device__ inline int ordered_split(int M, int N, int K, int tri, int* chunk) {
+    int ks = 1;
+    if (tri) {
+        ks = gram_split_rule(K, M, gram_resident());
+        *chunk = prod_chunk(K, ks);
+    } else {
+        sk_split(M, N, K, &ks, chunk);
+    }
+    return ks;
 }
 
 // C = alpha op(A) op(B) (+ beta C), or with tri the symmetric product of which
@@ -124,13 +183,13 @@ __device__ __forceinline__ int prod_split_warp(long M, long N, long K, int tri) 
 // desc (a captured step): M, N, K, lda, ldb, ldc in device memory; tc: sizes
 // that digits.cu takes are left to it.  An item is (tile, split); ks > 1:
 // partials to P (256 doubles an item), arrivals counted in cnt (zero between
-// products: the last arrival resets its tile's).  An 8 x 8 product outside
-// M x N or below the diagonal is skipped.
-template <bool TA, bool TB>
+// products: the last arrival resets its tile's).  ORDERED: a warp per 8 x 8 block; else the warps share the indices.  An 8 x 8
+// product outside M x N or below the diagonal is skipped.
+template <bool TA, bool TB, bool ORDERED>
 __global__ void __launch_bounds__(THREADS)
 prod_kernel(int M, int N, int K, double alpha, const double* __restrict__ A, long lda, const double* __restrict__ B,
-            long ldb, double beta, double* __restrict__ C, long ldc, int ks, double* __restrict__ P, int* cnt, int tri,
-            const int* __restrict__ desc, int tc) {
+            long ldb, double beta, double* __restrict__ C, long ldc, int ks, int chunk, double* __restrict__ P, int* cnt,
+            int tri, const int* __restrict__ desc, int tc) {
     if (desc) {
         M = desc[0];
         N = desc[1];
@@ -139,13 +198,14 @@ prod_kernel(int M, int N, int K, double alpha, const double* __restrict__ A, lon
         ldb = desc[4];
         ldc = desc[5];
         if (M <= 0 || N <= 0 || (tc && tc8_wanted(M, N, K))) return;
-        ks = prod_split_warp(M, N, K, tri);
+        ks = 1;
+        chunk = K;
+        if (P) ks = ordered_split(M, N, K, tri, &chunk);  // P null: an unsplit product
     }
-    __shared__ double red[4][BT * BT];
+    __shared__ double red[ORDERED ? 1 : 4][BT * BT];
     __shared__ int s_last;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const int TM = (M + BT - 1) / BT, TN = (N + BT - 1) / BT;
-    const int chunk = prod_chunk(K, ks);
     const long items = prod_tiles(M, N, tri) * ks;
     for (long item = blockIdx.x; item < items; item += gridDim.x) {
         const long tile = item / ks;
@@ -165,50 +225,79 @@ prod_kernel(int M, int N, int K, double alpha, const double* __restrict__ A, lon
         }
         const int m0 = tm * BT, n0 = tn * BT;
         const int kbeg = z * chunk, kend = min(K, kbeg + chunk);
-        const bool l1 = m0 + 8 < M, c1 = n0 + 8 < N;
-        const bool use10 = l1 && !(tri && tm == tn), use11 = l1 && c1;
-        double acc[2][2][2] = {};
-        // lane: row lane / 4 and index lane % 4 of the operands (rows past the
-        // last read the last: their outputs are not stored)
-        const int r0 = min(m0 + (lane >> 2), M - 1), r1 = min(m0 + 8 + (lane >> 2), M - 1);
-        const int q0 = min(n0 + (lane >> 2), N - 1), q1 = min(n0 + 8 + (lane >> 2), N - 1);
-        const double* a0 = TA ? A + r0 : A + (long)r0 * lda;
-        const double* a1 = TA ? A + r1 : A + (long)r1 * lda;
-        const double* b0 = TB ? B + (long)q0 * ldb : B + q0;
-        const double* b1 = TB ? B + (long)q1 * ldb : B + q1;
         const long sa = TA ? lda : 1, sb = TB ? 1 : ldb;
-        double x0 = 0.0, x1 = 0.0, y0 = 0.0, y1 = 0.0;
-        auto load = [&](int k) {
-            const int kk = k + (lane & 3);
-            const bool in = kk < kend;
-            x0 = in ? a0[kk * sa] : 0.0;
-            x1 = in && l1 ? a1[kk * sa] : 0.0;
-            y0 = in ? b0[kk * sb] : 0.0;
-            y1 = in && c1 ? b1[kk * sb] : 0.0;
-        };
-        int k = kbeg + 4 * warp;
-        if (k < kend) load(k);
-        for (; k < kend; k += BK) {
-            const double u0 = x0, u1 = x1, v0 = y0, v1 = y1;
-            if (k + BK < kend) load(k + BK);
-            dmma(acc[0][0], u0, v0);
-            if (c1) dmma(acc[0][1], u0, v1);
-            if (use10) dmma(acc[1][0], u1, v0);
-            if (use11) dmma(acc[1][1], u1, v1);
-        }
         __syncthreads();  // the item before has read red
+        if (ORDERED) {
+            const int mb = m0 + 8 * (warp >> 1), nb = n0 + 8 * (warp & 1);
+            double acc[2] = {0.0, 0.0};
+            if (mb < M && nb < N && !(tri && mb > nb)) {
+                // lane: row lane / 4 and index lane % 4 of the operands (rows
+                // past the last read the last: their outputs are not stored);
+                // the loads run two steps (1,024 clocks) ahead
+                const int r = min(mb + (lane >> 2), M - 1), q = min(nb + (lane >> 2), N - 1);
+                const double* a = (TA ? A + r : A + (long)r * lda);
+                const double* b = (TB ? B + (long)q * ldb : B + q);
+                double x[2], y[2];
+                auto load = [&](int k, int h) {
+                    const int kk = k + (lane & 3);
+                    x[h] = kk < kend ? a[kk * sa] : 0.0;
+                    y[h] = kk < kend ? b[kk * sb] : 0.0;
+                };
+                load(kbeg, 0);
+                load(kbeg + 4, 1);
+                for (int k = kbeg; k < kend; k += 8) {
+                    const double u0 = x[0], v0 = y[0], u1 = x[1], v1 = y[1];
+                    load(k + 8, 0);
+                    load(k + 12, 1);
+                    dmma(acc, u0, v0);
+                    if (k + 4 < kend) dmma(acc, u1, v1);
+                }
+            }
+            *reinterpret_cast<double2*>(&red[0][(8 * (warp >> 1) + (lane >> 2)) * BT + 8 * (warp & 1) + (lane & 3) * 2]) =
+                make_double2(acc[0], acc[1]);
+        } else {
+            const bool l1 = m0 + 8 < M, c1 = n0 + 8 < N;
+            const bool use10 = l1 && !(tri && tm == tn), use11 = l1 && c1;
+            double acc[2][2][2] = {};
+            const int r0 = min(m0 + (lane >> 2), M - 1), r1 = min(m0 + 8 + (lane >> 2), M - 1);
+            const int q0 = min(n0 + (lane >> 2), N - 1), q1 = min(n0 + 8 + (lane >> 2), N - 1);
+            const double* a0 = TA ? A + r0 : A + (long)r0 * lda;
+            const double* a1 = TA ? A + r1 : A + (long)r1 * lda;
+            const double* b0 = TB ? B + (long)q0 * ldb : B + q0;
+            const double* b1 = TB ? B + (long)q1 * ldb : B + q1;
+            double x0 = 0.0, x1 = 0.0, y0 = 0.0, y1 = 0.0;
+            auto load = [&](int k) {
+                const int kk = k + (lane & 3);
+                const bool in = kk < kend;
+                x0 = in ? a0[kk * sa] : 0.0;
+                x1 = in && l1 ? a1[kk * sa] : 0.0;
+                y0 = in ? b0[kk * sb] : 0.0;
+                y1 = in && c1 ? b1[kk * sb] : 0.0;
+            };
+            int k = kbeg + 4 * warp;
+            if (k < kend) load(k);
+            for (; k < kend; k += BK) {
+                const double u0 = x0, u1 = x1, v0 = y0, v1 = y1;
+                if (k + BK < kend) load(k + BK);
+                dmma(acc[0][0], u0, v0);
+                if (c1) dmma(acc[0][1], u0, v1);
+                if (use10) dmma(acc[1][0], u1, v0);
+                if (use11) dmma(acc[1][1], u1, v1);
+            }
 #pragma unroll
-        for (int i = 0; i < 2; ++i)
+            for (int i = 0; i < 2; ++i)
 #pragma unroll
-            for (int j = 0; j < 2; ++j)
-                *reinterpret_cast<double2*>(&red[warp][(8 * i + (lane >> 2)) * BT + 8 * j + (lane & 3) * 2]) =
-                    make_double2(acc[i][j][0], acc[i][j][1]);
+                for (int j = 0; j < 2; ++j)
+                    *reinterpret_cast<double2*>(&red[warp][(8 * i + (lane >> 2)) * BT + 8 * j + (lane & 3) * 2]) =
+                        make_double2(acc[i][j][0], acc[i][j][1]);
+        }
         __syncthreads();
         double v[2];
 #pragma unroll
         for (int h = 0; h < 2; ++h) {
             const int e = tid + h * THREADS;
-            v[h] = (red[0][e] + red[1][e]) + (red[2][e] + red[3][e]);
+            v[h] = ORDERED ? red[0][e]
+                           : (red[0][e] + red[ORDERED ? 0 : 1][e]) + (red[ORDERED ? 0 : 2][e] + red[ORDERED ? 0 : 3][e]);
         }
         if (ks > 1) {
             double* pt = P + tile * ks * (BT * BT);
@@ -343,20 +432,45 @@ inline int grid_for(long total, int threads = 256) {
     return (int)std::max<long>(1, std::min<long>(b, 152L * 32));
 }
 
-tt_status launch_prod(cudaStream_t s, bool ta, bool tb, int M, int N, int K, double alpha, const double* A, long lda,
-                      const double* B, long ldb, double beta, double* C, long ldc, int ks, double* P, int* cnt, int tri,
-                      const int* desc, int tc, long items) {
+struct ProdArgs {
+    int M, N, K;
+    double alpha;
+    const double* A;
+    long lda;
+    const double* B;
+    long ldb;
+    double beta;
+    double* C;
+    long ldc;
+    int ks, chunk;
+    double* P;
+    int *cnt, tri;
+    const int* desc;
+    int tc;
+};
+
+template <bool TA, bool TB>
+void launch_one(cudaStream_t s, bool ordered, unsigned grid, const ProdArgs& a) {
+    if (ordered)
+        prod_kernel<TA, TB, true><<<grid, THREADS, 0, s>>>(a.M, a.N, a.K, a.alpha, a.A, a.lda, a.B, a.ldb, a.beta, a.C,
+                                                          a.ldc, a.ks, a.chunk, a.P, a.cnt, a.tri, a.desc, a.tc);
+    else
+        prod_kernel<TA, TB, false><<<grid, THREADS, 0, s>>>(a.M, a.N, a.K, a.alpha, a.A, a.lda, a.B, a.ldb, a.beta, a.C,
+                                                           a.ldc, a.ks, a.chunk, a.P, a.cnt, a.tri, a.desc, a.tc);
+}
+
+tt_status launch_prod(cudaStream_t s, bool ta, bool tb, bool ordered, long items, const ProdArgs& a) {
     // more CTAs than fit at once let the scheduler level uneven tiles
     const unsigned grid = (unsigned)std::max(1L, std::min(items, 152L * 64));
     note_launch();
     if (ta && tb)
-        prod_kernel<true, true><<<grid, THREADS, 0, s>>>(M, N, K, alpha, A, lda, B, ldb, beta, C, ldc, ks, P, cnt, tri, desc, tc);
+        launch_one<true, true>(s, ordered, grid, a);
     else if (ta)
-        prod_kernel<true, false><<<grid, THREADS, 0, s>>>(M, N, K, alpha, A, lda, B, ldb, beta, C, ldc, ks, P, cnt, tri, desc, tc);
+        launch_one<true, false>(s, ordered, grid, a);
     else if (tb)
-        prod_kernel<false, true><<<grid, THREADS, 0, s>>>(M, N, K, alpha, A, lda, B, ldb, beta, C, ldc, ks, P, cnt, tri, desc, tc);
+        launch_one<false, true>(s, ordered, grid, a);
     else
-        prod_kernel<false, false><<<grid, THREADS, 0, s>>>(M, N, K, alpha, A, lda, B, ldb, beta, C, ldc, ks, P, cnt, tri, desc, tc);
+        launch_one<false, false>(s, ordered, grid, a);
     TT_CUDA_TRY(cudaGetLastError());
     return TT_OK;
 }
@@ -366,14 +480,14 @@ tt_status launch_prod(cudaStream_t s, bool ta, bool tb, int M, int N, int K, dou
 size_t split_doubles(long tiles, int ks) { return (size_t)tiles * ks * (BT * BT); }
 size_t split_scratch(long tiles, int ks) { return ks > 1 ? split_doubles(tiles, ks) + (size_t)(tiles + 1) / 2 : 0; }
 
-tt_status split_prod(cudaStream_t s, bool ta, bool tb, int M, int N, int K, double alpha, const double* A, long lda,
-                     const double* B, long ldb, double* C, long ldc, int ks, double* P, int* cnt, int tri) {
-    const long tiles = prod_tiles(M, N, tri);
-    if (ks > 1 && !cnt) {
-        cnt = reinterpret_cast<int*>(P + split_doubles(tiles, ks));
-        TT_CUDA_TRY(cudaMemsetAsync(cnt, 0, (size_t)tiles * sizeof(int), s));
+tt_status split_prod(cudaStream_t s, bool ta, bool tb, bool ordered, ProdArgs a) {
+    const long tiles = prod_tiles(a.M, a.N, a.tri);
+    if (tiles > PROD_COUNTERS) a.cnt = nullptr;
+    if (a.ks > 1 && !a.cnt) {
+        a.cnt = reinterpret_cast<int*>(a.P + split_doubles(tiles, a.ks));
+        TT_CUDA_TRY(cudaMemsetAsync(a.cnt, 0, (size_t)tiles * sizeof(int), s));
     }
-    return launch_prod(s, ta, tb, M, N, K, alpha, A, lda, B, ldb, 0.0, C, ldc, ks, P, cnt, tri, nullptr, 0, tiles * ks);
+    return launch_prod(s, ta, tb, ordered, tiles * a.ks, a);
 }
 
 }  // namespace
@@ -391,36 +505,70 @@ tt_status dgemm(cudaStream_t s, bool ta, bool tb, int M, int N, int K, double al
         return TT_OK;
     }
     if (M == 0 || N == 0) return TT_OK;
-    return launch_prod(s, ta, tb, M, N, K, alpha, A, lda, B, ldb, beta, C, ldc, 1, nullptr, nullptr, 0, nullptr, 0,
-                       prod_tiles(M, N, 0));
-}
-
-size_t dgemm_sk_scratch_doubles(int M, int N, int K) {
-    if (tc8_wanted(M, N, K)) return tc8_scratch_doubles(M, N, K, false);
-    if (M <= 0 || N <= 0 || K <= 0) return 0;
-    return split_scratch(prod_tiles(M, N, 0), prod_split(M, N, K, 0));
+    return launch_prod(s, ta, tb, true, prod_tiles(M, N, 0),
+                       ProdArgs{M, N, K, alpha, A, lda, B, ldb, beta, C, ldc, 1, K, nullptr, nullptr, 0, nullptr, 0});
 }
 
 tt_status dgemm_sk(cudaStream_t s, bool ta, bool tb, int M, int N, int K, double alpha,
                    const double* A, long lda, const double* B, long ldb, double* C, long ldc,
-                   DevBuf& scratch, int* status_dev, int* counters) {
-    if (tc8_wanted(M, N, K)) {
-        const tt_status st = tc8_gemm(s, ta, tb, M, N, K, alpha, A, lda, B, ldb, C, ldc, scratch, status_dev);
+                   DevBuf& scratch, const ProdCtx& ctx, bool split) {
+    if (ctx.digits && tc8_wanted(M, N, K)) {
+        const tt_status st = tc8_gemm(s, ta, tb, M, N, K, alpha, A, lda, B, ldb, C, ldc, scratch, ctx.status);
         if (st != TT_ERR_OOM) return st;  // without room for the digits: the FP64 pipe
     }
-    const int ks = M > 0 && N > 0 && K > 0 ? prod_split(M, N, K, 0) : 1;
+    int ks = 1, chunk = K;
+    if (split && M > 0 && N > 0 && K > 0) ks = ordered_split(M, N, K, 0, &chunk);
     if (ks == 1) return dgemm(s, ta, tb, M, N, K, alpha, A, lda, B, ldb, 0.0, C, ldc);
     TT_TRY(scratch.ensure(split_scratch(prod_tiles(M, N, 0), ks), s));
-    return split_prod(s, ta, tb, M, N, K, alpha, A, lda, B, ldb, C, ldc, ks, scratch.p, counters, 0);
+    return split_prod(s, ta, tb, true, ProdArgs{M, N, K, alpha, A, lda, B, ldb, 0.0, C, ldc, ks, chunk, scratch.p,
+                                                ctx.counters, 0, nullptr, 0});
+}
+
+tt_status gram(cudaStream_t s, int m, int n, const double* A, long lda, double* G, long ldg, DevBuf& partials,
+               const ProdCtx& ctx) {
+    if (n <= 0) return TT_OK;
+    if (ctx.digits && tc8_wanted(n, n, m)) {
+        const tt_status st = tc8_gram(s, m, n, A, lda, G, ldg, partials, ctx.status);
+        if (st != TT_ERR_OOM) return st;
+    }
+    if (m <= 0) {
+        for (int i = 0; i < n; ++i) fill(s, G + (long)i * ldg, n, 0.0);
+        return TT_OK;
+    }
+    int chunk = m;
+    const int ks = ordered_split(n, n, m, 1, &chunk);
+    TT_TRY(partials.ensure(split_scratch(prod_tiles(n, n, 1), ks), s));
+    // op(A) = A^T (stored m x n), op(B) = A
+    return split_prod(s, true, false, true, ProdArgs{n, n, m, 1.0, A, lda, A, lda, 0.0, G, ldg, ks, chunk, partials.p,
+                                                     ctx.counters, 1, nullptr, 0});
 }
 
 size_t gram_scratch_doubles(int m, int n) {
-    const int K = std::max(m, 1);
-    return split_scratch(prod_tiles(n, n, 1), prod_split(n, n, K, 1));
+    return split_scratch(prod_tiles(n, n, 1), gram_split_rule(std::max(m, 1), n, gram_resident()));
+}
+
+// ------------------------------------------------------------ library calls
+
+size_t gemm_call_doubles(int M, int N, int K) {
+    if (tc8_wanted(M, N, K)) return tc8_scratch_doubles(M, N, K, false);
+    return split_scratch(prod_tiles(M, N, 0), prod_split(M, N, K, 0));
+}
+
+tt_status gemm_call(cudaStream_t s, bool ta, bool tb, int M, int N, int K, double alpha, const double* A, long lda,
+                    const double* B, long ldb, double* C, long ldc, DevBuf& scratch) {
+    if (tc8_wanted(M, N, K)) return tc8_gemm(s, ta, tb, M, N, K, alpha, A, lda, B, ldb, C, ldc, scratch, nullptr);
+    const int ks = prod_split(M, N, K, 0);
+    return split_prod(s, ta, tb, false, ProdArgs{M, N, K, alpha, A, lda, B, ldb, 0.0, C, ldc, ks, prod_chunk(K, ks),
+                                                 scratch.p, nullptr, 0, nullptr, 0});
+}
+
+size_t gram_call_doubles(int m, int n) {
+    if (tc8_wanted(n, n, m)) return tc8_scratch_doubles(n, n, m, true);
+    return split_scratch(prod_tiles(n, n, 1), prod_split(n, n, std::max(m, 1), 1));
 }
 
 tt_status gram_fixed_scratch(cudaStream_t s, int m, int n, const double* A, long lda, double* G,
-                             long ldg, double* scratch, size_t scratch_doubles, int* counters) {
+                             long ldg, double* scratch, size_t scratch_doubles) {
     if (m < 0 || n < 0) {
         set_error("gram: negative size");
         return TT_ERR_ARG;
@@ -434,30 +582,71 @@ tt_status gram_fixed_scratch(cudaStream_t s, int m, int n, const double* A, long
     int ks = prod_split(n, n, m, 1);
     while (ks > 1 && split_scratch(tiles, ks) > scratch_doubles) --ks;
     ks = prod_final(m, ks);
-    // op(A) = A^T (stored m x n), op(B) = A
-    return split_prod(s, true, false, n, n, m, 1.0, A, lda, A, lda, G, ldg, ks, scratch, counters, 1);
+    return split_prod(s, true, false, false, ProdArgs{n, n, m, 1.0, A, lda, A, lda, 0.0, G, ldg, ks, prod_chunk(m, ks),
+                                                      scratch, nullptr, 1, nullptr, 0});
 }
 
+tt_status gram_call(cudaStream_t s, int m, int n, const double* A, long lda, double* G, long ldg, DevBuf& scratch) {
+    if (m > 0 && tc8_wanted(n, n, m)) {
+        const tt_status st = tc8_gram(s, m, n, A, lda, G, ldg, scratch, nullptr);
+        if (st != TT_ERR_OOM) return st;
+    }
+    TT_TRY(scratch.ensure(split_scratch(prod_tiles(n, n, 1), prod_split(n, n, std::max(m, 1), 1)), s));
+    return gram_fixed_scratch(s, m, n, A, lda, G, ldg, scratch.p, scratch.cap);
+}
+
+// ------------------------------------------------------------ captured steps
+
+// Doubles of partials (and counters, where the handle's are too few) that a
+// captured product of sizes up to these may use.
 size_t dyn_partials_need(int mode, int Mcap, int Ncap, int Kcap) {
-    // prod_limit: a split product has at most SPLIT_ITEMS items
-    return Mcap > 0 && Ncap > 0 && Kcap > BK ? (size_t)SPLIT_ITEMS * BT * BT : 0;
+    if (mode == 0 || Mcap <= 0 || Ncap <= 0 || Kcap <= 0) return 0;
+    size_t most = 0;
+    if (mode == 2) {
+        for (int n = 1; n <= Ncap; ++n)
+            most = std::max(most, split_doubles(prod_tiles(n, n, 1), gram_split_rule(Kcap, n, gram_resident())));
+    } else {
+        // sk_split's split is not monotone in K (the chunk is rounded), so
+        // bound it: below 152 64 x 64 tiles ceil(304 / tiles), the tuned entries
+        // of every K bucket up to Kcap, 64, or ceil(Kcap / 16)
+        const int TMc = (Mcap + 63) / 64, TNc = (Ncap + 63) / 64, kbmax = floor_log2(Kcap);
+        for (int tm = 1; tm <= TMc; ++tm)
+            for (int tn = 1; tn <= TNc && (long)tm * tn < 152; ++tn) {
+                const long tiles = (long)tm * tn;
+                long ks = (304 + tiles - 1) / tiles;
+                const int tb = floor_log2(tiles);
+                for (int kb = 0; tb < AT_TILE_BUCKETS && kb <= kbmax && kb < AT_K_BUCKETS; ++kb)
+                    ks = std::max<long>(ks, h_sk_table[tb * AT_K_BUCKETS + kb]);
+                ks = std::min(std::min(ks, 64L), (long)(Kcap + BK - 1) / BK);
+                most = std::max(most, split_doubles(tiles * 16, (int)ks));
+            }
+    }
+    const long tiles = prod_tiles(Mcap, Ncap, mode == 2);
+    return most + (tiles > PROD_COUNTERS ? (size_t)(tiles + 1) / 2 : 0);
 }
 
 tt_status dgemm_dyn(cudaStream_t s, bool ta, bool tb, const int* desc, int Mcap, int Ncap, int Kcap,
                     double alpha, const double* A, const double* B, double* C, double* P, size_t pcap, int mode,
-                    DevBuf& tcbuf, int* status_dev, int* counters) {
+                    DevBuf& tcbuf, const ProdCtx& ctx) {
     if (Mcap <= 0 || Ncap <= 0) return TT_OK;
     const int tri = mode == 2 ? 1 : 0;
-    const int tc = tc8_wanted(Mcap, Ncap, Kcap) ? 1 : 0;
-    if (tc) TT_TRY(tc8_dyn(s, ta, tb, desc, Mcap, Ncap, Kcap, alpha, A, B, C, tcbuf, status_dev, mode == 2));
-    if (dyn_partials_need(mode, Mcap, Ncap, Kcap) > pcap) {
+    const int tc = ctx.digits && tc8_wanted(Mcap, Ncap, Kcap) ? 1 : 0;
+    if (tc) TT_TRY(tc8_dyn(s, ta, tb, desc, Mcap, Ncap, Kcap, alpha, A, B, C, tcbuf, ctx.status, mode == 2));
+    const size_t need = dyn_partials_need(mode, Mcap, Ncap, Kcap);
+    if (need > pcap) {
         set_error("dgemm: the partials buffer of a captured product is smaller than its split needs");
         return TT_ERR_TOO_LARGE;
     }
-    // four CTAs an SM, or fewer where the capacity has no more items, walk
-    // whatever the device's sizes give
-    return launch_prod(s, ta, tb, 0, 0, 0, alpha, A, 0, B, 0, 0.0, C, 0, 1, P, counters, tri, desc, tc,
-                       std::min(152L * 4, prod_tiles(Mcap, Ncap, tri) * MAX_SPLIT));
+    const long tiles = prod_tiles(Mcap, Ncap, tri);
+    int* cnt = ctx.counters;
+    if (mode != 0 && tiles > PROD_COUNTERS) {
+        cnt = reinterpret_cast<int*>(P + need - (tiles + 1) / 2);
+        TT_CUDA_TRY(cudaMemsetAsync(cnt, 0, (size_t)tiles * sizeof(int), s));
+    }
+    // eight CTAs an SM, or fewer where the capacity has no more items, walk
+    // whatever the device's sizes give; mode 0 does not split
+    ProdArgs a{0, 0, 0, alpha, A, 0, B, 0, 0.0, C, 0, 1, 0, mode == 0 ? nullptr : P, cnt, tri, desc, tc};
+    return launch_prod(s, ta, tb, true, std::min(152L * 8, tiles * 64), a);
 }
 
 void scale_rows_dyn(cudaStream_t s, const int* desc, long total_cap, const double* in, const double* v, int mode,
@@ -465,17 +654,6 @@ void scale_rows_dyn(cudaStream_t s, const int* desc, long total_cap, const doubl
     if (total_cap <= 0) return;
     note_launch();
     scale_rows_dyn_kernel<<<grid_for(total_cap), 256, 0, s>>>(desc, in, v, mode, out);
-}
-
-tt_status gram(cudaStream_t s, int m, int n, const double* A, long lda, double* G, long ldg,
-               DevBuf& partials, int* status_dev, int* counters) {
-    if (n <= 0) return TT_OK;
-    if (tc8_wanted(n, n, m)) {
-        const tt_status st = tc8_gram(s, m, n, A, lda, G, ldg, partials, status_dev);
-        if (st != TT_ERR_OOM) return st;
-    }
-    TT_TRY(partials.ensure(gram_scratch_doubles(m, n), s));
-    return gram_fixed_scratch(s, m, n, A, lda, G, ldg, partials.p, partials.cap, counters);
 }
 
 void scale_rows(cudaStream_t s, int rows, int cols, const double* in, long ldi, const double* v,
@@ -565,7 +743,7 @@ tt_status autotune(cudaStream_t s, int* table_out) {
     const long Mmax = 64L << ((AT_TILE_BUCKETS - 1) / 2), Nmax = 64L << (AT_TILE_BUCKETS - 1 - (AT_TILE_BUCKETS - 1) / 2);
     const long Kmax = 1L << KB_MAX;
     double *A = nullptr, *B = nullptr, *C = nullptr, *P = nullptr;
-    const size_t pdbl = (size_t)SPLIT_ITEMS * BT * BT;
+    const size_t pdbl = (size_t)64 * Mmax * Nmax;
     int* cnt = nullptr;
     cudaEvent_t e0 = nullptr, e1 = nullptr;
     tt_status st = TT_OK;
@@ -583,8 +761,8 @@ tt_status autotune(cudaStream_t s, int* table_out) {
         cudaMallocAsync((void**)&B, Kmax * Nmax * sizeof(double), s) != cudaSuccess ||
         cudaMallocAsync((void**)&C, Mmax * Nmax * sizeof(double), s) != cudaSuccess ||
         cudaMallocAsync((void**)&P, pdbl * sizeof(double), s) != cudaSuccess ||
-        cudaMallocAsync((void**)&cnt, SPLIT_ITEMS * sizeof(int), s) != cudaSuccess ||
-        cudaMemsetAsync(cnt, 0, SPLIT_ITEMS * sizeof(int), s) != cudaSuccess ||
+        cudaMallocAsync((void**)&cnt, PROD_COUNTERS * sizeof(int), s) != cudaSuccess ||
+        cudaMemsetAsync(cnt, 0, PROD_COUNTERS * sizeof(int), s) != cudaSuccess ||
         cudaEventCreate(&e0) != cudaSuccess || cudaEventCreate(&e1) != cudaSuccess) {
         (void)cudaGetLastError();
         cleanup();
@@ -600,12 +778,15 @@ tt_status autotune(cudaStream_t s, int* table_out) {
             float best = 1e30f;
             int best_ks = 0;
             for (int ks = 1; ks <= 64 && ks <= std::max(1, K / (2 * BK)); ks *= 2) {
-                const int kk = prod_final(K, std::min(ks, prod_limit(prod_tiles(M, N, 0), K)));
+                int kchunk = (K + ks - 1) / ks;
+                kchunk = (kchunk + BK - 1) / BK * BK;
+                const int kk = (K + kchunk - 1) / kchunk;
                 float t = 1e30f;
                 for (int rep = 0; rep < 3; ++rep) {
                     cudaEventRecord(e0, s);
-                    st = launch_prod(s, false, false, M, N, K, 1.0, A, K, B, N, 0.0, C, N, kk, P, cnt, 0, nullptr, 0,
-                                     prod_tiles(M, N, 0) * kk);
+                    st = launch_prod(s, false, false, true, prod_tiles(M, N, 0) * kk,
+                                     ProdArgs{M, N, K, 1.0, A, K, B, N, 0.0, C, N, kk, kk > 1 ? kchunk : K, P, cnt, 0,
+                                              nullptr, 0});
                     cudaEventRecord(e1, s);
                     if (st < 0 || cudaEventSynchronize(e1) != cudaSuccess) {
                         if (st >= 0) st = TT_ERR_CUDA;

@@ -75,18 +75,27 @@ tt_status dgemm(cudaStream_t s, bool ta, bool tb, int M, int N, int K, double al
                 const double* A, long lda, const double* B, long ldb, double beta, double* C,
                 long ldc);
 
-// beta = 0 product: from digits (digits.cu) where tc8_wanted, else on the FP64
-// pipe with K split over CTAs by prod_split's rule.  counters (nullable):
-// SPLIT_ITEMS ints that are zero between products of one stream; without
-// them the arrival counters lie in scratch and cost a memset.
-constexpr long SPLIT_ITEMS = 4096;  // (tile, split) items of a split product, at most
-constexpr size_t SPLIT_DOUBLES = (256 + 1) * SPLIT_ITEMS;  // and its scratch
+// What a handle's products share: the device status word, PROD_COUNTERS arrival
+// counters (zero between products of the handle's stream; null: in the
+// product's scratch, for a memset) and whether digit products are taken.  The
+// problems of a batch do without: side by side they fill the FP64 pipes, and
+// 16 captured problems gained nothing from the digits' launches.
+constexpr long PROD_COUNTERS = 1 << 14;
+struct ProdCtx {
+    int* status = nullptr;
+    int* counters = nullptr;
+    bool digits = true;
+};
+// beta = 0 product of a rounding: from digits (digits.cu) where tc8_wanted,
+// else on the FP64 pipe, K split over CTAs by sk_split's rule (split) or not.
 tt_status dgemm_sk(cudaStream_t s, bool ta, bool tb, int M, int N, int K, double alpha,
                    const double* A, long lda, const double* B, long ldb, double* C, long ldc,
-                   DevBuf& scratch, int* status_dev = nullptr, int* counters = nullptr);
-
-// Scratch that a dgemm_sk of these sizes uses (0: none).
-size_t dgemm_sk_scratch_doubles(int M, int N, int K);
+                   DevBuf& scratch, const ProdCtx& ctx, bool split = true);
+// The same of a library call: the order of summation is free, the split the
+// cheapest.  Scratch of gemm_call_doubles.
+size_t gemm_call_doubles(int M, int N, int K);
+tt_status gemm_call(cudaStream_t s, bool ta, bool tb, int M, int N, int K, double alpha, const double* A, long lda,
+                    const double* B, long ldb, double* C, long ldc, DevBuf& scratch);
 
 // Autotuned split table (gemm.cu): buckets of floor(log2 tiles) < 8 and
 // floor(log2 K) < 22; autotune measures and installs it, autotune_install
@@ -96,30 +105,38 @@ tt_status autotune(cudaStream_t s, int* table_out);
 tt_status autotune_install(const int* table, int n);
 void autotune_read(int* table);
 
+// The split rules of the rounding's products (of K) and of its Gram (of the
+// rows, from the resident 64 x 64 tiles), shared by host and device.
+__host__ __device__ void sk_split(int M, int N, int K, int* ks_out, int* kchunk_out);
+__host__ __device__ int gram_split_rule(int m, int n, long resident);
+// splits of a large Gram dealt in many waves (gram_split_rule)
+constexpr int GRAM_MULTI_SPLITS = 64;
+
 // Products of a captured step, their sizes read from device memory: desc =
 // M, N, K, lda, ldb, ldc (Gram: n, n, m, lda, lda, ldg with A m x n), caps
-// bound every size the step can reach.  mode 1: dgemm_sk; 2: the Gram
-// G = A^T A.  The same split rules from the same sizes, so the same bits as
-// the host path.  P holds pcap doubles, at least dyn_partials_need (checked:
-// TT_ERR_TOO_LARGE); tcbuf: scratch of tc8_dyn, reserved ahead of the capture;
-// counters as in dgemm_sk.
+// bound every size the step can reach.  mode 0: dgemm_sk without a split; 1:
+// dgemm_sk; 2: the Gram G = A^T A.  The same bits as the host path for the
+// same sizes.  P holds pcap doubles, at least dyn_partials_need (checked:
+// TT_ERR_TOO_LARGE); tcbuf: scratch of tc8_dyn, reserved ahead of the capture.
 tt_status dgemm_dyn(cudaStream_t s, bool ta, bool tb, const int* desc, int Mcap, int Ncap, int Kcap,
                     double alpha, const double* A, const double* B, double* C, double* P, size_t pcap, int mode,
-                    DevBuf& tcbuf, int* status_dev, int* counters);
+                    DevBuf& tcbuf, const ProdCtx& ctx);
 size_t dyn_partials_need(int mode, int Mcap, int Ncap, int Kcap);
 // scale_rows with rows, cols, ldi, ldo = desc[0..3] (rows * cols <= total_cap)
 void scale_rows_dyn(cudaStream_t s, const int* desc, long total_cap, const double* in, const double* v, int mode,
                     double* out);
 
-// G = A^T A (A: m x n row-major, lda), as dgemm_sk: from digits or on the FP64
-// pipe split over rows.  partials is scratch grown as needed.
+// G = A^T A (A: m x n row-major, lda) of a rounding, as dgemm_sk with the rows
+// split by gram_split_rule.  partials is scratch grown as needed.
 tt_status gram(cudaStream_t s, int m, int n, const double* A, long lda, double* G, long ldg,
-               DevBuf& partials, int* status_dev = nullptr, int* counters = nullptr);
-size_t gram_scratch_doubles(int m, int n);
-// The FP64-pipe Gram in a fixed scratch: fewer splits where the partials would
-// not fit in scratch_doubles.
+               DevBuf& partials, const ProdCtx& ctx);
+// The same of a library call (as gemm_call), and on the FP64 pipe in a fixed
+// scratch: fewer splits where the partials would not fit in scratch_doubles.
+size_t gram_scratch_doubles(int m, int n);  // of gram on the FP64 pipe
+size_t gram_call_doubles(int m, int n);
+tt_status gram_call(cudaStream_t s, int m, int n, const double* A, long lda, double* G, long ldg, DevBuf& scratch);
 tt_status gram_fixed_scratch(cudaStream_t s, int m, int n, const double* A, long lda, double* G,
-                             long ldg, double* scratch, size_t scratch_doubles, int* counters = nullptr);
+                             long ldg, double* scratch, size_t scratch_doubles);
 // Measured FP64 tensor-pipe throughput (TFLOP/s).
 tt_status bench_fp64_mma(cudaStream_t s, double* tflops);
 // Measured BF16 mma.sync (m16n8k16, FP32 accumulate) throughput (TFLOP/s).
@@ -149,8 +166,8 @@ tt_status slgemm_nt(cudaStream_t s, long M, int N, int K, const double* A, long 
 // ---------------------------------------------------------------- FP64 products on tensor cores (digits.cu)
 // C = alpha op(A) op(B) and G = A^T A (A m x n) from exact integer digit
 // products: every sum exact, one rounding an entry (the header of digits.cu).
-// tc8_wanted is the rule by which dgemm_sk, gram and their captured forms
-// take it, from the sizes alone.  Below 16M terms (32 us of the FP64 pipe)
+// tc8_wanted is the rule by which dgemm_sk, gram, their captured forms and the
+// library calls take it, from the sizes alone.  Below 16M terms (32 us of the FP64 pipe)
 // the five or six launches cost more than they save; a contraction under 64
 // would not be rounded less often than the FP64 sum it replaces; the 64-bit
 // sums hold 2^26 indices.
@@ -247,6 +264,9 @@ tt_status syev_dyn(cudaStream_t s, const int* n_dev, int ncap, const double* G, 
 // failed factorisation, counts as zero)
 void truncation_decision_dyn(cudaStream_t s, const double* lamK, const int* kB_dev, double eps, int dm1,
                              int forced, int max_rank, double* delta2_dev, int* dec_i, double* dec_d);
+
+// A handle of a batch: as tt_create, its products without digits (ProdCtx).
+tt_status create_in_batch(const tt_problem_desc* desc, void* stream, tt_handle* out);
 
 // Captured steps of one handle (api.cu): graph_steps_begin checks the
 // conditions and launches nsteps replays without waiting; graph_steps_end
