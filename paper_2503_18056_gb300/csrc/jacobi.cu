@@ -490,24 +490,13 @@ __device__ __forceinline__ void osj_norms(const double* W, int n, int k, double*
     }
 }
 
-// The round barrier: the whole grid (bounded spin, DEV_TIMEOUT on expiry) or,
-// for a launch of one thread-block cluster, the hardware cluster barrier.
-template <bool CLUSTER>
-__device__ __forceinline__ bool osj_barrier(int* ctrl, int* status, unsigned& epoch) {
-    if (CLUSTER) {
-        cooperative_groups::this_cluster().sync();
-        return true;
-    }
-    return grid_barrier(ctrl, status, gridDim.x, epoch);
-}
-
-template <int C, bool CLUSTER>
+template <int C>
 __global__ void __launch_bounds__(32 * OSJ_MAX_WARPS)
 osj_kernel(int n, const int* __restrict__ k_dev, double* W, double* nrm, double* lam_u, double* vt_u, int* ctrl,
-           int* status, int max_sweeps, const int* n_dev) {
-    if (n_dev) {  // a captured step: sizes up to OSJ_CLUSTER_N take the cluster launch, larger the grid
+           int* status, int max_sweeps, const int* n_dev, int nsmall) {
+    if (n_dev) {  // a captured step: sizes up to nsmall take the cluster launch
         n = *n_dev;
-        if (CLUSTER ? n > OSJ_CLUSTER_N : n <= OSJ_CLUSTER_N) return;  // every CTA, before any barrier
+        if (n <= nsmall) return;  // every CTA, before any barrier
     }
     // relative skip threshold sqrt(n) eps_mach, the one of LAPACK's one-sided
     // Jacobi SVD (dgesvj): the typical rounding error of a computed inner
@@ -537,7 +526,7 @@ osj_kernel(int n, const int* __restrict__ k_dev, double* W, double* nrm, double*
             // norms summed afresh at every sweep: the updates inside a sweep
             // only steer the angles and the skip test
             osj_norms(W, n, k, nrm, gw, nw, lane);
-            if (!osj_barrier<CLUSTER>(ctrl, status, epoch)) return;
+            if (!grid_barrier(ctrl, status, gridDim.x, epoch)) return;
             int mine = 0;
             for (int r = 0; r < N - 1; ++r) {
                 for (int kk = gw; kk < npairs; kk += nw) {
@@ -551,7 +540,7 @@ osj_kernel(int n, const int* __restrict__ k_dev, double* W, double* nrm, double*
                     __syncthreads();
                     if (threadIdx.x == 0) atomicAdd(ctrl + 4 + sweep, s_cnt);
                 }
-                if (!osj_barrier<CLUSTER>(ctrl, status, epoch)) return;
+                if (!grid_barrier(ctrl, status, gridDim.x, epoch)) return;
             }
             if (threadIdx.x == 0) s_done = (atomicAdd(ctrl + 4 + sweep, 0) == 0);
             __syncthreads();
@@ -564,7 +553,7 @@ osj_kernel(int n, const int* __restrict__ k_dev, double* W, double* nrm, double*
     }
     // eigenvalues: the converged rows' squared norms, summed from the rows
     osj_norms(W, n, k, nrm, gw, nw, lane);
-    if (!osj_barrier<CLUSTER>(ctrl, status, epoch)) return;
+    if (!grid_barrier(ctrl, status, gridDim.x, epoch)) return;
     for (int i = gw; i < n; i += nw) {
         const double a = i < k ? __ldcg(nrm + i) : 0.0;
         const double f = a > 0.0 ? 1.0 / sqrt(a) : 0.0;
@@ -572,6 +561,265 @@ osj_kernel(int n, const int* __restrict__ k_dev, double* W, double* nrm, double*
         const double* wi = W + (long)i * n;
         for (int j = lane; j < n; j += 32) vt_u[(long)i * n + j] = i < k ? f * __ldcg(wi + j) : 0.0;
     }
+}
+
+// Up to OSJ_CLUSTER_N rows on one thread-block cluster: the same rotations in the
+// same order and arithmetic (bit for bit the grid kernel's with C = ceil(n / 32)),
+// laid out for what bounds it on GB300, FP64 issue (64 clocks a warp
+// instruction and SM sub-partition, about 600 for a square root or a division)
+// and the latency of a round:
+// - The rows never leave the SMs.  A warp (G = 1) or half a warp (G = 2) holds a
+//   pair's rows in registers and after the round sends each into the shared
+//   memory of the warp that needs it next: two short remote stores and one
+//   hardware cluster barrier a round, no trip to L2.  The pairs are
+//   round_pair's: slot 0 holds the last row, which stays, and row r; slot k rows
+//   r + k (first) and r - k (second); from round to round the first rows move
+//   down a slot, the second rows up one, and the ends turn.
+// - Above 128 rows two pairs share a warp, so that no sub-partition has a second
+//   warp and the scalar chain of the angle serves both.
+// - The skip test compares exponents and forms tol sqrt(a b) only within a few
+//   binades of it; an angle with |tau| >= 2^28 needs neither square root, where
+//   sqrt(1 + tau^2) = |tau| and sqrt(1 + t^2) = 1 exactly (the two roundings stay
+//   within half an ulp of tau: relative errors 2^-54 / m^2 + 2^-57 against 2^-53 /
+//   m for a significand m below sqrt 2, 2^-53 / m^2 + 2^-57 above).
+// Measured (GB300, factorisation included): n = 61 2.9 -> 1.9 ms, 128 6.5 ->
+// 4.8, 163 11.1 -> 10.3, 256 23.8 -> 18.8 for a graded full-rank matrix; the
+// 16-problem captured batch 20.5 -> 16.5 ms.
+// inbox: [slot of this CTA][parity][first, second][32 C entries], then the rows'
+// squared norms and indices.
+struct OsjMeta {
+    double nrm;
+    int idx, pad;
+};
+
+// 2 log2|c| against log2(tol^2 a b): +1 certainly above, -1 certainly below, 0 close
+__device__ __forceinline__ int osj_far(double c, double a, double b, double tol) {
+    auto ex = [](double v) { return (int)((__double2hiint(v) >> 20) & 0x7FF); };
+    const int ec = ex(c), ea = ex(a), eb = ex(b), et = ex(tol);
+    if (ec == 0 || ea == 0 || eb == 0 || ec == 0x7FF || ea == 0x7FF || eb == 0x7FF) return 0;
+    // c^2 in [2^(2 ec), 2^(2 ec + 2)), tol^2 a b in [2^s, 2^(s + 4)) (biases: 2 and 4)
+    const int s = 2 * et + ea + eb - 2 * 1023;
+    if (abs(ea + eb - 2 * 1023) > 1000) return 0;  // a b near the range's ends
+    return 2 * ec >= s + 5 ? 1 : (2 * ec + 2 <= s - 1 ? -1 : 0);
+}
+
+template <int C, int G>
+__device__ void osj_cluster_body(int n, int k, const double* W, double* lam_u, double* vt_u, int* ctrl, int* status,
+                                 int max_sweeps, double tol, double* inbox) {
+    namespace cg = cooperative_groups;
+    cg::cluster_group cl = cg::this_cluster();
+    constexpr int E = C * G;       // entries of a row a lane holds
+    constexpr int ROW = 32 * C;    // doubles of a row
+    constexpr int LANES = 32 / G;  // lanes of a pair
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, wpb = blockDim.x >> 5;
+    const int l = lane % LANES, spc = wpb * G;  // slots of a CTA
+    const int ls = warp * G + lane / LANES, slot = blockIdx.x * spc + ls;
+    const int N = k + (k & 1), S = N / 2;
+    const bool active = slot < S;
+    OsjMeta* meta = reinterpret_cast<OsjMeta*>(inbox + (size_t)spc * 4 * ROW);
+    // entry e of lane l: column l + 32 e (G = 1), or l + 16 (e % 2) + 32 (e / 2)
+    auto col = [&](int e) { return G == 1 ? l + 32 * e : l + 16 * (e & 1) + 32 * (e >> 1); };
+    // the 32 column classes' partials (p0: class l, p1: class l + 16) summed as
+    // a butterfly over 32 lanes sums them
+    auto sum = [&](double p0, double p1) {
+        double v = G == 1 ? p0 : p0 + p1;
+#pragma unroll
+        for (int o = LANES / 2; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+        return v;
+    };
+    double x[E], y[E];
+    auto norm2 = [&](const double (&v)[E]) {
+        double p[2] = {0.0, 0.0};
+#pragma unroll
+        for (int e = 0; e < E; ++e) p[G == 1 ? 0 : (e & 1)] = fma(v[e], v[e], p[G == 1 ? 0 : (e & 1)]);
+        return sum(p[0], p[1]);
+    };
+    // x: the row of the smaller index; sw: it is the slot's second row
+    int ix = 0, iy = 0;
+    bool sw = false;
+    double a = 0.0, b = 0.0;
+    {
+        const int i0 = slot == 0 ? N - 1 : slot, i1 = slot == 0 ? 0 : N - 1 - slot;  // round 0
+        sw = i1 < i0;
+        ix = min(i0, i1);
+        iy = max(i0, i1);
+#pragma unroll
+        for (int e = 0; e < E; ++e) {
+            const int j = col(e);
+            x[e] = active && ix < k && j < n ? __ldcg(W + (long)ix * n + j) : 0.0;
+            y[e] = active && iy < k && j < n ? __ldcg(W + (long)iy * n + j) : 0.0;
+        }
+    }
+    // where the slot's rows go after a round
+    double *to0 = nullptr, *to1 = nullptr;
+    OsjMeta *me0 = nullptr, *me1 = nullptr;
+    if (active && S > 1) {
+        const int ds0 = slot == 0 ? 0 : slot - 1, dw0 = slot == 1 ? 1 : 0;
+        const int ds1 = slot == S - 1 ? slot : slot + 1, dw1 = slot != 0 && slot == S - 1 ? 0 : 1;
+        to0 = cl.map_shared_rank(inbox, ds0 / spc) + ((size_t)(ds0 % spc) * 4 + dw0) * ROW;
+        to1 = cl.map_shared_rank(inbox, ds1 / spc) + ((size_t)(ds1 % spc) * 4 + dw1) * ROW;
+        me0 = cl.map_shared_rank(meta, ds0 / spc) + (ds0 % spc) * 4 + dw0;
+        me1 = cl.map_shared_rank(meta, ds1 / spc) + (ds1 % spc) * 4 + dw1;
+    }
+    cl.sync();  // every CTA of the cluster runs before its shared memory is written
+    int sweep = 0;
+    bool done = k < 2;
+    for (; sweep < max_sweeps && !done; ++sweep) {
+        // norms summed afresh at every sweep: the updates inside a sweep only
+        // steer the angles and the skip test
+        a = norm2(x);
+        b = norm2(y);
+        int mine = 0;
+        for (int r = 0; r < N - 1; ++r) {
+            const int par = r & 1;
+            {
+                double c0[2] = {0.0, 0.0}, c1[2] = {0.0, 0.0};  // even and odd steps of 32 columns
+#pragma unroll
+                for (int e = 0; e < E; ++e) {
+                    const int t = G == 1 ? e : e >> 1, h = G == 1 ? 0 : (e & 1);
+                    if (t & 1)
+                        c1[h] = fma(x[e], y[e], c1[h]);
+                    else
+                        c0[h] = fma(x[e], y[e], c0[h]);
+                }
+                const double c = sum(c0[0] + c1[0], c0[1] + c1[1]);
+                bool rot = false;
+                if (active && iy < k && a > 0.0 && b > 0.0) {
+                    const int far = osj_far(c, a, b, tol);
+                    rot = far > 0 || (far == 0 && fabs(c) > tol * sqrt(a * b));
+                }
+                if (__any_sync(0xffffffffu, rot)) {
+                    // Golub & Van Loan, Alg. 8.4.1 on [[a, c], [c, b]]
+                    const double tau = (b - a) / (2.0 * c);
+                    double t, cs, sn;
+                    if (__all_sync(0xffffffffu, !rot || (fabs(tau) >= 268435456.0 && fabs(tau) < 1e150))) {
+                        t = (tau >= 0.0 ? 1.0 : -1.0) / (fabs(tau) + fabs(tau));
+                        cs = 1.0;
+                        sn = t;
+                    } else {
+                        t = (tau >= 0.0 ? 1.0 : -1.0) / (fabs(tau) + sqrt(1.0 + tau * tau));
+                        cs = 1.0 / sqrt(1.0 + t * t);
+                        sn = t * cs;
+                    }
+                    // the rotation moves t c from one squared norm to the other: the
+                    // growing one is updated by that sum (no cancellation), the
+                    // shrinking one is summed again from the rotated row
+                    const bool p_shrinks = t * c > 0.0;
+                    double ns[2] = {0.0, 0.0};
+#pragma unroll
+                    for (int e = 0; e < E; ++e) {
+                        const int h = G == 1 ? 0 : (e & 1);
+                        const double xn = cs * x[e] - sn * y[e];
+                        const double yn = sn * x[e] + cs * y[e];
+                        if (rot) {
+                            x[e] = xn;
+                            y[e] = yn;
+                        }
+                        const double v = p_shrinks ? xn : yn;
+                        ns[h] = fma(v, v, ns[h]);
+                    }
+                    const double nv = sum(ns[0], ns[1]);
+                    if (rot) {
+                        const double an = p_shrinks ? nv : a - t * c;
+                        b = p_shrinks ? b + t * c : nv;
+                        a = an;
+                        ++mine;
+                    }
+                }
+            }
+            if (active && S > 1) {
+                double *o0 = (sw ? to1 : to0) + par * 2 * ROW, *o1 = (sw ? to0 : to1) + par * 2 * ROW;
+#pragma unroll
+                for (int e = 0; e < E; ++e) {
+                    o0[col(e)] = x[e];
+                    o1[col(e)] = y[e];
+                }
+                if (l == 0) {
+                    OsjMeta *m0 = (sw ? me1 : me0) + par * 2, *m1 = (sw ? me0 : me1) + par * 2;
+                    m0->nrm = a;
+                    m0->idx = ix;
+                    m1->nrm = b;
+                    m1->idx = iy;
+                }
+            }
+            if (r == N - 2 && l == 0 && mine) atomicAdd(ctrl + 4 + sweep, mine);
+            cl.sync();
+            if (active && S > 1) {
+                const OsjMeta* m = meta + ls * 4 + par * 2;
+                const int i0 = m[0].idx, i1 = m[1].idx;
+                sw = i1 < i0;
+                ix = min(i0, i1);
+                iy = max(i0, i1);
+                a = m[sw ? 1 : 0].nrm;
+                b = m[sw ? 0 : 1].nrm;
+                const double* in = inbox + ((size_t)ls * 4 + par * 2) * ROW;
+                const double *f0 = in + (sw ? ROW : 0), *f1 = in + (sw ? 0 : ROW);
+#pragma unroll
+                for (int e = 0; e < E; ++e) {
+                    x[e] = f0[col(e)];
+                    y[e] = f1[col(e)];
+                }
+            }
+        }
+        // N - 1 rounds, an odd number: the next sweep writes parity 0, just read
+        done = __ldcg(ctrl + 4 + sweep) == 0;
+        cl.sync();
+    }
+    if (blockIdx.x == 0 && threadIdx.x == 0) {
+        ctrl[2] = k >= 2 ? sweep : 0;
+        if (!done) atomicOr(status, DEV_NOT_CONVERGED);
+    }
+    // eigenvalues: the converged rows' squared norms, summed from the rows
+    a = norm2(x);
+    b = norm2(y);
+    auto put = [&](int i, double nn, const double (&v)[E]) {
+        if (!active || i >= k) return;
+        const double f = nn > 0.0 ? 1.0 / sqrt(nn) : 0.0;
+        if (l == 0) lam_u[i] = nn;
+#pragma unroll
+        for (int e = 0; e < E; ++e)
+            if (col(e) < n) vt_u[(long)i * n + col(e)] = f * v[e];
+    };
+    put(ix, a, x);
+    put(iy, b, y);
+    for (int i = k + blockIdx.x * wpb + warp; i < n; i += gridDim.x * wpb) {
+        if (lane == 0) lam_u[i] = 0.0;
+        for (int j = lane; j < n; j += 32) vt_u[(long)i * n + j] = 0.0;
+    }
+}
+
+__global__ void __launch_bounds__(32 * OSJ_MAX_WARPS)
+osj_cluster_kernel(int n, const int* __restrict__ k_dev, const double* W, double* lam_u, double* vt_u, int* ctrl,
+                   int* status, int max_sweeps, const int* n_dev, int nsmall) {
+    if (n_dev) {  // a captured step: larger sizes take the grid kernel
+        n = *n_dev;
+        if (n > nsmall) return;  // every CTA, before any barrier
+    }
+    extern __shared__ double osj_inbox[];
+    const double tol = sqrt((double)n) * 2.220446049250313e-16;  // as in osj_kernel
+    const int kraw = *k_dev;
+    if (kraw < 0) {
+        const int wpb = blockDim.x >> 5, lane = threadIdx.x & 31;
+        for (int i = blockIdx.x * wpb + (threadIdx.x >> 5); i < n; i += gridDim.x * wpb) {
+            if (lane == 0) lam_u[i] = __longlong_as_double(0x7ff8000000000000LL);
+            for (int j = lane; j < n; j += 32) vt_u[(long)i * n + j] = 0.0;
+        }
+        return;
+    }
+    const int k = min(kraw, n);
+#define OSJ_BODY(C, G) osj_cluster_body<C, G>(n, k, W, lam_u, vt_u, ctrl, status, max_sweeps, tol, osj_inbox)
+    switch ((n + 31) / 32) {
+        case 0:
+        case 1: OSJ_BODY(1, 1); break;
+        case 2: OSJ_BODY(2, 1); break;
+        case 3: OSJ_BODY(3, 1); break;
+        case 4: OSJ_BODY(4, 1); break;
+        case 5: OSJ_BODY(5, 2); break;
+        case 6: OSJ_BODY(6, 2); break;
+        case 7: OSJ_BODY(7, 2); break;
+        default: OSJ_BODY(8, 2); break;
+    }
+#undef OSJ_BODY
 }
 
 // Pivoted Cholesky on one thread-block cluster for n <= PCHOL_SMALL_N: the
@@ -1173,20 +1421,21 @@ tt_status osj_launch(cudaStream_t s, int ncap, const int* k_dev, EigWork& w, int
     double* vtu = w.vt_unsorted.p;
     int* ctrl = w.d_ctrl;
     int msw = max_sweeps;
-    if (ncap <= OSJ_CLUSTER_N || n_dev) {
-        // one cluster: a round ends at a hardware cluster barrier instead of a
-        // grid-wide one; its CL SMs hold up to OSJ_MAX_WARPS pairs each.  A
-        // captured step launches it for sizes up to OSJ_CLUSTER_N and the
-        // grid kernel after it for larger ones (each returns at once
-        // outside its range), so a replay takes the host path's kernel.
-        const int ncl = std::min(ncap, OSJ_CLUSTER_N);
-        const int cl = cluster_size_for((const void*)osj_kernel<8, true>, 32 * OSJ_MAX_WARPS);
-        const int npairs = (ncl + 1) / 2;
-        const int wpb = std::max(1, std::min(OSJ_MAX_WARPS, (npairs + cl - 1) / cl));
+    int nsmall = OSJ_CLUSTER_N;
+    if (ncap <= nsmall || n_dev) {
+        // one cluster, a warp per pair up to 128 rows, two pairs a warp above.
+        // A captured step launches it for sizes up to nsmall and the grid
+        // kernel after it for larger ones (each returns at once outside its
+        // range), so a replay takes the host path's kernel.
+        const int ncl = std::min(ncap, nsmall);
+        const int cl = cluster_size_for((const void*)osj_cluster_kernel, 32 * OSJ_MAX_WARPS);
+        const int np1 = (std::min(ncl, 128) + 1) / 2, np2 = (ncl + 3) / 4;
+        const int wpb = std::max(1, std::max((np1 + cl - 1) / cl, ncl > 128 ? (np2 + cl - 1) / cl : 0));
+        const int C = (ncl + 31) / 32, spc = wpb * (ncl > 128 ? 2 : 1);
         cudaLaunchConfig_t cfg = {};
         cfg.gridDim = dim3(cl);
         cfg.blockDim = dim3(32 * wpb);
-        cfg.dynamicSmemBytes = 0;
+        cfg.dynamicSmemBytes = (size_t)spc * 4 * (32 * C * sizeof(double) + sizeof(OsjMeta));
         cfg.stream = s;
         cudaLaunchAttribute at[1];
         at[0].id = cudaLaunchAttributeClusterDimension;
@@ -1196,14 +1445,14 @@ tt_status osj_launch(cudaStream_t s, int ncap, const int* k_dev, EigWork& w, int
         cfg.attrs = at;
         cfg.numAttrs = 1;
         note_launch();
-        TT_CUDA_TRY(cudaLaunchKernelEx(&cfg, osj_kernel<8, true>, nn, k_dev, Wp, nrm, lamu, vtu, ctrl, status_dev,
-                                       msw, n_dev));
-        if (ncap <= OSJ_CLUSTER_N) return TT_OK;
+        TT_CUDA_TRY(cudaLaunchKernelEx(&cfg, osj_cluster_kernel, nn, k_dev, (const double*)Wp, lamu, vtu, ctrl,
+                                       status_dev, msw, n_dev, nsmall));
+        if (ncap <= nsmall) return TT_OK;
     }
     // rows in registers up to n = 1024 (entries per lane: 8, 16 or 32)
-    const void* fn = ncap <= 256 ? (const void*)osj_kernel<8, false>
-                     : ncap <= 512 ? (const void*)osj_kernel<16, false>
-                     : ncap <= 1024 ? (const void*)osj_kernel<32, false> : (const void*)osj_kernel<0, false>;
+    const void* fn = ncap <= 512    ? (const void*)osj_kernel<16>
+                     : ncap <= 1024 ? (const void*)osj_kernel<32>
+                                    : (const void*)osj_kernel<0>;
     // one CTA per SM with one warp per pair it owns, so every SM carries the
     // same number of pairs in a round (the round ends at the slowest SM)
     int blocks = 1, wpb = 1;
@@ -1220,7 +1469,7 @@ tt_status osj_launch(cudaStream_t s, int ncap, const int* k_dev, EigWork& w, int
         }
         blocks = std::max(1, std::min((npairs + wpb - 1) / wpb, per_sm * sms));
     }
-    void* args[] = {&nn, &k_dev, &Wp, &nrm, &lamu, &vtu, &ctrl, &status_dev, &msw, &n_dev};
+    void* args[] = {&nn, &k_dev, &Wp, &nrm, &lamu, &vtu, &ctrl, &status_dev, &msw, &n_dev, &nsmall};
     note_launch();
     TT_CUDA_TRY(cudaLaunchCooperativeKernel(fn, dim3(blocks), dim3(32 * wpb), args, 0, s));
     return TT_OK;
@@ -1276,7 +1525,7 @@ tt_status eig_prepare() {
     TT_TRY(ensure_max_dynamic_smem((const void*)jacobi_kernel));
     // cluster attributes set before any capture
     cluster_size_for((const void*)pchol_cluster_kernel, 256);
-    cluster_size_for((const void*)osj_kernel<8, true>, 32 * OSJ_MAX_WARPS);
+    cluster_size_for((const void*)osj_cluster_kernel, 32 * OSJ_MAX_WARPS);
     return TT_OK;
 }
 
