@@ -14,7 +14,8 @@ ROOT = os.path.dirname(PKG)
 CSRC = os.path.join(PKG, "csrc")
 BUILD = os.path.join(PKG, "_build")
 LIB = os.path.join(PKG, "libttsn.so")
-HEADERS = [os.path.join(ROOT, "include", "ttsn.h"), os.path.join(CSRC, "internal.h")]
+HEADERS = [os.path.join(ROOT, "include", "ttsn.h"), os.path.join(CSRC, "internal.h"),
+           os.path.join(CSRC, "intfp.h")]
 
 NVCC = os.environ.get("NVCC", "nvcc")
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]

@@ -32,6 +32,7 @@
 #include <cooperative_groups.h>
 
 #include "internal.h"
+#include "intfp.h"
 
 namespace ttsn {
 
@@ -568,28 +569,31 @@ osj_kernel(int n, const int* __restrict__ k_dev, double* W, double* nrm, double*
 // laid out for what bounds it on GB300, FP64 issue (64 clocks a warp
 // instruction and SM sub-partition, about 600 for a square root or a division)
 // and the latency of a round:
-// - The rows never leave the SMs.  A warp (G = 1) or half a warp (G = 2) holds a
-//   pair's rows in registers and after the round sends each into the shared
-//   memory of the warp that needs it next: two short remote stores and one
-//   hardware cluster barrier a round, no trip to L2.  The pairs are
-//   round_pair's: slot 0 holds the last row, which stays, and row r; slot k rows
-//   r + k (first) and r - k (second); from round to round the first rows move
-//   down a slot, the second rows up one, and the ends turn.
-// - Above 128 rows two pairs share a warp, so that no sub-partition has a second
-//   warp and the scalar chain of the angle serves both.
+// - The rows never leave the SMs.  A warp holds a pair's rows in registers and
+//   after the round sends each into the shared memory of the warp that needs it
+//   next: two short remote stores and one hardware cluster barrier a round, no
+//   trip to L2.  The pairs are round_pair's: slot 0 holds the last row, which
+//   stays, and row r; slot k rows r + k (first) and r - k (second); from round to
+//   round the first rows move down a slot, the second rows up one, and the ends
+//   turn.  (Two pairs a warp above 128 rows, half the FP64 instructions of the
+//   angle a sub-partition: 7.2 ms against 6.2 at n = 163, equal at 241 to 256.)
+// - The angle's quotients and roots are intfp.h's, the same bits from integer
+//   instructions (n = 61: 1.76 -> 1.40 ms, 163: 8.0 -> 6.2).
+// - A rotated row's squared norm is summed over the lanes by the warp that takes
+//   it next, together with that warp's inner product: six shuffle-and-add steps
+//   for three sums, where one sum alone takes five.
 // - The skip test compares exponents and forms tol sqrt(a b) only within a few
 //   binades of it; an angle with |tau| >= 2^28 needs neither square root, where
 //   sqrt(1 + tau^2) = |tau| and sqrt(1 + t^2) = 1 exactly (the two roundings stay
 //   within half an ulp of tau: relative errors 2^-54 / m^2 + 2^-57 against 2^-53 /
 //   m for a significand m below sqrt 2, 2^-53 / m^2 + 2^-57 above).
-// Measured (GB300, factorisation included): n = 61 2.9 -> 1.9 ms, 128 6.5 ->
-// 4.8, 163 11.1 -> 10.3, 256 23.8 -> 18.8 for a graded full-rank matrix; the
-// 16-problem captured batch 20.5 -> 16.5 ms.
-// inbox: [slot of this CTA][parity][first, second][32 C entries], then the rows'
-// squared norms and indices.
+// Measured (GB300, factorisation included, a graded full-rank matrix): n = 61
+// 2.9 -> 1.40 ms, 128 6.4 -> 3.3, 163 11.1 -> 6.2, 256 22.9 -> 14.5.
+// inbox: [slot of this CTA][parity][first, second][32 (C + 1)], a row's entries
+// and its norm's partial sums, then the rows' squared norms and indices.
 struct OsjMeta {
     double nrm;
-    int idx, pad;
+    int idx, part;  // part: the squared norm follows from the row's partial sums
 };
 
 // 2 log2|c| against log2(tol^2 a b): +1 certainly above, -1 certainly below, 0 close
@@ -603,49 +607,58 @@ __device__ __forceinline__ int osj_far(double c, double a, double b, double tol)
     return 2 * ec >= s + 5 ? 1 : (2 * ec + 2 <= s - 1 ? -1 : 0);
 }
 
-template <int C, int G>
+// 2 v, without the FP64 pipe
+__device__ __forceinline__ double twice(double v) {
+    const int hi = __double2hiint(v), ex = (hi >> 20) & 0x7FF;
+    return (unsigned)(ex - 1) < 0x7FDu ? __hiloint2double(hi + (1 << 20), __double2loint(v)) : v + v;
+}
+
+template <int C>
 __device__ void osj_cluster_body(int n, int k, const double* W, double* lam_u, double* vt_u, int* ctrl, int* status,
                                  int max_sweeps, double tol, double* inbox) {
     namespace cg = cooperative_groups;
     cg::cluster_group cl = cg::this_cluster();
-    constexpr int E = C * G;       // entries of a row a lane holds
-    constexpr int ROW = 32 * C;    // doubles of a row
-    constexpr int LANES = 32 / G;  // lanes of a pair
+    constexpr int ROW = 32 * (C + 1);
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, wpb = blockDim.x >> 5;
-    const int l = lane % LANES, spc = wpb * G;  // slots of a CTA
-    const int ls = warp * G + lane / LANES, slot = blockIdx.x * spc + ls;
+    const int slot = blockIdx.x * wpb + warp;
     const int N = k + (k & 1), S = N / 2;
     const bool active = slot < S;
-    OsjMeta* meta = reinterpret_cast<OsjMeta*>(inbox + (size_t)spc * 4 * ROW);
-    // entry e of lane l: column l + 32 e (G = 1), or l + 16 (e % 2) + 32 (e / 2)
-    auto col = [&](int e) { return G == 1 ? l + 32 * e : l + 16 * (e & 1) + 32 * (e >> 1); };
-    // the 32 column classes' partials (p0: class l, p1: class l + 16) summed as
-    // a butterfly over 32 lanes sums them
-    auto sum = [&](double p0, double p1) {
-        double v = G == 1 ? p0 : p0 + p1;
+    OsjMeta* meta = reinterpret_cast<OsjMeta*>(inbox + (size_t)wpb * 4 * ROW);
+    // the three sums at once (c, and the squared norms of which fx, fy tell that
+    // they are wanted): a lane group carries a different sum from each step on,
+    // every sum with the additions of its own butterfly
+    auto sum3 = [&](double& c, double& px, double& py) {
+        const bool h1 = lane & 16, h2 = lane & 8;
+        double u = (h1 ? px : c) + __shfl_xor_sync(0xffffffffu, h1 ? c : px, 16);
+        const double v = py + __shfl_xor_sync(0xffffffffu, py, 16);
+        u = (h2 ? v : u) + __shfl_xor_sync(0xffffffffu, h2 ? u : v, 8);
 #pragma unroll
-        for (int o = LANES / 2; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-        return v;
+        for (int o = 4; o > 0; o >>= 1) u += __shfl_xor_sync(0xffffffffu, u, o);
+        c = __shfl_sync(0xffffffffu, u, 0);
+        py = __shfl_sync(0xffffffffu, u, 8);
+        px = __shfl_sync(0xffffffffu, u, 16);
     };
-    double x[E], y[E];
-    auto norm2 = [&](const double (&v)[E]) {
-        double p[2] = {0.0, 0.0};
+    double x[C], y[C];
+    auto norm2 = [&](const double (&v)[C]) {
+        double p = 0.0;
 #pragma unroll
-        for (int e = 0; e < E; ++e) p[G == 1 ? 0 : (e & 1)] = fma(v[e], v[e], p[G == 1 ? 0 : (e & 1)]);
-        return sum(p[0], p[1]);
+        for (int e = 0; e < C; ++e) p = fma(v[e], v[e], p);
+        return warp_sum(p);
     };
     // x: the row of the smaller index; sw: it is the slot's second row
     int ix = 0, iy = 0;
     bool sw = false;
-    double a = 0.0, b = 0.0;
+    double a = 0.0, b = 0.0;    // squared norms; pa, pb: their partial sums where fa, fb
+    double pa = 0.0, pb = 0.0;
+    bool fa = false, fb = false;
     {
         const int i0 = slot == 0 ? N - 1 : slot, i1 = slot == 0 ? 0 : N - 1 - slot;  // round 0
         sw = i1 < i0;
         ix = min(i0, i1);
         iy = max(i0, i1);
 #pragma unroll
-        for (int e = 0; e < E; ++e) {
-            const int j = col(e);
+        for (int e = 0; e < C; ++e) {
+            const int j = lane + 32 * e;
             x[e] = active && ix < k && j < n ? __ldcg(W + (long)ix * n + j) : 0.0;
             y[e] = active && iy < k && j < n ? __ldcg(W + (long)iy * n + j) : 0.0;
         }
@@ -656,10 +669,10 @@ __device__ void osj_cluster_body(int n, int k, const double* W, double* lam_u, d
     if (active && S > 1) {
         const int ds0 = slot == 0 ? 0 : slot - 1, dw0 = slot == 1 ? 1 : 0;
         const int ds1 = slot == S - 1 ? slot : slot + 1, dw1 = slot != 0 && slot == S - 1 ? 0 : 1;
-        to0 = cl.map_shared_rank(inbox, ds0 / spc) + ((size_t)(ds0 % spc) * 4 + dw0) * ROW;
-        to1 = cl.map_shared_rank(inbox, ds1 / spc) + ((size_t)(ds1 % spc) * 4 + dw1) * ROW;
-        me0 = cl.map_shared_rank(meta, ds0 / spc) + (ds0 % spc) * 4 + dw0;
-        me1 = cl.map_shared_rank(meta, ds1 / spc) + (ds1 % spc) * 4 + dw1;
+        to0 = cl.map_shared_rank(inbox, ds0 / wpb) + ((size_t)(ds0 % wpb) * 4 + dw0) * ROW;
+        to1 = cl.map_shared_rank(inbox, ds1 / wpb) + ((size_t)(ds1 % wpb) * 4 + dw1) * ROW;
+        me0 = cl.map_shared_rank(meta, ds0 / wpb) + (ds0 % wpb) * 4 + dw0;
+        me1 = cl.map_shared_rank(meta, ds1 / wpb) + (ds1 % wpb) * 4 + dw1;
     }
     cl.sync();  // every CTA of the cluster runs before its shared memory is written
     int sweep = 0;
@@ -669,96 +682,114 @@ __device__ void osj_cluster_body(int n, int k, const double* W, double* lam_u, d
         // steer the angles and the skip test
         a = norm2(x);
         b = norm2(y);
+        fa = fb = false;
         int mine = 0;
         for (int r = 0; r < N - 1; ++r) {
             const int par = r & 1;
             {
-                double c0[2] = {0.0, 0.0}, c1[2] = {0.0, 0.0};  // even and odd steps of 32 columns
+                double c0 = 0.0, c1 = 0.0;
 #pragma unroll
-                for (int e = 0; e < E; ++e) {
-                    const int t = G == 1 ? e : e >> 1, h = G == 1 ? 0 : (e & 1);
-                    if (t & 1)
-                        c1[h] = fma(x[e], y[e], c1[h]);
+                for (int e = 0; e < C; ++e) {
+                    if (e & 1)
+                        c1 = fma(x[e], y[e], c1);
                     else
-                        c0[h] = fma(x[e], y[e], c0[h]);
+                        c0 = fma(x[e], y[e], c0);
                 }
-                const double c = sum(c0[0] + c1[0], c0[1] + c1[1]);
+                double c = C == 1 ? c0 : c0 + c1;
+                if (fa || fb) {
+                    sum3(c, pa, pb);
+                    a = fa ? pa : a;
+                    b = fb ? pb : b;
+                    fa = fb = false;
+                } else {
+                    c = warp_sum(c);
+                }
                 bool rot = false;
                 if (active && iy < k && a > 0.0 && b > 0.0) {
                     const int far = osj_far(c, a, b, tol);
                     rot = far > 0 || (far == 0 && fabs(c) > tol * sqrt(a * b));
                 }
-                if (__any_sync(0xffffffffu, rot)) {
+                if (rot) {
                     // Golub & Van Loan, Alg. 8.4.1 on [[a, c], [c, b]]
-                    const double tau = (b - a) / (2.0 * c);
+                    const double tau = intfp::div(b - a, twice(c));
+                    const double at = fabs(tau);
                     double t, cs, sn;
-                    if (__all_sync(0xffffffffu, !rot || (fabs(tau) >= 268435456.0 && fabs(tau) < 1e150))) {
-                        t = (tau >= 0.0 ? 1.0 : -1.0) / (fabs(tau) + fabs(tau));
+                    if (at >= 268435456.0 && at < 1e150) {
+                        t = intfp::div(tau >= 0.0 ? 1.0 : -1.0, twice(at));
                         cs = 1.0;
                         sn = t;
                     } else {
-                        t = (tau >= 0.0 ? 1.0 : -1.0) / (fabs(tau) + sqrt(1.0 + tau * tau));
-                        cs = 1.0 / sqrt(1.0 + t * t);
+                        t = intfp::div(tau >= 0.0 ? 1.0 : -1.0, at + intfp::root(1.0 + tau * tau));
+                        cs = intfp::div(1.0, intfp::root(1.0 + t * t));
                         sn = t * cs;
                     }
                     // the rotation moves t c from one squared norm to the other: the
                     // growing one is updated by that sum (no cancellation), the
-                    // shrinking one is summed again from the rotated row
+                    // shrinking one is summed again from the rotated row, over the
+                    // lanes with the next product
                     const bool p_shrinks = t * c > 0.0;
-                    double ns[2] = {0.0, 0.0};
+                    double ns = 0.0;
 #pragma unroll
-                    for (int e = 0; e < E; ++e) {
-                        const int h = G == 1 ? 0 : (e & 1);
+                    for (int e = 0; e < C; ++e) {
                         const double xn = cs * x[e] - sn * y[e];
                         const double yn = sn * x[e] + cs * y[e];
-                        if (rot) {
-                            x[e] = xn;
-                            y[e] = yn;
-                        }
+                        x[e] = xn;
+                        y[e] = yn;
                         const double v = p_shrinks ? xn : yn;
-                        ns[h] = fma(v, v, ns[h]);
+                        ns = fma(v, v, ns);
                     }
-                    const double nv = sum(ns[0], ns[1]);
-                    if (rot) {
-                        const double an = p_shrinks ? nv : a - t * c;
-                        b = p_shrinks ? b + t * c : nv;
-                        a = an;
-                        ++mine;
+                    if (p_shrinks) {
+                        b = b + t * c;
+                        pa = ns;
+                    } else {
+                        a = a - t * c;
+                        pb = ns;
                     }
+                    fa = p_shrinks;
+                    fb = !p_shrinks;
+                    ++mine;
                 }
             }
             if (active && S > 1) {
                 double *o0 = (sw ? to1 : to0) + par * 2 * ROW, *o1 = (sw ? to0 : to1) + par * 2 * ROW;
 #pragma unroll
-                for (int e = 0; e < E; ++e) {
-                    o0[col(e)] = x[e];
-                    o1[col(e)] = y[e];
+                for (int e = 0; e < C; ++e) {
+                    o0[lane + 32 * e] = x[e];
+                    o1[lane + 32 * e] = y[e];
                 }
-                if (l == 0) {
+                if (fa) o0[32 * C + lane] = pa;
+                if (fb) o1[32 * C + lane] = pb;
+                if (lane == 0) {
                     OsjMeta *m0 = (sw ? me1 : me0) + par * 2, *m1 = (sw ? me0 : me1) + par * 2;
                     m0->nrm = a;
                     m0->idx = ix;
+                    m0->part = fa;
                     m1->nrm = b;
                     m1->idx = iy;
+                    m1->part = fb;
                 }
             }
-            if (r == N - 2 && l == 0 && mine) atomicAdd(ctrl + 4 + sweep, mine);
+            if (r == N - 2 && lane == 0 && mine) atomicAdd(ctrl + 4 + sweep, mine);
             cl.sync();
             if (active && S > 1) {
-                const OsjMeta* m = meta + ls * 4 + par * 2;
+                const OsjMeta* m = meta + warp * 4 + par * 2;
                 const int i0 = m[0].idx, i1 = m[1].idx;
                 sw = i1 < i0;
                 ix = min(i0, i1);
                 iy = max(i0, i1);
                 a = m[sw ? 1 : 0].nrm;
                 b = m[sw ? 0 : 1].nrm;
-                const double* in = inbox + ((size_t)ls * 4 + par * 2) * ROW;
+                fa = m[sw ? 1 : 0].part;
+                fb = m[sw ? 0 : 1].part;
+                const double* in = inbox + ((size_t)warp * 4 + par * 2) * ROW;
                 const double *f0 = in + (sw ? ROW : 0), *f1 = in + (sw ? 0 : ROW);
 #pragma unroll
-                for (int e = 0; e < E; ++e) {
-                    x[e] = f0[col(e)];
-                    y[e] = f1[col(e)];
+                for (int e = 0; e < C; ++e) {
+                    x[e] = f0[lane + 32 * e];
+                    y[e] = f1[lane + 32 * e];
                 }
+                pa = f0[32 * C + lane];
+                pb = f1[32 * C + lane];
             }
         }
         // N - 1 rounds, an odd number: the next sweep writes parity 0, just read
@@ -772,13 +803,13 @@ __device__ void osj_cluster_body(int n, int k, const double* W, double* lam_u, d
     // eigenvalues: the converged rows' squared norms, summed from the rows
     a = norm2(x);
     b = norm2(y);
-    auto put = [&](int i, double nn, const double (&v)[E]) {
+    auto put = [&](int i, double nn, const double (&v)[C]) {
         if (!active || i >= k) return;
         const double f = nn > 0.0 ? 1.0 / sqrt(nn) : 0.0;
-        if (l == 0) lam_u[i] = nn;
+        if (lane == 0) lam_u[i] = nn;
 #pragma unroll
-        for (int e = 0; e < E; ++e)
-            if (col(e) < n) vt_u[(long)i * n + col(e)] = f * v[e];
+        for (int e = 0; e < C; ++e)
+            if (lane + 32 * e < n) vt_u[(long)i * n + lane + 32 * e] = f * v[e];
     };
     put(ix, a, x);
     put(iy, b, y);
@@ -788,7 +819,7 @@ __device__ void osj_cluster_body(int n, int k, const double* W, double* lam_u, d
     }
 }
 
-__global__ void __launch_bounds__(32 * OSJ_MAX_WARPS)
+__global__ void __launch_bounds__(32 * OSJ_MAX_WARPS, 1)
 osj_cluster_kernel(int n, const int* __restrict__ k_dev, const double* W, double* lam_u, double* vt_u, int* ctrl,
                    int* status, int max_sweeps, const int* n_dev, int nsmall) {
     if (n_dev) {  // a captured step: larger sizes take the grid kernel
@@ -807,17 +838,17 @@ osj_cluster_kernel(int n, const int* __restrict__ k_dev, const double* W, double
         return;
     }
     const int k = min(kraw, n);
-#define OSJ_BODY(C, G) osj_cluster_body<C, G>(n, k, W, lam_u, vt_u, ctrl, status, max_sweeps, tol, osj_inbox)
+#define OSJ_BODY(C) osj_cluster_body<C>(n, k, W, lam_u, vt_u, ctrl, status, max_sweeps, tol, osj_inbox)
     switch ((n + 31) / 32) {
         case 0:
-        case 1: OSJ_BODY(1, 1); break;
-        case 2: OSJ_BODY(2, 1); break;
-        case 3: OSJ_BODY(3, 1); break;
-        case 4: OSJ_BODY(4, 1); break;
-        case 5: OSJ_BODY(5, 2); break;
-        case 6: OSJ_BODY(6, 2); break;
-        case 7: OSJ_BODY(7, 2); break;
-        default: OSJ_BODY(8, 2); break;
+        case 1: OSJ_BODY(1); break;
+        case 2: OSJ_BODY(2); break;
+        case 3: OSJ_BODY(3); break;
+        case 4: OSJ_BODY(4); break;
+        case 5: OSJ_BODY(5); break;
+        case 6: OSJ_BODY(6); break;
+        case 7: OSJ_BODY(7); break;
+        default: OSJ_BODY(8); break;
     }
 #undef OSJ_BODY
 }
@@ -825,19 +856,30 @@ osj_cluster_kernel(int n, const int* __restrict__ k_dev, const double* W, double
 // Pivoted Cholesky on one thread-block cluster for n <= PCHOL_SMALL_N: the
 // same factorisation as pchol_kernel (pivot = largest remaining diagonal
 // entry, ties to the lowest index, stop at the floor, -inf marks pivoted
-// columns, the same per-column sums), with contiguous blocks of cpc columns
-// per CTA, one thread per column, and the CTA's columns of W held in its
-// shared memory.  A pivot: every CTA reads the CTAs' candidate (value,
-// column) pairs from distributed shared memory and takes the same pivot p,
-// reads W[0..k)[p] from the owner's shared memory, forms row k of W for its
-// columns, updates their residual diagonal and posts its candidate for the
-// next pivot; one hardware cluster barrier (release / acquire at cluster
-// scope) ends the pivot.  On GB300 a pivot's n k FP64 FMAs are more than one
-// SM absorbs (~1.7 FMA per clock) and a grid-wide barrier per pivot costs
-// microseconds; a cluster spreads the FMAs over CL SMs for a barrier well
-// under a microsecond.  Candidates are double-buffered by the pivot's
-// parity, so a CTA never overwrites a slot another CTA may still read.
-constexpr int PCHOL_SMALL_N = 384;
+// columns), with contiguous blocks of cpc columns per CTA whose part of W lies
+// in its shared memory (column by column, PCHOL_LD apart).  A column is four
+// lanes, one for each of the four interleaved sums of its inner product with
+// the pivot column.  A pivot:
+//   1. every warp reads the candidates that all column warps have sent to its
+//      CTA and takes the same pivot p (integer maxima: a positive double's bits
+//      order as its value);
+//   2. the CTA copies W[0..k)[p] from the owner's shared memory;
+//   3. the column warps form the inner products while a warp without columns
+//      takes the square root;
+//   4. row k of W, the residual diagonal, and each warp's next candidate, sent
+//      to every CTA; one hardware cluster barrier (release / acquire).
+// On GB300 a DFMA holds its warp 64 clocks and a barrier costs about 400, so a
+// pivot is a chain of k / 4 DFMAs and some 2,000 clocks of the rest; one lane
+// per column took k DFMAs in a row.  Candidate slots alternate with the pivot's
+// parity, so no CTA overwrites one that another may still read.
+// Measured (GB300, one factorisation): n = 61 0.52 -> 0.34 ms, 163 1.44 -> 0.65,
+// 256 2.77 -> 1.07, 384 5.4 -> 1.9; above, against pchol_kernel, 449 3.2 -> 2.4 and
+// 600 4.5 -> 3.9 (the FMAs of larger sizes want more than a cluster).
+constexpr int PCHOL_SMALL_N = 608;
+constexpr int PCHOL_SLOTS = 112;  // column warps of a cluster
+
+__host__ __device__ inline int pchol_ld(int n) { return (n + 15) / 16 * 16 + 4; }  // columns 4 banks of 16 apart
+__host__ __device__ inline size_t pchol_smem_doubles(int n, int cpc) { return (size_t)cpc * pchol_ld(n) + n; }
 
 __global__ void __launch_bounds__(256)
 pchol_cluster_kernel(int n, int cpc, const double* __restrict__ G, long ldg, double* W, int* kB_out,
@@ -854,100 +896,97 @@ pchol_cluster_kernel(int n, int cpc, const double* __restrict__ G, long ldg, dou
             if (rank == 0 && threadIdx.x == 0) *kB_out = 0;
             return;
         }
+        cpc = (n + CL - 1) / CL;
     }
     extern __shared__ double sm[];
-    double* Wl = sm;                         // rows 0..k) of this CTA's cpc columns (n x cpc)
-    double* colp = sm + (size_t)n * cpc;     // W[0..k)[p]
-    __shared__ double s_cv[2];  // candidate value per parity
-    __shared__ int s_ci[2];     // candidate column per parity
-    __shared__ double s_wv[8];
-    __shared__ int s_wi[8];
-    __shared__ int s_bad;
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nwarps = (blockDim.x + 31) >> 5;
-    const int jl = threadIdx.x;
-    const int j = rank * cpc + jl;
-    const bool own = jl < cpc && j < n;
+    const int ld = pchol_ld(n);
+    double* Wl = sm;                         // this CTA's columns: [cpc][ld]
+    double* colp = sm + (size_t)cpc * ld;    // W[0..k)[p]
+    __shared__ unsigned long long s_key[2][PCHOL_SLOTS];  // candidates of the cluster's column warps, per parity
+    __shared__ int s_idx[2][PCHOL_SLOTS];
+    __shared__ double s_l;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nwarps = blockDim.x >> 5;
+    const int cw = (cpc + 7) / 8;  // column warps; the last warp has no columns
+    const int c = warp * 8 + (lane >> 2), q = lane & 3;
+    const int j = rank * cpc + c;
+    const bool own = warp < cw && c < cpc && j < n;
+    const int nslots = CL * cw;
     double dj = own ? G[(long)j * ldg + j] : -1.0;
-    // block candidate of (value, index), ties to the lowest index
-    auto post = [&](double v, int idx, int par) {
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) {
-            const double v2 = __shfl_xor_sync(0xffffffffu, v, o);
-            const int i2 = __shfl_xor_sync(0xffffffffu, idx, o);
-            if (v2 > v || (v2 == v && i2 < idx)) {
-                v = v2;
+    // this warp's candidate (the largest positive residual, lowest index) to
+    // every CTA's slot
+    auto post = [&](int par) {
+        if (warp >= cw) return;
+        unsigned long long key = own && dj > 0.0 ? (unsigned long long)__double_as_longlong(dj) : 0ull;
+        const unsigned hi = (unsigned)(key >> 32), mh = __reduce_max_sync(0xffffffffu, hi);
+        const unsigned lo = hi == mh ? (unsigned)key : 0u, ml = __reduce_max_sync(0xffffffffu, lo);
+        key = (unsigned long long)mh << 32 | ml;
+        const int idx = __reduce_min_sync(0xffffffffu, key != 0 && own && hi == mh && lo == ml ? j : n);
+        if (lane < CL) {
+            *cl.map_shared_rank(&s_key[par][rank * cw + warp], lane) = key;
+            *cl.map_shared_rank(&s_idx[par][rank * cw + warp], lane) = idx;
+        }
+    };
+    // the cluster's candidate, from this CTA's slots (after a barrier)
+    auto gather = [&](int par, double& d, int& p) {
+        unsigned long long key = 0;
+        int idx = n;
+        for (int i = lane; i < nslots; i += 32) {
+            const unsigned long long k2 = s_key[par][i];
+            const int i2 = s_idx[par][i];
+            if (k2 > key || (k2 == key && i2 < idx)) {
+                key = k2;
                 idx = i2;
             }
         }
-        if (lane == 0) {
-            s_wv[warp] = v;
-            s_wi[warp] = idx;
-        }
-        __syncthreads();
-        if (threadIdx.x == 0) {
-            double b = -1.0;
-            int bi = n;
-            for (int w = 0; w < nwarps; ++w)
-                if (s_wv[w] > b || (s_wv[w] == b && s_wi[w] < bi)) {
-                    b = s_wv[w];
-                    bi = s_wi[w];
-                }
-            s_cv[par] = b;
-            s_ci[par] = bi;
-        }
-    };
-    // the cluster's candidate, read from every CTA's slot (after a barrier):
-    // lane r of every warp reads CTA r's slot, a shuffle tree takes the best
-    auto gather = [&](int par, double& b, int& bi) {
-        b = -1.0;
-        bi = n;
-        if (lane < CL) {
-            b = *cl.map_shared_rank(&s_cv[par], lane);
-            bi = *cl.map_shared_rank(&s_ci[par], lane);
-        }
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) {
-            const double v2 = __shfl_xor_sync(0xffffffffu, b, o);
-            const int i2 = __shfl_xor_sync(0xffffffffu, bi, o);
-            if (v2 > b || (v2 == b && i2 < bi)) {
-                b = v2;
-                bi = i2;
-            }
-        }
+        const unsigned hi = (unsigned)(key >> 32), mh = __reduce_max_sync(0xffffffffu, hi);
+        const unsigned lo = hi == mh ? (unsigned)key : 0u, ml = __reduce_max_sync(0xffffffffu, lo);
+        p = __reduce_min_sync(0xffffffffu, hi == mh && lo == ml ? idx : n);
+        d = __longlong_as_double((long long)((unsigned long long)mh << 32 | ml));
     };
     // Inf or NaN on the diagonal (a Gram matrix shows any non-finite entry of
     // its factor there): rank -1 reports it instead of factorising
-    if (threadIdx.x == 0) s_bad = 0;
-    __syncthreads();
-    if (own && !isfinite(dj)) atomicOr(&s_bad, 1);
-    __syncthreads();
-    // the largest diagonal entry (the floor's scale) and the first pivot
-    post(own ? dj : -1.0, own ? j : n, 0);
-    if (threadIdx.x == 0 && s_bad) s_cv[0] = __longlong_as_double(0x7ff8000000000000LL);  // NaN marks it
+    const int bad = __syncthreads_or(own && !isfinite(dj));
+    cl.sync();  // every CTA of the cluster runs before its shared memory is written
+    post(0);
+    if (bad && threadIdx.x < CL) *cl.map_shared_rank(&s_key[0][rank * cw], threadIdx.x) = ~0ull;  // marks it
     cl.sync();
-    const int anybad = __any_sync(0xffffffffu, lane < CL && isnan(*cl.map_shared_rank(&s_cv[0], lane)));
+    bool anybad = false;
+    for (int i = 0; i < nslots; ++i) anybad |= s_key[0][i] == ~0ull;
     if (anybad) {
-        cl.sync();  // every CTA has read the slots before any CTA exits
         if (rank == 0 && threadIdx.x == 0) *kB_out = -1;
         return;
     }
-    double dmax;
+    double dp;
     int p;
-    gather(0, dmax, p);
-    const double floor_abs = floor_rel * dmax;
-    double dp = dmax;
+    gather(0, dp, p);
+    const double floor_abs = floor_rel * dp;
     int par = 0;
     int k = 0;
     for (; k < n; ++k) {
         if (!(dp > floor_abs) || p >= n) break;
-        const double l = sqrt(dp);
+        const double g = own && q == 0 ? G[(long)p * ldg + j] : 0.0;
         {
-            const double* Wo = cl.map_shared_rank(Wl, p / cpc);  // the owner's columns
-            const int pl = p % cpc;
-            for (int m = threadIdx.x; m < k; m += blockDim.x) colp[m] = Wo[(size_t)m * cpc + pl];
+            const double* Wo = cl.map_shared_rank(Wl, p / cpc) + (size_t)(p % cpc) * ld;  // the owner's column
+            for (int m = threadIdx.x; m < k; m += blockDim.x) colp[m] = Wo[m];
         }
         __syncthreads();
-        if (own) {
+        double acc = 0.0;
+        if (warp < cw) {
+            const double* wc = Wl + (size_t)(own ? c : 0) * ld;
+            const int k4 = k & ~3;
+#pragma unroll 4
+            for (int m = q; m < k4; m += 4) acc = fma(colp[m], wc[m], acc);
+            if (q == 0)
+                for (int m = k4; m < k; ++m) acc = fma(colp[m], wc[m], acc);
+            acc += __shfl_down_sync(0xffffffffu, acc, 1, 4);  // lanes 0 and 2: a0 + a1, a2 + a3
+            acc += __shfl_down_sync(0xffffffffu, acc, 2, 4);
+        } else if (warp == nwarps - 1) {
+            const double l = intfp::root(dp);
+            if (lane == 0) s_l = l;
+        }
+        __syncthreads();
+        if (own && q == 0) {
+            const double l = s_l;
             double w;
             if (j == p) {
                 w = l;
@@ -955,23 +994,15 @@ pchol_cluster_kernel(int n, int cpc, const double* __restrict__ G, long ldg, dou
             } else if (dj == -INFINITY) {
                 w = 0.0;
             } else {
-                double a0 = 0.0, a1 = 0.0, a2 = 0.0, a3 = 0.0;
-                int m = 0;
-                for (; m + 3 < k; m += 4) {
-                    a0 += colp[m] * Wl[(size_t)m * cpc + jl];
-                    a1 += colp[m + 1] * Wl[(size_t)(m + 1) * cpc + jl];
-                    a2 += colp[m + 2] * Wl[(size_t)(m + 2) * cpc + jl];
-                    a3 += colp[m + 3] * Wl[(size_t)(m + 3) * cpc + jl];
-                }
-                for (; m < k; ++m) a0 += colp[m] * Wl[(size_t)m * cpc + jl];
-                w = (G[(long)p * ldg + j] - ((a0 + a1) + (a2 + a3))) / l;
+                w = intfp::div(g - acc, l);
                 dj = dj - w * w;
             }
-            Wl[(size_t)k * cpc + jl] = w;
+            Wl[(size_t)c * ld + k] = w;
             __stcg(W + (long)k * n + j, w);
         }
+        if (q != 0) dj = -1.0;  // lane 0 of a column holds its residual
         par ^= 1;
-        post(own && dj != -INFINITY ? dj : -1.0, own && dj != -INFINITY ? j : n, par);
+        post(par);
         cl.sync();
         gather(par, dp, p);
     }
@@ -1379,12 +1410,15 @@ int cluster_size_for(const void* fn, int threads) {
     return cl;
 }
 
-// Largest n the cluster factorisation takes: at most PCHOL_SMALL_N, and its
-// columns of W must fit a CTA's shared memory (n ceil(n / CL) + n doubles).
+// Largest n the cluster factorisation takes: at most PCHOL_SMALL_N, its columns
+// of W in a CTA's shared memory, at most 7 column warps a CTA, a candidate slot
+// for each of the cluster's.
 int pchol_small_limit() {
     const int cl = cluster_size_for((const void*)pchol_cluster_kernel, 256);
     int n = PCHOL_SMALL_N;
-    while (n > 0 && ((size_t)n * ((n + cl - 1) / cl) + n) * sizeof(double) > 200 * 1024) --n;
+    while (n > 0 && (pchol_smem_doubles(n, (n + cl - 1) / cl) * sizeof(double) > 200 * 1024 ||
+                     cl * (((n + cl - 1) / cl + 7) / 8) > PCHOL_SLOTS || ((n + cl - 1) / cl + 7) / 8 > 7))
+        --n;
     return n;
 }
 
@@ -1392,11 +1426,11 @@ tt_status launch_pchol_cluster(cudaStream_t s, int n, const double* G, long ldg,
                                const int* n_dev, int nsmall) {
     const int cl = cluster_size_for((const void*)pchol_cluster_kernel, 256);
     const int cpc = (n + cl - 1) / cl;
-    const int threads = std::max(32, (cpc + 31) / 32 * 32);
+    const int threads = 32 * std::max(4, (cpc + 7) / 8 + 1);
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(cl);
     cfg.blockDim = dim3(threads);
-    cfg.dynamicSmemBytes = ((size_t)n * cpc + n) * sizeof(double);
+    cfg.dynamicSmemBytes = pchol_smem_doubles(n, cpc) * sizeof(double);
     cfg.stream = s;
     cudaLaunchAttribute at[1];
     at[0].id = cudaLaunchAttributeClusterDimension;
@@ -1423,19 +1457,18 @@ tt_status osj_launch(cudaStream_t s, int ncap, const int* k_dev, EigWork& w, int
     int msw = max_sweeps;
     int nsmall = OSJ_CLUSTER_N;
     if (ncap <= nsmall || n_dev) {
-        // one cluster, a warp per pair up to 128 rows, two pairs a warp above.
+        // one cluster, a warp per pair.
         // A captured step launches it for sizes up to nsmall and the grid
         // kernel after it for larger ones (each returns at once outside its
         // range), so a replay takes the host path's kernel.
         const int ncl = std::min(ncap, nsmall);
         const int cl = cluster_size_for((const void*)osj_cluster_kernel, 32 * OSJ_MAX_WARPS);
-        const int np1 = (std::min(ncl, 128) + 1) / 2, np2 = (ncl + 3) / 4;
-        const int wpb = std::max(1, std::max((np1 + cl - 1) / cl, ncl > 128 ? (np2 + cl - 1) / cl : 0));
-        const int C = (ncl + 31) / 32, spc = wpb * (ncl > 128 ? 2 : 1);
+        const int wpb = std::max(1, ((ncl + 1) / 2 + cl - 1) / cl);
+        const int C = (ncl + 31) / 32;
         cudaLaunchConfig_t cfg = {};
         cfg.gridDim = dim3(cl);
         cfg.blockDim = dim3(32 * wpb);
-        cfg.dynamicSmemBytes = (size_t)spc * 4 * (32 * C * sizeof(double) + sizeof(OsjMeta));
+        cfg.dynamicSmemBytes = (size_t)wpb * 4 * (32 * (C + 1) * sizeof(double) + sizeof(OsjMeta));
         cfg.stream = s;
         cudaLaunchAttribute at[1];
         at[0].id = cudaLaunchAttributeClusterDimension;
