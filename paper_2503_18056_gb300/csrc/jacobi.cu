@@ -400,39 +400,20 @@ __device__ __forceinline__ double warp_sum(double v) {
     return v;
 }
 
-// One pair: c = w_p . w_q, the rotation if it is needed, the rotated rows'
-// norms.  C > 0: the lane's n / 32 entries of both rows are held in registers
-// (all loads issued at once: one L2 round trip per pair); C == 0 streams the
-// rows (any n).  Returns whether it rotated.
-template <int C>
+// One pair of rows of any length, streamed from L2: c = w_p . w_q, the rotation
+// if it is needed, the rotated rows' norms.  Returns whether it rotated.
 __device__ __forceinline__ bool osj_pair(double* wp, double* wq, int n, int lane, double* nrm_p, double* nrm_q,
                                          double tol) {
-    double x[C > 0 ? C : 1], y[C > 0 ? C : 1];
-    double c;
-    if (C > 0) {
-#pragma unroll
-        for (int t = 0; t < C; ++t) {
-            const int j = lane + 32 * t;
-            x[t] = j < n ? __ldcg(wp + j) : 0.0;
-            y[t] = j < n ? __ldcg(wq + j) : 0.0;
-        }
-        double c0 = 0.0, c1 = 0.0;
-#pragma unroll
-        for (int t = 0; t < C; t += 2) {
-            c0 = fma(x[t], y[t], c0);
-            if (t + 1 < C) c1 = fma(x[t + 1], y[t + 1], c1);
-        }
-        c = warp_sum(c0 + c1);
-    } else {
-        double c0 = 0.0, c1 = 0.0;
+    double c0 = 0.0, c1 = 0.0;
+    {
         int j = lane;
         for (; j + 32 < n; j += 64) {
             c0 = fma(__ldcg(wp + j), __ldcg(wq + j), c0);
             c1 = fma(__ldcg(wp + j + 32), __ldcg(wq + j + 32), c1);
         }
         if (j < n) c0 = fma(__ldcg(wp + j), __ldcg(wq + j), c0);
-        c = warp_sum(c0 + c1);
     }
+    const double c = warp_sum(c0 + c1);
     const double a = __ldcg(nrm_p), b = __ldcg(nrm_q);
     if (!(a > 0.0 && b > 0.0 && fabs(c) > tol * sqrt(a * b))) return false;
     // Golub & Van Loan, Alg. 8.4.1 on [[a, c], [c, b]]
@@ -445,29 +426,14 @@ __device__ __forceinline__ bool osj_pair(double* wp, double* wq, int n, int lane
     // summed again from the rotated row
     const bool p_shrinks = t * c > 0.0;
     double ns = 0.0;
-    if (C > 0) {
-#pragma unroll
-        for (int t2 = 0; t2 < C; ++t2) {
-            const int j = lane + 32 * t2;
-            const double xn = cs * x[t2] - sn * y[t2];
-            const double yn = sn * x[t2] + cs * y[t2];
-            if (j < n) {
-                __stcg(wp + j, xn);
-                __stcg(wq + j, yn);
-            }
-            const double v = p_shrinks ? xn : yn;
-            ns = fma(v, v, ns);
-        }
-    } else {
-        for (int j = lane; j < n; j += 32) {
-            const double xo = __ldcg(wp + j), yo = __ldcg(wq + j);
-            const double xn = cs * xo - sn * yo;
-            const double yn = sn * xo + cs * yo;
-            __stcg(wp + j, xn);
-            __stcg(wq + j, yn);
-            const double v = p_shrinks ? xn : yn;
-            ns = fma(v, v, ns);
-        }
+    for (int j = lane; j < n; j += 32) {
+        const double xo = __ldcg(wp + j), yo = __ldcg(wq + j);
+        const double xn = cs * xo - sn * yo;
+        const double yn = sn * xo + cs * yo;
+        __stcg(wp + j, xn);
+        __stcg(wq + j, yn);
+        const double v = p_shrinks ? xn : yn;
+        ns = fma(v, v, ns);
     }
     ns = warp_sum(ns);
     if (lane == 0) {
@@ -491,11 +457,10 @@ __device__ __forceinline__ void osj_norms(const double* W, int n, int k, double*
     }
 }
 
-template <int C>
 __global__ void __launch_bounds__(32 * OSJ_MAX_WARPS)
 osj_kernel(int n, const int* __restrict__ k_dev, double* W, double* nrm, double* lam_u, double* vt_u, int* ctrl,
            int* status, int max_sweeps, const int* n_dev, int nsmall) {
-    if (n_dev) {  // a captured step: sizes up to nsmall take the cluster launch
+    if (n_dev) {  // a captured step: sizes up to nsmall take the launches before it
         n = *n_dev;
         if (n <= nsmall) return;  // every CTA, before any barrier
     }
@@ -534,7 +499,7 @@ osj_kernel(int n, const int* __restrict__ k_dev, double* W, double* nrm, double*
                     int p, q;
                     round_pair(N, r, kk, p, q);
                     if (q >= k) continue;
-                    if (osj_pair<C>(W + (long)p * n, W + (long)q * n, n, lane, nrm + p, nrm + q, tol)) ++mine;
+                    if (osj_pair(W + (long)p * n, W + (long)q * n, n, lane, nrm + p, nrm + q, tol)) ++mine;
                 }
                 if (r == N - 2) {
                     if (lane == 0 && mine) atomicAdd(&s_cnt, mine);
@@ -564,9 +529,8 @@ osj_kernel(int n, const int* __restrict__ k_dev, double* W, double* nrm, double*
     }
 }
 
-// Up to OSJ_CLUSTER_N rows on one thread-block cluster: the same rotations in the
-// same order and arithmetic (bit for bit the grid kernel's with C = ceil(n / 32)),
-// laid out for what bounds it on GB300, FP64 issue (64 clocks a warp
+// Up to OSJ_CLUSTER_N rows on one thread-block cluster: osj_kernel's rotations in
+// the same order, laid out for what bounds it on GB300, FP64 issue (64 clocks a warp
 // instruction and SM sub-partition, about 600 for a square root or a division)
 // and the latency of a round:
 // - The rows never leave the SMs.  A warp holds a pair's rows in registers and
@@ -613,6 +577,36 @@ __device__ __forceinline__ double twice(double v) {
     return (unsigned)(ex - 1) < 0x7FDu ? __hiloint2double(hi + (1 << 20), __double2loint(v)) : v + v;
 }
 
+// tan, cos and sin of the rotation that makes [[a, c], [c, b]] diagonal (Golub &
+// Van Loan, Alg. 8.4.1), c far from 0
+__device__ __forceinline__ void osj_angle(double a, double b, double c, double& t, double& cs, double& sn) {
+    const double tau = intfp::div(b - a, twice(c));
+    const double at = fabs(tau);
+    if (at >= 268435456.0 && at < 1e150) {
+        t = intfp::div(tau >= 0.0 ? 1.0 : -1.0, twice(at));
+        cs = 1.0;
+        sn = t;
+    } else {
+        t = intfp::div(tau >= 0.0 ? 1.0 : -1.0, at + intfp::root(1.0 + tau * tau));
+        cs = intfp::div(1.0, intfp::root(1.0 + t * t));
+        sn = t * cs;
+    }
+}
+
+// Three sums over a warp at once: a group of lanes carries a different one from
+// each step on, every sum with the additions of its own butterfly.
+__device__ __forceinline__ void osj_sum3(double& c, double& px, double& py, int lane) {
+    const bool h1 = lane & 16, h2 = lane & 8;
+    double u = (h1 ? px : c) + __shfl_xor_sync(0xffffffffu, h1 ? c : px, 16);
+    const double v = py + __shfl_xor_sync(0xffffffffu, py, 16);
+    u = (h2 ? v : u) + __shfl_xor_sync(0xffffffffu, h2 ? u : v, 8);
+#pragma unroll
+    for (int o = 4; o > 0; o >>= 1) u += __shfl_xor_sync(0xffffffffu, u, o);
+    c = __shfl_sync(0xffffffffu, u, 0);
+    py = __shfl_sync(0xffffffffu, u, 8);
+    px = __shfl_sync(0xffffffffu, u, 16);
+}
+
 template <int C>
 __device__ void osj_cluster_body(int n, int k, const double* W, double* lam_u, double* vt_u, int* ctrl, int* status,
                                  int max_sweeps, double tol, double* inbox) {
@@ -624,20 +618,6 @@ __device__ void osj_cluster_body(int n, int k, const double* W, double* lam_u, d
     const int N = k + (k & 1), S = N / 2;
     const bool active = slot < S;
     OsjMeta* meta = reinterpret_cast<OsjMeta*>(inbox + (size_t)wpb * 4 * ROW);
-    // the three sums at once (c, and the squared norms of which fx, fy tell that
-    // they are wanted): a lane group carries a different sum from each step on,
-    // every sum with the additions of its own butterfly
-    auto sum3 = [&](double& c, double& px, double& py) {
-        const bool h1 = lane & 16, h2 = lane & 8;
-        double u = (h1 ? px : c) + __shfl_xor_sync(0xffffffffu, h1 ? c : px, 16);
-        const double v = py + __shfl_xor_sync(0xffffffffu, py, 16);
-        u = (h2 ? v : u) + __shfl_xor_sync(0xffffffffu, h2 ? u : v, 8);
-#pragma unroll
-        for (int o = 4; o > 0; o >>= 1) u += __shfl_xor_sync(0xffffffffu, u, o);
-        c = __shfl_sync(0xffffffffu, u, 0);
-        py = __shfl_sync(0xffffffffu, u, 8);
-        px = __shfl_sync(0xffffffffu, u, 16);
-    };
     double x[C], y[C];
     auto norm2 = [&](const double (&v)[C]) {
         double p = 0.0;
@@ -697,7 +677,7 @@ __device__ void osj_cluster_body(int n, int k, const double* W, double* lam_u, d
                 }
                 double c = C == 1 ? c0 : c0 + c1;
                 if (fa || fb) {
-                    sum3(c, pa, pb);
+                    osj_sum3(c, pa, pb, lane);
                     a = fa ? pa : a;
                     b = fb ? pb : b;
                     fa = fb = false;
@@ -710,19 +690,8 @@ __device__ void osj_cluster_body(int n, int k, const double* W, double* lam_u, d
                     rot = far > 0 || (far == 0 && fabs(c) > tol * sqrt(a * b));
                 }
                 if (rot) {
-                    // Golub & Van Loan, Alg. 8.4.1 on [[a, c], [c, b]]
-                    const double tau = intfp::div(b - a, twice(c));
-                    const double at = fabs(tau);
                     double t, cs, sn;
-                    if (at >= 268435456.0 && at < 1e150) {
-                        t = intfp::div(tau >= 0.0 ? 1.0 : -1.0, twice(at));
-                        cs = 1.0;
-                        sn = t;
-                    } else {
-                        t = intfp::div(tau >= 0.0 ? 1.0 : -1.0, at + intfp::root(1.0 + tau * tau));
-                        cs = intfp::div(1.0, intfp::root(1.0 + t * t));
-                        sn = t * cs;
-                    }
+                    osj_angle(a, b, c, t, cs, sn);
                     // the rotation moves t c from one squared norm to the other: the
                     // growing one is updated by that sum (no cancellation), the
                     // shrinking one is summed again from the rotated row, over the
@@ -851,6 +820,225 @@ osj_cluster_kernel(int n, const int* __restrict__ k_dev, const double* W, double
         default: OSJ_BODY(8); break;
     }
 #undef OSJ_BODY
+}
+
+// OSJ_CLUSTER_N < n <= OSJ_GRID_N: the same rotations with the rows in L2, over all
+// SMs.  A sub-partition issues an FP64 warp instruction in 64 clocks and an SM has
+// four, so a CTA is four warps and a pair takes as many of them as there are:
+// G = 4 with one pair a CTA, 2 with two, else 1 (a warp's entries of a row:
+// n / (32 G)).  With a warp a pair and 32 entries a lane whatever n, a round of
+// 451 rows of 713 took 11.8 us.
+// There is no grid barrier between rounds.  A round's pairs are round_pair's, in
+// which a slot's two rows come from the slots beside it, so a pair waits for its two
+// neighbours' count of finished rounds (a store with release, a load with acquire)
+// and a slow pair delays only those near it.  Every CTA is resident (cooperative
+// launch) and every wait is bounded: a warp whose wait ran out sets DEV_TIMEOUT
+// and waits no more, and the grid barrier after the sweep ends the kernel.
+// nrm[i]: row i's squared norm, or -1 where part[i] holds its partial sums, to be
+// summed over the lanes with the next inner product.
+// Measured (GB300, factorisation included): graded full-rank matrices n = 300 25.1 ->
+// 14.0 ms, 449 39.2 -> 31.5, 608 76.8 -> 48.8; rank 451 of 713 47 -> 34; rank 311
+// of 311 20 -> 12.
+constexpr int OSJ_GRID_N = 1024;
+constexpr int OSJ_FLAG = 8;  // ints between two slots' counts: a sector each
+
+template <int E, int G>
+__device__ bool osj_grid_body(int n, int k, double* W, double* nrm, double* part, int* flags, int* ctrl, int* status,
+                              int max_sweeps, double tol, int& sweeps) {
+    __shared__ double s_red[4][4];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int N = k + (k & 1), S = N / 2;
+    const int b = (S + gridDim.x - 1) / gridDim.x;  // pairs of a CTA, at most 4 / G
+    const int g = warp / G, w = warp % G, slot = blockIdx.x * b + g;
+    const bool active = g < b && slot < S;
+    const int ne = (n + 32 * G - 1) / (32 * G);
+    int* mine_flag = flags + (long)slot * OSJ_FLAG;
+    const int* near = flags + (long)(slot + (lane & 1 ? 1 : -1)) * OSJ_FLAG;  // lanes 0 and 1 watch the neighbours
+    const bool watch = active && lane < 2 && (lane & 1 ? slot + 1 < S : slot > 0);
+    auto group_sync = [&]() {
+        if (G == 1)
+            __syncwarp();
+        else
+            asm volatile("bar.sync %0, %1;" ::"r"(g + 1), "r"(32 * G) : "memory");
+    };
+    // sums over the pair's warps of up to three values
+    auto across = [&](int m, double& v0, double& v1, double& v2) {
+        if (G == 1) return;
+        if (lane == 0) {
+            s_red[warp][0] = v0;
+            if (m > 1) {
+                s_red[warp][1] = v1;
+                s_red[warp][2] = v2;
+            }
+        }
+        group_sync();
+        const int w0 = g * G, i = lane & 3;  // a lane a value
+        double u = s_red[w0][i] + s_red[w0 + 1][i];
+        if (G == 4) u += s_red[w0 + (G == 4 ? 2 : 0)][i] + s_red[w0 + (G == 4 ? 3 : 0)][i];
+        v0 = __shfl_sync(0xffffffffu, u, 0);
+        if (m > 1) {
+            v1 = __shfl_sync(0xffffffffu, u, 1);
+            v2 = __shfl_sync(0xffffffffu, u, 2);
+        }
+    };
+    if (active && w == 0 && lane == 0) *mine_flag = 0;
+    unsigned epoch = 0;
+    if (!grid_barrier(ctrl, status, gridDim.x, epoch)) return false;
+    bool late = false, done = k < 2;
+    int sweep = 0, round = 0;  // round: rounds since the kernel's start
+    for (; sweep < max_sweeps && !done; ++sweep) {
+        int mine = 0;
+        for (int r = 0; active && r < N - 1; ++r, ++round) {
+            if (r > 0 && !late) {
+                int it = 0;
+                while (!__all_sync(0xffffffffu, !watch || (int)ld_acquire(reinterpret_cast<const unsigned*>(near)) >= round)) {
+                    if (++it > SPIN_LIMIT) {
+                        late = true;
+                        if (lane == 0) atomicOr(status, DEV_TIMEOUT);
+                        break;
+                    }
+                }
+                __syncwarp();
+            }
+            int p, q;
+            round_pair(N, r, slot, p, q);
+            const bool both = q < k;
+            double* wp = W + (long)p * n + 32 * w + lane;
+            double* wq = W + (long)q * n + 32 * w + lane;
+            double x[E], y[E];
+            bool rot = false;
+            if (both) {
+                const int left = n - 32 * w - lane;  // columns from this lane's first
+#pragma unroll
+                for (int e = 0; e < E; ++e)
+                    if (e < ne) {
+                        x[e] = 32 * G * e < left ? __ldcg(wp + 32 * G * e) : 0.0;
+                        y[e] = 32 * G * e < left ? __ldcg(wq + 32 * G * e) : 0.0;
+                    }
+                double a = __ldcg(nrm + p), bb = __ldcg(nrm + q);
+                double pa = __ldcg(part + (long)p * 128 + 32 * w + lane), pb = __ldcg(part + (long)q * 128 + 32 * w + lane);
+                double c0 = 0.0, c1 = 0.0;
+#pragma unroll
+                for (int e = 0; e < E; ++e)
+                    if (e < ne) {
+                        if (e & 1)
+                            c1 = fma(x[e], y[e], c1);
+                        else
+                            c0 = fma(x[e], y[e], c0);
+                    }
+                double c = c0 + c1;
+                bool fa = a < 0.0, fb = bb < 0.0;
+                if (r == 0) {  // norms summed afresh at every sweep
+                    pa = pb = 0.0;
+#pragma unroll
+                    for (int e = 0; e < E; ++e)
+                        if (e < ne) {
+                            pa = fma(x[e], x[e], pa);
+                            pb = fma(y[e], y[e], pb);
+                        }
+                    fa = fb = true;
+                }
+                const bool sums = fa || fb;
+                if (sums) {
+                    osj_sum3(c, pa, pb, lane);
+                    across(3, c, pa, pb);
+                    a = fa ? pa : a;
+                    bb = fb ? pb : bb;
+                } else {
+                    c = warp_sum(c);
+                    across(1, c, pa, pb);
+                }
+                if (a > 0.0 && bb > 0.0) {
+                    const int far = osj_far(c, a, bb, tol);
+                    rot = far > 0 || (far == 0 && fabs(c) > tol * sqrt(a * bb));
+                }
+                if (rot) {
+                    double t, cs, sn;
+                    osj_angle(a, bb, c, t, cs, sn);
+                    const bool p_shrinks = t * c > 0.0;
+                    double ns = 0.0;
+#pragma unroll
+                    for (int e = 0; e < E; ++e)
+                        if (e < ne) {
+                            const double xn = cs * x[e] - sn * y[e];
+                            const double yn = sn * x[e] + cs * y[e];
+                            if (32 * G * e < left) {
+                                __stcg(wp + 32 * G * e, xn);
+                                __stcg(wq + 32 * G * e, yn);
+                            }
+                            const double v = p_shrinks ? xn : yn;
+                            ns = fma(v, v, ns);
+                        }
+                    __stcg(part + (long)(p_shrinks ? p : q) * 128 + 32 * w + lane, ns);
+                    const double grown = p_shrinks ? bb + t * c : a - t * c;
+                    a = p_shrinks ? -1.0 : grown;
+                    bb = p_shrinks ? grown : -1.0;
+                    ++mine;
+                }
+                if ((rot || sums) && w == 0 && lane == 0) {
+                    __stcg(nrm + p, a);
+                    __stcg(nrm + q, bb);
+                }
+            } else if (r == 0) {  // the row that sits a round out
+                double ns = 0.0;
+                for (int j = 32 * w + lane; j < n; j += 32 * G) {
+                    const double v = __ldcg(W + (long)p * n + j);
+                    ns = fma(v, v, ns);
+                }
+                __stcg(part + (long)p * 128 + 32 * w + lane, ns);
+                if (w == 0 && lane == 0) __stcg(nrm + p, -1.0);
+            }
+            group_sync();
+            if (w == 0 && lane == 0)
+                asm volatile("st.release.gpu.global.s32 [%0], %1;" ::"l"(mine_flag), "r"(round + 1) : "memory");
+        }
+        if (active && w == 0 && lane == 0 && mine) atomicAdd(ctrl + 4 + sweep, mine);
+        if (!grid_barrier(ctrl, status, gridDim.x, epoch)) return false;
+        done = __ldcg(ctrl + 4 + sweep) == 0;
+    }
+    sweeps = k >= 2 ? sweep : 0;
+    if (!done && blockIdx.x == 0 && threadIdx.x == 0) atomicOr(status, DEV_NOT_CONVERGED);
+    return true;
+}
+
+__global__ void __launch_bounds__(128, 1)
+osj_grid_kernel(int n, const int* __restrict__ k_dev, double* W, double* nrm, double* lam_u, double* vt_u, int* ctrl,
+                int* status, int max_sweeps, const int* n_dev, int nsmall, int nlarge, double* part, int* flags) {
+    if (n_dev) {  // a captured step: other sizes take the launches beside it
+        n = *n_dev;
+        if (n <= nsmall || n > nlarge) return;  // every CTA, before any barrier
+    }
+    const double tol = sqrt((double)n) * 2.220446049250313e-16;  // as in osj_kernel
+    const int lane = threadIdx.x & 31, gw = blockIdx.x * 4 + (threadIdx.x >> 5), nw = gridDim.x * 4;
+    const int kraw = *k_dev;
+    const int k = min(kraw, n);
+    int sweeps = 0;
+    if (kraw >= 0) {
+        const int b = ((k + 1) / 2 + gridDim.x - 1) / gridDim.x;
+        bool ok;
+        if (b <= 1)
+            ok = osj_grid_body<OSJ_GRID_N / 128, 4>(n, k, W, nrm, part, flags, ctrl, status, max_sweeps, tol, sweeps);
+        else if (b == 2)
+            ok = osj_grid_body<OSJ_GRID_N / 64, 2>(n, k, W, nrm, part, flags, ctrl, status, max_sweeps, tol, sweeps);
+        else
+            ok = osj_grid_body<OSJ_GRID_N / 32, 1>(n, k, W, nrm, part, flags, ctrl, status, max_sweeps, tol, sweeps);
+        if (!ok) return;
+        if (blockIdx.x == 0 && threadIdx.x == 0) ctrl[2] = sweeps;
+    }
+    // eigenvalues: the converged rows' squared norms, summed from the rows
+    for (int i = gw; i < n; i += nw) {
+        double a = 0.0;
+        if (i < k) {
+            for (int j = lane; j < n; j += 32) {
+                const double v = __ldcg(W + (long)i * n + j);
+                a = fma(v, v, a);
+            }
+            a = warp_sum(a);
+        }
+        const double f = a > 0.0 ? 1.0 / sqrt(a) : 0.0;
+        if (lane == 0) lam_u[i] = kraw < 0 ? __longlong_as_double(0x7ff8000000000000LL) : a;
+        for (int j = lane; j < n; j += 32) vt_u[(long)i * n + j] = i < k ? f * __ldcg(W + (long)i * n + j) : 0.0;
+    }
 }
 
 // Pivoted Cholesky on one thread-block cluster for n <= PCHOL_SMALL_N: the
@@ -1482,26 +1670,42 @@ tt_status osj_launch(cudaStream_t s, int ncap, const int* k_dev, EigWork& w, int
                                        status_dev, msw, n_dev, nsmall));
         if (ncap <= nsmall) return TT_OK;
     }
-    // rows in registers up to n = 1024 (entries per lane: 8, 16 or 32)
-    const void* fn = ncap <= 512    ? (const void*)osj_kernel<16>
-                     : ncap <= 1024 ? (const void*)osj_kernel<32>
-                                    : (const void*)osj_kernel<0>;
-    // one CTA per SM with one warp per pair it owns, so every SM carries the
-    // same number of pairs in a round (the round ends at the slowest SM)
-    int blocks = 1, wpb = 1;
-    {
-        int dev = 0, sms = 0, per_sm = 0;
-        TT_CUDA_TRY(cudaGetDevice(&dev));
-        TT_CUDA_TRY(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
-        const int npairs = (ncap + 1) / 2;
-        wpb = std::max(1, std::min(OSJ_MAX_WARPS, (npairs + sms - 1) / sms));
-        TT_CUDA_TRY(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, fn, 32 * wpb, 0));
+    int dev = 0, sms = 0;
+    TT_CUDA_TRY(cudaGetDevice(&dev));
+    TT_CUDA_TRY(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
+    auto resident = [&](const void* fn, int threads, int& blocks) -> tt_status {
+        int per_sm = 0;
+        TT_CUDA_TRY(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, fn, threads, 0));
         if (per_sm < 1) {
             set_error("one-sided Jacobi kernel cannot be resident");
             return TT_ERR_CUDA;
         }
-        blocks = std::max(1, std::min((npairs + wpb - 1) / wpb, per_sm * sms));
+        blocks = per_sm * sms;
+        return TT_OK;
+    };
+    int blocks = 1;
+    int nlarge = std::min(OSJ_GRID_N, 8 * sms);  // at most four pairs a CTA
+    if (ncap <= nlarge || n_dev) {
+        // a CTA per SM whatever n: the pairs' split over warps follows from it and
+        // from the rank alone, so a replay's sums are the host path's.  Scratch:
+        // pchol's, free by now
+        const void* fn = (const void*)osj_grid_kernel;
+        TT_TRY(resident(fn, 128, blocks));
+        double* part = w.g1.p;                           // 128 a row
+        int* flags = reinterpret_cast<int*>(w.psd.p);  // OSJ_FLAG ints a pair of rows
+        void* args[] = {&nn, &k_dev, &Wp, &nrm, &lamu, &vtu, &ctrl, &status_dev, &msw, &n_dev, &nsmall, &nlarge, &part, &flags};
+        note_launch();
+        TT_CUDA_TRY(cudaLaunchCooperativeKernel(fn, dim3(sms), dim3(128), args, 0, s));
+        if (ncap <= nlarge) return TT_OK;
+        nsmall = nlarge;
     }
+    // one CTA per SM with one warp per pair it owns, so every SM carries the
+    // same number of pairs in a round (the round ends at the slowest SM)
+    const void* fn = (const void*)osj_kernel;
+    const int npairs = (ncap + 1) / 2;
+    const int wpb = std::max(1, std::min(OSJ_MAX_WARPS, (npairs + sms - 1) / sms));
+    TT_TRY(resident(fn, 32 * wpb, blocks));
+    blocks = std::max(1, std::min((npairs + wpb - 1) / wpb, blocks));
     void* args[] = {&nn, &k_dev, &Wp, &nrm, &lamu, &vtu, &ctrl, &status_dev, &msw, &n_dev, &nsmall};
     note_launch();
     TT_CUDA_TRY(cudaLaunchCooperativeKernel(fn, dim3(blocks), dim3(32 * wpb), args, 0, s));
