@@ -24,10 +24,8 @@
 // the sizes where it is used (tc8_wanted) have K >= 64.
 //
 // Measured (GB300, CUDA events, against the FP64 pipe's kernels): Gram of
-// 500,000 x 449 143 -> 8.9 ms, error against the exact product 1.3e-15 ->
-// 2.7e-16; 200,000 x 577 times 577 x 96 22.4 -> 2.6 ms, 8.0e-16 -> 5.4e-16;
-// 128^3 FP64 step at ranks 64 -> 128 870 -> 89 ms; 500^2 step at R = 876
-// 385 -> 79 ms.
+// 500,000 x 449 143 -> 5.7 ms, error against the exact product 1.3e-15 ->
+// 2.7e-16; 200,000 x 577 times 577 x 96 22.4 -> 1.8 ms, 8.0e-16 -> 5.4e-16.
 //
 // Inf, NaN and rows whose largest entry is outside 2^+-900 cannot be split:
 // the exponent scans latch a device flag and an FP64-pipe kernel behind the
@@ -52,15 +50,22 @@ constexpr int RB = 64;                         // rows of an image block
 constexpr int DIG_BYTES = RB * T_K * 2;        // one digit of one block and stage: 4096
 constexpr int BLK_BYTES = S8 * DIG_BYTES;      // 32768
 constexpr int A_BYTES = 2 * BLK_BYTES, B_BYTES = BLK_BYTES, STAGE_BYTES = A_BYTES + B_BYTES;
-constexpr int SLOT_BYTES = 3 * DIG_BYTES;      // A digit s (128 rows) and B digit 7 - s (64 rows)
+// A stage is refilled in two groups of digit pairs (A's digit s with B's digit
+// 7 - s): 0 and 1 (15 of the 36 products), then the others
+constexpr int GROUPS = 2;
+__host__ __device__ constexpr int group_start(int g) { return g == 0 ? 0 : g == 1 ? 2 : S8; }
 constexpr int DRAIN_WARPS = 16;
 constexpr int THREADS8 = 32 * (2 + DRAIN_WARPS);
 constexpr int DCOLS = T_N / (DRAIN_WARPS / 4);  // columns of a drain thread: 16
 constexpr unsigned TMEM_COLS = 512;
 constexpr long long SPIN = 1LL << 26;
 constexpr size_t SMEM8 = (size_t)T_STAGES * STAGE_BYTES + 1024 /* barriers */ + 1024 /* alignment */;
-// digit images of one pass over an operand: a longer operand goes in chunks
-constexpr long IMG_LIMIT = 1L << 27;
+// Digit images of one pass over an operand; a longer operand goes in chunks.  A
+// chunk costs its launches and a last wave: with images of 2^26, 2^27, 2^28, 2^29
+// and 2^30 bytes the Gram of 500,000 x 449 took 10.3, 9.1, 8.5, 8.4 and 8.6 ms and
+// 200,000 x 577 times 577 x 96 3.0, 2.6, 2.1, 2.1 and 2.5 (before the present
+// issue loop and split), although only the smaller ones stay in the 129 MB L2.
+constexpr long IMG_LIMIT = 1L << 28;
 
 __device__ __forceinline__ unsigned smem_addr(const void* p) { return (unsigned)__cvta_generic_to_shared(p); }
 __device__ __forceinline__ void bar_init(unsigned a, unsigned count) {
@@ -235,23 +240,24 @@ __device__ __forceinline__ u64 biased56(double v, int e) {
 // images (v0 in the low half): the biased digits u of both go into one word
 // as the BF16 pair 128 + u, one packed subtraction of 192 (128 for the
 // leading digit) leaves the digits exactly, and the signs are flipped in.
+__device__ __forceinline__ unsigned digit_pair(u64 F0, u64 F1, int s) {  // without the signs
+    const __nv_bfloat162 lead = __floats2bfloat162_rn(128.0f, 128.0f), rest = __floats2bfloat162_rn(192.0f, 192.0f);
+    const unsigned u0 = (unsigned)(F0 >> (7 * (7 - s))) & 0x7Fu;
+    const unsigned u1 = (unsigned)(F1 >> (7 * (7 - s))) & 0x7Fu;
+    const unsigned p = 0x43004300u | u0 | (u1 << 16);
+    __nv_bfloat162 x;
+    memcpy(&x, &p, 4);
+    const __nv_bfloat162 d = __hsub2(x, s == 0 ? lead : rest);
+    unsigned r;
+    memcpy(&r, &d, 4);
+    return r;
+}
 __device__ __forceinline__ void digits8x2(double v0, double v1, int e0, int e1, unsigned (&w)[S8]) {
     const u64 F0 = biased56(v0, e0), F1 = biased56(v1, e1);
     const unsigned sg = ((unsigned)((u64)__double_as_longlong(v0) >> 48) & 0x8000u) |
                         ((unsigned)((u64)__double_as_longlong(v1) >> 32) & 0x80000000u);
-    const __nv_bfloat162 lead = __floats2bfloat162_rn(128.0f, 128.0f), rest = __floats2bfloat162_rn(192.0f, 192.0f);
 #pragma unroll
-    for (int s = 0; s < S8; ++s) {
-        const unsigned u0 = (unsigned)(F0 >> (7 * (7 - s))) & 0x7Fu;
-        const unsigned u1 = (unsigned)(F1 >> (7 * (7 - s))) & 0x7Fu;
-        const unsigned p = 0x43004300u | u0 | (u1 << 16);
-        __nv_bfloat162 x;
-        memcpy(&x, &p, 4);
-        const __nv_bfloat162 d = __hsub2(x, s == 0 ? lead : rest);
-        unsigned r;
-        memcpy(&r, &d, 4);
-        w[s] = r ^ sg;
-    }
+    for (int s = 0; s < S8; ++s) w[s] = digit_pair(F0, F1, s) ^ sg;
 }
 // Byte offset of (row r, index k) in a swizzled digit tile of 64-byte rows
 __device__ __forceinline__ unsigned swz(int r, int k) {
@@ -384,9 +390,11 @@ __global__ void __launch_bounds__(256) split_rows_long_kernel(Prod p, Side o, in
 }
 
 // Rows that are the columns of a stored matrix (the Gram's operand): column
-// maxima, then the digits of a chunk of its rows.  A thread splits 16 rows of
-// one column, so that a warp reads 32 neighbouring columns of a row at a time
-// and stores one 32-byte sector a digit and lane.
+// maxima, then the digits of a chunk of its rows.  A thread splits 8 rows of one
+// column, so that a warp reads 32 neighbouring columns of a row at a time, and
+// stores 16 bytes a digit.  Bound by the latency of its loads: 8 rows fit 64
+// registers, four CTAs an SM (49,152 x 449: 156 us, 3.7 TB/s; with 16 rows a
+// thread, 128 registers and two CTAs 251 us, with 48 registers and spills 230).
 __global__ void __launch_bounds__(256) strided_max_kernel(Prod p, Side o) {
     p.Mc = p.M;
     if (!resolve(p)) return;
@@ -418,7 +426,7 @@ __global__ void __launch_bounds__(256) strided_max_kernel(Prod p, Side o) {
         }
     }
 }
-__global__ void __launch_bounds__(256, 2) split_strided_kernel(Prod p, Side o, int* flag) {
+__global__ void __launch_bounds__(256, 4) split_strided_kernel(Prod p, Side o, int* flag) {
     if (!resolve(p)) return;
     long i0, rows, rpad, ld;
     side_sizes(p, o, i0, rows, rpad, ld);
@@ -432,27 +440,25 @@ __global__ void __launch_bounds__(256, 2) split_strided_kernel(Prod p, Side o, i
             e = split_exp(o.mx[i0 + j], flag);
             if (blockIdx.y == 0 && threadIdx.x < 32) o.e[i0 + j] = e;
         }
-        const long groups = (long)nst * 2;
+        const long groups = (long)nst * 4;
         for (long g = (long)blockIdx.y * 8 + (threadIdx.x >> 5); g < groups; g += (long)gridDim.y * 8) {
-            const long k0 = g * 16;
-            unsigned w[S8][8];
+            const long k0 = g * 8;
+            u64 F[8];
+            unsigned sg[4];
 #pragma unroll
-            for (int r = 0; r < 16; r += 2) {
-                const double v0 = j < rows && k0 + r < Kc ? A[(k0 + r) * ld + j] : 0.0;
-                const double v1 = j < rows && k0 + r + 1 < Kc ? A[(k0 + r + 1) * ld + j] : 0.0;
-                unsigned wd[S8];
-                digits8x2(v0, v1, e, e, wd);
+            for (int r = 0; r < 8; ++r) F[r] = j < rows && k0 + r < Kc ? (u64)__double_as_longlong(__ldcs(A + (k0 + r) * ld + j)) : 0ull;
 #pragma unroll
-                for (int s = 0; s < S8; ++s) w[s][r / 2] = wd[s];
+            for (int r = 0; r < 8; ++r) {
+                const unsigned sign = ((unsigned)(F[r] >> 48) & 0x8000u) << (16 * (r & 1));
+                sg[r >> 1] = r & 1 ? sg[r >> 1] | sign : sign;
+                F[r] = biased56(__longlong_as_double((long long)F[r]), e);
             }
-            const int r = (int)(j & 63), st = (int)(g >> 1), half = (int)(g & 1) * 16;
-            unsigned char* d = tile_at(o.img, j >> 6, nst, st, 0);
-            const unsigned o0 = swz(r, half), o1 = swz(r, half + 8);
+            unsigned char* d = tile_at(o.img, j >> 6, nst, (int)(g >> 2), 0) + swz((int)(j & 63), (int)(g & 3) * 8);
 #pragma unroll
-            for (int s = 0; s < S8; ++s) {
-                *reinterpret_cast<uint4*>(d + s * DIG_BYTES + o0) = make_uint4(w[s][0], w[s][1], w[s][2], w[s][3]);
-                *reinterpret_cast<uint4*>(d + s * DIG_BYTES + o1) = make_uint4(w[s][4], w[s][5], w[s][6], w[s][7]);
-            }
+            for (int s = 0; s < S8; ++s)
+                *reinterpret_cast<uint4*>(d + s * DIG_BYTES) =
+                    make_uint4(digit_pair(F[0], F[1], s) ^ sg[0], digit_pair(F[2], F[3], s) ^ sg[1],
+                               digit_pair(F[4], F[5], s) ^ sg[2], digit_pair(F[6], F[7], s) ^ sg[3]);
         }
     }
 }
@@ -506,18 +512,24 @@ __device__ __forceinline__ void tile_of(long t, int nb, bool tri, long& mb, int&
 }
 
 // One CTA per SM walks (split of the contraction, output tile) items.  Warp 0
-// copies: slot s of a stage is A's digit s and B's digit 7 - s, the pair that
-// the MMAs of digit s use last, so a slot is refilled for the stage after next
-// as soon as those MMAs are done (a commit per digit) and loads are always in
-// flight.  Warp 1 issues: eight FP32 accumulators of 128 x 64 (one per level,
-// all 512 TMEM columns); the digit tiles of B lie back to back, so A's digit
-// s meets up to four of B's digits in one MMA of N <= 256 whose levels are
-// neighbouring column ranges.  Sixteen warps drain a block's accumulators into
-// 64-bit integers (a float-to-int and a wide multiply-add a value) and, at
-// an item's end, write the FP64 results while the next item's MMAs run.
+// copies: A's digit s and B's digit 7 - s are the pair that the MMAs of digit s
+// use last, so a group of pairs is refilled for the stage after next as soon as
+// the MMAs of its last digit are done (a commit per group).  Warp 1 issues: eight
+// FP32 accumulators of 128 x 64 (one per level, all 512 TMEM columns); the digit
+// tiles of B lie back to back, so A's digit s meets up to four of B's digits in
+// one MMA of N <= 256 whose levels are neighbouring column ranges.  Sixteen warps
+// drain a block's accumulators into 64-bit integers (a float-to-int and a wide
+// multiply-add a value) and, at an item's end, write the FP64 results while the
+// next item's MMAs run.
 //
-// What bounds it: shared memory.  Per 16 indices the MMAs read 120 KB of
-// operands and 48 KB arrive, 168 KB or 1312 clocks against 1152 of MMA.
+// What bounds it: the tensor cores (74% of their cycles; 1184 clocks of MMA per
+// 16 indices against 937 of operand reads and 375 of arrivals in shared memory),
+// then the drains, which the MMAs wait for: TMEM holds one set of accumulators.
+// The issuing thread must not be what bounds it: with a rolled loop, descriptors
+// computed per MMA and a commit per digit a stage took 4600 clocks even without
+// loads (tensor cores at 45%); unrolled, with descriptors that are constants from
+// the stage's, about 2900.  196,608 x 512 times 512 x 512: 4.1 -> 2.6 ms; commits
+// per stage 8, 4, 3, 2, 1 with the rolled loop: 3.84, 4.02, 3.94, 3.59, 3.55 ms.
 __global__ void __launch_bounds__(THREADS8, 1)
 tc8_kernel(Prod p, const unsigned char* __restrict__ At, const int* __restrict__ eA,
            const unsigned char* __restrict__ Bt, const int* __restrict__ eB, double alpha, double* __restrict__ C,
@@ -537,7 +549,7 @@ tc8_kernel(Prod p, const unsigned char* __restrict__ At, const int* __restrict__
     const unsigned pad = ((raw_s + 1023u) & ~1023u) - raw_s;
     const unsigned sb = raw_s + pad;
     u64* bars = reinterpret_cast<u64*>(raw + pad + T_STAGES * STAGE_BYTES);
-    // bars: [0,1] stage full, [2 + 8 st + s] slot empty, [18] accumulators full,
+    // bars: [0,1] stage full, [2 + 8 st + q] group q empty, [18] accumulators full,
     // [19] accumulators drained, [20] every MMA done
     unsigned* tmem_slot = reinterpret_cast<unsigned*>(bars + 24);
     volatile int* flags = reinterpret_cast<volatile int*>(tmem_slot + 2);  // abort, stages issued, consumed
@@ -549,7 +561,7 @@ tc8_kernel(Prod p, const unsigned char* __restrict__ At, const int* __restrict__
     if ((long)blockIdx.x >= items) return;
     if (threadIdx.x == 0) {
         for (int i = 0; i < 21; ++i)
-            bar_init(smem_addr(&bars[i]), i < 2 ? (unsigned)S8 : (i == 19 ? (unsigned)DRAIN_WARPS : 1u));
+            bar_init(smem_addr(&bars[i]), i < 2 ? (unsigned)GROUPS : (i == 19 ? (unsigned)DRAIN_WARPS : 1u));
         flags[0] = flags[1] = flags[2] = 0;
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
@@ -582,16 +594,20 @@ tc8_kernel(Prod p, const unsigned char* __restrict__ At, const int* __restrict__
                     const unsigned char* a0 = At + (2 * mb * nst + it) * (long)BLK_BYTES;
                     const unsigned char* a1 = a0 + (long)nst * BLK_BYTES;
                     const unsigned char* b0 = Bt + ((long)kb * nst + it) * BLK_BYTES;
-                    for (int s = 0; s < S8; ++s) {
-                        if (!stop && !bar_wait(smem_addr(&bars[2 + 8 * st + s]), ph ^ 1u, status, flags)) stop = true;
+                    for (int q = 0; q < GROUPS; ++q) {
+                        if (!stop && !bar_wait(smem_addr(&bars[2 + 8 * st + q]), ph ^ 1u, status, flags)) stop = true;
                         if (stop) {  // the stage's barrier completes with what was issued
                             bar_arrive(full);
                             continue;
                         }
-                        bar_expect(full, (unsigned)SLOT_BYTES);
-                        bulk_g2s(dst + s * 2 * DIG_BYTES, a0 + s * DIG_BYTES, DIG_BYTES, full);
-                        bulk_g2s(dst + s * 2 * DIG_BYTES + DIG_BYTES, a1 + s * DIG_BYTES, DIG_BYTES, full);
-                        bulk_g2s(dst + A_BYTES + (7 - s) * DIG_BYTES, b0 + (7 - s) * DIG_BYTES, DIG_BYTES, full);
+                        const int s0 = group_start(q), s1 = group_start(q + 1);
+                        bar_expect(full, (unsigned)(3 * (s1 - s0) * DIG_BYTES));
+                        for (int s = s0; s < s1; ++s) {
+                            bulk_g2s(dst + s * 2 * DIG_BYTES, a0 + s * DIG_BYTES, DIG_BYTES, full);
+                            bulk_g2s(dst + s * 2 * DIG_BYTES + DIG_BYTES, a1 + s * DIG_BYTES, DIG_BYTES, full);
+                        }
+                        bulk_g2s(dst + A_BYTES + (S8 - s1) * DIG_BYTES, b0 + (S8 - s1) * DIG_BYTES,
+                                 (unsigned)((s1 - s0) * DIG_BYTES), full);
                     }
                     flags[1] = (int)(g + 1);
                 }
@@ -620,20 +636,25 @@ tc8_kernel(Prod p, const unsigned char* __restrict__ At, const int* __restrict__
                     }
                     flags[2] = (int)(g + 1);
                     fence_after();
-                    const unsigned aB = sb + (unsigned)(st * STAGE_BYTES), bB = aB + A_BYTES;
-#pragma unroll 1
+                    // every MMA's descriptors are the stage's plus a constant: one
+                    // thread issues 24 MMAs a stage, a few instructions each
+                    const u64 ad0 = opdesc(sb + (unsigned)(st * STAGE_BYTES));
+                    const unsigned acc0 = first ? 0u : 1u;
+#pragma unroll
                     for (int s = 0; s < S8; ++s) {
 #pragma unroll
                         for (int kk = 0; kk < 2; ++kk) {
-                            const u64 ad = opdesc(aB + (unsigned)(s * 2 * DIG_BYTES + kk * 32));
-                            const unsigned acc = (first && s == 0 && kk == 0) ? 0u : 1u;
+                            const u64 ad = ad0 + (u64)((s * 2 * DIG_BYTES + kk * 32) >> 4);
+#pragma unroll
                             for (int t0 = 0; t0 < S8 - s; t0 += 4) {
-                                const int c = min(4, S8 - s - t0);
-                                const u64 bd = opdesc(bB + (unsigned)(t0 * DIG_BYTES + kk * 32));
-                                mma8(tmem + (unsigned)((s + t0) * T_N), ad, bd, mmadesc(c * T_N), acc);
+                                const u64 bd = ad0 + (u64)((A_BYTES + t0 * DIG_BYTES + kk * 32) >> 4);
+                                mma8(tmem + (unsigned)((s + t0) * T_N), ad, bd,
+                                     mmadesc((S8 - s - t0 < 4 ? S8 - s - t0 : 4) * T_N), s == 0 && kk == 0 ? acc0 : 1u);
                             }
                         }
-                        mma_commit(smem_addr(&bars[2 + 8 * st + s]));
+#pragma unroll
+                        for (int q = 0; q < GROUPS; ++q)
+                            if (s == group_start(q + 1) - 1) mma_commit(smem_addr(&bars[2 + 8 * st + q]));
                     }
                     if (((it - st0) % T_BLK) == T_BLK - 1 || it == st1 - 1) {
                         mma_commit(smem_addr(&bars[18]));
