@@ -835,7 +835,9 @@ osj_cluster_kernel(int n, const int* __restrict__ k_dev, const double* W, double
 // launch) and every wait is bounded: a warp whose wait ran out sets DEV_TIMEOUT
 // and waits no more, and the grid barrier after the sweep ends the kernel.
 // nrm[i]: row i's squared norm, or -1 where part[i] holds its partial sums, to be
-// summed over the lanes with the next inner product.
+// summed over the lanes with the next inner product.  Of a rotation's two new norms
+// the shrinking one is summed again only where it halved, an eighth of the FP64
+// instructions of a rotating pair less (rank 451 of 713: 34 -> 31 ms).
 // Measured (GB300, factorisation included): graded full-rank matrices n = 300 25.1 ->
 // 14.0 ms, 449 39.2 -> 31.5, 608 76.8 -> 48.8; rank 451 of 713 47 -> 34; rank 311
 // of 311 20 -> 12.
@@ -955,24 +957,39 @@ __device__ bool osj_grid_body(int n, int k, double* W, double* nrm, double* part
                 if (rot) {
                     double t, cs, sn;
                     osj_angle(a, bb, c, t, cs, sn);
-                    const bool p_shrinks = t * c > 0.0;
-                    double ns = 0.0;
+                    // the shrinking row's norm is summed again only where it lost
+                    // more than half (the formula cancels no further)
+                    const double tc = t * c;
+                    const bool p_shrinks = tc > 0.0;
+                    const double old = p_shrinks ? a : bb;
+                    a -= tc;
+                    bb += tc;
+                    const bool resum = __double2hiint(p_shrinks ? a : bb) < __double2hiint(old) - (1 << 20);
 #pragma unroll
                     for (int e = 0; e < E; ++e)
                         if (e < ne) {
                             const double xn = cs * x[e] - sn * y[e];
-                            const double yn = sn * x[e] + cs * y[e];
+                            y[e] = sn * x[e] + cs * y[e];
+                            x[e] = xn;
                             if (32 * G * e < left) {
-                                __stcg(wp + 32 * G * e, xn);
-                                __stcg(wq + 32 * G * e, yn);
+                                __stcg(wp + 32 * G * e, x[e]);
+                                __stcg(wq + 32 * G * e, y[e]);
                             }
-                            const double v = p_shrinks ? xn : yn;
-                            ns = fma(v, v, ns);
                         }
-                    __stcg(part + (long)(p_shrinks ? p : q) * 128 + 32 * w + lane, ns);
-                    const double grown = p_shrinks ? bb + t * c : a - t * c;
-                    a = p_shrinks ? -1.0 : grown;
-                    bb = p_shrinks ? grown : -1.0;
+                    if (resum) {
+                        double ns = 0.0;
+#pragma unroll
+                        for (int e = 0; e < E; ++e)
+                            if (e < ne) {
+                                const double v = p_shrinks ? x[e] : y[e];
+                                ns = fma(v, v, ns);
+                            }
+                        __stcg(part + (long)(p_shrinks ? p : q) * 128 + 32 * w + lane, ns);
+                        if (p_shrinks)
+                            a = -1.0;
+                        else
+                            bb = -1.0;
+                    }
                     ++mine;
                 }
                 if ((rot || sums) && w == 0 && lane == 0) {
