@@ -533,9 +533,15 @@ tt_status tt_create_shard(const tt_problem_desc* desc, void* stream, int plane_b
  * ------------------------------------------------------------------------ */
 
 /*
- * tt_dgemm: C = alpha op(A) op(B) + beta C in FP64 on the FP64 tensor pipe
- * (mma m8n8k4), row-major, op(X) = X if trans_x == 0 else X^T; op(A) is M x K,
+ * tt_dgemm: C = alpha op(A) op(B) + beta C in FP64, row-major, op(X) = X if trans_x == 0 else X^T; op(A) is M x K,
  * op(B) is K x N, C is M x N with leading dimensions lda, ldb, ldc.
+ * beta = 0 and more than about 16M terms: exact integer digit products on the
+ * BF16 tensor cores, an entry off by at most K 2^-51 max|a_i| max|b_j| (rows of
+ * op(A), columns of op(B)); operands for which that is far above the sum
+ * |a||b| (rows whose large entries are few or meet small ones), Inf, NaN and
+ * extreme scales are recomputed on the FP64 tensor pipe (mma m8n8k4), which
+ * takes all other calls.  Reproducible to the bit.  Device scratch from the
+ * library's own pool, which keeps up to 512 MB between calls.
  */
 tt_status tt_dgemm(int trans_a, int trans_b, int M, int N, int K, double alpha,
                    const double* A_dev, int lda, const double* B_dev, int ldb, double beta,
@@ -543,10 +549,10 @@ tt_status tt_dgemm(int trans_a, int trans_b, int M, int N, int K, double alpha,
 
 /*
  * tt_gram: G = A^T A for a tall row-major A (m x n, leading dimension lda), the
- * left Gram matrix of App. A.2 (G_A = A^T A).  Split over the m rows with a
- * fixed-order reduction, so the result is bitwise reproducible; G (n x n,
- * leading dimension ldg) is exactly symmetric.  Uses device scratch of
- * (number of row splits) * n * n doubles allocated by the library.
+ * left Gram matrix of App. A.2 (G_A = A^T A).  Digit products or the FP64
+ * tensor pipe as in tt_dgemm (rows are A's columns), split over the m rows with
+ * a fixed-order reduction, so the result is bitwise reproducible; G (n x n,
+ * leading dimension ldg) is exactly symmetric.  Scratch as in tt_dgemm.
  */
 tt_status tt_gram(int m, int n, const double* A_dev, int lda, double* G_dev, int ldg, void* stream);
 

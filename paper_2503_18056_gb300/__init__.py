@@ -635,7 +635,8 @@ class TTSNBatch:
 
 
 def dgemm(A, B, trans_a=False, trans_b=False, alpha=1.0, stream=None):
-    """C = alpha op(A) op(B) on the FP64 tensor pipe (library kernel)."""
+    """C = alpha op(A) op(B) in FP64 (library kernels: digit products on the BF16
+    tensor cores for large products, else the FP64 tensor pipe)."""
     A, B = _dev(A), _dev(B)
     M = A.shape[1] if trans_a else A.shape[0]
     K = A.shape[0] if trans_a else A.shape[1]

@@ -25,11 +25,21 @@
 //
 // Measured (GB300, CUDA events, against the FP64 pipe's kernels): Gram of
 // 500,000 x 449 143 -> 5.7 ms, error against the exact product 1.3e-15 ->
-// 2.7e-16; 200,000 x 577 times 577 x 96 22.4 -> 1.8 ms, 8.0e-16 -> 5.4e-16.
+// 2.7e-16; 200,000 x 577 times 577 x 96 22.4 -> 1.8 ms, 8.0e-16 -> 5.5e-16.
 //
 // Inf, NaN and rows whose largest entry is outside 2^+-900 cannot be split:
 // the exponent scans latch a device flag and an FP64-pipe kernel behind the
 // product, which otherwise returns at once, recomputes it.
+//
+// An entry far below its row's maximum keeps few digits, which matters where
+// small entries meet large ones (A times the identity, disjoint supports): the
+// sum |a||b| is then far below K max|a_i| max|b_j|, which bounds the error.  The
+// rounding needs its Grams to eps ||A||^2 only; a library call is also held to
+// the sum's scale: the split counts each row's entries above 2^-9 of its
+// maximum, and unless every pair of rows has K / 16 indices where both are
+// (tc8_lost), the product is recomputed on the FP64 pipe (the count and the
+// check: 200,000 x 577 times 577 x 96 1.73 -> 1.78 ms, the Gram of 500,000 x 449
+// 5.68 -> 5.70).
 #include <cuda.h>
 #include <cuda_bf16.h>
 
@@ -276,7 +286,10 @@ struct Side {
     u64* mx;           // row maxima (where they are found ahead of the split)
     int* e;            // row exponents
     unsigned char* img;
+    int* large;  // a guarded call: each row's entries of at least 2^(e - 10)
+    int* worst;  // and the most that a row falls short of K (split_rows_kernel; spread_kernel)
 };
+constexpr u64 F_LARGE = (1ull << 46) + 0x1020408102040ull;  // biased56 of 2^(e - 10)
 __device__ __forceinline__ void side_sizes(const Prod& p, const Side& o, long& i0, long& rows, long& rpad, long& ld) {
     i0 = o.isB ? 0 : p.i0;
     rows = o.isB ? p.N : p.Mc;
@@ -319,6 +332,14 @@ __global__ void __launch_bounds__(256) split_rows_kernel(Prod p, Side o, int* fl
         }
         const int e = split_exp(mx, flag);
         if (lane == 0 && r < rows) o.e[i0 + r] = e;
+        if (o.worst && mx != 0) {
+            int c = 0;
+#pragma unroll
+            for (int t = 0; t < V; ++t)
+                c += ((int)(mag(v[t][0]) >> 52) >= e - 10 + 1023) + ((int)(mag(v[t][1]) >> 52) >= e - 10 + 1023);
+            c = K - __reduce_add_sync(0xffffffffu, c);
+            if (lane == 0 && c > *(volatile int*)o.worst) atomicMax(o.worst, c);
+        }
         const unsigned off = swz((int)(r & 63), 2 * (lane & 15));
 #pragma unroll
         for (int t = 0; t < V; ++t) {
@@ -381,6 +402,13 @@ __global__ void __launch_bounds__(256) split_rows_long_kernel(Prod p, Side o, in
             if (k < Kc) v0 = A[r * ld + k];
             if (k + 1 < Kc) v1 = A[r * ld + k + 1];
         }
+        if (o.large) {  // 16 lanes a row, whole warps (total is a multiple of 32)
+            const int lim = e - 10 + 1023;
+            const unsigned b0 = __ballot_sync(0xffffffffu, (int)(mag(v0) >> 52) >= lim);
+            const unsigned b1 = __ballot_sync(0xffffffffu, (int)(mag(v1) >> 52) >= lim);
+            const unsigned half = threadIdx.x & 16 ? 0xffff0000u : 0xffffu;
+            if (kw == 0 && r < rows) atomicAdd(o.large + i0 + r, __popc(b0 & half) + __popc(b1 & half));
+        }
         unsigned w[S8];
         digits8x2(v0, v1, e, e, w);
         unsigned char* d = tile_at(o.img, r >> 6, nst, st, 0) + swz((int)(r & 63), 2 * kw);
@@ -426,7 +454,9 @@ __global__ void __launch_bounds__(256) strided_max_kernel(Prod p, Side o) {
         }
     }
 }
+template <bool GUARD>
 __global__ void __launch_bounds__(256, 4) split_strided_kernel(Prod p, Side o, int* flag) {
+    __shared__ int s_large[GUARD ? 32 : 1];
     if (!resolve(p)) return;
     long i0, rows, rpad, ld;
     side_sizes(p, o, i0, rows, rpad, ld);
@@ -439,6 +469,11 @@ __global__ void __launch_bounds__(256, 4) split_strided_kernel(Prod p, Side o, i
         if (j < rows) {
             e = split_exp(o.mx[i0 + j], flag);
             if (blockIdx.y == 0 && threadIdx.x < 32) o.e[i0 + j] = e;
+        }
+        if (GUARD) {
+            __syncthreads();
+            if (threadIdx.x < 32) s_large[threadIdx.x] = 0;
+            __syncthreads();
         }
         const long groups = (long)nst * 4;
         for (long g = (long)blockIdx.y * 8 + (threadIdx.x >> 5); g < groups; g += (long)gridDim.y * 8) {
@@ -453,6 +488,12 @@ __global__ void __launch_bounds__(256, 4) split_strided_kernel(Prod p, Side o, i
                 sg[r >> 1] = r & 1 ? sg[r >> 1] | sign : sign;
                 F[r] = biased56(__longlong_as_double((long long)F[r]), e);
             }
+            if (GUARD) {
+                int c = 0;
+#pragma unroll
+                for (int r = 0; r < 8; ++r) c += F[r] >= F_LARGE;
+                atomicAdd(&s_large[threadIdx.x & 31], c);
+            }
             unsigned char* d = tile_at(o.img, j >> 6, nst, (int)(g >> 2), 0) + swz((int)(j & 63), (int)(g & 3) * 8);
 #pragma unroll
             for (int s = 0; s < S8; ++s)
@@ -460,7 +501,21 @@ __global__ void __launch_bounds__(256, 4) split_strided_kernel(Prod p, Side o, i
                     make_uint4(digit_pair(F[0], F[1], s) ^ sg[0], digit_pair(F[2], F[3], s) ^ sg[1],
                                digit_pair(F[4], F[5], s) ^ sg[2], digit_pair(F[6], F[7], s) ^ sg[3]);
         }
+        if (GUARD) {
+            __syncthreads();
+            if (threadIdx.x < 32 && j < rows && s_large[threadIdx.x]) atomicAdd(o.large + i0 + j, s_large[threadIdx.x]);
+        }
     }
+}
+
+// *worst: the most indices of a nonzero row that are not large
+__global__ void __launch_bounds__(256) spread_kernel(long rows, int K, const int* __restrict__ large,
+                                                     const u64* __restrict__ mx, int* worst) {
+    int w = 0;
+    for (long r = blockIdx.x * 256L + threadIdx.x; r < rows; r += gridDim.x * 256L)
+        if (mx[r] != 0) w = max(w, K - large[r]);
+    w = __reduce_max_sync(0xffffffffu, w);
+    if ((threadIdx.x & 31) == 0 && w > *(volatile int*)worst) atomicMax(worst, w);
 }
 
 // ------------------------------------------------------------------ product
@@ -821,7 +876,7 @@ Plan make_plan(long M, long N, long K, bool gram) {
     const long nst = stages(p.Kc);
     p.Mc = gram ? M : std::min(M, std::max((long)T_M, IMG_LIMIT / (2L * S8 * nst * T_K) / T_M * T_M));
     p.planes = gram || p.Kc < K || split_limit(M, N, (int)nst) > 1;
-    p.head = (size_t)up(256 + 8 * (M + N) + 4 * (M + N) + 64, 1024);
+    p.head = (size_t)up(256 + 8 * (M + N) + 4 * (M + N) + 4 * (M + N) + 64, 1024);
     p.imgB = (size_t)(Np * nst * T_K * 2 * S8);
     p.imgA = gram ? 0 : (size_t)(up(p.Mc, T_M) * nst * T_K * 2 * S8);
     p.part = p.planes ? 16 * (size_t)std::max(M * N, std::min(M * N * MAX_SPLITS, PLANE_ELEMS)) : 0;
@@ -832,7 +887,7 @@ Plan make_plan(long M, long N, long K, bool gram) {
 // descriptor's).
 tt_status run(cudaStream_t s, bool ta, bool tb, long M, long N, long K, double alpha, const double* A, long lda,
               const double* B, long ldb, double* C, long ldc, DevBuf& scratch, int* status_dev, bool gram,
-              const int* desc) {
+              const int* desc, const int** gate) {
     const Plan q = make_plan(M, N, K, gram);
     // slack to bring the base to a 1024-byte boundary (a pool may give 256)
     TT_TRY(scratch.ensure((q.bytes() + 1024 + 7) / 8, s));
@@ -840,9 +895,11 @@ tt_status run(cudaStream_t s, bool ta, bool tb, long M, long N, long K, double a
     int* flag = reinterpret_cast<int*>(base);
     u64* mx = reinterpret_cast<u64*>(base + 256);
     int* ex = reinterpret_cast<int*>(mx + M + N);
-    Side a{A, 0, ta ? 1 : 0, mx, ex, base + q.head + q.imgB};
-    Side b{B, 1, tb ? 0 : 1, mx + M, ex + M, base + q.head};
-    if (gram) a = Side{A, 0, 1, mx, ex, base + q.head};
+    int* large = gate ? ex + M + N : nullptr;
+    int* worst = gate ? flag + 1 : nullptr;
+    Side a{A, 0, ta ? 1 : 0, mx, ex, base + q.head + q.imgB, large, worst};
+    Side b{B, 1, tb ? 0 : 1, mx + M, ex + M, base + q.head, gate ? large + M : nullptr, gate ? worst + 1 : nullptr};
+    if (gram) a.img = base + q.head;
     longlong2* planes = q.planes ? reinterpret_cast<longlong2*>(base + q.head + q.imgA + q.imgB) : nullptr;
     const int* eB = gram ? ex : b.e;
     Prod p{M, N, K, lda, ldb, ldc, desc, 0, q.Kc, 0, q.Mc, gram ? 1 : 0, q.Mc};
@@ -850,8 +907,9 @@ tt_status run(cudaStream_t s, bool ta, bool tb, long M, long N, long K, double a
     TT_CUDA_TRY(cudaGetDevice(&dev));
     TT_CUDA_TRY(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
     TT_TRY(ensure_max_dynamic_smem((const void*)tc8_kernel));
-    // the flag and, where atomics find them, the maxima start at zero
+    // the flag and, where atomics find them, the maxima and counts start at zero
     TT_CUDA_TRY(cudaMemsetAsync(flag, 0, 256 + (a.strided || b.strided ? 8 * (size_t)(M + N) : 0), s));
+    if (gate) TT_CUDA_TRY(cudaMemsetAsync(large, 0, 4 * (size_t)(M + N), s));
     const bool fusable = K <= FUSED_K;  // a captured step launches both forms when K may be longer
     auto maxima = [&](const Side& o) {
         const long rows = o.isB ? N : M;
@@ -867,9 +925,12 @@ tt_status run(cudaStream_t s, bool ta, bool tb, long M, long N, long K, double a
         const long rows = o.isB ? N : std::min(q.Mc, M - p.i0), rpad = up(rows, T_M);
         const int nst = stages(q.Kc);
         if (o.strided) {
+            const dim3 grid(blocks_for((rpad + 31) / 32, 4096), blocks_for(((long)nst * 2 + 7) / 8, 2048));
             note_launch();
-            split_strided_kernel<<<dim3(blocks_for((rpad + 31) / 32, 4096), blocks_for(((long)nst * 2 + 7) / 8, 2048)),
-                                   256, 0, s>>>(p, o, flag);
+            if (gate)
+                split_strided_kernel<true><<<grid, 256, 0, s>>>(p, o, flag);
+            else
+                split_strided_kernel<false><<<grid, 256, 0, s>>>(p, o, flag);
             return;
         }
         if (!fusable) {
@@ -925,6 +986,19 @@ tt_status run(cudaStream_t s, bool ta, bool tb, long M, long N, long K, double a
         note_launch();
         tc8_reduce_kernel<<<blocks_for((M * N + 255) / 256, 152L * 16), 256, 0, s>>>(p, planes, a.e, eB, spc, alpha, C);
     }
+    if (gate) {  // the caller recomputes what is lost
+        auto spread = [&](const Side& o) {
+            const long rows = o.isB ? N : M;
+            if (!o.strided && fusable) return;  // found by the split
+            note_launch();
+            spread_kernel<<<blocks_for((rows + 255) / 256, 152), 256, 0, s>>>(rows, (int)K, o.large, o.mx, o.worst);
+        };
+        spread(a);
+        if (!gram) spread(b);
+        TT_CUDA_TRY(cudaGetLastError());
+        *gate = flag;
+        return TT_OK;
+    }
     note_launch();
     fallback_kernel<<<152 * 4, FB * FB, 0, s>>>(flag, p, ta ? 1 : 0, tb ? 1 : 0, alpha, A, B, C);
     TT_CUDA_TRY(cudaGetLastError());
@@ -938,18 +1012,19 @@ size_t tc8_scratch_doubles(long M, long N, long K, bool gram) {
 }
 
 tt_status tc8_gemm(cudaStream_t s, bool ta, bool tb, long M, long N, long K, double alpha, const double* A, long lda,
-                   const double* B, long ldb, double* C, long ldc, DevBuf& scratch, int* status_dev) {
-    return run(s, ta, tb, M, N, K, alpha, A, lda, B, ldb, C, ldc, scratch, status_dev, false, nullptr);
+                   const double* B, long ldb, double* C, long ldc, DevBuf& scratch, int* status_dev,
+                   const int** gate) {
+    return run(s, ta, tb, M, N, K, alpha, A, lda, B, ldb, C, ldc, scratch, status_dev, false, nullptr, gate);
 }
 
 tt_status tc8_gram(cudaStream_t s, long m, long n, const double* A, long lda, double* G, long ldg, DevBuf& scratch,
-                   int* status_dev) {
-    return run(s, true, false, n, n, m, 1.0, A, lda, A, lda, G, ldg, scratch, status_dev, true, nullptr);
+                   int* status_dev, const int** gate) {
+    return run(s, true, false, n, n, m, 1.0, A, lda, A, lda, G, ldg, scratch, status_dev, true, nullptr, gate);
 }
 
 tt_status tc8_dyn(cudaStream_t s, bool ta, bool tb, const int* desc, long Mcap, long Ncap, long Kcap, double alpha,
                   const double* A, const double* B, double* C, DevBuf& scratch, int* status_dev, bool gram) {
-    return run(s, ta, tb, Mcap, Ncap, Kcap, alpha, A, 0, B, 0, C, 0, scratch, status_dev, gram, desc);
+    return run(s, ta, tb, Mcap, Ncap, Kcap, alpha, A, 0, B, 0, C, 0, scratch, status_dev, gram, desc, nullptr);
 }
 
 }  // namespace ttsn

@@ -181,7 +181,8 @@ __host__ __device__ inline int ordered_split(int M, int N, int K, int tri, int* 
 // C = alpha op(A) op(B) (+ beta C), or with tri the symmetric product of which
 // only the tiles on and above the diagonal are formed (both halves stored).
 // desc (a captured step): M, N, K, lda, ldb, ldc in device memory; tc: sizes
-// that digits.cu takes are left to it.  An item is (tile, split); ks > 1:
+// that digits.cu takes are left to it.  gate: behind a digit product, which it
+// replaces where that lost accuracy (tc8_lost).  An item is (tile, split); ks > 1:
 // partials to P (256 doubles an item), arrivals counted in cnt (zero between
 // products: the last arrival resets its tile's).  ORDERED: a warp per 8 x 8 block; else the warps share the indices.  An 8 x 8
 // product outside M x N or below the diagonal is skipped.
@@ -189,7 +190,8 @@ template <bool TA, bool TB, bool ORDERED>
 __global__ void __launch_bounds__(THREADS)
 prod_kernel(int M, int N, int K, double alpha, const double* __restrict__ A, long lda, const double* __restrict__ B,
             long ldb, double beta, double* __restrict__ C, long ldc, int ks, int chunk, double* __restrict__ P, int* cnt,
-            int tri, const int* __restrict__ desc, int tc) {
+            int tri, const int* __restrict__ desc, int tc, const int* __restrict__ gate) {
+    if (gate && !tc8_lost(gate, K, tri != 0)) return;
     if (desc) {
         M = desc[0];
         N = desc[1];
@@ -447,16 +449,17 @@ struct ProdArgs {
     int *cnt, tri;
     const int* desc;
     int tc;
+    const int* gate = nullptr;
 };
 
 template <bool TA, bool TB>
 void launch_one(cudaStream_t s, bool ordered, unsigned grid, const ProdArgs& a) {
     if (ordered)
         prod_kernel<TA, TB, true><<<grid, THREADS, 0, s>>>(a.M, a.N, a.K, a.alpha, a.A, a.lda, a.B, a.ldb, a.beta, a.C,
-                                                          a.ldc, a.ks, a.chunk, a.P, a.cnt, a.tri, a.desc, a.tc);
+                                                          a.ldc, a.ks, a.chunk, a.P, a.cnt, a.tri, a.desc, a.tc, a.gate);
     else
         prod_kernel<TA, TB, false><<<grid, THREADS, 0, s>>>(a.M, a.N, a.K, a.alpha, a.A, a.lda, a.B, a.ldb, a.beta, a.C,
-                                                           a.ldc, a.ks, a.chunk, a.P, a.cnt, a.tri, a.desc, a.tc);
+                                                           a.ldc, a.ks, a.chunk, a.P, a.cnt, a.tri, a.desc, a.tc, a.gate);
 }
 
 tt_status launch_prod(cudaStream_t s, bool ta, bool tb, bool ordered, long items, const ProdArgs& a) {
@@ -550,21 +553,26 @@ size_t gram_scratch_doubles(int m, int n) {
 // ------------------------------------------------------------ library calls
 
 size_t gemm_call_doubles(int M, int N, int K) {
-    if (tc8_wanted(M, N, K)) return tc8_scratch_doubles(M, N, K, false);
-    return split_scratch(prod_tiles(M, N, 0), prod_split(M, N, K, 0));
+    return (tc8_wanted(M, N, K) ? tc8_scratch_doubles(M, N, K, false) : 0) +
+           split_scratch(prod_tiles(M, N, 0), prod_split(M, N, K, 0));
 }
 
 tt_status gemm_call(cudaStream_t s, bool ta, bool tb, int M, int N, int K, double alpha, const double* A, long lda,
                     const double* B, long ldb, double* C, long ldc, DevBuf& scratch) {
-    if (tc8_wanted(M, N, K)) return tc8_gemm(s, ta, tb, M, N, K, alpha, A, lda, B, ldb, C, ldc, scratch, nullptr);
     const int ks = prod_split(M, N, K, 0);
+    const int* gate = nullptr;
+    double* P = scratch.p;
+    if (tc8_wanted(M, N, K)) {
+        TT_TRY(tc8_gemm(s, ta, tb, M, N, K, alpha, A, lda, B, ldb, C, ldc, scratch, nullptr, &gate));
+        P += tc8_scratch_doubles(M, N, K, false);
+    }
     return split_prod(s, ta, tb, false, ProdArgs{M, N, K, alpha, A, lda, B, ldb, 0.0, C, ldc, ks, prod_chunk(K, ks),
-                                                 scratch.p, nullptr, 0, nullptr, 0});
+                                                 P, nullptr, 0, nullptr, 0, gate});
 }
 
 size_t gram_call_doubles(int m, int n) {
-    if (tc8_wanted(n, n, m)) return tc8_scratch_doubles(n, n, m, true);
-    return split_scratch(prod_tiles(n, n, 1), prod_split(n, n, std::max(m, 1), 1));
+    return (tc8_wanted(n, n, m) ? tc8_scratch_doubles(n, n, m, true) : 0) +
+           split_scratch(prod_tiles(n, n, 1), prod_split(n, n, std::max(m, 1), 1));
 }
 
 tt_status gram_fixed_scratch(cudaStream_t s, int m, int n, const double* A, long lda, double* G,
@@ -588,7 +596,16 @@ tt_status gram_fixed_scratch(cudaStream_t s, int m, int n, const double* A, long
 
 tt_status gram_call(cudaStream_t s, int m, int n, const double* A, long lda, double* G, long ldg, DevBuf& scratch) {
     if (m > 0 && tc8_wanted(n, n, m)) {
-        const tt_status st = tc8_gram(s, m, n, A, lda, G, ldg, scratch, nullptr);
+        const size_t own = tc8_scratch_doubles(n, n, m, true);
+        tt_status st = scratch.ensure(gram_call_doubles(m, n), s);
+        const int* gate = nullptr;
+        if (st >= 0) st = tc8_gram(s, m, n, A, lda, G, ldg, scratch, nullptr, &gate);
+        if (st >= 0) {
+            const int ks = prod_split(n, n, m, 1);
+            return split_prod(s, true, false, false, ProdArgs{n, n, m, 1.0, A, lda, A, lda, 0.0, G, ldg, ks,
+                                                              prod_chunk(m, ks), scratch.p + own, nullptr, 1, nullptr, 0,
+                                                              gate});
+        }
         if (st != TT_ERR_OOM) return st;
     }
     TT_TRY(scratch.ensure(split_scratch(prod_tiles(n, n, 1), prod_split(n, n, std::max(m, 1), 1)), s));

@@ -176,10 +176,19 @@ __host__ __device__ inline bool tc8_wanted(long M, long N, long K) {
            (N <= 16384 || K <= 16384) && M * N >= (16000000L + K - 1) / K;
 }
 size_t tc8_scratch_doubles(long M, long N, long K, bool gram);
+// gate (null: a rounding's product, complete on return): set to three device
+// ints for tc8_lost, and the caller recomputes the product where that holds.
 tt_status tc8_gemm(cudaStream_t s, bool ta, bool tb, long M, long N, long K, double alpha, const double* A, long lda,
-                   const double* B, long ldb, double* C, long ldc, DevBuf& scratch, int* status_dev);
+                   const double* B, long ldb, double* C, long ldc, DevBuf& scratch, int* status_dev,
+                   const int** gate = nullptr);
 tt_status tc8_gram(cudaStream_t s, long m, long n, const double* A, long lda, double* G, long ldg, DevBuf& scratch,
-                   int* status_dev);
+                   int* status_dev, const int** gate = nullptr);
+// Some row could not be split (gate[0]), or two rows may have fewer than K / 16
+// indices where both are large (gate[1], gate[2]: the most indices that a row of
+// op(A), a column of op(B) is small at; the Gram has one operand).
+__device__ inline bool tc8_lost(const int* gate, int K, bool gram) {
+    return gate[0] != 0 || (long)gate[1] + (gram ? gate[1] : gate[2]) > K - K / 16;
+}
 // The captured form: sizes from desc (as dgemm_dyn's), at most the capacities;
 // does nothing for sizes that tc8_wanted leaves to the FP64 pipe.
 tt_status tc8_dyn(cudaStream_t s, bool ta, bool tb, const int* desc, long Mcap, long Ncap, long Kcap, double alpha,

@@ -130,3 +130,31 @@ def test_captured_steps_above_the_digit_sizes_equal_host_steps(ttsn):
         assert a.step()["ranks"] == b.step()["ranks"]
     assert 96 * 90 * (5 * a.ranks()[1] + 1) ** 2 > 16e6
     assert torch.equal(a.full(), b.full())
+
+
+@pytest.mark.parametrize("M,N,K", [(300, 260, 260), (2100, 1100, 1100), (260, 300, 2000)])
+@pytest.mark.parametrize("ta,tb", [(False, False), (True, False), (False, True), (True, True)])
+def test_small_entries_that_meet_large_ones_keep_their_accuracy(ttsn, M, N, K, ta, tb):
+    """A @ (a selection of columns) gives A's entries, whatever their range in a
+    row: the sums hold one term, so nothing is rounded."""
+    rng = np.random.default_rng(K)
+    A = rng.standard_normal((M, K)) * 10.0 ** (-40 * rng.random((M, K)))
+    pick = rng.integers(0, K, N)
+    B = np.zeros((K, N))
+    B[pick, np.arange(N)] = 1.0
+    got = _call(ttsn, A.T.copy() if ta else A, B.T.copy() if tb else B, ta, tb)
+    assert np.array_equal(got, A[:, pick])
+
+
+@pytest.mark.parametrize("m,n", [(900, 140), (30001, 65)])
+def test_gram_of_columns_that_are_large_at_different_rows(ttsn, m, n):
+    """Positive entries: the FP64 pipe's sums are off by m eps relative at most,
+    and so is the reference's."""
+    import torch
+
+    rng = np.random.default_rng(m)
+    A = 1e-18 * (1.0 + rng.random((m, n)))
+    A[np.arange(n) * (m // n), np.arange(n)] = 1.0
+    G = ttsn.gram(torch.as_tensor(A, device="cuda")).cpu().numpy()
+    ref = A.T @ A
+    assert np.all(np.abs(G - ref) <= 2 * m * np.finfo(float).eps * ref) and np.array_equal(G, G.T)
