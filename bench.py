@@ -768,11 +768,10 @@ def run_batch(args, torch, ttsn):
             "ranks_last_min_max": [min(min(r) for r in ranks), max(max(r) for r in ranks)]}
 
 
-# ncu DRAM read + write bytes of one left-Gram launch at the bench's rank cap
-# (2,097,152 x 897), scaled by the rows from an ncu capture (dram__bytes_read
-# and _write) of the same kernel and split (64 row splits) on a 500,000 x 897
-# operand: 23.26 GB.
-GRAM_LEFT_CAP_TRAFFIC = (23020594176 + 235760896) * 2097152 / 500000
+# ncu DRAM read + write bytes of one left Gram at the bench's rank cap (2,097,152
+# x 897), scaled by the rows from an ncu capture (dram__bytes_read and _write) of
+# the same kernels on a 500,000 x 897 operand: 28.78 GB.
+GRAM_LEFT_CAP_TRAFFIC = (19971342592 + 8811881216) * 2097152 / 500000
 
 
 def roofline_of(prof, fp64_peak, peaks):
@@ -788,18 +787,29 @@ def roofline_of(prof, fp64_peak, peaks):
         traffic = GRAM_LEFT_CAP_TRAFFIC if name == "gram_left" else None
         return name, {"bound": "tensor", "achieved": achieved, "peak": peak, "unit": "TFLOP/s",
                       "frac": achieved / peak if peak else None, "traffic": traffic,
-                      "traffic_note": "ncu DRAM read+write bytes of one capped 2,097,152 x 897 launch (scaled "
+                      "traffic_note": "ncu DRAM read+write bytes of one capped 2,097,152 x 897 Gram (scaled "
                                       "by the rows from a 500,000 x 897 capture)" if traffic else None,
                       "kernel": name, "dtype": "f64", "avg_phase_ms": avg_ms,
                       "launches": ph["launches"], "calls": ph["calls"],
                       "peak_source": "measured FP64 tensor pipe (mma.m8n8k4.f64 chains on all SMs, "
-                                     "tt_bench_fp64_mma); MEASURED_PEAKS.json has no FP64 figure"}
+                                     "tt_bench_fp64_mma); MEASURED_PEAKS.json has no FP64 figure; large "
+                                     "products run as exact digit products on the BF16 tensor cores, so "
+                                     "frac may exceed 1",
+                      "digits": digit_roofline(ph, peaks)}
     achieved = ph["bytes"] / (ph["ms"] * 1e-3) / 1e9
     peak = peaks.get("hbm_gbs", 6800.0)
     return name, {"bound": "hbm", "achieved": achieved, "peak": peak, "unit": "GB/s",
                   "frac": achieved / peak, "traffic": None, "kernel": name, "avg_phase_ms": avg_ms,
                   "launches": ph["launches"], "calls": ph["calls"],
                   "peak_source": "MEASURED_PEAKS.json hbm_gbs"}
+
+
+def digit_roofline(ph, peaks):
+    """The phase as digit products (36 BF16 products per FP64 term of the
+    algorithmic count, csrc/digits.cu) against the sustained BF16 throughput."""
+    peak = peaks.get("bf16_tflops_sustained") or peaks.get("bf16_tflops") or 1700.0
+    ex = 36.0 * ph["flops"] / (ph["ms"] * 1e-3) / 1e12
+    return {"achieved": ex, "peak": peak, "unit": "TFLOP/s", "frac": ex / peak}
 
 
 def cpu_baseline(p, budget_s, gpu_step_ms):
