@@ -15,7 +15,7 @@ CSRC = os.path.join(PKG, "csrc")
 BUILD = os.path.join(PKG, "_build")
 LIB = os.path.join(PKG, "libttsn.so")
 HEADERS = [os.path.join(ROOT, "include", "ttsn.h"), os.path.join(CSRC, "internal.h"),
-           os.path.join(CSRC, "intfp.h")]
+           os.path.join(CSRC, "intfp.h"), os.path.join(CSRC, "digits_plan.h")]
 
 NVCC = os.environ.get("NVCC", "nvcc")
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]

@@ -1553,7 +1553,7 @@ tt_status graph_reserve(tt_ctx* h) {
         for (const auto& q : c) {
             part = std::max(part, dyn_partials_need(q[0], q[1], q[2], q[3]));
             if (tc8_wanted(q[1], q[2], q[3]))
-                tcs = std::max(tcs, tc8_scratch_doubles(q[1], q[2], q[3], q[0] == 2));
+                tcs = std::max(tcs, tc8_scratch_doubles(q[1], q[2], q[3], q[0] == 2, true));
         }
     }
     struct Need {

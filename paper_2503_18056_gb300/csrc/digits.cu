@@ -53,11 +53,9 @@ namespace ttsn {
 
 namespace {
 
-constexpr int S8 = 8;
-constexpr int T_M = 128, T_N = 64, T_K = 32;  // output tile; contraction indices of a stage
-constexpr int T_BLK = 16;                     // stages of an exact block (512 indices)
+using namespace digits;
+
 constexpr int T_STAGES = 2;
-constexpr int RB = 64;                         // rows of an image block
 constexpr int DIG_BYTES = RB * T_K * 2;        // one digit of one block and stage: 4096
 constexpr int BLK_BYTES = S8 * DIG_BYTES;      // 32768
 constexpr int A_BYTES = 2 * BLK_BYTES, B_BYTES = BLK_BYTES, STAGE_BYTES = A_BYTES + B_BYTES;
@@ -71,12 +69,6 @@ constexpr int DCOLS = T_N / (DRAIN_WARPS / 4);  // columns of a drain thread: 16
 constexpr unsigned TMEM_COLS = 512;
 constexpr long long SPIN = 1LL << 26;
 constexpr size_t SMEM8 = (size_t)T_STAGES * STAGE_BYTES + 1024 /* barriers */ + 1024 /* alignment */;
-// Digit images of one pass over an operand; a longer operand goes in chunks.  A
-// chunk costs its launches and a last wave: with images of 2^26, 2^27, 2^28, 2^29
-// and 2^30 bytes the Gram of 500,000 x 449 took 10.3, 9.1, 8.5, 8.4 and 8.6 ms and
-// 200,000 x 577 times 577 x 96 3.0, 2.6, 2.1, 2.1 and 2.5 (before the present
-// issue loop and split), although only the smaller ones stay in the 129 MB L2.
-constexpr long IMG_LIMIT = 1L << 28;
 
 __device__ __forceinline__ unsigned smem_addr(const void* p) { return (unsigned)__cvta_generic_to_shared(p); }
 __device__ __forceinline__ void bar_init(unsigned a, unsigned count) {
@@ -173,41 +165,7 @@ __device__ __forceinline__ bool resolve(Prod& p) {
     p.Mc = p.Mc < p.M - p.i0 ? p.Mc : p.M - p.i0;
     return p.Mc > 0 && p.k0 < p.K;
 }
-__host__ __device__ inline long up(long x, long m) { return (x + m - 1) / m * m; }
-__host__ __device__ inline int stages(long Kc) { return (int)((Kc + T_K - 1) / T_K); }
-__host__ __device__ inline long tiles_of(long M, long N, int gram) {
-    const long nb = (N + T_N - 1) / T_N;
-    if (!gram) return (M + T_M - 1) / T_M * nb;
-    const long h = (nb + 1) / 2;  // rows of 128: nb, nb - 2, ... tiles
-    return h * nb - h * (h - 1);
-}
-
-// Splits of a chunk's contraction: stages per split.  The time of a launch is
-// about its waves of one CTA per SM times the stages of a split and one more
-// for an item's end; a plane costs its write and its read in the reduction.
-// A split has at least four stages, and the planes at most PLANE_ELEMS entries.
-constexpr long PLANE_ELEMS = 1L << 23;
-constexpr int MAX_SPLITS = 64;
-__host__ __device__ inline int split_limit(long M, long N, int nst) {
-    long k = PLANE_ELEMS / (M * N);
-    if (k > nst / 4) k = nst / 4;
-    if (k > MAX_SPLITS) k = MAX_SPLITS;
-    return k < 1 ? 1 : (int)k;
-}
-__host__ __device__ inline unsigned split_cost(int k, long ntiles, int nst) {
-    const int spc = (nst + k - 1) / k, kk = (nst + spc - 1) / spc;
-    const long waves = (ntiles * kk + 151) / 152;
-    const long c = waves * (spc + 1) * 64 + kk;
-    return c > 0x03ffffffL ? 0x03ffffffu : (unsigned)c;
-}
-int split_stages(long M, long N, long ntiles, int nst) {
-    const int lim = split_limit(M, N, nst);
-    int best = 1;
-    for (int k = 2; k <= lim; ++k)
-        if (split_cost(k, ntiles, nst) < split_cost(best, ntiles, nst)) best = k;
-    return (nst + best - 1) / best;
-}
-// the same choice made by one warp
+// split_stages as one warp makes it
 __device__ __forceinline__ int split_stages_warp(long M, long N, long ntiles, int nst) {
     const int lim = split_limit(M, N, nst), lane = threadIdx.x & 31;
     unsigned key = 0xffffffffu;
@@ -597,7 +555,8 @@ tc8_kernel(Prod p, const unsigned char* __restrict__ At, const int* __restrict__
     const long ntiles = tiles_of(M, N, p.gram);
     // a captured step decides the split here (from the first chunk, as the
     // reduction does)
-    if (p.desc) spc = split_stages_warp(p.M, N, tiles_of(p.Mc0, N, p.gram), stages(p.Kc < p.K ? p.Kc : p.K));
+    if (p.desc)
+        spc = planes ? split_stages_warp(p.M, N, tiles_of(p.Mc0, N, p.gram), stages(p.Kc < p.K ? p.Kc : p.K)) : nst;
     const bool accumulate = p.k0 > 0;
     const bool whole = planes == nullptr || (p.desc && !p.gram && p.K <= p.Kc && spc >= nst);
     extern __shared__ unsigned char raw[];
@@ -808,7 +767,7 @@ tc8_kernel(Prod p, const unsigned char* __restrict__ At, const int* __restrict__
 __global__ void __launch_bounds__(256)
 tc8_reduce_kernel(Prod p, const longlong2* __restrict__ planes, const int* __restrict__ eA,
                   const int* __restrict__ eB, int spc, double alpha, double* __restrict__ C) {
-    if (!resolve(p)) return;
+    if (!resolve(p) || !planes) return;  // without planes tc8_kernel has written C
     const int nst = stages(p.Kc < p.K ? p.Kc : p.K);
     if (p.desc) {
         spc = split_stages_warp(p.M, p.N, tiles_of(p.Mc0, p.N, p.gram), nst);
@@ -859,37 +818,12 @@ fallback_kernel(const int* __restrict__ flag, Prod p, int ta, int tb, double alp
 
 unsigned blocks_for(long work, long cap) { return (unsigned)std::max<long>(1, std::min<long>(work, cap)); }
 
-// Chunks and scratch of a product of at most these sizes.
-struct Plan {
-    long Kc, Mc;
-    bool planes;                         // several splits or chunks of K possible
-    size_t head, imgA, imgB, part;       // bytes: flag, maxima and exponents; images; planes
-    size_t bytes() const { return head + imgA + imgB + part; }
-};
-Plan make_plan(long M, long N, long K, bool gram) {
-    Plan p;
-    const long Np = up(N, gram ? T_M : RB);
-    // images of about IMG_LIMIT bytes each: a long contraction is cut along K
-    // (for an operand of up to 1024 rows), a tall A along its rows
-    const long wide = std::max(up(std::min(M, 1024L), T_M), Np);
-    const long kmax = std::max(16384L, IMG_LIMIT / (2 * S8 * wide) / (T_K * T_BLK) * (T_K * T_BLK));
-    p.Kc = K <= kmax ? K : up((K + (K + kmax - 1) / kmax - 1) / ((K + kmax - 1) / kmax), T_K * T_BLK);
-    const long nst = stages(p.Kc);
-    p.Mc = gram ? M : std::min(M, std::max((long)T_M, IMG_LIMIT / (2L * S8 * nst * T_K) / T_M * T_M));
-    p.planes = gram || p.Kc < K || split_limit(M, N, (int)nst) > 1;
-    p.head = (size_t)up(256 + 8 * (M + N) + 4 * (M + N) + 4 * (M + N) + 64, 1024);
-    p.imgB = (size_t)(Np * nst * T_K * 2 * S8);
-    p.imgA = gram ? 0 : (size_t)(up(p.Mc, T_M) * nst * T_K * 2 * S8);
-    p.part = p.planes ? 16 * (size_t)std::max(M * N, std::min(M * N * MAX_SPLITS, PLANE_ELEMS)) : 0;
-    return p;
-}
-
 // desc: a captured product of sizes up to M, N, K (then lda, ldb, ldc are the
 // descriptor's).
 tt_status run(cudaStream_t s, bool ta, bool tb, long M, long N, long K, double alpha, const double* A, long lda,
               const double* B, long ldb, double* C, long ldc, DevBuf& scratch, int* status_dev, bool gram,
               const int* desc, const int** gate) {
-    const Plan q = make_plan(M, N, K, gram);
+    const Plan q = make_plan(M, N, K, gram, desc != nullptr);
     // slack to bring the base to a 1024-byte boundary (a pool may give 256)
     TT_TRY(scratch.ensure((q.bytes() + 1024 + 7) / 8, s));
     unsigned char* base = reinterpret_cast<unsigned char*>(((uintptr_t)scratch.p + 1023) & ~(uintptr_t)1023);
@@ -901,7 +835,7 @@ tt_status run(cudaStream_t s, bool ta, bool tb, long M, long N, long K, double a
     Side a{A, 0, ta ? 1 : 0, mx, ex, base + q.head + q.imgB, large, worst};
     Side b{B, 1, tb ? 0 : 1, mx + M, ex + M, base + q.head, gate ? large + M : nullptr, gate ? worst + 1 : nullptr};
     if (gram) a.img = base + q.head;
-    longlong2* planes = q.planes ? reinterpret_cast<longlong2*>(base + q.head + q.imgA + q.imgB) : nullptr;
+    longlong2* planes = q.part ? reinterpret_cast<longlong2*>(base + q.head + q.imgA + q.imgB) : nullptr;
     const int* eB = gram ? ex : b.e;
     Prod p{M, N, K, lda, ldb, ldc, desc, 0, q.Kc, 0, q.Mc, gram ? 1 : 0, q.Mc};
     int dev = 0, sms = 152;
@@ -1008,8 +942,8 @@ tt_status run(cudaStream_t s, bool ta, bool tb, long M, long N, long K, double a
 
 }  // namespace
 
-size_t tc8_scratch_doubles(long M, long N, long K, bool gram) {
-    return (make_plan(M, N, K, gram).bytes() + 1024 + 7) / 8;
+size_t tc8_scratch_doubles(long M, long N, long K, bool gram, bool captured) {
+    return (make_plan(M, N, K, gram, captured).bytes() + 1024 + 7) / 8;
 }
 
 tt_status tc8_gemm(cudaStream_t s, bool ta, bool tb, long M, long N, long K, double alpha, const double* A, long lda,

@@ -8,6 +8,7 @@
 #include <string>
 
 #include "../../include/ttsn.h"
+#include "digits_plan.h"
 
 namespace ttsn {
 
@@ -167,15 +168,9 @@ tt_status slgemm_nt(cudaStream_t s, long M, int N, int K, const double* A, long 
 // C = alpha op(A) op(B) and G = A^T A (A m x n) from exact integer digit
 // products: every sum exact, one rounding an entry (the header of digits.cu).
 // tc8_wanted is the rule by which dgemm_sk, gram, their captured forms and the
-// library calls take it, from the sizes alone.  Below 16M terms (32 us of the FP64 pipe)
-// the five or six launches cost more than they save; a contraction under 64
-// would not be rounded less often than the FP64 sum it replaces; the 64-bit
-// sums hold 2^26 indices.
-__host__ __device__ inline bool tc8_wanted(long M, long N, long K) {
-    return K >= 64 && K <= (1L << 26) && M >= 32 && N >= 16 && N <= (1L << 20) && M * N <= (1L << 40) &&
-           (N <= 16384 || K <= 16384) && M * N >= (16000000L + K - 1) / K;
-}
-size_t tc8_scratch_doubles(long M, long N, long K, bool gram);
+// library calls take it, from the sizes alone.  captured: the scratch of a captured
+// product of sizes up to these.
+size_t tc8_scratch_doubles(long M, long N, long K, bool gram, bool captured = false);
 // gate (null: a rounding's product, complete on return): set to three device
 // ints for tc8_lost, and the caller recomputes the product where that holds.
 tt_status tc8_gemm(cudaStream_t s, bool ta, bool tb, long M, long N, long K, double alpha, const double* A, long lda,

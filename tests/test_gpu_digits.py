@@ -158,3 +158,39 @@ def test_gram_of_columns_that_are_large_at_different_rows(ttsn, m, n):
     G = ttsn.gram(torch.as_tensor(A, device="cuda")).cpu().numpy()
     ref = A.T @ A
     assert np.all(np.abs(G - ref) <= 2 * m * np.finfo(float).eps * ref) and np.array_equal(G, G.T)
+
+
+@pytest.mark.parametrize("r1,r2", [(46, 20), (52, 48), (64, 24)])
+def test_captured_steps_that_split_where_their_capacity_does_not(ttsn, r1, r2):
+    """256^2 cells, 32 x 64 ordinates, cap 128: the core update and Theta* G_B are
+    split at these ranks but not at the cap's sizes.  A short time step keeps the ranks."""
+    import torch
+
+    import workloads
+
+    p = workloads.problem("small_2d", n=(256, 256), n_theta=32, n_phi=64, eps=1e-4, bc=1)
+    p["max_rank"], p["dt"] = 128, 1e-9
+    g = torch.Generator(device="cuda").manual_seed(r1)
+
+    def rnd(*shape):
+        return torch.randn(*shape, generator=g, device="cuda", dtype=torch.float64)
+
+    # an isotropic field in equilibrium and modes without angular mean, every
+    # direction of both bonds well above eps
+    X, Th, Ph = 0.05 * rnd(1, 256 * 256, r1), rnd(r1, 32, r2), rnd(r2, 64, 1)
+    X[0, :, 0] = torch.as_tensor(p["T0"].reshape(-1), device="cuda") ** 4 / (4 * np.pi)
+    Ph -= Ph.mean(1, keepdim=True)
+    Ph[0] = 1.0
+    Th[0], Th[:, :, 0], Th[0, :, 0] = 0.0, 0.0, 1.0
+    a, b = ttsn.TTSN.from_problem(p), ttsn.TTSN.from_problem(p)
+    b.set_graph(True)
+    for h in (a, b):
+        h.set_cores([X, Th, Ph])
+        h.set_T(p["T0"])
+    for _ in range(2):
+        ia, ib = a.step(), b.step()
+        assert ia["ranks"] == ib["ranks"] and r1 <= ia["ranks"][1] <= r1 + 1
+    for x, y in zip(a.cores(), b.cores()):
+        assert torch.equal(torch.as_tensor(x), torch.as_tensor(y))
+    (Ea, Ta, ta), (Eb, Tb, tb) = a.energy(), b.energy()
+    assert torch.equal(Ea, Eb) and torch.equal(Ta, Tb) and ta == tb
