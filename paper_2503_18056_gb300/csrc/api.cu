@@ -1541,7 +1541,7 @@ tt_status graph_reserve(tt_ctx* h) {
     const long Gm = std::max(G1, G2);
     // partials of the captured split products: the largest need over the
     // (mode, M, N, K) capacities of graph_step_body's products
-    size_t part = 1, tcs = 1;
+    size_t part = 1, tcs = 0;
     {
         const int c[][4] = {{1, (int)G2, (int)G2, (int)np},       {1, (int)G1, (int)G1, (int)(nt * G2)},
                             {2, (int)G1, (int)G1, (int)nc},       {1, (int)G1, (int)G1, (int)G1},
@@ -1552,7 +1552,7 @@ tt_status graph_reserve(tt_ctx* h) {
                             {1, (int)(c1 * nt), (int)c2, (int)G2}};
         for (const auto& q : c) {
             part = std::max(part, dyn_partials_need(q[0], q[1], q[2], q[3]));
-            if (tc8_wanted(q[1], q[2], q[3]))
+            if (h->prod.digits && tc8_wanted(q[1], q[2], q[3]))
                 tcs = std::max(tcs, tc8_scratch_doubles(q[1], q[2], q[3], q[0] == 2, true));
         }
     }
@@ -1571,9 +1571,15 @@ tt_status graph_reserve(tt_ctx* h) {
         {&h->eig.lam_unsorted, Gm}, {&h->eig.abc, 3 * (Gm + 1)}, {&h->eig.cs, Gm + 1},
         {&h->eig.psd, 3 * Gm + 2},
         {&h->dyn_part, (long)part},
-        {&h->dyn_tc, (long)tcs},
     };
     for (auto& x : need) TT_TRY(x.b->ensure((size_t)std::max<long>(x.n, 1), s, /*keep=*/true));
+    if (tcs) {
+        const tt_status st = h->dyn_tc.ensure(tcs, s);
+        if (st == TT_ERR_OOM)
+            h->prod.digits = false;  // without room for the digits: host and captured steps on the FP64 pipe
+        else
+            TT_TRY(st);
+    }
     TT_TRY(eig_reserve(h->eig, s));
     TT_TRY(h->dyn_buf.ensure((size_t)(DYN_INTS + 1) / 2 + 16, s));
     h->dyn = reinterpret_cast<int*>(h->dyn_buf.p);
@@ -2411,10 +2417,11 @@ tt_status create_impl(const tt_problem_desc* desc, void* stream, const tt_alloca
             // digit images and planes of the capped step's products; a handle
             // without room for them runs on the FP64 pipe
             const long c[][4] = {{1, R1, R1, nc}, {0, nc, cap1, R1}, {0, R1 * D.n_theta, R2, R2},
-                                 {0, R1, R1, D.n_theta * R2}, {0, cap1, D.n_theta * R2, R1}};
+                                 {0, R1, R1, D.n_theta * R2}, {0, cap1, D.n_theta * R2, R1}, {0, R1, R1, R1},
+                                 {1, R2, R2, cap1 * D.n_theta}, {0, cap1 * D.n_theta, cap2, R2}};
             size_t need = 0;
             for (const auto& q : c)
-                if (tc8_wanted(q[1], q[2], q[3])) need = std::max(need, tc8_scratch_doubles(q[1], q[2], q[3], q[0] != 0));
+                if (tc8_wanted(q[1], q[2], q[3])) need = std::max(need, tc8_reserve_doubles(q[1], q[2], q[3], q[0] != 0));
             const tt_status ps = need ? h->partials.ensure(need, s) : TT_OK;
             if (ps < 0 && ps != TT_ERR_OOM) TT_CREATE_TRY(ps);
         }

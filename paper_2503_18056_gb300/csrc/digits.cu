@@ -946,6 +946,10 @@ size_t tc8_scratch_doubles(long M, long N, long K, bool gram, bool captured) {
     return (make_plan(M, N, K, gram, captured).bytes() + 1024 + 7) / 8;
 }
 
+size_t tc8_reserve_doubles(long M, long N, long K, bool gram) {
+    return (reserve_bytes(M, N, K, gram) + 1024 + 7) / 8;
+}
+
 tt_status tc8_gemm(cudaStream_t s, bool ta, bool tb, long M, long N, long K, double alpha, const double* A, long lda,
                    const double* B, long ldb, double* C, long ldc, DevBuf& scratch, int* status_dev,
                    const int** gate) {

@@ -109,5 +109,18 @@ inline Plan make_plan(long M, long N, long K, bool gram, bool captured) {
     return p;
 }
 
+// Bytes that hold the scratch of every product of sizes up to these: a smaller
+// operand goes in fewer or longer chunks and may split more often, so no size's
+// own plan bounds the others'.
+inline size_t reserve_bytes(long M, long N, long K, bool gram) {
+    const long Np = up(N, gram ? T_M : RB), Kp = up(K, T_K), row = 2 * S8;
+    const long imgB = least(Np * Kp, most(IMG_LIMIT / row, 16384 * Np)) * row;
+    const long imgA = gram ? 0 : least(up(M, T_M) * Kp, IMG_LIMIT / row) * row;
+    const long splits = least(stages(K) / 4, MAX_SPLITS);
+    long elems = gram || K > 16384 ? M * N : 0;
+    if (splits > 1) elems = most(elems, least(M * N * splits, PLANE_ELEMS));
+    return (size_t)(up(256 + 16 * (M + N) + 64, 1024) + imgA + imgB + 16 * elems);
+}
+
 }  // namespace digits
 }  // namespace ttsn

@@ -171,6 +171,8 @@ tt_status slgemm_nt(cudaStream_t s, long M, int N, int K, const double* A, long 
 // library calls take it, from the sizes alone.  captured: the scratch of a captured
 // product of sizes up to these.
 size_t tc8_scratch_doubles(long M, long N, long K, bool gram, bool captured = false);
+// and of any product of sizes up to these
+size_t tc8_reserve_doubles(long M, long N, long K, bool gram);
 // gate (null: a rounding's product, complete on return): set to three device
 // ints for tc8_lost, and the caller recomputes the product where that holds.
 tt_status tc8_gemm(cudaStream_t s, bool ta, bool tb, long M, long N, long K, double alpha, const double* A, long lda,

@@ -57,6 +57,7 @@ int main() {
                         check(q, true, gram, Mc, Nc, Kc, M, N, K);
                         const Plan own = make_plan(M, N, K, gram, false);
                         check(own, false, gram, M, N, K, M, N, K);
+                        if (own.bytes() > reserve_bytes(Mc, Nc, Kc, gram)) fail("reservation", Mc, Nc, Kc, M, N, K);
                     };
                     one(gramL, true, G1, G1, nc, R1, R1, nc);
                     for (long r : {1L, 7L, r1 / 2, r1, (r1 + c1) / 2, c1})
@@ -84,10 +85,16 @@ int main() {
             for (long f = 1; f <= 64; f *= 2)
                 for (long h = 1; h <= 64; h *= 2) {
                     const long n = most(1, s[1] / f), k = most(1, s[2] / h);
-                    for (long m : {M, most(1, M / f), most(1, M / 3)})
+                    for (long m : {M, most(1, M / f), most(1, M / 3)}) {
                         check(cap, true, gram, M, s[1], s[2], gram ? n : m, n, k);
+                        if (make_plan(gram ? n : m, n, k, gram, false).bytes() > reserve_bytes(M, s[1], s[2], gram))
+                            fail("reservation", M, s[1], s[2], m, n, k);
+                    }
                 }
         }
+    // a small problem's products (32^2 cells, 8 x 16 ordinates, cap 128) hold no planes
+    // that their contraction cannot be split into
+    if (reserve_bytes(641, 641, 1024, true) > (80u << 20)) fail("small Gram", 641, 641, 1024, 641, 641, 1024);
     std::printf("%ld\n", bad);
     return bad != 0;
 }
