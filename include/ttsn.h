@@ -568,6 +568,16 @@ tt_status tt_gram(int m, int n, const double* A_dev, int lda, double* G_dev, int
 tt_status tt_wait_probe(void* stream);
 
 /*
+ * tt_digits_wait_probe: the same for the digit products of tt_dgemm, whose
+ * kernel's roles wait for one another with a bounded spin.  C = A B (row-major,
+ * no transposes, a size that tt_dgemm takes digit products for) with every such
+ * wait given up at once; the product behind it must find that and recompute C
+ * on the FP64 tensor pipe, so C is complete all the same.
+ */
+tt_status tt_digits_wait_probe(int M, int N, int K, const double* A_dev, const double* B_dev, double* C_dev,
+                               void* stream);
+
+/*
  * tt_pchol: pivoted Cholesky factor of a symmetric positive semidefinite n x n
  * matrix G (leading dimension ldg), the factor of the right Gram matrix that
  * the one-sided truncation uses (W^T W = G_B, App. A.2): the pivot is the

@@ -118,6 +118,7 @@ def _load():
         "tt_set_rounding": [vp, i],
         "tt_set_eigensolver": [vp, i],
         "tt_wait_probe": [vp],
+        "tt_digits_wait_probe": [i, i, i, vp, vp, vp, vp],
         "tt_profile": [vp, i],
         "tt_profile_read": [vp, i, dp, ctypes.POINTER(ctypes.c_longlong),
                             ctypes.POINTER(ctypes.c_longlong), dp, dp],
@@ -159,7 +160,7 @@ EXPORTED = ["tt_create", "tt_create_tt", "tt_sn_step", "tt_sn_step_ex", "tt_roun
             "tt_batch_handle", "tt_batch_sync", "tt_batch_destroy", "tt_tape_begin",
             "tt_tape_objective", "tt_sn_step_adjoint", "tt_tape_clear", "tt_set_sources",
             "tt_create_ex", "tt_get_cores", "tt_pchol", "tt_set_inflow", "tt_set_sketch",
-            "tt_set_rounding", "tt_set_eigensolver", "tt_wait_probe", "tt_create_shard", "tt_syev_ex", "tt_syev_psd", "tt_set_max_sweeps", "tt_set_graph",
+            "tt_set_rounding", "tt_set_eigensolver", "tt_wait_probe", "tt_digits_wait_probe", "tt_create_shard", "tt_syev_ex", "tt_syev_psd", "tt_set_max_sweeps", "tt_set_graph",
             "tt_batch_set_graph", "tt_autotune", "tt_set_autotune_table", "tt_get_autotune_table"]
 
 PHASES = ["transport", "gram_right", "eig", "gram_left", "small", "update", "energy"]

@@ -3126,6 +3126,17 @@ tt_status tt_gemm_nt_mixed(int M, int N, int K, const double* A, int lda, const 
     return TT_OK;
 }
 
+tt_status tt_digits_wait_probe(int M, int N, int K, const double* A, const double* B, double* C, void* stream) {
+    set_error("");
+    if (M < 0 || N < 0 || K < 0 || !tc8_wanted(M, N, K))
+        return fail(TT_ERR_ARG, "tt_digits_wait_probe: not a size that tt_dgemm takes digit products for");
+    if (!A || !B || !C) return fail(TT_ERR_ARG, "tt_digits_wait_probe: null pointer");
+    cudaStream_t s = (cudaStream_t)stream;
+    TempScratch t(gemm_call_doubles(M, N, K), s);
+    if (!t.ok()) return fail(TT_ERR_OOM, "tt_digits_wait_probe: no room for the product's scratch");
+    return gemm_call(s, false, false, M, N, K, 1.0, A, K, B, N, C, N, t.buf, true);
+}
+
 tt_status tt_wait_probe(void* stream) {
     set_error("");
     cudaStream_t s = (cudaStream_t)stream;

@@ -28,8 +28,9 @@
 // 2.7e-16; 200,000 x 577 times 577 x 96 22.4 -> 1.8 ms, 8.0e-16 -> 5.5e-16.
 //
 // Inf, NaN and rows whose largest entry is outside 2^+-900 cannot be split:
-// the exponent scans latch a device flag and an FP64-pipe kernel behind the
-// product, which otherwise returns at once, recomputes it.
+// the exponent scans latch a device flag, and so does a wait that ran out; an
+// FP64-pipe kernel behind the product, which otherwise returns at once,
+// recomputes it.
 //
 // An entry far below its row's maximum keeps few digits, which matters where
 // small entries meet large ones (A times the identity, disjoint supports): the
@@ -89,15 +90,25 @@ __device__ __forceinline__ bool bar_try(unsigned a, unsigned parity) {
         : "memory");
     return ok != 0;
 }
-// Bounded wait; false once the limit is reached (DEV_TIMEOUT latched, the
-// other roles told through *abort_flag) or another role has given up.
-__device__ __forceinline__ bool bar_wait(unsigned a, unsigned parity, int* status, volatile int* abort_flag) {
-    for (long long it = 0; it < SPIN; ++it) {
+// Where a wait that ran out is reported: the caller's status word (null: none)
+// and the product's flag, upon which the product is recomputed.
+struct Report {
+    int *status, *lost;
+    __device__ __forceinline__ void timeout() const {
+        if (status) atomicOr(status, DEV_TIMEOUT);
+        atomicOr(lost, 1);
+    }
+};
+// Bounded wait; false once the limit is reached (reported, the other roles told
+// through *abort_flag) or another role has given up.
+__device__ __forceinline__ bool bar_wait(unsigned a, unsigned parity, const Report& rep, volatile int* abort_flag,
+                                         long long limit = SPIN) {
+    for (long long it = 0; it < limit; ++it) {
         if (bar_try(a, parity)) return true;
         if (abort_flag && *abort_flag) return false;
         if (it > 64) __nanosleep(32);
     }
-    if (status) atomicOr(status, DEV_TIMEOUT);
+    rep.timeout();
     if (abort_flag) *abort_flag = 1;
     return false;
 }
@@ -547,7 +558,7 @@ __device__ __forceinline__ void tile_of(long t, int nb, bool tri, long& mb, int&
 __global__ void __launch_bounds__(THREADS8, 1)
 tc8_kernel(Prod p, const unsigned char* __restrict__ At, const int* __restrict__ eA,
            const unsigned char* __restrict__ Bt, const int* __restrict__ eB, double alpha, double* __restrict__ C,
-           longlong2* __restrict__ planes, int spc, int* status) {
+           longlong2* __restrict__ planes, int spc, Report rep, long long limit) {
     if (!resolve(p)) return;  // every thread, before any barrier
     const long M = p.Mc;
     const int N = (int)p.N;
@@ -610,7 +621,7 @@ tc8_kernel(Prod p, const unsigned char* __restrict__ At, const int* __restrict__
                     const unsigned char* a1 = a0 + (long)nst * BLK_BYTES;
                     const unsigned char* b0 = Bt + ((long)kb * nst + it) * BLK_BYTES;
                     for (int q = 0; q < GROUPS; ++q) {
-                        if (!stop && !bar_wait(smem_addr(&bars[2 + 8 * st + q]), ph ^ 1u, status, flags)) stop = true;
+                        if (!stop && !bar_wait(smem_addr(&bars[2 + 8 * st + q]), ph ^ 1u, rep, flags, limit)) stop = true;
                         if (stop) {  // the stage's barrier completes with what was issued
                             bar_arrive(full);
                             continue;
@@ -639,13 +650,13 @@ tc8_kernel(Prod p, const unsigned char* __restrict__ At, const int* __restrict__
                     const unsigned ph = (unsigned)(g / T_STAGES) & 1u;
                     const bool first = ((it - st0) % T_BLK) == 0;
                     if (first && gb > 0) {
-                        if (!bar_wait(smem_addr(&bars[19]), (unsigned)(gb - 1) & 1u, status, flags)) {
+                        if (!bar_wait(smem_addr(&bars[19]), (unsigned)(gb - 1) & 1u, rep, flags, limit)) {
                             stop = true;
                             break;
                         }
                         fence_after();
                     }
-                    if (!bar_wait(smem_addr(&bars[st]), ph, status, flags)) {
+                    if (!bar_wait(smem_addr(&bars[st]), ph, rep, flags, limit)) {
                         stop = true;
                         break;
                     }
@@ -678,7 +689,7 @@ tc8_kernel(Prod p, const unsigned char* __restrict__ At, const int* __restrict__
                 }
             }
             mma_commit(smem_addr(&bars[20]));
-            bar_wait(smem_addr(&bars[20]), 0u, status, nullptr);
+            bar_wait(smem_addr(&bars[20]), 0u, rep, nullptr);
         }
     } else {
         const int q = warp & 3;  // TMEM lanes 32 q .. 32 q + 31
@@ -695,7 +706,7 @@ tc8_kernel(Prod p, const unsigned char* __restrict__ At, const int* __restrict__
 #pragma unroll
             for (int c = 0; c < DCOLS; ++c) hi[c] = lo[c] = 0;
             for (int b = 0; b < blocks; ++b, ++gb) {
-                if (!__all_sync(0xffffffffu, bar_wait(smem_addr(&bars[18]), (unsigned)gb & 1u, status, flags))) {
+                if (!__all_sync(0xffffffffu, bar_wait(smem_addr(&bars[18]), (unsigned)gb & 1u, rep, flags, limit))) {
                     stop = true;
                     break;
                 }
@@ -753,7 +764,7 @@ tc8_kernel(Prod p, const unsigned char* __restrict__ At, const int* __restrict__
     __syncthreads();
     if (threadIdx.x == 0) {  // after an abort: copies in flight land before the CTA exits
         for (long g = flags[2]; g < flags[1]; ++g)
-            bar_wait(smem_addr(&bars[g % T_STAGES]), (unsigned)(g / T_STAGES) & 1u, status, nullptr);
+            bar_wait(smem_addr(&bars[g % T_STAGES]), (unsigned)(g / T_STAGES) & 1u, rep, nullptr);
     }
     __syncthreads();
     if (warp == 1) {
@@ -822,7 +833,7 @@ unsigned blocks_for(long work, long cap) { return (unsigned)std::max<long>(1, st
 // descriptor's).
 tt_status run(cudaStream_t s, bool ta, bool tb, long M, long N, long K, double alpha, const double* A, long lda,
               const double* B, long ldb, double* C, long ldc, DevBuf& scratch, int* status_dev, bool gram,
-              const int* desc, const int** gate) {
+              const int* desc, const int** gate, long long limit = SPIN) {
     const Plan q = make_plan(M, N, K, gram, desc != nullptr);
     // slack to bring the base to a 1024-byte boundary (a pool may give 256)
     TT_TRY(scratch.ensure((q.bytes() + 1024 + 7) / 8, s));
@@ -911,7 +922,7 @@ tt_status run(cudaStream_t s, bool ta, bool tb, long M, long N, long K, double a
             const long items = tiles_of(std::min(q.Mc, M - p.i0), N, gram) * ((nst0 + spc - 1) / spc);
             note_launch();
             tc8_kernel<<<desc ? sms : (int)std::min<long>(items, sms), THREADS8, SMEM8, s>>>(
-                p, a.img, a.e, b.img, eB, alpha, C, direct ? nullptr : planes, spc, status_dev);
+                p, a.img, a.e, b.img, eB, alpha, C, direct ? nullptr : planes, spc, Report{status_dev, flag}, limit);
             TT_CUDA_TRY(cudaGetLastError());
         }
     }
@@ -952,8 +963,9 @@ size_t tc8_reserve_doubles(long M, long N, long K, bool gram) {
 
 tt_status tc8_gemm(cudaStream_t s, bool ta, bool tb, long M, long N, long K, double alpha, const double* A, long lda,
                    const double* B, long ldb, double* C, long ldc, DevBuf& scratch, int* status_dev,
-                   const int** gate) {
-    return run(s, ta, tb, M, N, K, alpha, A, lda, B, ldb, C, ldc, scratch, status_dev, false, nullptr, gate);
+                   const int** gate, bool probe) {
+    return run(s, ta, tb, M, N, K, alpha, A, lda, B, ldb, C, ldc, scratch, status_dev, false, nullptr, gate,
+               probe ? 0 : SPIN);
 }
 
 tt_status tc8_gram(cudaStream_t s, long m, long n, const double* A, long lda, double* G, long ldg, DevBuf& scratch,

@@ -558,12 +558,12 @@ size_t gemm_call_doubles(int M, int N, int K) {
 }
 
 tt_status gemm_call(cudaStream_t s, bool ta, bool tb, int M, int N, int K, double alpha, const double* A, long lda,
-                    const double* B, long ldb, double* C, long ldc, DevBuf& scratch) {
+                    const double* B, long ldb, double* C, long ldc, DevBuf& scratch, bool probe) {
     const int ks = prod_split(M, N, K, 0);
     const int* gate = nullptr;
     double* P = scratch.p;
     if (tc8_wanted(M, N, K)) {
-        TT_TRY(tc8_gemm(s, ta, tb, M, N, K, alpha, A, lda, B, ldb, C, ldc, scratch, nullptr, &gate));
+        TT_TRY(tc8_gemm(s, ta, tb, M, N, K, alpha, A, lda, B, ldb, C, ldc, scratch, nullptr, &gate, probe));
         P += tc8_scratch_doubles(M, N, K, false);
     }
     return split_prod(s, ta, tb, false, ProdArgs{M, N, K, alpha, A, lda, B, ldb, 0.0, C, ldc, ks, prod_chunk(K, ks),

@@ -96,7 +96,7 @@ tt_status dgemm_sk(cudaStream_t s, bool ta, bool tb, int M, int N, int K, double
 // cheapest.  Scratch of gemm_call_doubles.
 size_t gemm_call_doubles(int M, int N, int K);
 tt_status gemm_call(cudaStream_t s, bool ta, bool tb, int M, int N, int K, double alpha, const double* A, long lda,
-                    const double* B, long ldb, double* C, long ldc, DevBuf& scratch);
+                    const double* B, long ldb, double* C, long ldc, DevBuf& scratch, bool probe = false);
 
 // Autotuned split table (gemm.cu): buckets of floor(log2 tiles) < 8 and
 // floor(log2 K) < 22; autotune measures and installs it, autotune_install
@@ -175,12 +175,13 @@ size_t tc8_scratch_doubles(long M, long N, long K, bool gram, bool captured = fa
 size_t tc8_reserve_doubles(long M, long N, long K, bool gram);
 // gate (null: a rounding's product, complete on return): set to three device
 // ints for tc8_lost, and the caller recomputes the product where that holds.
+// probe: every wait of the product's kernel gives up at once (tt_digits_wait_probe).
 tt_status tc8_gemm(cudaStream_t s, bool ta, bool tb, long M, long N, long K, double alpha, const double* A, long lda,
                    const double* B, long ldb, double* C, long ldc, DevBuf& scratch, int* status_dev,
-                   const int** gate = nullptr);
+                   const int** gate = nullptr, bool probe = false);
 tt_status tc8_gram(cudaStream_t s, long m, long n, const double* A, long lda, double* G, long ldg, DevBuf& scratch,
                    int* status_dev, const int** gate = nullptr);
-// Some row could not be split (gate[0]), or two rows may have fewer than K / 16
+// Some row could not be split or a wait ran out (gate[0]), or two rows may have fewer than K / 16
 // indices where both are large (gate[1], gate[2]: the most indices that a row of
 // op(A), a column of op(B) is small at; the Gram has one operand).
 __device__ inline bool tc8_lost(const int* gate, int K, bool gram) {

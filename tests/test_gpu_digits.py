@@ -194,3 +194,23 @@ def test_captured_steps_that_split_where_their_capacity_does_not(ttsn, r1, r2):
         assert torch.equal(torch.as_tensor(x), torch.as_tensor(y))
     (Ea, Ta, ta), (Eb, Tb, tb) = a.energy(), b.energy()
     assert torch.equal(Ea, Eb) and torch.equal(Ta, Tb) and ta == tb
+
+
+@pytest.mark.parametrize("M,N,K", [(300, 260, 260), (60, 50, 9000)])
+def test_product_whose_waits_run_out_is_recomputed(ttsn, M, N, K):
+    """Every wait of the digit kernel gives up at once and C is written by nothing
+    (written whole, or summed from planes that were not): the FP64 pipe's sum
+    replaces it, off by K eps sum |a||b| at most, as is the reference's."""
+    import torch
+
+    from paper_2503_18056_gb300 import _native
+
+    rng = np.random.default_rng(M)
+    A, B = rng.standard_normal((M, K)), rng.standard_normal((K, N))
+    a, b = torch.as_tensor(A, device="cuda"), torch.as_tensor(B, device="cuda")
+    c = torch.full((M, N), -7.0, dtype=torch.float64, device="cuda")
+    st = _native.lib.tt_digits_wait_probe(M, N, K, *(ctypes.c_void_p(x.data_ptr()) for x in (a, b, c)),
+                                          ctypes.c_void_p(torch.cuda.current_stream().cuda_stream))
+    assert st == 0
+    assert np.all(np.abs(c.cpu().numpy() - A @ B) <= 2 * K * np.finfo(float).eps * (np.abs(A) @ np.abs(B)))
+    assert torch.equal(torch.as_tensor(_call(ttsn, A, B, False, False), device="cuda"), ttsn.dgemm(a, b))
