@@ -27,10 +27,10 @@
 // 500,000 x 449 143 -> 5.7 ms, error against the exact product 1.3e-15 ->
 // 2.7e-16; 200,000 x 577 times 577 x 96 22.4 -> 1.8 ms, 8.0e-16 -> 5.5e-16.
 //
-// Inf, NaN and rows whose largest entry is outside 2^+-900 cannot be split:
-// the exponent scans latch a device flag, and so does a wait that ran out; an
-// FP64-pipe kernel behind the product, which otherwise returns at once,
-// recomputes it.
+// Rows that hold Inf or NaN or whose largest entry is outside 2^+-900 cannot be
+// split: their exponent is EXP_LOST, their digits are zero, and gemm.cu's
+// prod_kernel behind the product, which otherwise returns at once, recomputes the
+// 16 x 16 tiles that they reach (tc8_lost), or everything where a wait ran out.
 //
 // An entry far below its row's maximum keeps few digits, which matters where
 // small entries meet large ones (A times the identity, disjoint supports): the
@@ -96,7 +96,7 @@ struct Report {
     int *status, *lost;
     __device__ __forceinline__ void timeout() const {
         if (status) atomicOr(status, DEV_TIMEOUT);
-        atomicOr(lost, 1);
+        atomicOr(lost + LOST_ALL, 1);
     }
 };
 // Bounded wait; false once the limit is reached (reported, the other roles told
@@ -191,11 +191,14 @@ __device__ __forceinline__ int split_stages_warp(long M, long N, long ntiles, in
 // |v| as its bit pattern (ordered as the values; Inf and NaN above all).
 __device__ __forceinline__ u64 mag(double v) { return (u64)__double_as_longlong(v) & 0x7FFFFFFFFFFFFFFFull; }
 __device__ __forceinline__ u64 umax(u64 a, u64 b) { return a > b ? a : b; }
-// e with every |v| <= the maximum of this pattern below 2^(e - 1); *flag is
-// latched when the maximum is Inf, NaN or outside 2^+-900.
+// e with every |v| <= the maximum of this pattern below 2^(e - 1); EXP_LOST (and
+// flag latched) where it is Inf, NaN or outside 2^+-900.
 __device__ __forceinline__ int split_exp(u64 mx, int* flag) {
     const int ex = (int)(mx >> 52);
-    if (mx != 0 && (ex < 1023 - 900 || ex > 1023 + 900)) atomicOr(flag, 1);
+    if (mx != 0 && (ex < 1023 - 900 || ex > 1023 + 900)) {
+        atomicOr(flag + LOST_ROWS, 1);
+        return EXP_LOST;
+    }
     return mx == 0 ? 0 : ex - 1023 + 2;
 }
 
@@ -302,7 +305,7 @@ __global__ void __launch_bounds__(256) split_rows_kernel(Prod p, Side o, int* fl
         }
         const int e = split_exp(mx, flag);
         if (lane == 0 && r < rows) o.e[i0 + r] = e;
-        if (o.worst && mx != 0) {
+        if (o.worst && mx != 0 && e != EXP_LOST) {
             int c = 0;
 #pragma unroll
             for (int t = 0; t < V; ++t)
@@ -480,10 +483,10 @@ __global__ void __launch_bounds__(256, 4) split_strided_kernel(Prod p, Side o, i
 
 // *worst: the most indices of a nonzero row that are not large
 __global__ void __launch_bounds__(256) spread_kernel(long rows, int K, const int* __restrict__ large,
-                                                     const u64* __restrict__ mx, int* worst) {
+                                                     const u64* __restrict__ mx, const int* __restrict__ e, int* worst) {
     int w = 0;
     for (long r = blockIdx.x * 256L + threadIdx.x; r < rows; r += gridDim.x * 256L)
-        if (mx[r] != 0) w = max(w, K - large[r]);
+        if (mx[r] != 0 && e[r] != EXP_LOST) w = max(w, K - large[r]);
     w = __reduce_max_sync(0xffffffffu, w);
     if ((threadIdx.x & 31) == 0 && w > *(volatile int*)worst) atomicMax(worst, w);
 }
@@ -800,40 +803,13 @@ tc8_reduce_kernel(Prod p, const longlong2* __restrict__ planes, const int* __res
     }
 }
 
-// The product on the FP64 FMA pipe, only where the split latched *flag.
-constexpr int FB = 16;
-__global__ void __launch_bounds__(FB * FB)
-fallback_kernel(const int* __restrict__ flag, Prod p, int ta, int tb, double alpha, const double* __restrict__ A,
-                const double* __restrict__ B, double* __restrict__ C) {
-    if (*flag == 0) return;
-    p.Mc = p.M;
-    if (!resolve(p)) return;
-    const long ai = ta ? 1 : p.lda, ak = ta ? p.lda : 1, bj = tb ? p.ldb : 1, bk = tb ? 1 : p.ldb;
-    __shared__ double As[FB][FB + 1], Bs[FB][FB + 1];
-    const int ty = threadIdx.x / FB, tx = threadIdx.x % FB;
-    const long nb = (p.N + FB - 1) / FB, tiles = (p.M + FB - 1) / FB * nb;
-    for (long t = blockIdx.x; t < tiles; t += gridDim.x) {
-        const long i = t / nb * FB + ty, j0 = t % nb * FB, j = j0 + tx;
-        double acc = 0.0;
-        for (long k0 = 0; k0 < p.K; k0 += FB) {
-            As[ty][tx] = i < p.M && k0 + tx < p.K ? A[i * ai + (k0 + tx) * ak] : 0.0;
-            Bs[ty][tx] = j0 + ty < p.N && k0 + tx < p.K ? B[(j0 + ty) * bj + (k0 + tx) * bk] : 0.0;
-            __syncthreads();
-            const int kn = (int)min((long)FB, p.K - k0);
-            for (int k = 0; k < kn; ++k) acc = fma(As[ty][k], Bs[tx][k], acc);
-            __syncthreads();
-        }
-        if (i < p.M && j < p.N) C[i * p.ldc + j] = alpha * acc;
-    }
-}
-
 unsigned blocks_for(long work, long cap) { return (unsigned)std::max<long>(1, std::min<long>(work, cap)); }
 
 // desc: a captured product of sizes up to M, N, K (then lda, ldb, ldc are the
 // descriptor's).
 tt_status run(cudaStream_t s, bool ta, bool tb, long M, long N, long K, double alpha, const double* A, long lda,
               const double* B, long ldb, double* C, long ldc, DevBuf& scratch, int* status_dev, bool gram,
-              const int* desc, const int** gate, long long limit = SPIN) {
+              const int* desc, bool guard, Lost* lost, long long limit = SPIN) {
     const Plan q = make_plan(M, N, K, gram, desc != nullptr);
     // slack to bring the base to a 1024-byte boundary (a pool may give 256)
     TT_TRY(scratch.ensure((q.bytes() + 1024 + 7) / 8, s));
@@ -841,10 +817,10 @@ tt_status run(cudaStream_t s, bool ta, bool tb, long M, long N, long K, double a
     int* flag = reinterpret_cast<int*>(base);
     u64* mx = reinterpret_cast<u64*>(base + 256);
     int* ex = reinterpret_cast<int*>(mx + M + N);
-    int* large = gate ? ex + M + N : nullptr;
-    int* worst = gate ? flag + 1 : nullptr;
+    int* large = guard ? ex + M + N : nullptr;
+    int* worst = guard ? flag + LOST_WORST : nullptr;
     Side a{A, 0, ta ? 1 : 0, mx, ex, base + q.head + q.imgB, large, worst};
-    Side b{B, 1, tb ? 0 : 1, mx + M, ex + M, base + q.head, gate ? large + M : nullptr, gate ? worst + 1 : nullptr};
+    Side b{B, 1, tb ? 0 : 1, mx + M, ex + M, base + q.head, guard ? large + M : nullptr, guard ? worst + 1 : nullptr};
     if (gram) a.img = base + q.head;
     longlong2* planes = q.part ? reinterpret_cast<longlong2*>(base + q.head + q.imgA + q.imgB) : nullptr;
     const int* eB = gram ? ex : b.e;
@@ -855,7 +831,7 @@ tt_status run(cudaStream_t s, bool ta, bool tb, long M, long N, long K, double a
     TT_TRY(ensure_max_dynamic_smem((const void*)tc8_kernel));
     // the flag and, where atomics find them, the maxima and counts start at zero
     TT_CUDA_TRY(cudaMemsetAsync(flag, 0, 256 + (a.strided || b.strided ? 8 * (size_t)(M + N) : 0), s));
-    if (gate) TT_CUDA_TRY(cudaMemsetAsync(large, 0, 4 * (size_t)(M + N), s));
+    if (guard) TT_CUDA_TRY(cudaMemsetAsync(large, 0, 4 * (size_t)(M + N), s));
     const bool fusable = K <= FUSED_K;  // a captured step launches both forms when K may be longer
     auto maxima = [&](const Side& o) {
         const long rows = o.isB ? N : M;
@@ -873,7 +849,7 @@ tt_status run(cudaStream_t s, bool ta, bool tb, long M, long N, long K, double a
         if (o.strided) {
             const dim3 grid(blocks_for((rpad + 31) / 32, 4096), blocks_for(((long)nst * 2 + 7) / 8, 2048));
             note_launch();
-            if (gate)
+            if (guard)
                 split_strided_kernel<true><<<grid, 256, 0, s>>>(p, o, flag);
             else
                 split_strided_kernel<false><<<grid, 256, 0, s>>>(p, o, flag);
@@ -932,22 +908,18 @@ tt_status run(cudaStream_t s, bool ta, bool tb, long M, long N, long K, double a
         note_launch();
         tc8_reduce_kernel<<<blocks_for((M * N + 255) / 256, 152L * 16), 256, 0, s>>>(p, planes, a.e, eB, spc, alpha, C);
     }
-    if (gate) {  // the caller recomputes what is lost
+    if (guard) {
         auto spread = [&](const Side& o) {
             const long rows = o.isB ? N : M;
             if (!o.strided && fusable) return;  // found by the split
             note_launch();
-            spread_kernel<<<blocks_for((rows + 255) / 256, 152), 256, 0, s>>>(rows, (int)K, o.large, o.mx, o.worst);
+            spread_kernel<<<blocks_for((rows + 255) / 256, 152), 256, 0, s>>>(rows, (int)K, o.large, o.mx, o.e, o.worst);
         };
         spread(a);
         if (!gram) spread(b);
-        TT_CUDA_TRY(cudaGetLastError());
-        *gate = flag;
-        return TT_OK;
     }
-    note_launch();
-    fallback_kernel<<<152 * 4, FB * FB, 0, s>>>(flag, p, ta ? 1 : 0, tb ? 1 : 0, alpha, A, B, C);
     TT_CUDA_TRY(cudaGetLastError());
+    *lost = Lost{flag, ex, eB, guard ? 1 : 0, gram ? 1 : 0, reinterpret_cast<double*>(base + q.head)};
     return TT_OK;
 }
 
@@ -961,21 +933,23 @@ size_t tc8_reserve_doubles(long M, long N, long K, bool gram) {
     return (reserve_bytes(M, N, K, gram) + 1024 + 7) / 8;
 }
 
+size_t tc8_head_doubles(long M, long N) { return (make_plan(M, N, T_K, false, false).head + 1024 + 7) / 8; }
+
 tt_status tc8_gemm(cudaStream_t s, bool ta, bool tb, long M, long N, long K, double alpha, const double* A, long lda,
-                   const double* B, long ldb, double* C, long ldc, DevBuf& scratch, int* status_dev,
-                   const int** gate, bool probe) {
-    return run(s, ta, tb, M, N, K, alpha, A, lda, B, ldb, C, ldc, scratch, status_dev, false, nullptr, gate,
+                   const double* B, long ldb, double* C, long ldc, DevBuf& scratch, int* status_dev, bool guard,
+                   Lost* lost, bool probe) {
+    return run(s, ta, tb, M, N, K, alpha, A, lda, B, ldb, C, ldc, scratch, status_dev, false, nullptr, guard, lost,
                probe ? 0 : SPIN);
 }
 
 tt_status tc8_gram(cudaStream_t s, long m, long n, const double* A, long lda, double* G, long ldg, DevBuf& scratch,
-                   int* status_dev, const int** gate) {
-    return run(s, true, false, n, n, m, 1.0, A, lda, A, lda, G, ldg, scratch, status_dev, true, nullptr, gate);
+                   int* status_dev, bool guard, Lost* lost) {
+    return run(s, true, false, n, n, m, 1.0, A, lda, A, lda, G, ldg, scratch, status_dev, true, nullptr, guard, lost);
 }
 
 tt_status tc8_dyn(cudaStream_t s, bool ta, bool tb, const int* desc, long Mcap, long Ncap, long Kcap, double alpha,
-                  const double* A, const double* B, double* C, DevBuf& scratch, int* status_dev, bool gram) {
-    return run(s, ta, tb, Mcap, Ncap, Kcap, alpha, A, 0, B, 0, C, 0, scratch, status_dev, gram, desc, nullptr);
+                  const double* A, const double* B, double* C, DevBuf& scratch, int* status_dev, bool gram, Lost* lost) {
+    return run(s, ta, tb, Mcap, Ncap, Kcap, alpha, A, 0, B, 0, C, 0, scratch, status_dev, gram, desc, false, lost);
 }
 
 }  // namespace ttsn

@@ -180,18 +180,18 @@ __host__ __device__ inline int ordered_split(int M, int N, int K, int tri, int* 
 
 // C = alpha op(A) op(B) (+ beta C), or with tri the symmetric product of which
 // only the tiles on and above the diagonal are formed (both halves stored).
-// desc (a captured step): M, N, K, lda, ldb, ldc in device memory; tc: sizes
-// that digits.cu takes are left to it.  gate: behind a digit product, which it
-// replaces where that lost accuracy (tc8_lost).  An item is (tile, split); ks > 1:
+// desc (a captured step): M, N, K, lda, ldb, ldc in device memory.  lost: behind a
+// digit product (in a captured step of the sizes that take one), of which it
+// recomputes what tc8_lost says: everything, or the tiles with a lost row or
+// column.  An item is (tile, split); ks > 1:
 // partials to P (256 doubles an item), arrivals counted in cnt (zero between
-// products: the last arrival resets its tile's).  ORDERED: a warp per 8 x 8 block; else the warps share the indices.  An 8 x 8
-// product outside M x N or below the diagonal is skipped.
+// products: the last arrival resets its tile's).  ORDERED: a warp per 8 x 8
+// block; else the warps share the indices.  An 8 x 8 product outside M x N or below the diagonal is skipped.
 template <bool TA, bool TB, bool ORDERED>
 __global__ void __launch_bounds__(THREADS)
 prod_kernel(int M, int N, int K, double alpha, const double* __restrict__ A, long lda, const double* __restrict__ B,
             long ldb, double beta, double* __restrict__ C, long ldc, int ks, int chunk, double* __restrict__ P, int* cnt,
-            int tri, const int* __restrict__ desc, int tc, const int* __restrict__ gate) {
-    if (gate && !tc8_lost(gate, K, tri != 0)) return;
+            int tri, const int* __restrict__ desc, Lost lost) {
     if (desc) {
         M = desc[0];
         N = desc[1];
@@ -199,11 +199,14 @@ prod_kernel(int M, int N, int K, double alpha, const double* __restrict__ A, lon
         lda = desc[3];
         ldb = desc[4];
         ldc = desc[5];
-        if (M <= 0 || N <= 0 || (tc && tc8_wanted(M, N, K))) return;
+        if (M <= 0 || N <= 0) return;
         ks = 1;
         chunk = K;
         if (P) ks = ordered_split(M, N, K, tri, &chunk);  // P null: an unsplit product
     }
+    const bool behind = lost.flag && (!desc || tc8_wanted(M, N, K));
+    const int redo = behind ? tc8_lost(lost, K) : 2;
+    if (redo == 0) return;
     __shared__ double red[ORDERED ? 1 : 4][BT * BT];
     __shared__ int s_last;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
@@ -226,6 +229,10 @@ prod_kernel(int M, int N, int K, double alpha, const double* __restrict__ A, lon
             tn = (int)(tile % TN);
         }
         const int m0 = tm * BT, n0 = tn * BT;
+        if (redo == 1) {  // the same for every warp
+            const int e = lane < BT ? lost.a[min(m0 + lane, M - 1)] : lost.b[min(n0 + lane - BT, N - 1)];
+            if (!__any_sync(0xffffffffu, e == EXP_LOST)) continue;
+        }
         const int kbeg = z * chunk, kend = min(K, kbeg + chunk);
         const long sa = TA ? lda : 1, sb = TB ? 1 : ldb;
         __syncthreads();  // the item before has read red
@@ -448,23 +455,23 @@ struct ProdArgs {
     double* P;
     int *cnt, tri;
     const int* desc;
-    int tc;
-    const int* gate = nullptr;
+    Lost lost = {};
 };
 
 template <bool TA, bool TB>
 void launch_one(cudaStream_t s, bool ordered, unsigned grid, const ProdArgs& a) {
     if (ordered)
         prod_kernel<TA, TB, true><<<grid, THREADS, 0, s>>>(a.M, a.N, a.K, a.alpha, a.A, a.lda, a.B, a.ldb, a.beta, a.C,
-                                                          a.ldc, a.ks, a.chunk, a.P, a.cnt, a.tri, a.desc, a.tc, a.gate);
+                                                          a.ldc, a.ks, a.chunk, a.P, a.cnt, a.tri, a.desc, a.lost);
     else
         prod_kernel<TA, TB, false><<<grid, THREADS, 0, s>>>(a.M, a.N, a.K, a.alpha, a.A, a.lda, a.B, a.ldb, a.beta, a.C,
-                                                           a.ldc, a.ks, a.chunk, a.P, a.cnt, a.tri, a.desc, a.tc, a.gate);
+                                                           a.ldc, a.ks, a.chunk, a.P, a.cnt, a.tri, a.desc, a.lost);
 }
 
 tt_status launch_prod(cudaStream_t s, bool ta, bool tb, bool ordered, long items, const ProdArgs& a) {
-    // more CTAs than fit at once let the scheduler level uneven tiles
-    const unsigned grid = (unsigned)std::max(1L, std::min(items, 152L * 64));
+    // more CTAs than fit at once let the scheduler level uneven tiles; behind a
+    // digit product they seldom have any
+    const unsigned grid = (unsigned)std::max(1L, std::min(items, a.lost.flag && !a.desc ? 152L * 8 : 152L * 64));
     note_launch();
     if (ta && tb)
         launch_one<true, true>(s, ordered, grid, a);
@@ -482,6 +489,14 @@ tt_status launch_prod(cudaStream_t s, bool ta, bool tb, bool ordered, long items
 // the caller keeps none (zeroed ahead of the launch).
 size_t split_doubles(long tiles, int ks) { return (size_t)tiles * ks * (BT * BT); }
 size_t split_scratch(long tiles, int ks) { return ks > 1 ? split_doubles(tiles, ks) + (size_t)(tiles + 1) / 2 : 0; }
+
+// Scratch of a digit product and, behind its head, of the recomputation with ks
+// splits.
+size_t digits_doubles(long M, long N, long K, int tri, int ks) {
+    const size_t part = split_scratch(prod_tiles(M, N, tri), ks);
+    if (!tc8_wanted(M, N, K)) return part;
+    return std::max(tc8_scratch_doubles(M, N, K, tri != 0), tc8_head_doubles(M, N) + part);
+}
 
 tt_status split_prod(cudaStream_t s, bool ta, bool tb, bool ordered, ProdArgs a) {
     const long tiles = prod_tiles(a.M, a.N, a.tri);
@@ -509,41 +524,57 @@ tt_status dgemm(cudaStream_t s, bool ta, bool tb, int M, int N, int K, double al
     }
     if (M == 0 || N == 0) return TT_OK;
     return launch_prod(s, ta, tb, true, prod_tiles(M, N, 0),
-                       ProdArgs{M, N, K, alpha, A, lda, B, ldb, beta, C, ldc, 1, K, nullptr, nullptr, 0, nullptr, 0});
+                       ProdArgs{M, N, K, alpha, A, lda, B, ldb, beta, C, ldc, 1, K, nullptr, nullptr, 0, nullptr});
 }
 
 tt_status dgemm_sk(cudaStream_t s, bool ta, bool tb, int M, int N, int K, double alpha,
                    const double* A, long lda, const double* B, long ldb, double* C, long ldc,
                    DevBuf& scratch, const ProdCtx& ctx, bool split) {
-    if (ctx.digits && tc8_wanted(M, N, K)) {
-        const tt_status st = tc8_gemm(s, ta, tb, M, N, K, alpha, A, lda, B, ldb, C, ldc, scratch, ctx.status);
-        if (st != TT_ERR_OOM) return st;  // without room for the digits: the FP64 pipe
-    }
     int ks = 1, chunk = K;
     if (split && M > 0 && N > 0 && K > 0) ks = ordered_split(M, N, K, 0, &chunk);
+    const size_t part = split_scratch(prod_tiles(M, N, 0), ks);
+    if (ctx.digits && tc8_wanted(M, N, K)) {
+        Lost lost;
+        // without room for the digits: the FP64 pipe
+        tt_status st = scratch.ensure(digits_doubles(M, N, K, 0, ks), s);
+        if (st >= 0)
+            st = tc8_gemm(s, ta, tb, M, N, K, alpha, A, lda, B, ldb, C, ldc, scratch, ctx.status, false, &lost);
+        if (st >= 0)
+            return split_prod(s, ta, tb, true, ProdArgs{M, N, K, alpha, A, lda, B, ldb, 0.0, C, ldc, ks, chunk, lost.free,
+                                                        ctx.counters, 0, nullptr, lost});
+        if (st != TT_ERR_OOM) return st;
+    }
     if (ks == 1) return dgemm(s, ta, tb, M, N, K, alpha, A, lda, B, ldb, 0.0, C, ldc);
-    TT_TRY(scratch.ensure(split_scratch(prod_tiles(M, N, 0), ks), s));
+    TT_TRY(scratch.ensure(part, s));
     return split_prod(s, ta, tb, true, ProdArgs{M, N, K, alpha, A, lda, B, ldb, 0.0, C, ldc, ks, chunk, scratch.p,
-                                                ctx.counters, 0, nullptr, 0});
+                                                ctx.counters, 0, nullptr});
 }
 
 tt_status gram(cudaStream_t s, int m, int n, const double* A, long lda, double* G, long ldg, DevBuf& partials,
                const ProdCtx& ctx) {
     if (n <= 0) return TT_OK;
-    if (ctx.digits && tc8_wanted(n, n, m)) {
-        const tt_status st = tc8_gram(s, m, n, A, lda, G, ldg, partials, ctx.status);
-        if (st != TT_ERR_OOM) return st;
-    }
     if (m <= 0) {
         for (int i = 0; i < n; ++i) fill(s, G + (long)i * ldg, n, 0.0);
         return TT_OK;
     }
     int chunk = m;
     const int ks = ordered_split(n, n, m, 1, &chunk);
-    TT_TRY(partials.ensure(split_scratch(prod_tiles(n, n, 1), ks), s));
+    const size_t part = split_scratch(prod_tiles(n, n, 1), ks);
     // op(A) = A^T (stored m x n), op(B) = A
-    return split_prod(s, true, false, true, ProdArgs{n, n, m, 1.0, A, lda, A, lda, 0.0, G, ldg, ks, chunk, partials.p,
-                                                     ctx.counters, 1, nullptr, 0});
+    ProdArgs a{n, n, m, 1.0, A, lda, A, lda, 0.0, G, ldg, ks, chunk, nullptr, ctx.counters, 1, nullptr};
+    if (ctx.digits && tc8_wanted(n, n, m)) {
+        tt_status st = partials.ensure(digits_doubles(n, n, m, 1, ks), s);
+        if (st >= 0) st = tc8_gram(s, m, n, A, lda, G, ldg, partials, ctx.status, false, &a.lost);
+        if (st >= 0) {
+            a.P = a.lost.free;
+            return split_prod(s, true, false, true, a);
+        }
+        if (st != TT_ERR_OOM) return st;
+    }
+    TT_TRY(partials.ensure(part, s));
+    a.P = partials.p;
+    a.lost = {};
+    return split_prod(s, true, false, true, a);
 }
 
 size_t gram_scratch_doubles(int m, int n) {
@@ -552,27 +583,21 @@ size_t gram_scratch_doubles(int m, int n) {
 
 // ------------------------------------------------------------ library calls
 
-size_t gemm_call_doubles(int M, int N, int K) {
-    return (tc8_wanted(M, N, K) ? tc8_scratch_doubles(M, N, K, false) : 0) +
-           split_scratch(prod_tiles(M, N, 0), prod_split(M, N, K, 0));
-}
+size_t gemm_call_doubles(int M, int N, int K) { return digits_doubles(M, N, K, 0, prod_split(M, N, K, 0)); }
 
 tt_status gemm_call(cudaStream_t s, bool ta, bool tb, int M, int N, int K, double alpha, const double* A, long lda,
                     const double* B, long ldb, double* C, long ldc, DevBuf& scratch, bool probe) {
     const int ks = prod_split(M, N, K, 0);
-    const int* gate = nullptr;
-    double* P = scratch.p;
+    ProdArgs a{M, N, K, alpha, A, lda, B, ldb, 0.0, C, ldc, ks, prod_chunk(K, ks), scratch.p, nullptr, 0, nullptr};
     if (tc8_wanted(M, N, K)) {
-        TT_TRY(tc8_gemm(s, ta, tb, M, N, K, alpha, A, lda, B, ldb, C, ldc, scratch, nullptr, &gate, probe));
-        P += tc8_scratch_doubles(M, N, K, false);
+        TT_TRY(tc8_gemm(s, ta, tb, M, N, K, alpha, A, lda, B, ldb, C, ldc, scratch, nullptr, true, &a.lost, probe));
+        a.P = a.lost.free;
     }
-    return split_prod(s, ta, tb, false, ProdArgs{M, N, K, alpha, A, lda, B, ldb, 0.0, C, ldc, ks, prod_chunk(K, ks),
-                                                 P, nullptr, 0, nullptr, 0, gate});
+    return split_prod(s, ta, tb, false, a);
 }
 
 size_t gram_call_doubles(int m, int n) {
-    return (tc8_wanted(n, n, m) ? tc8_scratch_doubles(n, n, m, true) : 0) +
-           split_scratch(prod_tiles(n, n, 1), prod_split(n, n, std::max(m, 1), 1));
+    return digits_doubles(n, n, std::max(m, 1), 1, prod_split(n, n, std::max(m, 1), 1));
 }
 
 tt_status gram_fixed_scratch(cudaStream_t s, int m, int n, const double* A, long lda, double* G,
@@ -591,20 +616,18 @@ tt_status gram_fixed_scratch(cudaStream_t s, int m, int n, const double* A, long
     while (ks > 1 && split_scratch(tiles, ks) > scratch_doubles) --ks;
     ks = prod_final(m, ks);
     return split_prod(s, true, false, false, ProdArgs{n, n, m, 1.0, A, lda, A, lda, 0.0, G, ldg, ks, prod_chunk(m, ks),
-                                                      scratch, nullptr, 1, nullptr, 0});
+                                                      scratch, nullptr, 1, nullptr});
 }
 
 tt_status gram_call(cudaStream_t s, int m, int n, const double* A, long lda, double* G, long ldg, DevBuf& scratch) {
     if (m > 0 && tc8_wanted(n, n, m)) {
-        const size_t own = tc8_scratch_doubles(n, n, m, true);
+        const int ks = prod_split(n, n, m, 1);
+        ProdArgs a{n, n, m, 1.0, A, lda, A, lda, 0.0, G, ldg, ks, prod_chunk(m, ks), nullptr, nullptr, 1, nullptr};
         tt_status st = scratch.ensure(gram_call_doubles(m, n), s);
-        const int* gate = nullptr;
-        if (st >= 0) st = tc8_gram(s, m, n, A, lda, G, ldg, scratch, nullptr, &gate);
+        if (st >= 0) st = tc8_gram(s, m, n, A, lda, G, ldg, scratch, nullptr, true, &a.lost);
         if (st >= 0) {
-            const int ks = prod_split(n, n, m, 1);
-            return split_prod(s, true, false, false, ProdArgs{n, n, m, 1.0, A, lda, A, lda, 0.0, G, ldg, ks,
-                                                              prod_chunk(m, ks), scratch.p + own, nullptr, 1, nullptr, 0,
-                                                              gate});
+            a.P = a.lost.free;
+            return split_prod(s, true, false, false, a);
         }
         if (st != TT_ERR_OOM) return st;
     }
@@ -647,8 +670,9 @@ tt_status dgemm_dyn(cudaStream_t s, bool ta, bool tb, const int* desc, int Mcap,
                     DevBuf& tcbuf, const ProdCtx& ctx) {
     if (Mcap <= 0 || Ncap <= 0) return TT_OK;
     const int tri = mode == 2 ? 1 : 0;
-    const int tc = ctx.digits && tc8_wanted(Mcap, Ncap, Kcap) ? 1 : 0;
-    if (tc) TT_TRY(tc8_dyn(s, ta, tb, desc, Mcap, Ncap, Kcap, alpha, A, B, C, tcbuf, ctx.status, mode == 2));
+    Lost lost;
+    if (ctx.digits && tc8_wanted(Mcap, Ncap, Kcap))
+        TT_TRY(tc8_dyn(s, ta, tb, desc, Mcap, Ncap, Kcap, alpha, A, B, C, tcbuf, ctx.status, mode == 2, &lost));
     const size_t need = dyn_partials_need(mode, Mcap, Ncap, Kcap);
     if (need > pcap) {
         set_error("dgemm: the partials buffer of a captured product is smaller than its split needs");
@@ -662,7 +686,7 @@ tt_status dgemm_dyn(cudaStream_t s, bool ta, bool tb, const int* desc, int Mcap,
     }
     // eight CTAs an SM, or fewer where the capacity has no more items, walk
     // whatever the device's sizes give; mode 0 does not split
-    ProdArgs a{0, 0, 0, alpha, A, 0, B, 0, 0.0, C, 0, 1, 0, mode == 0 ? nullptr : P, cnt, tri, desc, tc};
+    ProdArgs a{0, 0, 0, alpha, A, 0, B, 0, 0.0, C, 0, 1, 0, mode == 0 ? nullptr : P, cnt, tri, desc, lost};
     return launch_prod(s, ta, tb, true, std::min(152L * 8, tiles * 64), a);
 }
 
@@ -803,7 +827,7 @@ tt_status autotune(cudaStream_t s, int* table_out) {
                     cudaEventRecord(e0, s);
                     st = launch_prod(s, false, false, true, prod_tiles(M, N, 0) * kk,
                                      ProdArgs{M, N, K, 1.0, A, K, B, N, 0.0, C, N, kk, kk > 1 ? kchunk : K, P, cnt, 0,
-                                              nullptr, 0});
+                                              nullptr});
                     cudaEventRecord(e1, s);
                     if (st < 0 || cudaEventSynchronize(e1) != cudaSuccess) {
                         if (st >= 0) st = TT_ERR_CUDA;

@@ -173,24 +173,42 @@ tt_status slgemm_nt(cudaStream_t s, long M, int N, int K, const double* A, long 
 size_t tc8_scratch_doubles(long M, long N, long K, bool gram, bool captured = false);
 // and of any product of sizes up to these
 size_t tc8_reserve_doubles(long M, long N, long K, bool gram);
-// gate (null: a rounding's product, complete on return): set to three device
-// ints for tc8_lost, and the caller recomputes the product where that holds.
+// What a digit product leaves to be recomputed by the caller (tc8_lost): flag
+// holds whether that is everything (LOST_ALL: a wait ran out) or rows of op(A) or
+// columns of op(B) whose exponent is EXP_LOST (LOST_ROWS), and of a guarded
+// product (a library call) the most indices that a row of op(A) and a column of
+// op(B) is small at (LOST_WORST).  free: the scratch behind tc8_head_doubles, in
+// which the recomputation's partials may go.
+constexpr int LOST_ALL = 0, LOST_ROWS = 1, LOST_WORST = 2;
+constexpr int EXP_LOST = 1 << 20;
+struct Lost {
+    const int* flag = nullptr;  // null: a product of its own
+    const int *a = nullptr, *b = nullptr;
+    int guard = 0, gram = 0;
+    double* free = nullptr;
+};
+#ifdef __CUDACC__
+// 2: everything is lost (of a guarded product also where two rows may have fewer
+// than K / 16 indices where both are large; the Gram has one operand), 1: some
+// rows, 0: nothing.
+__device__ inline int tc8_lost(const Lost& l, int K) {
+    if (l.flag[LOST_ALL] ||
+        (l.guard && (long)l.flag[LOST_WORST] + l.flag[LOST_WORST + (l.gram ? 0 : 1)] > K - K / 16))
+        return 2;
+    return l.flag[LOST_ROWS] ? 1 : 0;
+}
+#endif
+size_t tc8_head_doubles(long M, long N);
 // probe: every wait of the product's kernel gives up at once (tt_digits_wait_probe).
 tt_status tc8_gemm(cudaStream_t s, bool ta, bool tb, long M, long N, long K, double alpha, const double* A, long lda,
-                   const double* B, long ldb, double* C, long ldc, DevBuf& scratch, int* status_dev,
-                   const int** gate = nullptr, bool probe = false);
+                   const double* B, long ldb, double* C, long ldc, DevBuf& scratch, int* status_dev, bool guard,
+                   Lost* lost, bool probe = false);
 tt_status tc8_gram(cudaStream_t s, long m, long n, const double* A, long lda, double* G, long ldg, DevBuf& scratch,
-                   int* status_dev, const int** gate = nullptr);
-// Some row could not be split or a wait ran out (gate[0]), or two rows may have fewer than K / 16
-// indices where both are large (gate[1], gate[2]: the most indices that a row of
-// op(A), a column of op(B) is small at; the Gram has one operand).
-__device__ inline bool tc8_lost(const int* gate, int K, bool gram) {
-    return gate[0] != 0 || (long)gate[1] + (gram ? gate[1] : gate[2]) > K - K / 16;
-}
+                   int* status_dev, bool guard, Lost* lost);
 // The captured form: sizes from desc (as dgemm_dyn's), at most the capacities;
 // does nothing for sizes that tc8_wanted leaves to the FP64 pipe.
 tt_status tc8_dyn(cudaStream_t s, bool ta, bool tb, const int* desc, long Mcap, long Ncap, long Kcap, double alpha,
-                  const double* A, const double* B, double* C, DevBuf& scratch, int* status_dev, bool gram);
+                  const double* A, const double* B, double* C, DevBuf& scratch, int* status_dev, bool gram, Lost* lost);
 
 // Row scaling: out[i][j] = in[i][j] * f(v[i]) for i < rows, j < cols, where
 // mode 0: v, 1: sqrt(v), 2: 1/sqrt(v), 3: 1/v.  out may alias in.

@@ -214,3 +214,27 @@ def test_product_whose_waits_run_out_is_recomputed(ttsn, M, N, K):
     assert st == 0
     assert np.all(np.abs(c.cpu().numpy() - A @ B) <= 2 * K * np.finfo(float).eps * (np.abs(A) @ np.abs(B)))
     assert torch.equal(torch.as_tensor(_call(ttsn, A, B, False, False), device="cuda"), ttsn.dgemm(a, b))
+
+
+def test_rows_that_cannot_be_split_leave_the_others_as_they_are(ttsn):
+    """A row below 2^-900 or with an Inf and a column with a NaN are recomputed with
+    their 16 x 16 tiles; every other entry keeps the digit product's bits."""
+    rng = np.random.default_rng(1)
+    M, N, K = 300, 260, 300
+    A, B = rng.standard_normal((M, K)), rng.standard_normal((K, N))
+    plain = _call(ttsn, A, B, False, False)
+    X, Y = A.copy(), B.copy()
+    X[37] *= 1e-290
+    X[120, 5] = np.inf
+    Y[9, 201] = np.nan
+    got = _call(ttsn, X, Y, False, False)
+    with np.errstate(all="ignore"):
+        ref = X @ Y
+    rows, cols = np.ones(M, bool), np.ones(N, bool)
+    rows[32:48] = rows[112:128] = cols[192:208] = False
+    assert np.array_equal(got[np.ix_(rows, cols)], plain[np.ix_(rows, cols)])
+    assert np.array_equal(np.isnan(got), np.isnan(ref)) and np.array_equal(np.isinf(got), np.isinf(ref))
+    fine = np.isfinite(ref)
+    bound = (K + 1) * np.finfo(float).eps * (np.abs(A) @ np.abs(B))
+    bound[37] *= 1e-290
+    assert np.all(np.abs(got[fine] - ref[fine]) <= 2 * bound[fine])
