@@ -2423,7 +2423,7 @@ tt_status create_impl(const tt_problem_desc* desc, void* stream, const tt_alloca
             for (const auto& q : c)
                 if (tc8_wanted(q[1], q[2], q[3])) {
                     need = std::max(need, tc8_reserve_doubles(q[1], q[2], q[3], q[0] != 0));
-                    need = std::max(need, tc8_head_doubles(q[1], q[2]) +
+                    need = std::max(need, tc8_head_doubles(q[1], q[2], q[3], q[0] != 0) +
                                               dyn_partials_need(q[0] ? 2 : 1, (int)q[1], (int)q[2], (int)q[3]));
                 }
             const tt_status ps = need ? h->partials.ensure(need, s) : TT_OK;

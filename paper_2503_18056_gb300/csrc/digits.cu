@@ -5,27 +5,34 @@
 // from exact integer digit products (the error-free splitting of Ozaki, Ogita,
 // Oishi, Rump, Numer. Algorithms 59, 2012, with fixed-point digits):
 //
-//   Split.  Row i of op(A) and column j of op(B) carry a power of two each,
-//   |a_ik| < 2^(e_i - 1); a_ik 2^-e_i is rounded to 56-bit fixed point (an
-//   entry within a factor 8 of its row's maximum keeps all its 53 bits) and
-//   cut into S = 8 balanced base-128 digits, d_0 in [0, 64], the others in
-//   [-64, 63], each exact in BF16.
+//   Split.  Row i of op(A) and column j of op(B) carry a power of two each (of a
+//   contraction above 1024 indices, for every block of 512 of them: an entry is
+//   measured against its neighbours, not against the whole row), |a_ik| <
+//   2^(e_i - 1); a_ik 2^-e_i is rounded to 56-bit fixed point (an entry within a
+//   factor 8 of its row's maximum keeps all its 53 bits) and cut into S = 8
+//   balanced base-128 digits, d_0 in [0, 64], the others in [-64, 63], each exact
+//   in BF16.
 //   Products.  d_s d_t (at most 2^12) of level w = s + t <= 7 are summed by
 //   tcgen05.mma over at most 512 contraction indices: 8 pairs * 512 * 2^12 =
 //   2^24, so the FP32 accumulators hold exact integers.  The dropped levels
-//   are about 2^-56 of max|a_i| max|b_j| a term.
-//   Sums.  Every block's level sums are added as integers into two 64-bit
-//   accumulators an output (levels 0-3 and 4-7), also across splits and chunks
-//   of the contraction: the sum is exact and is rounded once to FP64, so the
-//   result does not depend on how the work is cut.
+//   are about 2^-56 of the maxima's product a term.
+//   Sums.  A block's level sums are added as integers (levels 0-3 and 4-7), and
+//   the blocks in fixed point under the rows' largest exponents (E_i, E_j), also
+//   across splits and chunks of the contraction: the sum is exact (a block more than
+//   2^8 below 2^(E_i + E_j) is cut off at 2^-71 of it) and is rounded once to FP64,
+//   so the result does not depend on how the work is cut (up to 16384 indices the
+//   cut follows from the sizes, above it lies between blocks).
 //
+// What is lost, the dropped levels and the rounding to 56 bits, is at most 9.1
+// 2^-58 2^(e_i + e_j) an index.
 // Against the FP64 pipe's running sum (an error of 2^-53 of the partial sum a
 // term) the result is nearer to the exact product from K of a few dozen on;
 // the sizes where it is used (tc8_wanted) have K >= 64.
 //
 // Measured (GB300, CUDA events, against the FP64 pipe's kernels): Gram of
-// 500,000 x 449 143 -> 5.7 ms, error against the exact product 1.3e-15 ->
-// 2.7e-16; 200,000 x 577 times 577 x 96 22.4 -> 1.8 ms, 8.0e-16 -> 5.5e-16.
+// 500,000 x 449 143 -> 5.95 ms (5.72 with one exponent a column), error against the
+// exact product 1.3e-15 -> 1.2e-16 (2.4e-16); 200,000 x 577 times 577 x 96 22.4 ->
+// 1.8 ms, 8.0e-16 -> 5.5e-16.
 //
 // Rows that hold Inf or NaN or whose largest entry is outside 2^+-900 cannot be
 // split: their exponent is EXP_LOST, their digits are zero, and gemm.cu's
@@ -34,9 +41,9 @@
 //
 // An entry far below its row's maximum keeps few digits, which matters where
 // small entries meet large ones (A times the identity, disjoint supports): the
-// sum |a||b| is then far below K max|a_i| max|b_j|, which bounds the error.  The
-// rounding needs its Grams to eps ||A||^2 only; a library call is also held to
-// the sum's scale: the split counts each row's entries above 2^-9 of its
+// sum |a||b| is then far below K max|a_i| max|b_j|, which bounds the error.  A
+// rounding's Gram is held to its columns' norms (gram_check_kernel in gemm.cu), a
+// library call to the sum's scale: the split counts each row's entries above 2^-9 of its
 // maximum, and unless every pair of rows has K / 16 indices where both are
 // (tc8_lost), the product is recomputed on the FP64 pipe (the count and the
 // check: 200,000 x 577 times 577 x 96 1.73 -> 1.78 ms, the Gram of 500,000 x 449
@@ -147,6 +154,11 @@ __device__ __forceinline__ void tmem_ld16(unsigned addr, unsigned (&r)[16]) {
           "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15])
         : "r"(addr));
 }
+__device__ __forceinline__ void tmem_ld4(unsigned addr, unsigned (&r)[4]) {
+    asm volatile("tcgen05.ld.sync.aligned.32x32b.x4.b32 {%0,%1,%2,%3}, [%4];"
+                 : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3])
+                 : "r"(addr));
+}
 __device__ __forceinline__ void tmem_wait_ld() { asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory"); }
 
 typedef unsigned long long u64;
@@ -177,13 +189,13 @@ __device__ __forceinline__ bool resolve(Prod& p) {
     return p.Mc > 0 && p.k0 < p.K;
 }
 // split_stages as one warp makes it
-__device__ __forceinline__ int split_stages_warp(long M, long N, long ntiles, int nst) {
-    const int lim = split_limit(M, N, nst), lane = threadIdx.x & 31;
+__device__ __forceinline__ int split_stages_warp(long M, long N, long ntiles, int nst, int unit) {
+    const int lim = split_limit(M, N, nst, unit), lane = threadIdx.x & 31;
     unsigned key = 0xffffffffu;
-    for (int k = lane + 1; k <= lim; k += 32) key = min(key, split_cost(k, ntiles, nst) * 64u + (unsigned)(k - 1));
+    for (int k = lane + 1; k <= lim; k += 32)
+        key = min(key, split_cost(k, ntiles, nst, unit) * 64u + (unsigned)(k - 1));
     key = __reduce_min_sync(0xffffffffu, key);
-    const int best = (int)(key & 63u) + 1;
-    return (nst + best - 1) / best;
+    return stages_of_split((int)(key & 63u) + 1, nst, unit);
 }
 
 // ------------------------------------------------------------------ split
@@ -200,6 +212,13 @@ __device__ __forceinline__ int split_exp(u64 mx, int* flag) {
         return EXP_LOST;
     }
     return mx == 0 ? 0 : ex - 1023 + 2;
+}
+// The same of a block of a row; its range is the row's matter.
+constexpr int EXP_ZERO = -EXP_LOST;  // nothing in it but zeros (and subnormals, which have no digits)
+// With it goes the number of the block's entries that have digits at all.
+__device__ __forceinline__ int block_word(u64 mx, int count) {
+    const int ex = (int)(mx >> 52);
+    return ((ex == 0 ? EXP_ZERO : ex - 1023 + 2) << 10) | count;
 }
 
 // The biased digits of v 2^-e as one integer: F = round(|v| 2^(56 - e)) < 2^55,
@@ -261,8 +280,11 @@ struct Side {
     unsigned char* img;
     int* large;  // a guarded call: each row's entries of at least 2^(e - 10)
     int* worst;  // and the most that a row falls short of K (split_rows_kernel; spread_kernel)
+    int* eb;     // K > ONE_EXP_K: the words of a row's blocks (block_word), a block after the other
+    long ebs;    // rows of eb
+    // the exponent for the digits of row i at index k, e the row's
+    __device__ __forceinline__ int block(int e, long k, long i) const { return e == EXP_LOST ? e : block_exp(eb[k / BLK_K * ebs + i]); }
 };
-constexpr u64 F_LARGE = (1ull << 46) + 0x1020408102040ull;  // biased56 of 2^(e - 10)
 __device__ __forceinline__ void side_sizes(const Prod& p, const Side& o, long& i0, long& rows, long& rpad, long& ld) {
     i0 = o.isB ? 0 : p.i0;
     rows = o.isB ? p.N : p.Mc;
@@ -328,33 +350,45 @@ __global__ void __launch_bounds__(256) split_rows_kernel(Prod p, Side o, int* fl
     }
 }
 
-// Longer rows in two passes: their maxima, then the digits of a chunk.
-constexpr int FUSED_K = 1024;
+// Longer rows in two passes: the maxima of their blocks, then the digits of a chunk.
 __global__ void __launch_bounds__(256) row_max_kernel(Prod p, Side o) {
     p.Mc = p.M;
-    if (!resolve(p) || (p.desc && p.K <= FUSED_K)) return;
+    if (!resolve(p) || p.K <= ONE_EXP_K) return;
     const long rows = o.isB ? p.N : p.M, ld = o.isB ? p.ldb : p.lda;
     const int lane = threadIdx.x & 31;
     const long nw = (long)gridDim.x * 8;
     for (long r = (long)blockIdx.x * 8 + (threadIdx.x >> 5); r < rows; r += nw) {
         const double* row = o.p + r * ld;
-        u64 m0 = 0, m1 = 0, m2 = 0, m3 = 0;
-        long k = lane;
-        for (; k + 96 < p.K; k += 128) {
-            m0 = umax(m0, mag(row[k]));
-            m1 = umax(m1, mag(row[k + 32]));
-            m2 = umax(m2, mag(row[k + 64]));
-            m3 = umax(m3, mag(row[k + 96]));
-        }
-        for (; k < p.K; k += 32) m0 = umax(m0, mag(row[k]));
-        m0 = umax(umax(m0, m1), umax(m2, m3));
+        u64 top = 0;
+        for (long kb = 0; kb * BLK_K < p.K; ++kb) {
+            const long k1 = min(p.K, (kb + 1) * BLK_K);
+            u64 m0 = 0, m1 = 0, m2 = 0, m3 = 0;
+            int c = 0;
+            auto see = [&](u64& m, long k) {
+                const u64 v = mag(row[k]);
+                m = umax(m, v);
+                c += (v >> 52) != 0;
+            };
+            long k = kb * BLK_K + lane;
+            for (; k + 96 < k1; k += 128) {
+                see(m0, k);
+                see(m1, k + 32);
+                see(m2, k + 64);
+                see(m3, k + 96);
+            }
+            for (; k < k1; k += 32) see(m0, k);
+            m0 = umax(umax(m0, m1), umax(m2, m3));
+            c = __reduce_add_sync(0xffffffffu, c);
 #pragma unroll
-        for (int q = 16; q > 0; q >>= 1) m0 = umax(m0, __shfl_xor_sync(0xffffffffu, m0, q));
-        if (lane == 0) o.mx[r] = m0;
+            for (int q = 16; q > 0; q >>= 1) m0 = umax(m0, __shfl_xor_sync(0xffffffffu, m0, q));
+            if (lane == 0) o.eb[kb * o.ebs + r] = block_word(m0, c);
+            top = umax(top, m0);
+        }
+        if (lane == 0) o.mx[r] = top;
     }
 }
 __global__ void __launch_bounds__(256) split_rows_long_kernel(Prod p, Side o, int* flag) {
-    if (!resolve(p) || (p.desc && p.K <= FUSED_K)) return;
+    if (!resolve(p) || p.K <= ONE_EXP_K) return;
     long i0, rows, rpad, ld;
     side_sizes(p, o, i0, rows, rpad, ld);
     const long Kc = p.Kc < p.K - p.k0 ? p.Kc : p.K - p.k0;
@@ -368,10 +402,11 @@ __global__ void __launch_bounds__(256) split_rows_long_kernel(Prod p, Side o, in
         const long r = q / nst;
         const long k = (long)st * T_K + 2 * kw;
         double v0 = 0.0, v1 = 0.0;
-        int e = 0;
+        int e = 0, eb = 0;
         if (r < rows) {
             e = split_exp(o.mx[i0 + r], flag);
             if (k == 0) o.e[i0 + r] = e;
+            eb = o.block(e, p.k0 + k, i0 + r);
             if (k < Kc) v0 = A[r * ld + k];
             if (k + 1 < Kc) v1 = A[r * ld + k + 1];
         }
@@ -383,7 +418,7 @@ __global__ void __launch_bounds__(256) split_rows_long_kernel(Prod p, Side o, in
             if (kw == 0 && r < rows) atomicAdd(o.large + i0 + r, __popc(b0 & half) + __popc(b1 & half));
         }
         unsigned w[S8];
-        digits8x2(v0, v1, e, e, w);
+        digits8x2(v0, v1, eb, eb, w);
         unsigned char* d = tile_at(o.img, r >> 6, nst, st, 0) + swz((int)(r & 63), 2 * kw);
 #pragma unroll
         for (int s = 0; s < S8; ++s) *reinterpret_cast<unsigned*>(d + s * DIG_BYTES) = w[s];
@@ -400,31 +435,49 @@ __global__ void __launch_bounds__(256) strided_max_kernel(Prod p, Side o) {
     p.Mc = p.M;
     if (!resolve(p)) return;
     const long n = o.isB ? p.N : p.M, ld = o.isB ? p.ldb : p.lda;
-    const long per = (p.K + gridDim.y - 1) / gridDim.y;
-    const long k0 = blockIdx.y * per, k1 = min(p.K, k0 + per);
+    // a block of indices after the other, or one range a CTA
+    const bool blocked = p.K > ONE_EXP_K;
+    const long per = blocked ? BLK_K : (p.K + gridDim.y - 1) / gridDim.y;
     __shared__ u64 part[8][32];
+    __shared__ int count[8][32];
     for (long jb = blockIdx.x * 32L; jb < n; jb += gridDim.x * 32L) {
         const long j = jb + (threadIdx.x & 31);
-        u64 m0 = 0, m1 = 0, m2 = 0, m3 = 0;
-        if (j < n) {
-            long k = k0 + (threadIdx.x >> 5);
-            for (; k + 24 < k1; k += 32) {
-                m0 = umax(m0, mag(o.p[k * ld + j]));
-                m1 = umax(m1, mag(o.p[(k + 8) * ld + j]));
-                m2 = umax(m2, mag(o.p[(k + 16) * ld + j]));
-                m3 = umax(m3, mag(o.p[(k + 24) * ld + j]));
+        u64 top = 0;
+        for (long kb = blockIdx.y; kb * per < p.K; kb += gridDim.y) {
+            const long k1 = min(p.K, (kb + 1) * per);
+            u64 m0 = 0, m1 = 0, m2 = 0, m3 = 0;
+            int c = 0;
+            auto see = [&](u64& m, long k) {
+                const u64 v = mag(o.p[k * ld + j]);
+                m = umax(m, v);
+                c += (v >> 52) != 0;
+            };
+            if (j < n) {
+                long k = kb * per + (threadIdx.x >> 5);
+                for (; k + 24 < k1; k += 32) {
+                    see(m0, k);
+                    see(m1, k + 8);
+                    see(m2, k + 16);
+                    see(m3, k + 24);
+                }
+                for (; k < k1; k += 8) see(m0, k);
             }
-            for (; k < k1; k += 8) m0 = umax(m0, mag(o.p[k * ld + j]));
-        }
-        __syncthreads();
-        part[threadIdx.x >> 5][threadIdx.x & 31] = umax(umax(m0, m1), umax(m2, m3));
-        __syncthreads();
-        if (threadIdx.x < 32 && j < n) {
-            u64 m = part[0][threadIdx.x];
+            __syncthreads();
+            part[threadIdx.x >> 5][threadIdx.x & 31] = umax(umax(m0, m1), umax(m2, m3));
+            count[threadIdx.x >> 5][threadIdx.x & 31] = c;
+            __syncthreads();
+            if (threadIdx.x < 32 && j < n) {
+                u64 m = part[0][threadIdx.x];
 #pragma unroll
-            for (int w = 1; w < 8; ++w) m = umax(m, part[w][threadIdx.x]);
-            if (m) atomicMax(o.mx + j, m);
+                for (int w = 1; w < 8; ++w) {
+                    m = umax(m, part[w][threadIdx.x]);
+                    c += count[w][threadIdx.x];
+                }
+                if (blocked) o.eb[kb * o.ebs + j] = block_word(m, c);
+                top = umax(top, m);
+            }
         }
+        if (threadIdx.x < 32 && j < n && top) atomicMax(o.mx + j, top);
     }
 }
 template <bool GUARD>
@@ -436,6 +489,7 @@ __global__ void __launch_bounds__(256, 4) split_strided_kernel(Prod p, Side o, i
     const long Kc = p.Kc < p.K - p.k0 ? p.Kc : p.K - p.k0;
     const int nst = stages(Kc);
     const double* A = o.p + i0 + p.k0 * ld;
+    const bool blocked = p.K > ONE_EXP_K;
     for (long jb = blockIdx.x * 32L; jb < rpad; jb += gridDim.x * 32L) {
         const long j = jb + (threadIdx.x & 31);
         int e = 0;
@@ -453,19 +507,20 @@ __global__ void __launch_bounds__(256, 4) split_strided_kernel(Prod p, Side o, i
             const long k0 = g * 8;
             u64 F[8];
             unsigned sg[4];
+            const int eb = blocked && j < rows ? o.block(e, p.k0 + k0, i0 + j) : e;
 #pragma unroll
             for (int r = 0; r < 8; ++r) F[r] = j < rows && k0 + r < Kc ? (u64)__double_as_longlong(__ldcs(A + (k0 + r) * ld + j)) : 0ull;
+            if (GUARD) {
+                int c = 0;
+#pragma unroll
+                for (int r = 0; r < 8; ++r) c += (int)((F[r] >> 52) & 0x7FF) >= e - 10 + 1023;
+                atomicAdd(&s_large[threadIdx.x & 31], c);
+            }
 #pragma unroll
             for (int r = 0; r < 8; ++r) {
                 const unsigned sign = ((unsigned)(F[r] >> 48) & 0x8000u) << (16 * (r & 1));
                 sg[r >> 1] = r & 1 ? sg[r >> 1] | sign : sign;
-                F[r] = biased56(__longlong_as_double((long long)F[r]), e);
-            }
-            if (GUARD) {
-                int c = 0;
-#pragma unroll
-                for (int r = 0; r < 8; ++r) c += F[r] >= F_LARGE;
-                atomicAdd(&s_large[threadIdx.x & 31], c);
+                F[r] = biased56(__longlong_as_double((long long)F[r]), eb);
             }
             unsigned char* d = tile_at(o.img, j >> 6, nst, (int)(g >> 2), 0) + swz((int)(j & 63), (int)(g & 3) * 8);
 #pragma unroll
@@ -493,9 +548,29 @@ __global__ void __launch_bounds__(256) spread_kernel(long rows, int K, const int
 
 // ------------------------------------------------------------------ product
 
-// (hi 2^28 + lo) 2^(e - 63) rounded to nearest.
-__device__ __forceinline__ double digits_value(long long hi, long long lo, int e) {
-    __int128 t = ((__int128)hi << 28) + lo;
+// Sums: t stands for t 2^(e - 63 - ROOM), e the sum of the rows' exponents.  |t| is
+// below 2^(61 + ROOM) K, so 96 bits hold it; a thread keeps 96, planes 128.
+constexpr int ROOM = 8;
+__device__ __forceinline__ __int128 whole_sum(long long hi, long long lo) { return (((__int128)hi << 28) + lo) << ROOM; }
+struct Sum96 {
+    long long hi;
+    unsigned lo;
+    // + (h 2^28 + l) 2^(ROOM - r), r >= 0, rounded down
+    __device__ __forceinline__ void add(long long h, long long l, int r) {
+        const long long th = (l >> (32 - ROOM)) + (h << (28 + ROOM - 32));
+        const unsigned tl = (unsigned)l << ROOM;
+        const unsigned below = r < 32 ? __funnelshift_r(tl, (unsigned)th, r) : (unsigned)(th >> min(r - 32, 63));
+        const unsigned s = lo + below;
+        hi += (th >> min(r, 63)) + (s < below ? 1 : 0);
+        lo = s;
+    }
+    __device__ __forceinline__ __int128 value() const { return ((__int128)hi << 32) + lo; }
+};
+__device__ __forceinline__ __int128 join(longlong2 v) { return ((__int128)v.y << 64) + (u64)v.x; }
+__device__ __forceinline__ longlong2 parts(__int128 t) { return make_longlong2((long long)(u64)t, (long long)(t >> 64)); }
+
+// t 2^(e - 63 - ROOM) rounded to nearest.
+__device__ __forceinline__ double digits_value(__int128 t, int e) {
     const bool neg = t < 0;
     unsigned __int128 u = neg ? (unsigned __int128)(-t) : (unsigned __int128)t;
     u64 uh = (u64)(u >> 64), ul = (u64)u;
@@ -505,7 +580,7 @@ __device__ __forceinline__ double digits_value(long long hi, long long lo, int e
     u <<= z;
     u64 m = (u64)(u >> 64);
     const u64 rest = (u64)u;
-    int ex = e - 63 + 127 - z;  // exponent of the leading bit
+    int ex = e - 63 - ROOM + 127 - z;  // exponent of the leading bit
     const u64 low = (m & 0x7FF) | (rest ? 1ull : 0ull);
     m >>= 11;  // 53 bits
     if (low > 0x400 || (low == 0x400 && (m & 1))) {
@@ -558,11 +633,14 @@ __device__ __forceinline__ void tile_of(long t, int nb, bool tri, long& mb, int&
 // loads (tensor cores at 45%); unrolled, with descriptors that are constants from
 // the stage's, about 2900.  196,608 x 512 times 512 x 512: 4.1 -> 2.6 ms; commits
 // per stage 8, 4, 3, 2, 1 with the rolled loop: 3.84, 4.02, 3.94, 3.59, 3.55 ms.
+template <bool BLOCKED>
 __global__ void __launch_bounds__(THREADS8, 1)
-tc8_kernel(Prod p, const unsigned char* __restrict__ At, const int* __restrict__ eA,
-           const unsigned char* __restrict__ Bt, const int* __restrict__ eB, double alpha, double* __restrict__ C,
+tc8_kernel(Prod p, const unsigned char* __restrict__ At, const int* __restrict__ eA, const int* __restrict__ ebA,
+           long ebsA, const unsigned char* __restrict__ Bt, const int* __restrict__ eB, const int* __restrict__ ebB,
+           long ebsB, double alpha, double* __restrict__ C,
            longlong2* __restrict__ planes, int spc, Report rep, long long limit) {
-    if (!resolve(p)) return;  // every thread, before any barrier
+    // every thread, before any barrier; a captured step launches both forms
+    if (!resolve(p) || (p.K > ONE_EXP_K) != BLOCKED) return;
     const long M = p.Mc;
     const int N = (int)p.N;
     const int nst = stages(p.Kc < p.K - p.k0 ? p.Kc : p.K - p.k0);
@@ -570,7 +648,9 @@ tc8_kernel(Prod p, const unsigned char* __restrict__ At, const int* __restrict__
     // a captured step decides the split here (from the first chunk, as the
     // reduction does)
     if (p.desc)
-        spc = planes ? split_stages_warp(p.M, N, tiles_of(p.Mc0, N, p.gram), stages(p.Kc < p.K ? p.Kc : p.K)) : nst;
+        spc = planes ? split_stages_warp(p.M, N, tiles_of(p.Mc0, N, p.gram), stages(p.Kc < p.K ? p.Kc : p.K),
+                                         split_unit(p.K))
+                     : nst;
     const bool accumulate = p.k0 > 0;
     const bool whole = planes == nullptr || (p.desc && !p.gram && p.K <= p.Kc && spc >= nst);
     extern __shared__ unsigned char raw[];
@@ -651,7 +731,8 @@ tc8_kernel(Prod p, const unsigned char* __restrict__ At, const int* __restrict__
                 for (int it = st0; it < st1; ++it, ++g) {
                     const int st = (int)(g % T_STAGES);
                     const unsigned ph = (unsigned)(g / T_STAGES) & 1u;
-                    const bool first = ((it - st0) % T_BLK) == 0;
+                    const int at = BLOCKED ? it : it - st0;
+                    const bool first = it == st0 || at % T_BLK == 0;
                     if (first && gb > 0) {
                         if (!bar_wait(smem_addr(&bars[19]), (unsigned)(gb - 1) & 1u, rep, flags, limit)) {
                             stop = true;
@@ -685,7 +766,7 @@ tc8_kernel(Prod p, const unsigned char* __restrict__ At, const int* __restrict__
                         for (int q = 0; q < GROUPS; ++q)
                             if (s == group_start(q + 1) - 1) mma_commit(smem_addr(&bars[2 + 8 * st + q]));
                     }
-                    if (((it - st0) % T_BLK) == T_BLK - 1 || it == st1 - 1) {
+                    if (at % T_BLK == T_BLK - 1 || it == st1 - 1) {
                         mma_commit(smem_addr(&bars[18]));
                         ++gb;
                     }
@@ -704,47 +785,99 @@ tc8_kernel(Prod p, const unsigned char* __restrict__ At, const int* __restrict__
             int kb;
             tile_of(item % ntiles, nb, p.gram != 0, mb, kb);
             const int sp = (int)(item / ntiles);
-            const int blocks = (min(nst, (sp + 1) * spc) - sp * spc + T_BLK - 1) / T_BLK;
-            long long hi[DCOLS], lo[DCOLS];
+            const int st0 = sp * spc, st1 = min(nst, st0 + spc);
+            const int b0 = BLOCKED ? st0 / T_BLK : 0, b1 = BLOCKED ? (st1 - 1) / T_BLK + 1 : (st1 - st0 + T_BLK - 1) / T_BLK;
+            const long i = mb * T_M + 32 * q + lane;
+            const int col0 = kb * T_N + c0;
+            long long hi[BLOCKED ? 1 : DCOLS], lo[BLOCKED ? 1 : DCOLS];  // sums of levels 0-3 and 4-7
+            Sum96 all[BLOCKED ? DCOLS : 1];
 #pragma unroll
-            for (int c = 0; c < DCOLS; ++c) hi[c] = lo[c] = 0;
-            for (int b = 0; b < blocks; ++b, ++gb) {
+            for (int c = 0; c < DCOLS; ++c) {
+                if (BLOCKED)
+                    all[BLOCKED ? c : 0] = Sum96{0, 0u};
+                else
+                    hi[BLOCKED ? 0 : c] = lo[BLOCKED ? 0 : c] = 0;
+            }
+            for (int b = b0; b < b1; ++b, ++gb) {
+                int below = 0;              // the block's exponents below the rows': of the row,
+                unsigned bcol[DCOLS / 4];  // of the columns, a byte each
+                if (BLOCKED) {
+                    const long blk = p.k0 / BLK_K + b;
+                    if (i < M) below = min(max(eA[p.i0 + i] - block_exp(ebA[blk * ebsA + p.i0 + i]), 0), 127);
+#pragma unroll
+                    for (int c = 0; c < DCOLS; ++c) {
+                        const int v = col0 + c < N ? min(max(eB[col0 + c] - block_exp(ebB[blk * ebsB + col0 + c]), 0), 127) : 0;
+                        bcol[c / 4] = c % 4 ? bcol[c / 4] | (unsigned)v << (8 * (c % 4)) : (unsigned)v;
+                    }
+                }
                 if (!__all_sync(0xffffffffu, bar_wait(smem_addr(&bars[18]), (unsigned)gb & 1u, rep, flags, limit))) {
                     stop = true;
                     break;
                 }
                 fence_after();
                 const unsigned ta = tmem + ((unsigned)(32 * q) << 16) + (unsigned)c0;
+                if (!BLOCKED) {
 #pragma unroll
-                for (int w = 0; w < S8; ++w) {
-                    unsigned r[16];
-                    tmem_ld16(ta + (unsigned)(w * T_N), r);
-                    tmem_wait_ld();
-                    const int scale = 1 << (7 * (3 - (w & 3)));
+                    for (int w = 0; w < S8; ++w) {
+                        unsigned r[16];
+                        tmem_ld16(ta + (unsigned)(w * T_N), r);
+                        tmem_wait_ld();
+                        const int scale = 1 << (7 * (3 - (w & 3)));
 #pragma unroll
-                    for (int c = 0; c < DCOLS; ++c) {
-                        const long long v = (long long)__float2int_rn(__uint_as_float(r[c])) * scale;
-                        if (w < 4)
-                            hi[c] += v;
-                        else
-                            lo[c] += v;
+                        for (int c = 0; c < DCOLS; ++c) {
+                            const long long v = (long long)__float2int_rn(__uint_as_float(r[c])) * scale;
+                            if (w < 4)
+                                hi[BLOCKED ? 0 : c] += v;
+                            else
+                                lo[BLOCKED ? 0 : c] += v;
+                        }
+                    }
+                } else {  // a few columns at a time: every block has its shifts
+#pragma unroll
+                    for (int c = 0; c < DCOLS; c += 4) {
+                        unsigned r[S8][4];
+#pragma unroll
+                        for (int w = 0; w < S8; ++w) tmem_ld4(ta + (unsigned)(w * T_N + c), r[w]);
+                        tmem_wait_ld();
+                        if (c + 4 == DCOLS) {  // the accumulators are read: the next block may start
+                            fence_before();
+                            __syncwarp();
+                            if (lane == 0) bar_arrive(smem_addr(&bars[19]));
+                        }
+#pragma unroll
+                        for (int u = 0; u < 4; ++u) {
+                            long long h = 0, l = 0;
+#pragma unroll
+                            for (int w = 0; w < S8; ++w) {
+                                const long long v =
+                                    (long long)__float2int_rn(__uint_as_float(r[w][u])) * (1 << (7 * (3 - (w & 3))));
+                                if (w < 4)
+                                    h += v;
+                                else
+                                    l += v;
+                            }
+                            all[BLOCKED ? c + u : 0].add(h, l, below + (int)((bcol[c / 4] >> (8 * u)) & 0xFFu));
+                        }
                     }
                 }
-                fence_before();
-                __syncwarp();
-                if (lane == 0) bar_arrive(smem_addr(&bars[19]));
+                if (!BLOCKED) {
+                    fence_before();
+                    __syncwarp();
+                    if (lane == 0) bar_arrive(smem_addr(&bars[19]));
+                }
             }
             if (stop) break;
-            const long i = mb * T_M + 32 * q + lane;
+            auto sum = [&](int c) {
+                return BLOCKED ? all[BLOCKED ? c : 0].value() : whole_sum(hi[BLOCKED ? 0 : c], lo[BLOCKED ? 0 : c]);
+            };
             if (i < M && !flags[0]) {
-                const int col0 = kb * T_N + c0;
                 if (whole) {
                     const int ea = eA[p.i0 + i];
                     double* out = C + (p.i0 + i) * p.ldc;
 #pragma unroll
                     for (int c = 0; c < DCOLS; ++c)
                         if (col0 + c < N) {
-                            const double v = digits_value(hi[c], lo[c], ea + eB[col0 + c]);
+                            const double v = digits_value(sum(c), ea + eB[col0 + c]);
                             out[col0 + c] = alpha == 1.0 ? v : alpha * v;
                         }
                 } else {
@@ -752,13 +885,8 @@ tc8_kernel(Prod p, const unsigned char* __restrict__ At, const int* __restrict__
 #pragma unroll
                     for (int c = 0; c < DCOLS; ++c)
                         if (col0 + c < N) {
-                            longlong2 v = make_longlong2(hi[c], lo[c]);
-                            if (accumulate) {
-                                const longlong2 u = out[col0 + c];
-                                v.x += u.x;
-                                v.y += u.y;
-                            }
-                            out[col0 + c] = v;
+                            const __int128 v = sum(c);
+                            out[col0 + c] = parts(accumulate ? v + join(out[col0 + c]) : v);
                         }
                 }
             }
@@ -784,7 +912,7 @@ tc8_reduce_kernel(Prod p, const longlong2* __restrict__ planes, const int* __res
     if (!resolve(p) || !planes) return;  // without planes tc8_kernel has written C
     const int nst = stages(p.Kc < p.K ? p.Kc : p.K);
     if (p.desc) {
-        spc = split_stages_warp(p.M, p.N, tiles_of(p.Mc0, p.N, p.gram), nst);
+        spc = split_stages_warp(p.M, p.N, tiles_of(p.Mc0, p.N, p.gram), nst, split_unit(p.K));
         if (!p.gram && p.K <= p.Kc && spc >= nst) return;  // written whole
     }
     const int ksp = (nst + spc - 1) / spc;
@@ -792,13 +920,9 @@ tc8_reduce_kernel(Prod p, const longlong2* __restrict__ planes, const int* __res
     for (long t = blockIdx.x * (long)blockDim.x + threadIdx.x; t < total; t += (long)gridDim.x * blockDim.x) {
         const long i = t / p.N, j = t % p.N;
         const long src = p.gram && j < i ? j * p.N + i : t;
-        longlong2 v = planes[src];
-        for (int z = 1; z < ksp; ++z) {
-            const longlong2 u = planes[z * total + src];
-            v.x += u.x;
-            v.y += u.y;
-        }
-        const double x = digits_value(v.x, v.y, eA[i] + eB[j]);
+        __int128 v = join(planes[src]);
+        for (int z = 1; z < ksp; ++z) v += join(planes[z * total + src]);
+        const double x = digits_value(v, eA[i] + eB[j]);
         C[i * p.ldc + j] = alpha == 1.0 ? x : alpha * x;
     }
 }
@@ -816,28 +940,35 @@ tt_status run(cudaStream_t s, bool ta, bool tb, long M, long N, long K, double a
     unsigned char* base = reinterpret_cast<unsigned char*>(((uintptr_t)scratch.p + 1023) & ~(uintptr_t)1023);
     int* flag = reinterpret_cast<int*>(base);
     u64* mx = reinterpret_cast<u64*>(base + 256);
-    int* ex = reinterpret_cast<int*>(mx + M + N);
-    int* large = guard ? ex + M + N : nullptr;
+    const long nrows = gram ? M : M + N;
+    int* ex = reinterpret_cast<int*>(mx + nrows);
+    int* large = guard ? ex + nrows : nullptr;
     int* worst = guard ? flag + LOST_WORST : nullptr;
-    Side a{A, 0, ta ? 1 : 0, mx, ex, base + q.head + q.imgB, large, worst};
-    Side b{B, 1, tb ? 0 : 1, mx + M, ex + M, base + q.head, guard ? large + M : nullptr, guard ? worst + 1 : nullptr};
-    if (gram) a.img = base + q.head;
+    int* eb = ex + 2 * nrows;  // behind the counts
+    Side a{A, 0, ta ? 1 : 0, mx, ex, base + q.head + q.imgB, large, worst, eb, M};
+    Side b{B, 1, tb ? 0 : 1, mx + M, ex + M, base + q.head, guard ? large + M : nullptr, guard ? worst + 1 : nullptr,
+           eb + (K + BLK_K - 1) / BLK_K * M, N};
+    if (gram) {
+        a.img = base + q.head;
+        b = a;
+    }
     longlong2* planes = q.part ? reinterpret_cast<longlong2*>(base + q.head + q.imgA + q.imgB) : nullptr;
-    const int* eB = gram ? ex : b.e;
     Prod p{M, N, K, lda, ldb, ldc, desc, 0, q.Kc, 0, q.Mc, gram ? 1 : 0, q.Mc};
     int dev = 0, sms = 152;
     TT_CUDA_TRY(cudaGetDevice(&dev));
     TT_CUDA_TRY(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
-    TT_TRY(ensure_max_dynamic_smem((const void*)tc8_kernel));
+    TT_TRY(ensure_max_dynamic_smem((const void*)tc8_kernel<false>));
+    TT_TRY(ensure_max_dynamic_smem((const void*)tc8_kernel<true>));
     // the flag and, where atomics find them, the maxima and counts start at zero
-    TT_CUDA_TRY(cudaMemsetAsync(flag, 0, 256 + (a.strided || b.strided ? 8 * (size_t)(M + N) : 0), s));
-    if (guard) TT_CUDA_TRY(cudaMemsetAsync(large, 0, 4 * (size_t)(M + N), s));
-    const bool fusable = K <= FUSED_K;  // a captured step launches both forms when K may be longer
+    TT_CUDA_TRY(cudaMemsetAsync(flag, 0, 256 + (a.strided || b.strided ? 8 * (size_t)nrows : 0), s));
+    if (guard) TT_CUDA_TRY(cudaMemsetAsync(large, 0, 4 * (size_t)nrows, s));
+    const bool fusable = K <= ONE_EXP_K;  // a captured step launches both forms when K may be longer
     auto maxima = [&](const Side& o) {
         const long rows = o.isB ? N : M;
         if (o.strided) {
             note_launch();
-            strided_max_kernel<<<dim3(blocks_for((rows + 31) / 32, 4096), blocks_for(K / 256, 512)), 256, 0, s>>>(p, o);
+            strided_max_kernel<<<dim3(blocks_for((rows + 31) / 32, 4096), blocks_for(K / (fusable ? 256 : BLK_K), 512)), 256, 0, s>>>(
+                p, o);
         } else if (!fusable) {
             note_launch();
             row_max_kernel<<<blocks_for((rows + 7) / 8, 152L * 64), 256, 0, s>>>(p, o);
@@ -861,7 +992,7 @@ tt_status run(cudaStream_t s, bool ta, bool tb, long M, long N, long K, double a
             if (!desc) return;
         }
         const unsigned grid = blocks_for((rpad + 7) / 8, 152L * 64);
-        const int need = std::min(nst, FUSED_K / T_K);
+        const int need = std::min(nst, ONE_EXP_K / T_K);
         // by value one instance, the smallest that holds the row; a captured
         // product launches each that a size up to its capacity may need
         if (desc ? true : need <= 4) {
@@ -882,7 +1013,7 @@ tt_status run(cudaStream_t s, bool ta, bool tb, long M, long N, long K, double a
         }
     };
     const int nst0 = stages(q.Kc);
-    const int spc = split_stages(M, N, tiles_of(q.Mc, N, gram), nst0);
+    const int spc = split_stages(M, N, tiles_of(q.Mc, N, gram), nst0, split_unit(K));
     const bool direct = !desc && !gram && q.Kc >= K && spc >= nst0;
     maxima(a);
     if (!gram) maxima(b);
@@ -896,9 +1027,14 @@ tt_status run(cudaStream_t s, bool ta, bool tb, long M, long N, long K, double a
             p.Mc = q.Mc;
             split(a);
             const long items = tiles_of(std::min(q.Mc, M - p.i0), N, gram) * ((nst0 + spc - 1) / spc);
-            note_launch();
-            tc8_kernel<<<desc ? sms : (int)std::min<long>(items, sms), THREADS8, SMEM8, s>>>(
-                p, a.img, a.e, b.img, eB, alpha, C, direct ? nullptr : planes, spc, Report{status_dev, flag}, limit);
+            auto product = [&](auto kernel) {
+                note_launch();
+                kernel<<<desc ? sms : (int)std::min<long>(items, sms), THREADS8, SMEM8, s>>>(
+                    p, a.img, a.e, a.eb, a.ebs, b.img, b.e, b.eb, b.ebs, alpha, C, direct ? nullptr : planes, spc,
+                    Report{status_dev, flag}, limit);
+            };
+            if (fusable || (desc && p.k0 == 0)) product(tc8_kernel<false>);
+            if (!fusable) product(tc8_kernel<true>);
             TT_CUDA_TRY(cudaGetLastError());
         }
     }
@@ -906,7 +1042,7 @@ tt_status run(cudaStream_t s, bool ta, bool tb, long M, long N, long K, double a
     p.Mc = q.Mc;
     if (!direct) {
         note_launch();
-        tc8_reduce_kernel<<<blocks_for((M * N + 255) / 256, 152L * 16), 256, 0, s>>>(p, planes, a.e, eB, spc, alpha, C);
+        tc8_reduce_kernel<<<blocks_for((M * N + 255) / 256, 152L * 16), 256, 0, s>>>(p, planes, a.e, b.e, spc, alpha, C);
     }
     if (guard) {
         auto spread = [&](const Side& o) {
@@ -919,7 +1055,7 @@ tt_status run(cudaStream_t s, bool ta, bool tb, long M, long N, long K, double a
         if (!gram) spread(b);
     }
     TT_CUDA_TRY(cudaGetLastError());
-    *lost = Lost{flag, ex, eB, guard ? 1 : 0, gram ? 1 : 0, reinterpret_cast<double*>(base + q.head)};
+    *lost = Lost{flag, a.e, b.e, guard ? 1 : 0, gram ? 1 : 0, reinterpret_cast<double*>(base + q.head), mx, a.eb, a.ebs};
     return TT_OK;
 }
 
@@ -933,7 +1069,7 @@ size_t tc8_reserve_doubles(long M, long N, long K, bool gram) {
     return (reserve_bytes(M, N, K, gram) + 1024 + 7) / 8;
 }
 
-size_t tc8_head_doubles(long M, long N) { return (make_plan(M, N, T_K, false, false).head + 1024 + 7) / 8; }
+size_t tc8_head_doubles(long M, long N, long K, bool gram) { return (head_bytes(M, N, K, gram) + 1024 + 7) / 8; }
 
 tt_status tc8_gemm(cudaStream_t s, bool ta, bool tb, long M, long N, long K, double alpha, const double* A, long lda,
                    const double* B, long ldb, double* C, long ldc, DevBuf& scratch, int* status_dev, bool guard,

@@ -31,6 +31,9 @@ constexpr int S8 = 8;
 constexpr int T_M = 128, T_N = 64, T_K = 32;  // output tile; contraction indices of a stage
 constexpr int T_BLK = 16;                     // stages of an exact block (512 indices)
 constexpr int RB = 64;                        // rows of an image block
+// A contraction of up to ONE_EXP_K indices has one power of two a row, a longer
+// one an own for each BLK_K of them.
+constexpr int BLK_K = T_K * T_BLK, ONE_EXP_K = 1024;
 // Digit images of one pass over an operand; a longer operand goes in chunks.  A
 // chunk costs its launches and a last wave: with images of 2^26, 2^27, 2^28, 2^29
 // and 2^30 bytes the Gram of 500,000 x 449 took 10.3, 9.1, 8.5, 8.4 and 8.6 ms and
@@ -53,25 +56,31 @@ TTSN_HD long tiles_of(long M, long N, int gram) {
 // about its waves of one CTA per SM times the stages of a split and one more
 // for an item's end; a plane costs its write and its read in the reduction.
 // A split has at least four stages, and the planes at most PLANE_ELEMS entries.
+// A contraction that may go in chunks is split between exact blocks, so that the
+// blocks' sums, and with them the result's bits, do not depend on the chunks
+// (unit: stages that stay together).
 constexpr long PLANE_ELEMS = 1L << 23;
 constexpr int MAX_SPLITS = 64;
-TTSN_HD int split_limit(long M, long N, int nst) {
+constexpr long CHUNK_MIN = 16384;  // no shorter contraction goes in chunks
+TTSN_HD int split_unit(long K) { return K > CHUNK_MIN ? T_BLK : 1; }
+TTSN_HD int split_limit(long M, long N, int nst, int unit) {
     long k = PLANE_ELEMS / (M * N);
-    k = least(k, least(nst / 4, MAX_SPLITS));
+    k = least(k, least(nst / most(4, unit), MAX_SPLITS));
     return k < 1 ? 1 : (int)k;
 }
-TTSN_HD unsigned split_cost(int k, long ntiles, int nst) {
-    const int spc = (nst + k - 1) / k, kk = (nst + spc - 1) / spc;
+TTSN_HD int stages_of_split(int k, int nst, int unit) { return (int)up((nst + k - 1) / k, unit); }
+TTSN_HD unsigned split_cost(int k, long ntiles, int nst, int unit) {
+    const int spc = stages_of_split(k, nst, unit), kk = (nst + spc - 1) / spc;
     const long waves = (ntiles * kk + 151) / 152;
     const long c = waves * (spc + 1) * 64 + kk;
     return c > 0x03ffffffL ? 0x03ffffffu : (unsigned)c;
 }
-TTSN_HD int split_stages(long M, long N, long ntiles, int nst) {
-    const int lim = split_limit(M, N, nst);
+TTSN_HD int split_stages(long M, long N, long ntiles, int nst, int unit) {
+    const int lim = split_limit(M, N, nst, unit);
     int best = 1;
     for (int k = 2; k <= lim; ++k)
-        if (split_cost(k, ntiles, nst) < split_cost(best, ntiles, nst)) best = k;
-    return (nst + best - 1) / best;
+        if (split_cost(k, ntiles, nst, unit) < split_cost(best, ntiles, nst, unit)) best = k;
+    return stages_of_split(best, nst, unit);
 }
 
 // Chunks and scratch of a product.  A captured product (captured) has these
@@ -83,13 +92,19 @@ struct Plan {
     size_t head, imgA, imgB, part;  // bytes: flags, maxima and exponents; images; planes (0: none)
     size_t bytes() const { return head + imgA + imgB + part; }
 };
+// Flags; per row its largest entry, exponent and count of large entries, and
+// the exponents of its blocks.
+inline size_t head_bytes(long M, long N, long K, bool gram) {
+    const long rows = gram ? M : M + N;
+    return (size_t)up(256 + 16 * rows + (K > ONE_EXP_K ? 4 * rows * ((K + BLK_K - 1) / BLK_K) : 0) + 64, 1024);
+}
 inline Plan make_plan(long M, long N, long K, bool gram, bool captured) {
     Plan p;
     const long Np = up(N, gram ? T_M : RB);
     // images of about IMG_LIMIT bytes each: a long contraction is cut along K
     // (for an operand of up to 1024 rows), a tall A along its rows
     const long wide = most(up(least(M, 1024L), T_M), Np);
-    const long kmax = most(16384L, IMG_LIMIT / (2 * S8 * wide) / (T_K * T_BLK) * (T_K * T_BLK));
+    const long kmax = most(CHUNK_MIN, IMG_LIMIT / (2 * S8 * wide) / (T_K * T_BLK) * (T_K * T_BLK));
     p.Kc = K <= kmax ? K : up((K + (K + kmax - 1) / kmax - 1) / ((K + kmax - 1) / kmax), T_K * T_BLK);
     const int nst = stages(p.Kc);
     p.Mc = gram ? M : least(M, most((long)T_M, IMG_LIMIT / (2L * S8 * nst * T_K) / T_M * T_M));
@@ -99,10 +114,10 @@ inline Plan make_plan(long M, long N, long K, bool gram, bool captured) {
         const long most_splits = least(nst / 4, MAX_SPLITS);
         if (most_splits > 1) elems = most(elems, least(M * N * most_splits, PLANE_ELEMS));
     } else {
-        const int spc = split_stages(M, N, tiles_of(p.Mc, N, gram), nst);
+        const int spc = split_stages(M, N, tiles_of(p.Mc, N, gram), nst, split_unit(K));
         if (spc < nst) elems = M * N * ((nst + spc - 1) / spc);
     }
-    p.head = (size_t)up(256 + 8 * (M + N) + 4 * (M + N) + 4 * (M + N) + 64, 1024);
+    p.head = head_bytes(M, N, K, gram);
     p.imgB = (size_t)(Np * nst * T_K * 2 * S8);
     p.imgA = gram ? 0 : (size_t)(up(p.Mc, T_M) * nst * T_K * 2 * S8);
     p.part = 16 * (size_t)elems;
@@ -114,12 +129,12 @@ inline Plan make_plan(long M, long N, long K, bool gram, bool captured) {
 // own plan bounds the others'.
 inline size_t reserve_bytes(long M, long N, long K, bool gram) {
     const long Np = up(N, gram ? T_M : RB), Kp = up(K, T_K), row = 2 * S8;
-    const long imgB = least(Np * Kp, most(IMG_LIMIT / row, 16384 * Np)) * row;
+    const long imgB = least(Np * Kp, most(IMG_LIMIT / row, CHUNK_MIN * Np)) * row;
     const long imgA = gram ? 0 : least(up(M, T_M) * Kp, IMG_LIMIT / row) * row;
     const long splits = least(stages(K) / 4, MAX_SPLITS);
-    long elems = gram || K > 16384 ? M * N : 0;
+    long elems = gram || K > CHUNK_MIN ? M * N : 0;
     if (splits > 1) elems = most(elems, least(M * N * splits, PLANE_ELEMS));
-    return (size_t)(up(256 + 16 * (M + N) + 64, 1024) + imgA + imgB + 16 * elems);
+    return head_bytes(M, N, K, gram) + (size_t)(imgA + imgB + 16 * elems);
 }
 
 }  // namespace digits

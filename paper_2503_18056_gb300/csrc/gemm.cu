@@ -339,6 +339,51 @@ prod_kernel(int M, int N, int K, double alpha, const double* __restrict__ A, lon
     }
 }
 
+// Behind a rounding's digit Gram G: a column is lost where the digits' error may
+// exceed that of the FP64 sums it stands for, relative to the column's own norm.
+// A digit Gram's entry (i, j) is off by at most sqrt(Q_i Q_j), Q_i = 9.1 2^-58
+// sum_blocks c_block 4^e_block (c: entries that are not zero), the FP64 pipe's by chunk
+// 2^-53 |a_i| |a_j| (chunk: rows of a split); a column stays where Q_i <= chunk 2^-53
+// |a_i|^2, above about 2,400 rows a split always.  So a column is recomputed (its row
+// and column of G, prod_kernel) only where few of its blocks' entries make up its
+// norm, and G keeps its relative accuracy under any scaling of the columns, which
+// the eigenvalues of W G W^T take over, whatever the rounding's tolerance.
+// A warp a column.
+__global__ void __launch_bounds__(256)
+gram_check_kernel(int n, int K, const double* __restrict__ G, long ldg, const int* __restrict__ desc, Lost lost) {
+    if (desc) {
+        n = desc[0];
+        K = desc[2];
+        ldg = desc[5];
+        if (!tc8_wanted(n, n, K)) return;
+    }
+    int chunk;
+    ordered_split(n, n, K, 1, &chunk);
+    const int lane = threadIdx.x & 31;
+    for (int i = blockIdx.x * 8 + (threadIdx.x >> 5); i < n; i += gridDim.x * 8) {
+        const int e = lost.a[i];
+        if (lost.mx[i] == 0 || e == EXP_LOST) continue;
+        // sum_blocks c_block 4^(e_block - e) in units of 2^-30 (at least one an entry): the
+        // same in any order
+        unsigned long long sum = 0;
+        if (K > digits::ONE_EXP_K) {
+            for (long b = lane; b * digits::BLK_K < K; b += 32) {
+                const int w = lost.eb[b * lost.ebs + i];
+                sum += (unsigned long long)block_count(w) << (30 - 2 * min(max(e - block_exp(w), 0), 15));
+            }
+#pragma unroll
+            for (int o = 16; o > 0; o >>= 1) sum += __shfl_xor_sync(0xffffffffu, sum, o);
+        } else {
+            sum = (unsigned long long)K << 30;
+        }
+        const double most = 0x1p-30 * (double)sum * (9.1 / 32.0) / chunk;
+        if (lane == 0 && !(most <= scalbn(G[(long)i * ldg + i], -2 * e))) {
+            lost.a[i] = EXP_LOST;
+            atomicOr(lost.flag + LOST_ROWS, 1);
+        }
+    }
+}
+
 // out[i][j] = in[i][j] * f(v[i]) with rows, cols, ldi, ldo = desc[0..3]
 __global__ void scale_rows_dyn_kernel(const int* __restrict__ desc, const double* in, const double* v, int mode,
                                       double* out) {
@@ -495,7 +540,7 @@ size_t split_scratch(long tiles, int ks) { return ks > 1 ? split_doubles(tiles, 
 size_t digits_doubles(long M, long N, long K, int tri, int ks) {
     const size_t part = split_scratch(prod_tiles(M, N, tri), ks);
     if (!tc8_wanted(M, N, K)) return part;
-    return std::max(tc8_scratch_doubles(M, N, K, tri != 0), tc8_head_doubles(M, N) + part);
+    return std::max(tc8_scratch_doubles(M, N, K, tri != 0), tc8_head_doubles(M, N, K, tri != 0) + part);
 }
 
 tt_status split_prod(cudaStream_t s, bool ta, bool tb, bool ordered, ProdArgs a) {
@@ -550,6 +595,12 @@ tt_status dgemm_sk(cudaStream_t s, bool ta, bool tb, int M, int N, int K, double
                                                 ctx.counters, 0, nullptr});
 }
 
+// Between the digit Gram and its recomputation.
+static void gram_check(cudaStream_t s, int n, int K, const double* G, long ldg, const int* desc, const Lost& lost) {
+    note_launch();
+    gram_check_kernel<<<std::max(1, std::min(n / 8, 152)), 256, 0, s>>>(n, K, G, ldg, desc, lost);
+}
+
 tt_status gram(cudaStream_t s, int m, int n, const double* A, long lda, double* G, long ldg, DevBuf& partials,
                const ProdCtx& ctx) {
     if (n <= 0) return TT_OK;
@@ -566,6 +617,7 @@ tt_status gram(cudaStream_t s, int m, int n, const double* A, long lda, double* 
         tt_status st = partials.ensure(digits_doubles(n, n, m, 1, ks), s);
         if (st >= 0) st = tc8_gram(s, m, n, A, lda, G, ldg, partials, ctx.status, false, &a.lost);
         if (st >= 0) {
+            gram_check(s, n, m, G, ldg, nullptr, a.lost);
             a.P = a.lost.free;
             return split_prod(s, true, false, true, a);
         }
@@ -673,6 +725,7 @@ tt_status dgemm_dyn(cudaStream_t s, bool ta, bool tb, const int* desc, int Mcap,
     Lost lost;
     if (ctx.digits && tc8_wanted(Mcap, Ncap, Kcap))
         TT_TRY(tc8_dyn(s, ta, tb, desc, Mcap, Ncap, Kcap, alpha, A, B, C, tcbuf, ctx.status, mode == 2, &lost));
+    if (lost.flag && tri) gram_check(s, Ncap, Kcap, C, 0, desc, lost);
     const size_t need = dyn_partials_need(mode, Mcap, Ncap, Kcap);
     if (need > pcap) {
         set_error("dgemm: the partials buffer of a captured product is smaller than its split needs");

@@ -178,14 +178,21 @@ size_t tc8_reserve_doubles(long M, long N, long K, bool gram);
 // columns of op(B) whose exponent is EXP_LOST (LOST_ROWS), and of a guarded
 // product (a library call) the most indices that a row of op(A) and a column of
 // op(B) is small at (LOST_WORST).  free: the scratch behind tc8_head_doubles, in
-// which the recomputation's partials may go.
+// which the recomputation's partials may go.  mx, eb, ebs: the Gram's columns' largest
+// entries and their blocks' words (gram_check_kernel): the exponent and, in the
+// low ten bits, the number of entries with digits.
 constexpr int LOST_ALL = 0, LOST_ROWS = 1, LOST_WORST = 2;
 constexpr int EXP_LOST = 1 << 20;
+__host__ __device__ inline int block_exp(int word) { return word >> 10; }
+__host__ __device__ inline int block_count(int word) { return word & 1023; }
 struct Lost {
-    const int* flag = nullptr;  // null: a product of its own
-    const int *a = nullptr, *b = nullptr;
+    int* flag = nullptr;  // null: a product of its own
+    int *a = nullptr, *b = nullptr;
     int guard = 0, gram = 0;
     double* free = nullptr;
+    const unsigned long long* mx = nullptr;
+    const int* eb = nullptr;
+    long ebs = 0;
 };
 #ifdef __CUDACC__
 // 2: everything is lost (of a guarded product also where two rows may have fewer
@@ -198,7 +205,7 @@ __device__ inline int tc8_lost(const Lost& l, int K) {
     return l.flag[LOST_ROWS] ? 1 : 0;
 }
 #endif
-size_t tc8_head_doubles(long M, long N);
+size_t tc8_head_doubles(long M, long N, long K, bool gram);
 // probe: every wait of the product's kernel gives up at once (tt_digits_wait_probe).
 tt_status tc8_gemm(cudaStream_t s, bool ta, bool tb, long M, long N, long K, double alpha, const double* A, long lda,
                    const double* B, long ldb, double* C, long ldc, DevBuf& scratch, int* status_dev, bool guard,

@@ -26,14 +26,17 @@ static void fail(const char* what, long Mc, long Nc, long Kc, long M, long N, lo
 static void check(const Plan& q, bool captured, bool gram, long Mc, long Nc, long Kc, long M, long N, long K) {
     const long chunk = least(q.Kc, K), rows = least(q.Mc, M);
     const int nst = stages(chunk);
-    const int spc = split_stages(M, N, tiles_of(rows, N, gram), nst), ks = (nst + spc - 1) / spc;
+    const int spc = split_stages(M, N, tiles_of(rows, N, gram), nst, split_unit(K)), ks = (nst + spc - 1) / spc;
     const bool whole = !gram && K <= q.Kc && ks == 1;
     if (!whole && q.part < 16ull * M * N * ks) fail(q.part ? "planes too small" : "no planes", Mc, Nc, Kc, M, N, K);
-    if (q.part && captured && ks > 1 && stages(q.Kc) >= 8 && split_limit(Mc, Nc, stages(q.Kc)) == 1) ++split_under_unsplit;
+    if (q.part && captured && ks > 1 && stages(q.Kc) >= 8 && split_limit(Mc, Nc, stages(q.Kc), split_unit(Kc)) == 1) ++split_under_unsplit;
     const size_t stage = 2ull * S8 * T_K;
     if (up(N, gram ? T_M : RB) * nst * stage > q.imgB) fail("image B", Mc, Nc, Kc, M, N, K);
     if (!gram && up(rows, T_M) * nst * stage > q.imgA) fail("image A", Mc, Nc, Kc, M, N, K);
-    if (q.head < 256 + 16ull * (M + N)) fail("head", Mc, Nc, Kc, M, N, K);
+    const size_t side = gram ? M : M + N;
+    if (q.head < 256 + 16 * side + (K > ONE_EXP_K ? 4 * side * ((K + BLK_K - 1) / BLK_K) : 0)) fail("head", Mc, Nc, Kc, M, N, K);
+    // a contraction that goes in chunks is cut between exact blocks
+    if (K > q.Kc && (q.Kc % BLK_K || spc % T_BLK)) fail("cut", Mc, Nc, Kc, M, N, K);
     if (q.Kc < Kc && q.Kc % (T_K * T_BLK)) fail("chunk", Mc, Nc, Kc, M, N, K);
 }
 int main() {

@@ -238,3 +238,52 @@ def test_rows_that_cannot_be_split_leave_the_others_as_they_are(ttsn):
     bound = (K + 1) * np.finfo(float).eps * (np.abs(A) @ np.abs(B))
     bound[37] *= 1e-290
     assert np.all(np.abs(got[fine] - ref[fine]) <= 2 * bound[fine])
+
+
+@pytest.mark.parametrize("rows", [262144, 2097152])
+@pytest.mark.parametrize("where", ["one", "patch", "scattered"])
+@pytest.mark.parametrize("eps", [1e-6, 1e-7])
+def test_rounding_of_point_like_columns_keeps_its_tolerance(ttsn, rows, where, eps):
+    """Large entries in a few rows over a background of 2^-28, whose singular values are
+    1e-8 to 1e-6 of the norm: one scale a column would lose the background's products.
+    The rounding must do as well as with a Gram from FP64 sums (gram_noalloc, with the
+    same eigensolver and truncation), which itself cannot resolve all of these."""
+    import torch
+
+    n = 40
+    r = torch.arange(rows, device="cuda", dtype=torch.float64)
+    f = torch.arange(1, n + 1, device="cuda", dtype=torch.float64)
+    A = 2.0 ** -28 * torch.cos(2 * np.pi * (r[:, None] + 0.5) * f[None, :] / rows)
+    at = {"one": [12345], "patch": range(70000, 70006), "scattered": range(100, rows, rows // 60)}[where]
+    A[list(at)] += 1.0
+    tt = ttsn.TensorTrain([A[None].contiguous(), torch.eye(n, device="cuda", dtype=torch.float64)[:, :, None].contiguous()])
+    tt.round(eps=eps)
+    err = float(torch.linalg.norm(tt.full().reshape(rows, n) - A) / torch.linalg.norm(A))
+    lam, V, _ = ttsn.syev_psd(ttsn.gram_noalloc(A))
+    tail = torch.flip(torch.cumsum(torch.flip(lam, (0,)), 0), (0,))
+    r64 = min(int((tail > eps * eps * lam.sum()).sum()), int((lam > n * 2.0 ** -52 * lam[0]).sum()))
+    err64 = float(torch.linalg.norm(A - (A @ V[:r64].T) @ V[:r64]) / torch.linalg.norm(A))
+    assert err <= 1.1 * max(eps, err64)
+
+
+def test_gram_of_long_columns_whose_blocks_differ_in_scale(ttsn):
+    """Blocks of 512 rows scaled by powers of two over +-60 binary orders, integer
+    entries, so every block's sum is an integer times a power of two.  The sum is off
+    by its last rounding and, for each of the 80 blocks, by at most 2^-71 of
+    2^(e_i + e_j) <= 16 max|a_i| max|a_j|."""
+    import torch
+
+    rng = np.random.default_rng(3)
+    m, n = 40960, 48
+    A = rng.integers(-(1 << 12), 1 << 12, (m, n)).astype(float)
+    s = 2.0 ** np.repeat(rng.integers(-60, 61, (m // 512, 1)), 512, axis=0)
+    G = ttsn.gram(torch.as_tensor(A * s, device="cuda")).cpu().numpy()
+    ref = np.zeros((n, n), np.longdouble)
+    for b in range(m // 512):
+        blk = A[512 * b:512 * b + 512].astype(np.int64)
+        ref += (blk.T @ blk).astype(np.longdouble) * np.longdouble(s[512 * b, 0]) ** 2
+    mx = np.abs(A * s).max(0)
+    # (the guard may send it to the FP64 pipe: its sum's bound)
+    fp64 = m * np.finfo(float).eps * (np.abs(A * s).T @ np.abs(A * s))
+    assert np.all(np.abs(G - ref) <= np.maximum(80 * 2.0 ** -67 * mx[:, None] * mx[None, :] + 2.0 ** -53 * np.abs(ref), fp64))
+    assert np.array_equal(G, G.T)
