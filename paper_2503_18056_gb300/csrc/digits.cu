@@ -1055,7 +1055,8 @@ tt_status run(cudaStream_t s, bool ta, bool tb, long M, long N, long K, double a
         if (!gram) spread(b);
     }
     TT_CUDA_TRY(cudaGetLastError());
-    *lost = Lost{flag, a.e, b.e, guard ? 1 : 0, gram ? 1 : 0, reinterpret_cast<double*>(base + q.head), mx, a.eb, a.ebs};
+    *lost = Lost{flag, a.e, b.e, guard ? 1 : 0, gram ? 1 : 0, reinterpret_cast<double*>(base + q.head), mx, a.eb, a.ebs,
+                 gram && !guard ? reinterpret_cast<float*>(ex + nrows) : nullptr};
     return TT_OK;
 }
 

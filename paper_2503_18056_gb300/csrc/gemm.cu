@@ -230,8 +230,15 @@ prod_kernel(int M, int N, int K, double alpha, const double* __restrict__ A, lon
         }
         const int m0 = tm * BT, n0 = tn * BT;
         if (redo == 1) {  // the same for every warp
-            const int e = lane < BT ? lost.a[min(m0 + lane, M - 1)] : lost.b[min(n0 + lane - BT, N - 1)];
-            if (!__any_sync(0xffffffffu, e == EXP_LOST)) continue;
+            const int i = lane < BT ? min(m0 + lane, M - 1) : min(n0 + lane - BT, N - 1);
+            if (lost.rho) {
+                unsigned r = __float_as_uint(lost.rho[i]);  // not negative: ordered as integers
+                const unsigned a = __reduce_max_sync(0xffffffffu, lane < BT ? r : 0u);
+                const unsigned b = __reduce_max_sync(0xffffffffu, lane < BT ? 0u : r);
+                if (!(__uint_as_float(a) * __uint_as_float(b) > 1.0f)) continue;
+            } else if (!__any_sync(0xffffffffu, (lane < BT ? lost.a[i] : lost.b[i]) == EXP_LOST)) {
+                continue;
+            }
         }
         const int kbeg = z * chunk, kend = min(K, kbeg + chunk);
         const long sa = TA ? lda : 1, sb = TB ? 1 : ldb;
@@ -339,15 +346,16 @@ prod_kernel(int M, int N, int K, double alpha, const double* __restrict__ A, lon
     }
 }
 
-// Behind a rounding's digit Gram G: a column is lost where the digits' error may
-// exceed that of the FP64 sums it stands for, relative to the column's own norm.
-// A digit Gram's entry (i, j) is off by at most sqrt(Q_i Q_j), Q_i = 9.1 2^-58
-// sum_blocks c_block 4^e_block (c: entries that are not zero), the FP64 pipe's by chunk
-// 2^-53 |a_i| |a_j| (chunk: rows of a split); a column stays where Q_i <= chunk 2^-53
-// |a_i|^2, above about 2,400 rows a split always.  So a column is recomputed (its row
-// and column of G, prod_kernel) only where few of its blocks' entries make up its
-// norm, and G keeps its relative accuracy under any scaling of the columns, which
-// the eigenvalues of W G W^T take over, whatever the rounding's tolerance.
+// Behind a rounding's digit Gram G: entries are lost where the digits' error may
+// exceed that of the FP64 sums they stand for, relative to the two columns' norms.
+// Entry (i, j) is off by at most sqrt(Q_i Q_j), Q_i = 9.1 2^-58 sum_blocks c_block
+// 4^e_block (c: entries that are not zero), the FP64 pipe's by chunk 2^-53 |a_i| |a_j|
+// (chunk: rows of a split).  So with rho_i = sqrt(Q_i / (chunk 2^-53 |a_i|^2)) an
+// entry stays where rho_i rho_j <= 1, always above about 2,400 rows a split, and the
+// others' tiles are recomputed (prod_kernel): columns of whose blocks' entries few
+// make up the norm, against one another.  G keeps its relative accuracy under any
+// scaling of the columns, which the eigenvalues of W G W^T take over, whatever the
+// rounding's tolerance.
 // A warp a column.
 __global__ void __launch_bounds__(256)
 gram_check_kernel(int n, int K, const double* __restrict__ G, long ldg, const int* __restrict__ desc, Lost lost) {
@@ -362,7 +370,11 @@ gram_check_kernel(int n, int K, const double* __restrict__ G, long ldg, const in
     const int lane = threadIdx.x & 31;
     for (int i = blockIdx.x * 8 + (threadIdx.x >> 5); i < n; i += gridDim.x * 8) {
         const int e = lost.a[i];
-        if (lost.mx[i] == 0 || e == EXP_LOST) continue;
+        if (lost.mx[i] == 0 || e == EXP_LOST) {
+            // no product with a lost column stays, however small the other's rho
+            if (lane == 0) lost.rho[i] = e == EXP_LOST ? __int_as_float(0x7f800000) : 1e-30f;
+            continue;
+        }
         // sum_blocks c_block 4^(e_block - e) in units of 2^-30 (at least one an entry): the
         // same in any order
         unsigned long long sum = 0;
@@ -376,10 +388,13 @@ gram_check_kernel(int n, int K, const double* __restrict__ G, long ldg, const in
         } else {
             sum = (unsigned long long)K << 30;
         }
-        const double most = 0x1p-30 * (double)sum * (9.1 / 32.0) / chunk;
-        if (lane == 0 && !(most <= scalbn(G[(long)i * ldg + i], -2 * e))) {
-            lost.a[i] = EXP_LOST;
-            atomicOr(lost.flag + LOST_ROWS, 1);
+        const double q = 0x1p-30 * (double)sum * (9.1 / 32.0) / chunk;
+        const double r2 = q / scalbn(G[(long)i * ldg + i], -2 * e);
+        if (lane == 0) {
+            // rounded up; what is not a number or not positive (a diagonal entry cannot be) is lost
+            const float r = r2 >= 0.0 ? __fsqrt_ru(__double2float_ru(r2)) : __int_as_float(0x7f800000);
+            lost.rho[i] = fmaxf(r, 1e-30f);
+            if (r > 1.0f) atomicOr(lost.flag + LOST_ROWS, 1);
         }
     }
 }

@@ -180,7 +180,9 @@ size_t tc8_reserve_doubles(long M, long N, long K, bool gram);
 // op(B) is small at (LOST_WORST).  free: the scratch behind tc8_head_doubles, in
 // which the recomputation's partials may go.  mx, eb, ebs: the Gram's columns' largest
 // entries and their blocks' words (gram_check_kernel): the exponent and, in the
-// low ten bits, the number of entries with digits.
+// low ten bits, the number of entries with digits.  rho: what gram_check_kernel
+// makes of them, an entry is lost where rho_i rho_j > 1 (not looked at in a guarded
+// product).
 constexpr int LOST_ALL = 0, LOST_ROWS = 1, LOST_WORST = 2;
 constexpr int EXP_LOST = 1 << 20;
 __host__ __device__ inline int block_exp(int word) { return word >> 10; }
@@ -193,6 +195,7 @@ struct Lost {
     const unsigned long long* mx = nullptr;
     const int* eb = nullptr;
     long ebs = 0;
+    float* rho = nullptr;
 };
 #ifdef __CUDACC__
 // 2: everything is lost (of a guarded product also where two rows may have fewer

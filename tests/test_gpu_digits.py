@@ -267,23 +267,65 @@ def test_rounding_of_point_like_columns_keeps_its_tolerance(ttsn, rows, where, e
 
 
 def test_gram_of_long_columns_whose_blocks_differ_in_scale(ttsn):
-    """Blocks of 512 rows scaled by powers of two over +-60 binary orders, integer
-    entries, so every block's sum is an integer times a power of two.  The sum is off
-    by its last rounding and, for each of the 80 blocks, by at most 2^-71 of
+    """Blocks of 512 rows scaled by powers of two, a few of them far below the others,
+    integer entries, so every block's sum is an integer times a power of two.  The sum
+    is off by its last rounding and, for each of the 80 blocks, by at most 2^-71 of
     2^(e_i + e_j) <= 16 max|a_i| max|a_j|."""
     import torch
 
     rng = np.random.default_rng(3)
     m, n = 40960, 48
     A = rng.integers(-(1 << 12), 1 << 12, (m, n)).astype(float)
-    s = 2.0 ** np.repeat(rng.integers(-60, 61, (m // 512, 1)), 512, axis=0)
+    down = np.where(np.arange(m // 512) % 8 == 3, rng.integers(10, 61, m // 512), rng.integers(0, 5, m // 512))
+    s = 2.0 ** -np.repeat(down, 512)[:, None].astype(float)
     G = ttsn.gram(torch.as_tensor(A * s, device="cuda")).cpu().numpy()
     ref = np.zeros((n, n), np.longdouble)
     for b in range(m // 512):
         blk = A[512 * b:512 * b + 512].astype(np.int64)
         ref += (blk.T @ blk).astype(np.longdouble) * np.longdouble(s[512 * b, 0]) ** 2
     mx = np.abs(A * s).max(0)
-    # (the guard may send it to the FP64 pipe: its sum's bound)
-    fp64 = m * np.finfo(float).eps * (np.abs(A * s).T @ np.abs(A * s))
-    assert np.all(np.abs(G - ref) <= np.maximum(80 * 2.0 ** -67 * mx[:, None] * mx[None, :] + 2.0 ** -53 * np.abs(ref), fp64))
+    assert np.all(np.abs(G - ref) <= 80 * 2.0 ** -67 * mx[:, None] * mx[None, :] + 2.0 ** -53 * np.abs(ref))
     assert np.array_equal(G, G.T)
+
+
+def _gauged(rng, shape, ranks, decades):
+    """Cores of a TT, and those of the same tensor with a graded power-of-two gauge on
+    every bond."""
+    r = [1] + ranks + [1]
+    cores = [rng.standard_normal((r[k], shape[k], r[k + 1])) for k in range(len(shape))]
+    other = [c.copy() for c in cores]
+    for k in range(len(shape) - 1):
+        D = 2.0 ** np.round(decades * np.log2(10.0) * rng.random(r[k + 1]))
+        other[k] *= D
+        other[k + 1] /= D[:, None, None]
+    return cores, other
+
+
+def test_graded_gauge_does_not_change_the_full_tensor(ttsn):
+    """Scaling a core's columns by D and the next core's rows by 1 / D, powers of two
+    over eight decades, changes no rounding error of a sum over the bond."""
+    import torch
+
+    cores, other = _gauged(np.random.default_rng(7), (3000, 64, 40), [90, 90], 8)
+    assert torch.equal(ttsn.TensorTrain(cores).full(), ttsn.TensorTrain(other).full())
+
+
+def test_rounding_with_a_graded_gauge_gives_an_orthonormal_core(ttsn):
+    """A' = A P_A with P_A from the eigenvectors of K = W G_A W^T: its columns are
+    orthonormal to the rounding of K, n^2 eps lambda_1, relative to its smallest
+    eigenvalue, whatever the bonds' gauge (six decades here); with a scale a row and
+    not the bond's, the digit products would lose the gauge's decades."""
+    import torch
+
+    cores, other = _gauged(np.random.default_rng(8), (3000, 64, 40), [90, 90], 6)
+    for c in (cores, other):
+        tt = ttsn.TensorTrain(c)
+        X = tt.full().reshape(3000, -1)
+        tt.round(eps=1e-6)
+        A = tt.cores()[0].reshape(3000, -1)
+        r = A.shape[1]
+        sv = torch.linalg.svdvals(X)
+        bound = 90 ** 2 * 2.0 ** -52 * float(sv[0] / sv[r - 1]) ** 2
+        assert r == 90 and bound < 1e-9
+        assert float((A.T @ A - torch.eye(r, device=A.device, dtype=A.dtype)).abs().max()) <= bound
+        assert float(torch.linalg.norm(tt.full().reshape(3000, -1) - X) / torch.linalg.norm(X)) <= 1e-6
