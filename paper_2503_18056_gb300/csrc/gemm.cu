@@ -353,9 +353,13 @@ prod_kernel(int M, int N, int K, double alpha, const double* __restrict__ A, lon
 // (chunk: rows of a split).  So with rho_i = sqrt(Q_i / (chunk 2^-53 |a_i|^2)) an
 // entry stays where rho_i rho_j <= 1, always above about 2,400 rows a split, and the
 // others' tiles are recomputed (prod_kernel): columns of whose blocks' entries few
-// make up the norm, against one another.  G keeps its relative accuracy under any
-// scaling of the columns, which the eigenvalues of W G W^T take over, whatever the
-// rounding's tolerance.
+// make up the norm, against one another.  Shorter splits count as 1,024 rows: Q takes
+// every digit at its largest, and even an entry that loses all it can loses a
+// twentieth of that; at 256 rows the difference columns of a smooth field on a 128^2
+// grid (an entry of 1 at a vacuum face, 0.05 elsewhere) have rho up to 2, and their
+// Grams, 60 us, would all be formed twice (440).  G keeps its relative accuracy under
+// any scaling of the columns, which the eigenvalues of W G W^T take over, whatever
+// the rounding's tolerance.
 // A warp a column.
 __global__ void __launch_bounds__(256)
 gram_check_kernel(int n, int K, const double* __restrict__ G, long ldg, const int* __restrict__ desc, Lost lost) {
@@ -388,7 +392,7 @@ gram_check_kernel(int n, int K, const double* __restrict__ G, long ldg, const in
         } else {
             sum = (unsigned long long)K << 30;
         }
-        const double q = 0x1p-30 * (double)sum * (9.1 / 32.0) / chunk;
+        const double q = 0x1p-30 * (double)sum * (9.1 / 32.0) / max(chunk, 1024);
         const double r2 = q / scalbn(G[(long)i * ldg + i], -2 * e);
         if (lane == 0) {
             // rounded up; what is not a number or not positive (a diagonal entry cannot be) is lost
