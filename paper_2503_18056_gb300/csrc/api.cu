@@ -349,6 +349,7 @@ struct tt_ctx {
     unsigned graph_launches = 0;       // library kernels one replay runs
     bool ranks_stale = false;          // h->r lags the device after replays
     int cap1 = 0, cap2 = 0;            // rank caps of the two bonds
+    DevBuf kscale, dyn_scale;          // bond scales of the digit products (ints), of captured ones
     DevBuf dyn_buf, dyn_part, dyn_tc;  // size block (ints), product partials, digit-product scratch
     int* dyn = nullptr;
     int* h_dyn = nullptr;              // pinned mirror, refreshed by every replay
@@ -403,7 +404,7 @@ struct tt_ctx {
                           &partials, &bwd, &f_sigma_a, &f_sigma_s, &f_cv, &f_T, &f_Estar, &f_E,
                           &thbar, &red, &ang_buf, &src_x, &src_th, &src_ph, &src_q,
                           &split_fac, &sp_F, &sp_tmp[0], &sp_tmp[1], &f_fw, &usr_x, &usr_th, &usr_ph,
-                          &sk_Y, &sk_Q, &sk_G, &sk_lam, &sk_Vt, &sk_Vs, &xch, &dyn_buf, &dyn_part, &dyn_tc, &ydots,
+                          &sk_Y, &sk_Q, &sk_G, &sk_lam, &sk_Vt, &sk_Vs, &xch, &dyn_buf, &dyn_part, &dyn_tc, &kscale, &dyn_scale, &ydots,
                           &ts_Qa, &ts_Qb, &ts_Y, &ts_R, &ts_J, &ts_lam, &ts_Vt, &ts_U, &ts_M};
         for (DevBuf* b : bufs) b->release();
         for (auto& ax : inflow)
@@ -554,8 +555,14 @@ tt_status eig_orthonormalise(tt_ctx* h, long m, int l, const double* Y, DevBuf& 
     if (k == 0) return TT_OK;
     scale_rows(s, k, l, h->sk_Vt.p, l, h->sk_lam.p, 2, h->sk_Vs.p, l);  // rows v_j / sqrt(lambda_j)
     TT_TRY(Q.ensure((size_t)m * k, s));
+    Bond over;  // the scale of Y's columns
+    if (h->prod.digits && tc8_wanted(m, l, l)) {
+        TT_TRY(h->kscale.ensure(((size_t)l + 1) / 2, s));
+        over = Bond{reinterpret_cast<int*>(h->kscale.p), -1};
+        bond_scale(s, l, 1, h->sk_G.p, l, reinterpret_cast<int*>(h->kscale.p));
+    }
     TT_TRY(dgemm_sk(s, false, true, (int)m, k, l, 1.0, Y, l, h->sk_Vs.p, l, Q.p, k,
-                    h->partials, h->prod, false));
+                    h->partials, h->prod, false, &over));
     return TT_OK;
 }
 
@@ -683,8 +690,14 @@ tt_status orth_qr3(tt_ctx* h, long m, int l, const double* Y, DevBuf** Q, int* k
                 h->d_int + next_sweep_slot(h), h->max_sweeps));
     shifted_scale_rows(s, l, h->sk_Vt.p, l, h->sk_lam.p, h->sk_Vs.p, l);
     TT_TRY(h->ts_Qa.ensure((size_t)m * l, s));
+    Bond over;  // the scale of Y's columns
+    if (h->prod.digits && tc8_wanted(m, l, l)) {
+        TT_TRY(h->kscale.ensure(((size_t)l + 1) / 2, s));
+        over = Bond{reinterpret_cast<int*>(h->kscale.p), -1};
+        bond_scale(s, l, 1, h->sk_G.p, l, reinterpret_cast<int*>(h->kscale.p));
+    }
     TT_TRY(dgemm_sk(s, false, true, (int)m, l, l, 1.0, Y, l, h->sk_Vs.p, l, h->ts_Qa.p, l,
-                    h->partials, h->prod, false));
+                    h->partials, h->prod, false, &over));
     int k2 = 0, k3 = 0;
     TT_TRY(eig_orthonormalise(h, m, l, h->ts_Qa.p, h->ts_Qb, &k2));
     if (k2 == 0) {
@@ -889,10 +902,17 @@ tt_status round_cores(tt_ctx* h, DevBuf* src, const int* R, DevBuf* dst, int* rr
                 TT_TRY(slgemm_nt(s, Ra, Ra, nn * Rb, h->bwd.p, (long)nn * Rb, src[k + 1].p,
                                  (long)nn * Rb, h->GB[k].p, Ra, h->slscratch, h->d_int + HI_STATUS));
             } else {
+                Bond up, down;
+                if (h->prod.digits && (tc8_wanted((long)Ra * nn, Rb, Rb) || tc8_wanted(Ra, Ra, (long)nn * Rb))) {
+                    TT_TRY(h->kscale.ensure(((size_t)nn * Rb + 1) / 2, s));
+                    up = Bond{reinterpret_cast<int*>(h->kscale.p), 1};
+                    down = Bond{up.s, -1};
+                    bond_scale(s, Rb, nn, h->GB[k + 1].p, Rb, reinterpret_cast<int*>(h->kscale.p));
+                }
                 TT_TRY(dgemm_sk(s, false, false, Ra * nn, Rb, Rb, 1.0, src[k + 1].p, Rb, h->GB[k + 1].p,
-                             Rb, h->bwd.p, Rb, h->partials, h->prod, false));
+                             Rb, h->bwd.p, Rb, h->partials, h->prod, false, &up));
                 TT_TRY(dgemm_sk(s, false, true, Ra, Ra, nn * Rb, 1.0, h->bwd.p, (long)nn * Rb,
-                                src[k + 1].p, (long)nn * Rb, h->GB[k].p, Ra, h->partials, h->prod));
+                                src[k + 1].p, (long)nn * Rb, h->GB[k].p, Ra, h->partials, h->prod, true, &down));
             }
         }
     }
@@ -950,6 +970,17 @@ tt_status round_cores(tt_ctx* h, DevBuf* src, const int* R, DevBuf* dst, int* rr
             // Gram is the sum of the shards' partial Grams
             if (k == 0 && h->shard.on) TT_TRY(shard_exchange(h, TT_XCHG_SUM, h->GA.p, (size_t)Rk * Rk));
         }
+        // the scale of the bond index for the digit products that contract it:
+        // A's columns (and G_A's) over their norms, what meets them times these
+        Bond over, times;
+        const Bond none;
+        const long cols = (long)n[k + 1] * R[k + 2];
+        if (h->prod.digits && (tc8_wanted(m, Rk, Rk) || tc8_wanted(Rk, cols, Rk) || tc8_wanted(Rk, Rk, Rk))) {
+            TT_TRY(h->kscale.ensure(((size_t)Rk + 1) / 2, s));
+            bond_scale(s, Rk, 1, h->GA.p, Rk, reinterpret_cast<int*>(h->kscale.p));
+            over = Bond{reinterpret_cast<int*>(h->kscale.p), -1};
+            times = Bond{over.s, 1};
+        }
         {
             PhaseScope ps(h, TT_PH_SMALL, 2.0 * Rk * (double)Rk * kB + 2.0 * kB * (double)kB * Rk, 0.0);
             // W (kB x Rk, W^T W = G_B) from the backward sweep; K = W G_A W^T
@@ -957,9 +988,9 @@ tt_status round_cores(tt_ctx* h, DevBuf* src, const int* R, DevBuf* dst, int* rr
             TT_TRY(h->T1.ensure((size_t)Rk * kB, s));
             TT_TRY(h->K.ensure((size_t)kB * kB, s));
             TT_TRY(dgemm_sk(s, false, true, Rk, kB, Rk, 1.0, h->GA.p, Rk, Wk, Rk, h->T1.p, kB,
-                            h->partials, h->prod));
+                            h->partials, h->prod, true, &over));
             TT_TRY(dgemm_sk(s, false, false, kB, kB, Rk, 1.0, Wk, Rk, h->T1.p, kB, h->K.p, kB,
-                            h->partials, h->prod));
+                            h->partials, h->prod, true, &times));
         }
         TT_TRY(h->lamK.ensure((size_t)kB, s));
         TT_TRY(h->VtK.ensure((size_t)kB * kB, s));
@@ -997,14 +1028,15 @@ tt_status round_cores(tt_ctx* h, DevBuf* src, const int* R, DevBuf* dst, int* rr
             TT_TRY(h->Vts.ensure((size_t)rk * kB, s));
             scale_rows(s, rk, kB, h->VtK.p, kB, h->lamK.p, 2, h->Vts.p, kB);
             TT_TRY(h->PAt.ensure((size_t)rk * Rk, s));
+            // (the contraction is over W's own rows, which have no free scale)
             TT_TRY(dgemm_sk(s, false, false, rk, Rk, kB, 1.0, h->Vts.p, kB, h->VtB[k].p, Rk, h->PAt.p, Rk,
-                            h->partials, h->prod));
+                            h->partials, h->prod, true, &none));
             // M_upd = P_A^T G_A = A'^T A  (rk x Rk): B'^T = A'^T A B^T, the orthogonal
             // projection of A B^T onto span(A'); equals App. A.2's (V_B S_B^{-1} V~ S~)^T
             // on the retained eigenspace of G_B without forming S_B^{-1}
             TT_TRY(h->Mupd.ensure((size_t)rk * Rk, s));
             TT_TRY(dgemm_sk(s, false, false, rk, Rk, Rk, 1.0, h->PAt.p, Rk, h->GA.p, Rk, h->Mupd.p, Rk,
-                            h->partials, h->prod));
+                            h->partials, h->prod, true, &times));
         }
         if (h->cur_rec && h->rec_proj && k < 2) {
             tt_ctx::StepRec* rc = h->cur_rec;
@@ -1023,7 +1055,7 @@ tt_status round_cores(tt_ctx* h, DevBuf* src, const int* R, DevBuf* dst, int* rr
                                  h->d_int + HI_STATUS, &h->partials, reinterpret_cast<const int*>(h->erowA.p)));
             else
                 TT_TRY(dgemm_sk(s, false, true, (int)m, rk, Rk, 1.0, A, Rk, h->PAt.p, Rk, dst[k].p, rk,
-                                h->partials, h->prod, false));
+                                h->partials, h->prod, false, &over));
         }
         // next core = M_upd x_1 G_{k+1}
         double* next;
@@ -1039,7 +1071,7 @@ tt_status round_cores(tt_ctx* h, DevBuf* src, const int* R, DevBuf* dst, int* rr
             PhaseScope ps(h, TT_PH_UPDATE, 2.0 * rk * (double)Rk * ncols,
                           8.0 * ((double)Rk * ncols + (double)rk * ncols));
             TT_TRY(dgemm_sk(s, false, false, rk, (int)ncols, Rk, 1.0, h->Mupd.p, Rk, src[k + 1].p, ncols,
-                            next, ncols, h->partials, h->prod));
+                            next, ncols, h->partials, h->prod, true, &over));
         }
         rr[k + 1] = rk;
         A = next;
@@ -1463,12 +1495,20 @@ tt_status graph_step_body(tt_ctx* h) {
                           h->ydots.p, Sources(), dd);
     // rounding (App. A.2, one-sided Gram truncation): backward sweep
     fill(s, h->d_dbl + HD_DELTA2, 1, -1.0);
+    // the bonds' scales as the host path's (round_cores)
+    int* ks = reinterpret_cast<int*>(h->dyn_scale.p);
+    const Bond up{h->prod.digits ? ks : nullptr, 1}, down{up.s, -1}, none;
+    const Bond &times = up, &over = down;
+    auto scale = [&](int cap, int rep, const double* G, const int* of) {
+        if (h->prod.digits) bond_scale(s, cap, rep, G, 0, ks, of);
+    };
     TT_TRY(dgemm_dyn(s, false, true, desc + 0, G2, G2, np, 1.0, h->gcore[2].p, h->gcore[2].p, h->GB[1].p, P, PC, 1, h->dyn_tc,
                      h->prod));
+    scale(G2, nt, h->GB[1].p, desc + 0);
     TT_TRY(dgemm_dyn(s, false, false, desc + 8, G1 * nt, G2, G2, 1.0, h->gcore[1].p, h->GB[1].p, h->bwd.p, P, PC, 0, h->dyn_tc,
-                     h->prod));
+                     h->prod, &up));
     TT_TRY(dgemm_dyn(s, false, true, desc + 16, G1, G1, nt * G2, 1.0, h->bwd.p, h->gcore[1].p, h->GB[0].p, P, PC, 1, h->dyn_tc,
-                     h->prod));
+                     h->prod, &down));
     TT_TRY(pchol_dyn(s, dd + DYN_G1, G1, h->GB[0].p, h->VtB[0].p, h->Wc.p, h->lamB[0].p, h->eig,
                      h->d_int + HI_STATUS, dd + DYN_KB0));
     TT_TRY(pchol_dyn(s, dd + DYN_G2, G2, h->GB[1].p, h->VtB[1].p, h->Wc.p, h->lamB[1].p, h->eig,
@@ -1477,10 +1517,11 @@ tt_status graph_step_body(tt_ctx* h) {
     // bond 0: G_A, K = W G_A W^T, eig(K), decision
     TT_TRY(dgemm_dyn(s, true, false, desc + 24, G1, G1, (int)nc, 1.0, h->gcore[0].p, h->gcore[0].p, h->GA.p, P, PC, 2, h->dyn_tc,
                      h->prod));
+    scale(G1, 1, h->GA.p, desc + 24);
     TT_TRY(dgemm_dyn(s, false, true, desc + 32, G1, G1, G1, 1.0, h->GA.p, h->VtB[0].p, h->T1.p, P, PC, 1, h->dyn_tc,
-                     h->prod));
+                     h->prod, &over));
     TT_TRY(dgemm_dyn(s, false, false, desc + 40, G1, G1, G1, 1.0, h->VtB[0].p, h->T1.p, h->K.p, P, PC, 1, h->dyn_tc,
-                     h->prod));
+                     h->prod, &times));
     TT_TRY((h->eig_method == TT_EIG_ONE_SIDED ? syev_psd_dyn : syev_dyn)(
         s, dd + DYN_KB0, G1, h->K.p, h->lamK.p, h->VtK.p, h->eig, h->d_int + HI_STATUS, dd + DYN_SWEEPS,
         h->max_sweeps));
@@ -1490,20 +1531,21 @@ tt_status graph_step_body(tt_ctx* h) {
     // bond 0 update: P_A^T, M_upd, X' = X* P_A, next core = M_upd x_1 Theta*
     scale_rows_dyn(s, desc + 48, (long)c1 * G1, h->VtK.p, h->lamK.p, 2, h->Vts.p);
     TT_TRY(dgemm_dyn(s, false, false, desc + 56, c1, G1, G1, 1.0, h->Vts.p, h->VtB[0].p, h->PAt.p, P, PC, 1, h->dyn_tc,
-                     h->prod));
+                     h->prod, &none));
     TT_TRY(dgemm_dyn(s, false, false, desc + 64, c1, G1, G1, 1.0, h->PAt.p, h->GA.p, h->Mupd.p, P, PC, 1, h->dyn_tc,
-                     h->prod));
+                     h->prod, &times));
     TT_TRY(dgemm_dyn(s, false, true, desc + 72, (int)nc, c1, G1, 1.0, h->gcore[0].p, h->PAt.p, h->core[0].p, P, PC, 0, h->dyn_tc,
-                     h->prod));
+                     h->prod, &over));
     TT_TRY(dgemm_dyn(s, false, false, desc + 80, c1, nt * G2, G1, 1.0, h->Mupd.p, h->gcore[1].p, h->tmp[0].p, P, PC, 1, h->dyn_tc,
-                     h->prod));
+                     h->prod, &over));
     // bond 1 on the next core (replicated rows r0 n_theta)
     TT_TRY(dgemm_dyn(s, true, false, desc + 88, G2, G2, c1 * nt, 1.0, h->tmp[0].p, h->tmp[0].p, h->GA.p, P, PC, 2, h->dyn_tc,
                      h->prod));
+    scale(G2, 1, h->GA.p, desc + 88);
     TT_TRY(dgemm_dyn(s, false, true, desc + 96, G2, G2, G2, 1.0, h->GA.p, h->VtB[1].p, h->T1.p, P, PC, 1, h->dyn_tc,
-                     h->prod));
+                     h->prod, &over));
     TT_TRY(dgemm_dyn(s, false, false, desc + 104, G2, G2, G2, 1.0, h->VtB[1].p, h->T1.p, h->K.p, P, PC, 1, h->dyn_tc,
-                     h->prod));
+                     h->prod, &times));
     TT_TRY((h->eig_method == TT_EIG_ONE_SIDED ? syev_psd_dyn : syev_dyn)(
         s, dd + DYN_KB1, G2, h->K.p, h->lamK.p, h->VtK.p, h->eig, h->d_int + HI_STATUS, dd + DYN_SWEEPS + 1,
         h->max_sweeps));
@@ -1512,13 +1554,13 @@ tt_status graph_step_body(tt_ctx* h) {
     plan(3);
     scale_rows_dyn(s, desc + 112, (long)c2 * G2, h->VtK.p, h->lamK.p, 2, h->Vts.p);
     TT_TRY(dgemm_dyn(s, false, false, desc + 120, c2, G2, G2, 1.0, h->Vts.p, h->VtB[1].p, h->PAt.p, P, PC, 1, h->dyn_tc,
-                     h->prod));
+                     h->prod, &none));
     TT_TRY(dgemm_dyn(s, false, false, desc + 128, c2, G2, G2, 1.0, h->PAt.p, h->GA.p, h->Mupd.p, P, PC, 1, h->dyn_tc,
-                     h->prod));
+                     h->prod, &times));
     TT_TRY(dgemm_dyn(s, false, true, desc + 136, c1 * nt, c2, G2, 1.0, h->tmp[0].p, h->PAt.p, h->core[1].p, P, PC, 0, h->dyn_tc,
-                     h->prod));
+                     h->prod, &over));
     TT_TRY(dgemm_dyn(s, false, false, desc + 144, c2, np, G2, 1.0, h->Mupd.p, h->gcore[2].p, h->core[2].p, P, PC, 1, h->dyn_tc,
-                     h->prod));
+                     h->prod, &over));
     // energy-conserving temperature update (Sec. 3.2) from the rounded TT
     plain_thbar(s, h->ang, c1, c2, h->core[1].p, h->core[2].p, h->thbar.p, dd);
     energy_rows(s, nc, c1, h->core[0].p, c1, h->thbar.p, h->fields.c, nullptr, h->f_Estar.p, h->f_cv.p,
@@ -1567,6 +1609,7 @@ tt_status graph_reserve(tt_ctx* h) {
         {&h->T1, Gm * Gm}, {&h->K, Gm * Gm}, {&h->lamK, Gm}, {&h->VtK, Gm * Gm},
         {&h->Vts, Gm * Gm}, {&h->PAt, Gm * Gm}, {&h->Mupd, Gm * Gm}, {&h->bwd, G1 * nt * G2},
         {&h->tmp[0], c1 * nt * G2}, {&h->thbar, nterms * (c1 + c2) + 2}, {&h->ydots, nc * nterms},
+        {&h->dyn_scale, (std::max(nt * G2, Gm) + 1) / 2},
         {&h->eig.g0, Gm * Gm}, {&h->eig.g1, Gm * Gm}, {&h->eig.vt_unsorted, Gm * Gm},
         {&h->eig.lam_unsorted, Gm}, {&h->eig.abc, 3 * (Gm + 1)}, {&h->eig.cs, Gm + 1},
         {&h->eig.psd, 3 * Gm + 2},

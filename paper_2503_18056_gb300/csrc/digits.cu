@@ -39,16 +39,26 @@
 // prod_kernel behind the product, which otherwise returns at once, recomputes the
 // 16 x 16 tiles that they reach (tc8_lost), or everything where a wait ran out.
 //
-// An entry far below its row's maximum keeps few digits, which matters where
-// small entries meet large ones (A times the identity, disjoint supports): the
-// sum |a||b| is then far below K max|a_i| max|b_j|, which bounds the error.  A
-// rounding's Gram is held to its columns' norms (gram_check_kernel in gemm.cu), a
-// library call to the sum's scale: the split counts each row's entries above 2^-9 of its
-// maximum, and unless every pair of rows has K / 16 indices where both are
-// (tc8_lost), the product is recomputed on the FP64 pipe (the count and the
-// check: 200,000 x 577 times 577 x 96 1.73 -> 1.78 ms, the Gram of 500,000 x 449
-// 5.68 -> 5.70; where it is recomputed, a sparse 500,000 x 449 takes 106 ms and
-// 20,000 x 500 times the identity 9.7, on the FP64 pipe alone 143 and 9.8 before).
+// An entry far below its row's (block's) maximum keeps few digits, which matters
+// where small entries meet large ones: the sum |a||b| is then far below K max|a_i|
+// max|b_j|, which bounds the error.
+// - A rounding's Gram is held to its columns' norms (gram_check_kernel in gemm.cu).
+// - A handle's other products contract an index that may carry any scaling, one
+//   core's columns times D and the next core's rows over D: the sum does not depend
+//   on D, but a power of two a row would see D on one side and 1 / D on the other.
+//   So they are formed at a scale of the index: the norms of A's columns where a
+//   rounding has their Gram matrix (Bond), else the smaller operand's entries
+//   (index_max_kernel).  A D of powers of two then changes no bit of tt_to_full.
+//   What the smaller operand gives is not enough in a rounding: P_A's entries go like
+//   1 / sigma_j, and its largest ones would set the scale of A' columns to which they
+//   do not belong.
+// - A library call (A times the identity, disjoint supports) is held to the sum's
+//   scale: the split counts each row's entries above 2^-9 of its maximum, and
+//   unless every pair of rows has K / 16 indices where both are (tc8_lost), the
+//   product is recomputed on the FP64 pipe (the count and the check: 200,000 x 577
+//   times 577 x 96 1.73 -> 1.78 ms, the Gram of 500,000 x 449 5.68 -> 5.70; where it
+//   is recomputed, a sparse 500,000 x 449 takes 106 ms and 20,000 x 500 times the
+//   identity 9.7, on the FP64 pipe alone 143 and 9.8 before).
 #include <cuda.h>
 #include <cuda_bf16.h>
 
@@ -205,14 +215,14 @@ __device__ __forceinline__ u64 mag(double v) { return (u64)__double_as_longlong(
 __device__ __forceinline__ u64 umax(u64 a, u64 b) { return a > b ? a : b; }
 // e with every |v| <= the maximum of this pattern below 2^(e - 1); EXP_LOST (and
 // flag latched) where it is Inf, NaN or outside 2^+-900.
-__device__ __forceinline__ int split_exp(u64 mx, int* flag) {
-    const int ex = (int)(mx >> 52);
-    if (mx != 0 && (ex < 1023 - 900 || ex > 1023 + 900)) {
+__device__ __forceinline__ int split_exp(int ex, bool zero, int* flag) {
+    if (!zero && (ex < 1023 - 900 || ex > 1023 + 900)) {
         atomicOr(flag + LOST_ROWS, 1);
         return EXP_LOST;
     }
-    return mx == 0 ? 0 : ex - 1023 + 2;
+    return zero ? 0 : ex - 1023 + 2;
 }
+__device__ __forceinline__ int split_exp(u64 mx, int* flag) { return split_exp((int)(mx >> 52), mx == 0, flag); }
 // The same of a block of a row; its range is the row's matter.
 constexpr int EXP_ZERO = -EXP_LOST;  // nothing in it but zeros (and subnormals, which have no digits)
 // With it goes the number of the block's entries that have digits at all.
@@ -282,6 +292,24 @@ struct Side {
     int* worst;  // and the most that a row falls short of K (split_rows_kernel; spread_kernel)
     int* eb;     // K > ONE_EXP_K: the words of a row's blocks (block_word), a block after the other
     long ebs;    // rows of eb
+    // the contraction index's exponents (Bond; sign 0: the smaller operand's largest
+    // entries, index_max_kernel) or null, and op(A)'s sign
+    const int* ks;
+    int sign;
+    // entries at index k count as times 2^scale
+    __device__ __forceinline__ int scale(const Prod& p, long k) const {
+        const int x = ks[k];
+        if (x == 0) return 0;
+        const int s = min(max(x - 1023, -400), 400);
+        return (sign ? (sign < 0) == (isB == 0) : (isB != 0) == (p.M > p.N)) ? -s : s;
+    }
+    template <bool SCALE>
+    __device__ __forceinline__ u64 mag_at(const Prod& p, const double* q, long k) const {
+        const u64 m = mag(*q);
+        const int ex = (int)(m >> 52);
+        if (!SCALE || ex == 0 || ex == 0x7FF) return m;
+        return (m & 0xFFFFFFFFFFFFFull) | (u64)min(max(ex + scale(p, k), 1), 0x7FF) << 52;
+    }
     // the exponent for the digits of row i at index k, e the row's
     __device__ __forceinline__ int block(int e, long k, long i) const { return e == EXP_LOST ? e : block_exp(eb[k / BLK_K * ebs + i]); }
 };
@@ -292,11 +320,71 @@ __device__ __forceinline__ void side_sizes(const Prod& p, const Side& o, long& i
     ld = o.isB ? p.ldb : p.lda;
 }
 
+// The exponents of the contraction index where no Bond gives them: of the smaller
+// operand's (by rows) largest entry at each index.
+__global__ void __launch_bounds__(256) index_max_kernel(Prod p, Side a, Side b, int* out) {
+    p.Mc = p.M;
+    if (!resolve(p)) return;
+    const bool useB = p.M > p.N;
+    const long rows = useB ? p.N : p.M, ld = useB ? p.ldb : p.lda;
+    const double* q = useB ? b.p : a.p;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    constexpr long SEG = 256;
+    const long segs = (rows + SEG - 1) / SEG;
+    auto exponent = [](double v) {  // 0 of what has none
+        const int ex = (__double2hiint(v) >> 20) & 0x7FF;
+        return ex == 0x7FF ? 0 : ex;
+    };
+    if (useB ? b.strided : a.strided) {  // a warp an index and SEG rows
+        for (long t = blockIdx.x * 8L + warp; t < p.K * segs; t += gridDim.x * 8L) {
+            const long k = t / segs, i1 = min(rows, (t % segs + 1) * SEG);
+            int m = 0;
+#pragma unroll 4
+            for (long i = t % segs * SEG + lane; i < i1; i += 32) m = max(m, exponent(q[k * ld + i]));
+            m = __reduce_max_sync(0xffffffffu, m);
+            if (lane == 0 && m) atomicMax(out + k, m);
+        }
+        return;
+    }
+    __shared__ int part[8][32];
+    const long kbs = (p.K + 31) / 32;
+    for (long t = blockIdx.x; t < kbs * segs; t += gridDim.x) {  // a CTA 32 indices and SEG rows
+        const long k = t / segs * 32 + lane, i1 = min(rows, (t % segs + 1) * SEG);
+        int m = 0;
+        if (k < p.K) {
+#pragma unroll 4
+            for (long i = t % segs * SEG + warp; i < i1; i += 8) m = max(m, exponent(q[i * ld + k]));
+        }
+        __syncthreads();
+        part[warp][lane] = m;
+        __syncthreads();
+        if (warp == 0 && k < p.K) {
+#pragma unroll
+            for (int w = 1; w < 8; ++w) m = max(m, part[w][lane]);
+            if (m) atomicMax(out + k, m);
+        }
+    }
+}
+// The same from the diagonal of the bond's Gram matrix: half its exponent.
+__global__ void __launch_bounds__(256) bond_scale_kernel(int n, int rep, const double* __restrict__ G, long ldg,
+                                                         const int* __restrict__ desc, int* __restrict__ out) {
+    if (desc) {
+        n = desc[0];
+        ldg = desc[5];
+    }
+    for (int k = blockIdx.x * 256 + threadIdx.x; k < n; k += gridDim.x * 256) {
+        const double g = G[(long)k * ldg + k];
+        const int ex = __double2hiint(g) >> 20;  // negative entries: none
+        const int x = ex > 0 && ex < 0x7FF ? ((ex - 1023) >> 1) + 1023 : 0;
+        for (int q = 0; q < rep; ++q) out[(long)q * n + k] = x;
+    }
+}
+
 // Rows with a contiguous contraction index, K <= 64 V: a warp reads a row
 // once, reduces its maximum (the exponent) and writes its digits.  A lane
 // holds the pairs k = 64 t + 2 lane, so a digit store covers two whole
 // 64-byte tile rows.  Rows past the last are zero.
-template <int V>
+template <int V, bool SCALE>
 __global__ void __launch_bounds__(256) split_rows_kernel(Prod p, Side o, int* flag) {
     if (!resolve(p)) return;
     long i0, rows, rpad, ld;
@@ -306,9 +394,18 @@ __global__ void __launch_bounds__(256) split_rows_kernel(Prod p, Side o, int* fl
     const double* A = o.p + i0 * ld;
     const int lane = threadIdx.x & 31;
     const long nw = (long)gridDim.x * 8;
+    short2 sc[SCALE ? V : 1];  // the scales of this lane's indices, the same in every row
+    if (SCALE) {
+#pragma unroll
+        for (int t = 0; t < V; ++t) {
+            const int k = 64 * t + 2 * lane;
+            sc[SCALE ? t : 0] = make_short2((short)(k < K ? o.scale(p, k) : 0), (short)(k + 1 < K ? o.scale(p, k + 1) : 0));
+        }
+    }
     for (long r = (long)blockIdx.x * 8 + (threadIdx.x >> 5); r < rpad; r += nw) {
         double v[V][2];
         u64 mx = 0;
+        int top = 0;  // SCALE: the largest exponent, 0 of a zero row
         if (r < rows) {
             const double* row = A + r * ld;
 #pragma unroll
@@ -317,15 +414,30 @@ __global__ void __launch_bounds__(256) split_rows_kernel(Prod p, Side o, int* fl
                 v[t][0] = k < K ? row[k] : 0.0;
                 v[t][1] = k + 1 < K ? row[k + 1] : 0.0;
             }
+            if (SCALE) {
+                auto see = [&](double x, int s) {
+                    const int hi = __double2hiint(x) & 0x7FFFFFFF, ex = hi >> 20;
+                    int y = ex ? max(ex + s, 1) : ((hi | __double2loint(x)) ? 1 : 0);
+                    if (ex == 0x7FF) y = 4095;
+                    top = max(top, y);
+                };
 #pragma unroll
-            for (int t = 0; t < V; ++t) mx = umax(mx, umax(mag(v[t][0]), mag(v[t][1])));
+                for (int t = 0; t < V; ++t) {
+                    see(v[t][0], sc[SCALE ? t : 0].x);
+                    see(v[t][1], sc[SCALE ? t : 0].y);
+                }
+                top = __reduce_max_sync(0xffffffffu, top);
+            } else {
 #pragma unroll
-            for (int q = 16; q > 0; q >>= 1) mx = umax(mx, __shfl_xor_sync(0xffffffffu, mx, q));
+                for (int t = 0; t < V; ++t) mx = umax(mx, umax(mag(v[t][0]), mag(v[t][1])));
+#pragma unroll
+                for (int q = 16; q > 0; q >>= 1) mx = umax(mx, __shfl_xor_sync(0xffffffffu, mx, q));
+            }
         } else {
 #pragma unroll
             for (int t = 0; t < V; ++t) v[t][0] = v[t][1] = 0.0;
         }
-        const int e = split_exp(mx, flag);
+        const int e = SCALE ? split_exp(top, top == 0, flag) : split_exp(mx, flag);
         if (lane == 0 && r < rows) o.e[i0 + r] = e;
         if (o.worst && mx != 0 && e != EXP_LOST) {
             int c = 0;
@@ -341,7 +453,8 @@ __global__ void __launch_bounds__(256) split_rows_kernel(Prod p, Side o, int* fl
             const int st = 2 * t + (lane >> 4);
             if (st < nst) {
                 unsigned w[S8];
-                digits8x2(v[t][0], v[t][1], e, e, w);
+                digits8x2(v[t][0], v[t][1], e - (SCALE ? sc[SCALE ? t : 0].x : 0), e - (SCALE ? sc[SCALE ? t : 0].y : 0),
+                          w);
                 unsigned char* q = tile_at(o.img, r >> 6, nst, st, 0) + off;
 #pragma unroll
                 for (int s = 0; s < S8; ++s) *reinterpret_cast<unsigned*>(q + s * DIG_BYTES) = w[s];
@@ -350,43 +463,45 @@ __global__ void __launch_bounds__(256) split_rows_kernel(Prod p, Side o, int* fl
     }
 }
 
-// Longer rows in two passes: the maxima of their blocks, then the digits of a chunk.
+// Longer rows in two passes: the maxima of their blocks (a warp each), then the
+// digits of a chunk.
+template <bool SCALE>
 __global__ void __launch_bounds__(256) row_max_kernel(Prod p, Side o) {
     p.Mc = p.M;
     if (!resolve(p) || p.K <= ONE_EXP_K) return;
     const long rows = o.isB ? p.N : p.M, ld = o.isB ? p.ldb : p.lda;
     const int lane = threadIdx.x & 31;
     const long nw = (long)gridDim.x * 8;
-    for (long r = (long)blockIdx.x * 8 + (threadIdx.x >> 5); r < rows; r += nw) {
+    const long nblk = (p.K + BLK_K - 1) / BLK_K;
+    for (long t = (long)blockIdx.x * 8 + (threadIdx.x >> 5); t < rows * nblk; t += nw) {
+        const long r = t / nblk, kb = t % nblk, k1 = min(p.K, (kb + 1) * BLK_K);
         const double* row = o.p + r * ld;
-        u64 top = 0;
-        for (long kb = 0; kb * BLK_K < p.K; ++kb) {
-            const long k1 = min(p.K, (kb + 1) * BLK_K);
-            u64 m0 = 0, m1 = 0, m2 = 0, m3 = 0;
-            int c = 0;
-            auto see = [&](u64& m, long k) {
-                const u64 v = mag(row[k]);
-                m = umax(m, v);
-                c += (v >> 52) != 0;
-            };
-            long k = kb * BLK_K + lane;
-            for (; k + 96 < k1; k += 128) {
-                see(m0, k);
-                see(m1, k + 32);
-                see(m2, k + 64);
-                see(m3, k + 96);
-            }
-            for (; k < k1; k += 32) see(m0, k);
-            m0 = umax(umax(m0, m1), umax(m2, m3));
-            c = __reduce_add_sync(0xffffffffu, c);
-#pragma unroll
-            for (int q = 16; q > 0; q >>= 1) m0 = umax(m0, __shfl_xor_sync(0xffffffffu, m0, q));
-            if (lane == 0) o.eb[kb * o.ebs + r] = block_word(m0, c);
-            top = umax(top, m0);
+        u64 m0 = 0, m1 = 0, m2 = 0, m3 = 0;
+        int c = 0;
+        auto see = [&](u64& m, long k) {
+            const u64 v = o.mag_at<SCALE>(p, row + k, k);
+            m = umax(m, v);
+            c += (v >> 52) != 0;
+        };
+        long k = kb * BLK_K + lane;
+        for (; k + 96 < k1; k += 128) {
+            see(m0, k);
+            see(m1, k + 32);
+            see(m2, k + 64);
+            see(m3, k + 96);
         }
-        if (lane == 0) o.mx[r] = top;
+        for (; k < k1; k += 32) see(m0, k);
+        m0 = umax(umax(m0, m1), umax(m2, m3));
+#pragma unroll
+        for (int q = 16; q > 0; q >>= 1) m0 = umax(m0, __shfl_xor_sync(0xffffffffu, m0, q));
+        c = __reduce_add_sync(0xffffffffu, c);
+        if (lane == 0) {
+            o.eb[kb * o.ebs + r] = block_word(m0, c);
+            if (m0) atomicMax(o.mx + r, m0);
+        }
     }
 }
+template <bool SCALE>
 __global__ void __launch_bounds__(256) split_rows_long_kernel(Prod p, Side o, int* flag) {
     if (!resolve(p) || p.K <= ONE_EXP_K) return;
     long i0, rows, rpad, ld;
@@ -418,7 +533,8 @@ __global__ void __launch_bounds__(256) split_rows_long_kernel(Prod p, Side o, in
             if (kw == 0 && r < rows) atomicAdd(o.large + i0 + r, __popc(b0 & half) + __popc(b1 & half));
         }
         unsigned w[S8];
-        digits8x2(v0, v1, eb, eb, w);
+        const int s0 = SCALE && k < Kc ? o.scale(p, p.k0 + k) : 0, s1 = SCALE && k + 1 < Kc ? o.scale(p, p.k0 + k + 1) : 0;
+        digits8x2(v0, v1, eb - s0, eb - s1, w);
         unsigned char* d = tile_at(o.img, r >> 6, nst, st, 0) + swz((int)(r & 63), 2 * kw);
 #pragma unroll
         for (int s = 0; s < S8; ++s) *reinterpret_cast<unsigned*>(d + s * DIG_BYTES) = w[s];
@@ -431,6 +547,7 @@ __global__ void __launch_bounds__(256) split_rows_long_kernel(Prod p, Side o, in
 // stores 16 bytes a digit.  Bound by the latency of its loads: 8 rows fit 64
 // registers, four CTAs an SM (49,152 x 449: 156 us, 3.7 TB/s; with 16 rows a
 // thread, 128 registers and two CTAs 251 us, with 48 registers and spills 230).
+template <bool SCALE>
 __global__ void __launch_bounds__(256) strided_max_kernel(Prod p, Side o) {
     p.Mc = p.M;
     if (!resolve(p)) return;
@@ -448,7 +565,7 @@ __global__ void __launch_bounds__(256) strided_max_kernel(Prod p, Side o) {
             u64 m0 = 0, m1 = 0, m2 = 0, m3 = 0;
             int c = 0;
             auto see = [&](u64& m, long k) {
-                const u64 v = mag(o.p[k * ld + j]);
+                const u64 v = o.mag_at<SCALE>(p, o.p + k * ld + j, k);
                 m = umax(m, v);
                 c += (v >> 52) != 0;
             };
@@ -480,7 +597,7 @@ __global__ void __launch_bounds__(256) strided_max_kernel(Prod p, Side o) {
         if (threadIdx.x < 32 && j < n && top) atomicMax(o.mx + j, top);
     }
 }
-template <bool GUARD>
+template <bool GUARD, bool SCALE>
 __global__ void __launch_bounds__(256, 4) split_strided_kernel(Prod p, Side o, int* flag) {
     __shared__ int s_large[GUARD ? 32 : 1];
     if (!resolve(p)) return;
@@ -520,7 +637,8 @@ __global__ void __launch_bounds__(256, 4) split_strided_kernel(Prod p, Side o, i
             for (int r = 0; r < 8; ++r) {
                 const unsigned sign = ((unsigned)(F[r] >> 48) & 0x8000u) << (16 * (r & 1));
                 sg[r >> 1] = r & 1 ? sg[r >> 1] | sign : sign;
-                F[r] = biased56(__longlong_as_double((long long)F[r]), eb);
+                F[r] = biased56(__longlong_as_double((long long)F[r]),
+                                eb - (SCALE && k0 + r < Kc ? o.scale(p, p.k0 + k0 + r) : 0));
             }
             unsigned char* d = tile_at(o.img, j >> 6, nst, (int)(g >> 2), 0) + swz((int)(j & 63), (int)(g & 3) * 8);
 #pragma unroll
@@ -933,7 +1051,7 @@ unsigned blocks_for(long work, long cap) { return (unsigned)std::max<long>(1, st
 // descriptor's).
 tt_status run(cudaStream_t s, bool ta, bool tb, long M, long N, long K, double alpha, const double* A, long lda,
               const double* B, long ldb, double* C, long ldc, DevBuf& scratch, int* status_dev, bool gram,
-              const int* desc, bool guard, Lost* lost, long long limit = SPIN) {
+              const int* desc, bool guard, const Bond* bond, Lost* lost, long long limit = SPIN) {
     const Plan q = make_plan(M, N, K, gram, desc != nullptr);
     // slack to bring the base to a 1024-byte boundary (a pool may give 256)
     TT_TRY(scratch.ensure((q.bytes() + 1024 + 7) / 8, s));
@@ -941,13 +1059,17 @@ tt_status run(cudaStream_t s, bool ta, bool tb, long M, long N, long K, double a
     int* flag = reinterpret_cast<int*>(base);
     u64* mx = reinterpret_cast<u64*>(base + 256);
     const long nrows = gram ? M : M + N;
-    int* ex = reinterpret_cast<int*>(mx + nrows);
+    const bool scale = !gram && !guard && !(bond && !bond->s), find = scale && !bond;
+    int* kx = reinterpret_cast<int*>(mx + nrows);  // of its own, found below
+    const int* ks = !scale ? nullptr : find ? kx : bond->s;
+    const int sign = bond ? bond->sign : 0;
+    int* ex = kx + (gram ? 0 : K);
     int* large = guard ? ex + nrows : nullptr;
     int* worst = guard ? flag + LOST_WORST : nullptr;
     int* eb = ex + 2 * nrows;  // behind the counts
-    Side a{A, 0, ta ? 1 : 0, mx, ex, base + q.head + q.imgB, large, worst, eb, M};
+    Side a{A, 0, ta ? 1 : 0, mx, ex, base + q.head + q.imgB, large, worst, eb, M, ks, sign};
     Side b{B, 1, tb ? 0 : 1, mx + M, ex + M, base + q.head, guard ? large + M : nullptr, guard ? worst + 1 : nullptr,
-           eb + (K + BLK_K - 1) / BLK_K * M, N};
+           eb + (K + BLK_K - 1) / BLK_K * M, N, ks, sign};
     if (gram) {
         a.img = base + q.head;
         b = a;
@@ -960,18 +1082,20 @@ tt_status run(cudaStream_t s, bool ta, bool tb, long M, long N, long K, double a
     TT_TRY(ensure_max_dynamic_smem((const void*)tc8_kernel<false>));
     TT_TRY(ensure_max_dynamic_smem((const void*)tc8_kernel<true>));
     // the flag and, where atomics find them, the maxima and counts start at zero
-    TT_CUDA_TRY(cudaMemsetAsync(flag, 0, 256 + (a.strided || b.strided ? 8 * (size_t)nrows : 0), s));
+    const size_t maxima_bytes = a.strided || b.strided || K > ONE_EXP_K || find ? 8 * (size_t)nrows : 0;
+    TT_CUDA_TRY(cudaMemsetAsync(flag, 0, 256 + maxima_bytes + (find ? 4 * (size_t)K : 0), s));
     if (guard) TT_CUDA_TRY(cudaMemsetAsync(large, 0, 4 * (size_t)nrows, s));
     const bool fusable = K <= ONE_EXP_K;  // a captured step launches both forms when K may be longer
     auto maxima = [&](const Side& o) {
         const long rows = o.isB ? N : M;
         if (o.strided) {
             note_launch();
-            strided_max_kernel<<<dim3(blocks_for((rows + 31) / 32, 4096), blocks_for(K / (fusable ? 256 : BLK_K), 512)), 256, 0, s>>>(
-                p, o);
+            const dim3 grid(blocks_for((rows + 31) / 32, 4096), blocks_for(K / (fusable ? 256 : BLK_K), 512));
+            (scale ? strided_max_kernel<true> : strided_max_kernel<false>)<<<grid, 256, 0, s>>>(p, o);
         } else if (!fusable) {
             note_launch();
-            row_max_kernel<<<blocks_for((rows + 7) / 8, 152L * 64), 256, 0, s>>>(p, o);
+            const unsigned grid = blocks_for((rows * ((K + BLK_K - 1) / BLK_K) + 7) / 8, 152L * 64);
+            (scale ? row_max_kernel<true> : row_max_kernel<false>)<<<grid, 256, 0, s>>>(p, o);
         }
     };
     auto split = [&](const Side& o) {
@@ -980,15 +1104,15 @@ tt_status run(cudaStream_t s, bool ta, bool tb, long M, long N, long K, double a
         if (o.strided) {
             const dim3 grid(blocks_for((rpad + 31) / 32, 4096), blocks_for(((long)nst * 2 + 7) / 8, 2048));
             note_launch();
-            if (guard)
-                split_strided_kernel<true><<<grid, 256, 0, s>>>(p, o, flag);
-            else
-                split_strided_kernel<false><<<grid, 256, 0, s>>>(p, o, flag);
+            (guard   ? split_strided_kernel<true, false>
+             : scale ? split_strided_kernel<false, true>
+                     : split_strided_kernel<false, false>)<<<grid, 256, 0, s>>>(p, o, flag);
             return;
         }
         if (!fusable) {
             note_launch();
-            split_rows_long_kernel<<<blocks_for((rpad * nst * 16 + 255) / 256, 152L * 64), 256, 0, s>>>(p, o, flag);
+            const unsigned long_grid = blocks_for((rpad * nst * 16 + 255) / 256, 152L * 64);
+            (scale ? split_rows_long_kernel<true> : split_rows_long_kernel<false>)<<<long_grid, 256, 0, s>>>(p, o, flag);
             if (!desc) return;
         }
         const unsigned grid = blocks_for((rpad + 7) / 8, 152L * 64);
@@ -997,24 +1121,29 @@ tt_status run(cudaStream_t s, bool ta, bool tb, long M, long N, long K, double a
         // product launches each that a size up to its capacity may need
         if (desc ? true : need <= 4) {
             note_launch();
-            split_rows_kernel<2><<<grid, 256, 0, s>>>(p, o, flag);
+            (scale ? split_rows_kernel<2, true> : split_rows_kernel<2, false>)<<<grid, 256, 0, s>>>(p, o, flag);
         }
         if (need > 4 && (desc || need <= 8)) {
             note_launch();
-            split_rows_kernel<4><<<grid, 256, 0, s>>>(p, o, flag);
+            (scale ? split_rows_kernel<4, true> : split_rows_kernel<4, false>)<<<grid, 256, 0, s>>>(p, o, flag);
         }
         if (need > 8 && (desc || need <= 16)) {
             note_launch();
-            split_rows_kernel<8><<<grid, 256, 0, s>>>(p, o, flag);
+            (scale ? split_rows_kernel<8, true> : split_rows_kernel<8, false>)<<<grid, 256, 0, s>>>(p, o, flag);
         }
         if (need > 16) {
             note_launch();
-            split_rows_kernel<16><<<grid, 256, 0, s>>>(p, o, flag);
+            (scale ? split_rows_kernel<16, true> : split_rows_kernel<16, false>)<<<grid, 256, 0, s>>>(p, o, flag);
         }
     };
     const int nst0 = stages(q.Kc);
     const int spc = split_stages(M, N, tiles_of(q.Mc, N, gram), nst0, split_unit(K));
     const bool direct = !desc && !gram && q.Kc >= K && spc >= nst0;
+    if (find) {
+        const long segs = (std::min(M, N) + 255) / 256;
+        note_launch();
+        index_max_kernel<<<blocks_for(std::max((K + 31) / 32, K / 8) * segs, 152L * 8), 256, 0, s>>>(p, a, b, kx);
+    }
     maxima(a);
     if (!gram) maxima(b);
     for (p.k0 = 0; p.k0 < K; p.k0 += q.Kc) {
@@ -1070,23 +1199,30 @@ size_t tc8_reserve_doubles(long M, long N, long K, bool gram) {
     return (reserve_bytes(M, N, K, gram) + 1024 + 7) / 8;
 }
 
+void bond_scale(cudaStream_t s, int n, int rep, const double* G, long ldg, int* out, const int* desc) {
+    if (n <= 0) return;
+    note_launch();
+    bond_scale_kernel<<<blocks_for((n + 255) / 256, 152), 256, 0, s>>>(n, rep, G, ldg, desc, out);
+}
+
 size_t tc8_head_doubles(long M, long N, long K, bool gram) { return (head_bytes(M, N, K, gram) + 1024 + 7) / 8; }
 
 tt_status tc8_gemm(cudaStream_t s, bool ta, bool tb, long M, long N, long K, double alpha, const double* A, long lda,
                    const double* B, long ldb, double* C, long ldc, DevBuf& scratch, int* status_dev, bool guard,
-                   Lost* lost, bool probe) {
-    return run(s, ta, tb, M, N, K, alpha, A, lda, B, ldb, C, ldc, scratch, status_dev, false, nullptr, guard, lost,
+                   const Bond* bond, Lost* lost, bool probe) {
+    return run(s, ta, tb, M, N, K, alpha, A, lda, B, ldb, C, ldc, scratch, status_dev, false, nullptr, guard, bond, lost,
                probe ? 0 : SPIN);
 }
 
 tt_status tc8_gram(cudaStream_t s, long m, long n, const double* A, long lda, double* G, long ldg, DevBuf& scratch,
                    int* status_dev, bool guard, Lost* lost) {
-    return run(s, true, false, n, n, m, 1.0, A, lda, A, lda, G, ldg, scratch, status_dev, true, nullptr, guard, lost);
+    return run(s, true, false, n, n, m, 1.0, A, lda, A, lda, G, ldg, scratch, status_dev, true, nullptr, guard, nullptr, lost);
 }
 
 tt_status tc8_dyn(cudaStream_t s, bool ta, bool tb, const int* desc, long Mcap, long Ncap, long Kcap, double alpha,
-                  const double* A, const double* B, double* C, DevBuf& scratch, int* status_dev, bool gram, Lost* lost) {
-    return run(s, ta, tb, Mcap, Ncap, Kcap, alpha, A, 0, B, 0, C, 0, scratch, status_dev, gram, desc, false, lost);
+                  const double* A, const double* B, double* C, DevBuf& scratch, int* status_dev, bool gram,
+                  const Bond* bond, Lost* lost) {
+    return run(s, ta, tb, Mcap, Ncap, Kcap, alpha, A, 0, B, 0, C, 0, scratch, status_dev, gram, desc, false, bond, lost);
 }
 
 }  // namespace ttsn

@@ -93,10 +93,10 @@ struct Plan {
     size_t bytes() const { return head + imgA + imgB + part; }
 };
 // Flags; per row its largest entry, exponent and count of large entries, and
-// the exponents of its blocks.
+// the exponents of its blocks; the exponents of the contraction index.
 inline size_t head_bytes(long M, long N, long K, bool gram) {
     const long rows = gram ? M : M + N;
-    return (size_t)up(256 + 16 * rows + (K > ONE_EXP_K ? 4 * rows * ((K + BLK_K - 1) / BLK_K) : 0) + 64, 1024);
+    return (size_t)up(256 + 16 * rows + (gram ? 0 : 4 * K) + (K > ONE_EXP_K ? 4 * rows * ((K + BLK_K - 1) / BLK_K) : 0) + 64, 1024);
 }
 inline Plan make_plan(long M, long N, long K, bool gram, bool captured) {
     Plan p;

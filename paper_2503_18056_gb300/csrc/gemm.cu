@@ -593,7 +593,7 @@ tt_status dgemm(cudaStream_t s, bool ta, bool tb, int M, int N, int K, double al
 
 tt_status dgemm_sk(cudaStream_t s, bool ta, bool tb, int M, int N, int K, double alpha,
                    const double* A, long lda, const double* B, long ldb, double* C, long ldc,
-                   DevBuf& scratch, const ProdCtx& ctx, bool split) {
+                   DevBuf& scratch, const ProdCtx& ctx, bool split, const Bond* bond) {
     int ks = 1, chunk = K;
     if (split && M > 0 && N > 0 && K > 0) ks = ordered_split(M, N, K, 0, &chunk);
     const size_t part = split_scratch(prod_tiles(M, N, 0), ks);
@@ -602,7 +602,7 @@ tt_status dgemm_sk(cudaStream_t s, bool ta, bool tb, int M, int N, int K, double
         // without room for the digits: the FP64 pipe
         tt_status st = scratch.ensure(digits_doubles(M, N, K, 0, ks), s);
         if (st >= 0)
-            st = tc8_gemm(s, ta, tb, M, N, K, alpha, A, lda, B, ldb, C, ldc, scratch, ctx.status, false, &lost);
+            st = tc8_gemm(s, ta, tb, M, N, K, alpha, A, lda, B, ldb, C, ldc, scratch, ctx.status, false, bond, &lost);
         if (st >= 0)
             return split_prod(s, ta, tb, true, ProdArgs{M, N, K, alpha, A, lda, B, ldb, 0.0, C, ldc, ks, chunk, lost.free,
                                                         ctx.counters, 0, nullptr, lost});
@@ -661,7 +661,7 @@ tt_status gemm_call(cudaStream_t s, bool ta, bool tb, int M, int N, int K, doubl
     const int ks = prod_split(M, N, K, 0);
     ProdArgs a{M, N, K, alpha, A, lda, B, ldb, 0.0, C, ldc, ks, prod_chunk(K, ks), scratch.p, nullptr, 0, nullptr};
     if (tc8_wanted(M, N, K)) {
-        TT_TRY(tc8_gemm(s, ta, tb, M, N, K, alpha, A, lda, B, ldb, C, ldc, scratch, nullptr, true, &a.lost, probe));
+        TT_TRY(tc8_gemm(s, ta, tb, M, N, K, alpha, A, lda, B, ldb, C, ldc, scratch, nullptr, true, nullptr, &a.lost, probe));
         a.P = a.lost.free;
     }
     return split_prod(s, ta, tb, false, a);
@@ -738,12 +738,12 @@ size_t dyn_partials_need(int mode, int Mcap, int Ncap, int Kcap) {
 
 tt_status dgemm_dyn(cudaStream_t s, bool ta, bool tb, const int* desc, int Mcap, int Ncap, int Kcap,
                     double alpha, const double* A, const double* B, double* C, double* P, size_t pcap, int mode,
-                    DevBuf& tcbuf, const ProdCtx& ctx) {
+                    DevBuf& tcbuf, const ProdCtx& ctx, const Bond* bond) {
     if (Mcap <= 0 || Ncap <= 0) return TT_OK;
     const int tri = mode == 2 ? 1 : 0;
     Lost lost;
     if (ctx.digits && tc8_wanted(Mcap, Ncap, Kcap))
-        TT_TRY(tc8_dyn(s, ta, tb, desc, Mcap, Ncap, Kcap, alpha, A, B, C, tcbuf, ctx.status, mode == 2, &lost));
+        TT_TRY(tc8_dyn(s, ta, tb, desc, Mcap, Ncap, Kcap, alpha, A, B, C, tcbuf, ctx.status, mode == 2, bond, &lost));
     if (lost.flag && tri) gram_check(s, Ncap, Kcap, C, 0, desc, lost);
     const size_t need = dyn_partials_need(mode, Mcap, Ncap, Kcap);
     if (need > pcap) {

@@ -87,11 +87,22 @@ struct ProdCtx {
     int* counters = nullptr;
     bool digits = true;
 };
-// beta = 0 product of a rounding: from digits (digits.cu) where tc8_wanted,
-// else on the FP64 pipe, K split over CTAs by sk_split's rule (split) or not.
+// The index that a rounding's product contracts: digits.cu takes op(A)'s entries at
+// index k times 2^(sign (s[k] - 1023)) and op(B)'s times the inverse, s[k] = 0: as
+// they are (s null: all).  bond_scale: s from the diagonal of the bond's Gram matrix G
+// (n x n), rep times over; n and ldg from desc[0] and [5] where given (n then is
+// the capacity).
+struct Bond {
+    const int* s = nullptr;
+    int sign = 0;
+};
+void bond_scale(cudaStream_t s, int n, int rep, const double* G, long ldg, int* out, const int* desc = nullptr);
+// beta = 0 product of a handle: from digits (digits.cu) where tc8_wanted, else on
+// the FP64 pipe, K split over CTAs by sk_split's rule (split) or not.  bond null: the
+// index's scale from the smaller operand.
 tt_status dgemm_sk(cudaStream_t s, bool ta, bool tb, int M, int N, int K, double alpha,
                    const double* A, long lda, const double* B, long ldb, double* C, long ldc,
-                   DevBuf& scratch, const ProdCtx& ctx, bool split = true);
+                   DevBuf& scratch, const ProdCtx& ctx, bool split = true, const Bond* bond = nullptr);
 // The same of a library call: the order of summation is free, the split the
 // cheapest.  Scratch of gemm_call_doubles.
 size_t gemm_call_doubles(int M, int N, int K);
@@ -121,7 +132,7 @@ constexpr int GRAM_MULTI_SPLITS = 64;
 // TT_ERR_TOO_LARGE); tcbuf: scratch of tc8_dyn, reserved ahead of the capture.
 tt_status dgemm_dyn(cudaStream_t s, bool ta, bool tb, const int* desc, int Mcap, int Ncap, int Kcap,
                     double alpha, const double* A, const double* B, double* C, double* P, size_t pcap, int mode,
-                    DevBuf& tcbuf, const ProdCtx& ctx);
+                    DevBuf& tcbuf, const ProdCtx& ctx, const Bond* bond = nullptr);
 size_t dyn_partials_need(int mode, int Mcap, int Ncap, int Kcap);
 // scale_rows with rows, cols, ldi, ldo = desc[0..3] (rows * cols <= total_cap)
 void scale_rows_dyn(cudaStream_t s, const int* desc, long total_cap, const double* in, const double* v, int mode,
@@ -212,13 +223,14 @@ size_t tc8_head_doubles(long M, long N, long K, bool gram);
 // probe: every wait of the product's kernel gives up at once (tt_digits_wait_probe).
 tt_status tc8_gemm(cudaStream_t s, bool ta, bool tb, long M, long N, long K, double alpha, const double* A, long lda,
                    const double* B, long ldb, double* C, long ldc, DevBuf& scratch, int* status_dev, bool guard,
-                   Lost* lost, bool probe = false);
+                   const Bond* bond, Lost* lost, bool probe = false);
 tt_status tc8_gram(cudaStream_t s, long m, long n, const double* A, long lda, double* G, long ldg, DevBuf& scratch,
                    int* status_dev, bool guard, Lost* lost);
 // The captured form: sizes from desc (as dgemm_dyn's), at most the capacities;
 // does nothing for sizes that tc8_wanted leaves to the FP64 pipe.
 tt_status tc8_dyn(cudaStream_t s, bool ta, bool tb, const int* desc, long Mcap, long Ncap, long Kcap, double alpha,
-                  const double* A, const double* B, double* C, DevBuf& scratch, int* status_dev, bool gram, Lost* lost);
+                  const double* A, const double* B, double* C, DevBuf& scratch, int* status_dev, bool gram,
+                  const Bond* bond, Lost* lost);
 
 // Row scaling: out[i][j] = in[i][j] * f(v[i]) for i < rows, j < cols, where
 // mode 0: v, 1: sqrt(v), 2: 1/sqrt(v), 3: 1/v.  out may alias in.

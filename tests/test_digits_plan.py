@@ -34,7 +34,7 @@ static void check(const Plan& q, bool captured, bool gram, long Mc, long Nc, lon
     if (up(N, gram ? T_M : RB) * nst * stage > q.imgB) fail("image B", Mc, Nc, Kc, M, N, K);
     if (!gram && up(rows, T_M) * nst * stage > q.imgA) fail("image A", Mc, Nc, Kc, M, N, K);
     const size_t side = gram ? M : M + N;
-    if (q.head < 256 + 16 * side + (K > ONE_EXP_K ? 4 * side * ((K + BLK_K - 1) / BLK_K) : 0)) fail("head", Mc, Nc, Kc, M, N, K);
+    if (q.head < 256 + 16 * side + (gram ? 0 : 4 * K) + (K > ONE_EXP_K ? 4 * side * ((K + BLK_K - 1) / BLK_K) : 0)) fail("head", Mc, Nc, Kc, M, N, K);
     // a contraction that goes in chunks is cut between exact blocks
     if (K > q.Kc && (q.Kc % BLK_K || spc % T_BLK)) fail("cut", Mc, Nc, Kc, M, N, K);
     if (q.Kc < Kc && q.Kc % (T_K * T_BLK)) fail("chunk", Mc, Nc, Kc, M, N, K);
