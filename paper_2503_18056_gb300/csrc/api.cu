@@ -2106,7 +2106,7 @@ struct ShardArgs {
 };
 
 tt_status create_impl(const tt_problem_desc* desc, void* stream, const tt_allocator* alloc,
-                      const ShardArgs* sh, tt_handle* out, bool digits = true) {
+                      const ShardArgs* sh, tt_handle* out) {
     if (!desc || !out) return fail(TT_ERR_ARG, "tt_create: null argument");
     if (alloc && (!alloc->alloc || !alloc->free))
         return fail(TT_ERR_ARG, "tt_create_ex: allocator needs both alloc and free");
@@ -2188,7 +2188,6 @@ tt_status create_impl(const tt_problem_desc* desc, void* stream, const tt_alloca
     }
     AllocScope alloc_scope_(h->alloc_ptr());
     cudaStream_t s = (cudaStream_t)stream;
-    h->prod.digits = digits;
     tt_status st = h->init_common(s);
     if (st < 0) {
         delete h;
@@ -2456,7 +2455,7 @@ tt_status create_impl(const tt_problem_desc* desc, void* stream, const tt_alloca
         TT_CREATE_TRY(h->GA.ensure((size_t)(R1 * R1), s));
         TT_CREATE_TRY(h->partials.ensure(D.precision == TT_MIXED ? slgram_scratch_doubles((int)nc, (int)R1)
                                                                  : gram_scratch_doubles((int)nc, (int)R1), s));
-        if (D.precision != TT_MIXED && digits) {
+        if (D.precision != TT_MIXED) {
             // digit images and planes of the capped step's products; a handle
             // without room for them runs on the FP64 pipe
             const long c[][4] = {{1, R1, R1, nc}, {0, nc, cap1, R1}, {0, R1 * D.n_theta, R2, R2},
@@ -3354,10 +3353,3 @@ tt_status tt_bench_bf16_mma(double* tflops_host, void* stream) {
 }
 
 }  // extern "C"
-
-namespace ttsn {
-tt_status create_in_batch(const tt_problem_desc* desc, void* stream, tt_handle* out) {
-    set_error("");
-    return create_impl(desc, stream, nullptr, nullptr, out, false);
-}
-}  // namespace ttsn

@@ -1,5 +1,5 @@
 // Batched form: many independent TT-S_N problems of uneven sizes stepped
-// together.  Each problem is a full handle on its own CUDA stream;
+// together.  Each problem is a full handle (tt_create) on its own CUDA stream;
 // a pool of host threads advances the problems concurrently, so the small
 // per-problem kernels of different problems overlap on the GPU and each
 // problem's rank decisions wait only for its own stream.  With captured steps
@@ -71,7 +71,7 @@ tt_status tt_batch_create(const tt_problem_desc* descs, int count, int threads, 
         }
         b->streams.push_back(s);
         tt_handle h = nullptr;
-        tt_status st = create_in_batch(&descs[i], s, &h);
+        tt_status st = tt_create(&descs[i], s, &h);
         if (st < 0) {
             std::string msg = std::string("tt_batch_create: problem ") + std::to_string(i) + ": " + tt_last_error();
             delete b;

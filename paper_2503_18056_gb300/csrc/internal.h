@@ -78,9 +78,11 @@ tt_status dgemm(cudaStream_t s, bool ta, bool tb, int M, int N, int K, double al
 
 // What a handle's products share: the device status word, PROD_COUNTERS arrival
 // counters (zero between products of the handle's stream; null: in the
-// product's scratch, for a memset) and whether digit products are taken.  The
-// problems of a batch do without: side by side they fill the FP64 pipes, and
-// 16 captured problems gained nothing from the digits' launches.
+// product's scratch, for a memset) and whether digit products are taken (not by a
+// captured handle that found no room for them).  The sizes decide (tc8_wanted), not
+// whether a problem is alone or in a batch: the same bits.  16 problems of 48^2 to
+// 128^2 cells side by side, 4 steps: 13.9 ms with digits and host threads (14.7
+// without), 14.2 captured (13.9); alone at cap 48, 128^2: 7.8 ms a step (8.8).
 constexpr long PROD_COUNTERS = 1 << 14;
 struct ProdCtx {
     int* status = nullptr;
@@ -311,9 +313,6 @@ tt_status syev_dyn(cudaStream_t s, const int* n_dev, int ncap, const double* G, 
 // failed factorisation, counts as zero)
 void truncation_decision_dyn(cudaStream_t s, const double* lamK, const int* kB_dev, double eps, int dm1,
                              int forced, int max_rank, double* delta2_dev, int* dec_i, double* dec_d);
-
-// A handle of a batch: as tt_create, its products without digits (ProdCtx).
-tt_status create_in_batch(const tt_problem_desc* desc, void* stream, tt_handle* out);
 
 // Captured steps of one handle (api.cu): graph_steps_begin checks the
 // conditions and launches nsteps replays without waiting; graph_steps_end

@@ -63,3 +63,21 @@ def test_batch_of_the_64_problem_workload_builds_and_steps(ttsn):
         assert max(info["ranks"]) <= p["max_rank"]
         E, T, _ = batch.problem(i).energy()
         assert np.isfinite(E.cpu().numpy()).all() and np.isfinite(T.cpu().numpy()).all()
+
+
+@pytest.mark.parametrize("graph", [False, True])
+def test_batch_equals_individual_runs_bitwise_at_digit_product_sizes(ttsn, graph):
+    """Grids whose products have more than 16M terms: the rule by which they are digit
+    products is the sizes', not the batch's."""
+    ps = [workloads.problem("small_2d", n=(m, m), n_theta=16, n_phi=32, eps=1e-6, max_rank=cap)
+          for m, cap in ((128, 48), (160, 48), (96, 64))]
+    batch = ttsn.TTSNBatch(ps, threads=3)
+    batch.set_graph(graph)
+    infos = batch.step(4)
+    for i, p in enumerate(ps):
+        alone = ttsn.TTSN.from_problem(p)
+        info = alone.step(4)
+        assert info["ranks"] == infos[i]["ranks"]
+        assert p["n"][0] ** 2 * (5 * info["ranks"][1] + 1) ** 2 > 16e6
+        for x, y in zip(alone.cores(), batch.problem(i).cores()):
+            assert np.array_equal(x.cpu().numpy(), y.cpu().numpy())
