@@ -41,3 +41,34 @@ def test_syev_psd_and_pchol(n, full):
     U = V[lam > 0]
     # unit rows, orthogonal to the skip threshold sqrt(n) eps and the rounding of the product
     assert np.abs(U @ U.T - np.eye(len(U))).max() <= 8 * (n + 1) * EPS
+
+
+# pairs of a CTA (four warps a pair up to twice the SMs' rows, then two), the grid
+# kernel's longest rows and the streaming kernel above them
+@pytest.mark.parametrize("n,rank", [(304, 304), (305, 305), (700, 300), (1024, 1024), (1024, 500), (1025, 1025), (1100, 1050)])
+def test_syev_psd_between_the_grid_kernels(n, rank):
+    K = graded(n, rank, n)
+    lam, V, _ = T.syev_psd(torch.tensor(K, device="cuda"))
+    lam, V = lam.cpu().numpy(), V.cpu().numpy()
+    tol = 64 * (n + 1) * EPS * lam[0]
+    assert np.all(np.diff(lam) <= 0) and lam[-1] >= 0
+    assert np.abs(lam - np.linalg.eigvalsh(K)[::-1]).max() <= tol
+    assert np.abs((V.T * lam) @ V - K).max() <= tol
+    U = V[lam > 0]
+    assert np.abs(U @ U.T - np.eye(len(U))).max() <= 8 * (n + 1) * EPS
+
+
+def test_captured_eigensolves_below_a_capacity_above_the_grid_kernel():
+    """Cap 210 in 2D: 1,051 grown columns, so a captured step launches all three
+    kernels and each size takes the host path's."""
+    import workloads
+
+    p = workloads.problem("small_2d", n=(32, 30), n_theta=16, n_phi=32, eps=1e-6, bc=1)
+    p["max_rank"] = 210
+    a, b = T.TTSN.from_problem(p), T.TTSN.from_problem(p)
+    b.set_graph(True)
+    for _ in range(5):
+        assert a.step()["ranks"] == b.step()["ranks"]
+    assert 5 * a.ranks()[1] + 1 > 256
+    for x, y in zip(a.cores(), b.cores()):
+        assert torch.equal(torch.as_tensor(x), torch.as_tensor(y))
