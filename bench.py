@@ -785,17 +785,21 @@ def roofline_of(prof, fp64_peak, peaks):
         achieved = ph["flops"] / (ph["ms"] * 1e-3) / 1e12
         peak = fp64_peak
         traffic = GRAM_LEFT_CAP_TRAFFIC if name == "gram_left" else None
-        return name, {"bound": "tensor", "achieved": achieved, "peak": peak, "unit": "TFLOP/s",
-                      "frac": achieved / peak if peak else None, "traffic": traffic,
-                      "traffic_note": "ncu DRAM read+write bytes of one capped 2,097,152 x 897 Gram (scaled "
-                                      "by the rows from a 500,000 x 897 capture)" if traffic else None,
-                      "kernel": name, "dtype": "f64", "avg_phase_ms": avg_ms,
-                      "launches": ph["launches"], "calls": ph["calls"],
-                      "peak_source": "measured FP64 tensor pipe (mma.m8n8k4.f64 chains on all SMs, "
-                                     "tt_bench_fp64_mma); MEASURED_PEAKS.json has no FP64 figure; large "
-                                     "products run as exact digit products on the BF16 tensor cores, so "
-                                     "frac may exceed 1",
-                      "digits": digit_roofline(ph, peaks)}
+        roof = {"bound": "tensor", "achieved": achieved, "peak": peak, "unit": "TFLOP/s",
+                "frac": achieved / peak if peak else None, "traffic": traffic,
+                "traffic_note": "ncu DRAM read+write bytes of one capped 2,097,152 x 897 Gram (scaled "
+                                "by the rows from a 500,000 x 897 capture)" if traffic else None,
+                "kernel": name, "dtype": "f64", "avg_phase_ms": avg_ms,
+                "launches": ph["launches"], "calls": ph["calls"],
+                "peak_source": "measured FP64 tensor pipe (mma.m8n8k4.f64 chains on all SMs, "
+                               "tt_bench_fp64_mma); MEASURED_PEAKS.json has no FP64 figure"}
+        if peak and achieved > peak:
+            # above the FP64 pipe's peak the products ran as digit products: the rate
+            # executed on the BF16 tensor cores is the one with a roofline
+            roof.update(digit_roofline(ph, peaks))
+            roof.update(dtype="f64 from bf16 digit products", fp64_equivalent_tflops=achieved, fp64_pipe_tflops=peak,
+                        peak_source="MEASURED_PEAKS.json, sustained BF16 (36 digit products a term, csrc/digits.cu)")
+        return name, roof
     achieved = ph["bytes"] / (ph["ms"] * 1e-3) / 1e9
     peak = peaks.get("hbm_gbs", 6800.0)
     return name, {"bound": "hbm", "achieved": achieved, "peak": peak, "unit": "GB/s",

@@ -534,8 +534,9 @@ void launch_one(cudaStream_t s, bool ordered, unsigned grid, const ProdArgs& a) 
 
 tt_status launch_prod(cudaStream_t s, bool ta, bool tb, bool ordered, long items, const ProdArgs& a) {
     // more CTAs than fit at once let the scheduler level uneven tiles; behind a
-    // digit product they seldom have any
-    const unsigned grid = (unsigned)std::max(1L, std::min(items, a.lost.flag && !a.desc ? 152L * 8 : 152L * 64));
+    // rounding's digit product they seldom have any (a library call may lose all)
+    const bool idle = a.lost.flag && !a.lost.guard && !a.desc;
+    const unsigned grid = (unsigned)std::max(1L, std::min(items, idle ? 152L * 8 : 152L * 64));
     note_launch();
     if (ta && tb)
         launch_one<true, true>(s, ordered, grid, a);
