@@ -739,11 +739,11 @@ __device__ __forceinline__ void tile_of(long t, int nb, bool tri, long& mb, int&
 // FP32 accumulators of 128 x 64 (one per level, all 512 TMEM columns); the digit
 // tiles of B lie back to back, so A's digit s meets up to four of B's digits in
 // one MMA of N <= 256 whose levels are neighbouring column ranges.  Sixteen warps
-// drain a block's accumulators into 64-bit integers (a float-to-int and a wide
-// multiply-add a value) and, at an item's end, write the FP64 results while the
-// next item's MMAs run.
+// drain a block's accumulators into integers (a float-to-int and a wide multiply-add
+// a value, with an exponent a block also a shifted 96-bit addition an output) and, at
+// an item's end, write the FP64 results while the next item's MMAs run.
 //
-// What bounds it: the tensor cores (74% of their cycles; 1184 clocks of MMA per
+// What bounds it: the tensor cores (72% of their cycles; 1184 clocks of MMA per
 // 16 indices against 937 of operand reads and 375 of arrivals in shared memory),
 // then the drains, which the MMAs wait for: TMEM holds one set of accumulators.
 // The issuing thread must not be what bounds it: with a rolled loop, descriptors

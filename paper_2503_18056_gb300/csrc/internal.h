@@ -82,7 +82,8 @@ tt_status dgemm(cudaStream_t s, bool ta, bool tb, int M, int N, int K, double al
 // captured handle that found no room for them).  The sizes decide (tc8_wanted), not
 // whether a problem is alone or in a batch: the same bits.  16 problems of 48^2 to
 // 128^2 cells side by side, 4 steps: 13.9 ms with digits and host threads (14.7
-// without), 14.2 captured (13.9); alone at cap 48, 128^2: 7.8 ms a step (8.8).
+// without), 14.2 captured (13.9); 64 problems of 64^2 to 256^2, a step each: 13.4
+// ms (17.5), captured 17.2 (18.3); alone at cap 48, 128^2: 7.8 ms a step (8.8).
 constexpr long PROD_COUNTERS = 1 << 14;
 struct ProdCtx {
     int* status = nullptr;
