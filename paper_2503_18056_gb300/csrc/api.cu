@@ -1616,6 +1616,9 @@ tt_status graph_reserve(tt_ctx* h) {
         {&h->dyn_part, (long)part},
     };
     for (auto& x : need) TT_TRY(x.b->ensure((size_t)std::max<long>(x.n, 1), s, /*keep=*/true));
+    TT_TRY(eig_reserve(h->eig, s));
+    TT_TRY(h->dyn_buf.ensure((size_t)(DYN_INTS + 1) / 2 + 16, s));
+    h->dyn = reinterpret_cast<int*>(h->dyn_buf.p);
     if (tcs) {
         const tt_status st = h->dyn_tc.ensure(tcs, s);
         if (st == TT_ERR_OOM)
@@ -1623,9 +1626,6 @@ tt_status graph_reserve(tt_ctx* h) {
         else
             TT_TRY(st);
     }
-    TT_TRY(eig_reserve(h->eig, s));
-    TT_TRY(h->dyn_buf.ensure((size_t)(DYN_INTS + 1) / 2 + 16, s));
-    h->dyn = reinterpret_cast<int*>(h->dyn_buf.p);
     if (!h->h_dyn) TT_CUDA_TRY(cudaMallocHost(&h->h_dyn, DYN_INTS * sizeof(int)));
     if (!h->h_dyn_dec) TT_CUDA_TRY(cudaMallocHost(&h->h_dyn_dec, 8 * sizeof(double)));
     return TT_OK;
@@ -2455,22 +2455,6 @@ tt_status create_impl(const tt_problem_desc* desc, void* stream, const tt_alloca
         TT_CREATE_TRY(h->GA.ensure((size_t)(R1 * R1), s));
         TT_CREATE_TRY(h->partials.ensure(D.precision == TT_MIXED ? slgram_scratch_doubles((int)nc, (int)R1)
                                                                  : gram_scratch_doubles((int)nc, (int)R1), s));
-        if (D.precision != TT_MIXED) {
-            // digit images and planes of the capped step's products; a handle
-            // without room for them runs on the FP64 pipe
-            const long c[][4] = {{1, R1, R1, nc}, {0, nc, cap1, R1}, {0, R1 * D.n_theta, R2, R2},
-                                 {0, R1, R1, D.n_theta * R2}, {0, cap1, D.n_theta * R2, R1}, {0, R1, R1, R1},
-                                 {1, R2, R2, cap1 * D.n_theta}, {0, cap1 * D.n_theta, cap2, R2}};
-            size_t need = 0;
-            for (const auto& q : c)
-                if (tc8_wanted(q[1], q[2], q[3])) {
-                    need = std::max(need, tc8_reserve_doubles(q[1], q[2], q[3], q[0] != 0));
-                    need = std::max(need, tc8_head_doubles(q[1], q[2], q[3], q[0] != 0) +
-                                              dyn_partials_need(q[0] ? 2 : 1, (int)q[1], (int)q[2], (int)q[3]));
-                }
-            const tt_status ps = need ? h->partials.ensure(need, s) : TT_OK;
-            if (ps < 0 && ps != TT_ERR_OOM) TT_CREATE_TRY(ps);
-        }
         for (int k = 0; k < 2; ++k) {
             const long Rk = k == 0 ? R1 : R2;
             TT_CREATE_TRY(h->GB[k].ensure((size_t)(Rk * Rk), s));
@@ -2496,6 +2480,24 @@ tt_status create_impl(const tt_problem_desc* desc, void* stream, const tt_alloca
         if (D.precision == TT_MIXED) {
             TT_CREATE_TRY(h->slscratch.ensure((size_t)(nc + R1) / 2 + 2, s));
             TT_CREATE_TRY(h->erowA.ensure((size_t)(nc + 1) / 2, s));
+        }
+        if (D.precision != TT_MIXED) {
+            // digit images and planes of the capped step's products, after all that
+            // a step cannot do without; a handle without room for them runs on
+            // the FP64 pipe
+            const long c[][4] = {{1, R1, R1, nc}, {0, nc, cap1, R1}, {0, R1 * D.n_theta, R2, R2},
+                                 {0, R1, R1, D.n_theta * R2}, {0, cap1, D.n_theta * R2, R1}, {0, R1, R1, R1},
+                                 {1, R2, R2, cap1 * D.n_theta}, {0, cap1 * D.n_theta, cap2, R2}};
+            size_t need = 0;
+            for (const auto& q : c)
+                if (tc8_wanted(q[1], q[2], q[3])) {
+                    need = std::max(need, tc8_reserve_doubles(q[1], q[2], q[3], q[0] != 0));
+                    need = std::max(need, tc8_head_doubles(q[1], q[2], q[3], q[0] != 0) +
+                                              dyn_partials_need(q[0] ? 2 : 1, (int)q[1], (int)q[2], (int)q[3]));
+                }
+            if (need) TT_CREATE_TRY(h->kscale.ensure((size_t)(std::max(D.n_theta * R2, R1) + 1) / 2, s));
+            const tt_status ps = need ? h->partials.ensure(need, s) : TT_OK;
+            if (ps < 0 && ps != TT_ERR_OOM) TT_CREATE_TRY(ps);
         }
     }
     init_isotropic(s, nc, (D.Tr0 ? D.Tr0 : D.T0) + cell0, D.c, D.a_r, h->core[0].p);

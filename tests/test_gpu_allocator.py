@@ -113,3 +113,21 @@ def test_refused_allocation_is_out_of_memory_and_leaks_nothing(ttsn):
     for _ in range(4):
         again.step()
     assert torch.equal(again.full(), ref.full())
+
+
+def test_digit_scratch_is_reserved_after_what_a_step_cannot_do_without(ttsn):
+    """One byte less than a capped handle takes: only the digit products' scratch,
+    which the FP64 pipe does without, is refused, and the handle steps all the same.
+    Both runs round to eps."""
+    p = workloads.problem("small_2d", n=(96, 90), n_theta=16, n_phi=32, eps=1e-6, bc=1)
+    p["max_rank"] = 24
+    ample = _Budget(1 << 40)
+    ref = ttsn.TTSN.from_problem(p, allocator=ample)
+    taken = sum(ample.held.values())
+    tight = _Budget(taken - 1)
+    g = ttsn.TTSN.from_problem(p, allocator=tight)
+    assert sum(tight.held.values()) < taken - (8 << 20)
+    for _ in range(4):
+        assert ref.step()["ranks"] == g.step()["ranks"]
+    E, F = ref.energy()[0], g.energy()[0]
+    assert float((E - F).norm() / E.norm()) <= 4 * 1e-6
