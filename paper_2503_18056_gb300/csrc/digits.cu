@@ -296,11 +296,10 @@ struct Side {
     // entries, index_max_kernel) or null, and op(A)'s sign
     const int* ks;
     int sign;
-    // entries at index k count as times 2^scale
+    // entries at index k count as times 2^scale (an index that one operand does not have,
+    // exponent 0, at the limit: the other's entries there must not set its rows' scale)
     __device__ __forceinline__ int scale(const Prod& p, long k) const {
-        const int x = ks[k];
-        if (x == 0) return 0;
-        const int s = min(max(x - 1023, -400), 400);
+        const int s = min(max(ks[k] - 1023, -400), 400);
         return (sign ? (sign < 0) == (isB == 0) : (isB != 0) == (p.M > p.N)) ? -s : s;
     }
     template <bool SCALE>

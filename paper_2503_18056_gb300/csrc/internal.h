@@ -91,8 +91,8 @@ struct ProdCtx {
     bool digits = true;
 };
 // The index that a rounding's product contracts: digits.cu takes op(A)'s entries at
-// index k times 2^(sign (s[k] - 1023)) and op(B)'s times the inverse, s[k] = 0: as
-// they are (s null: all).  bond_scale: s from the diagonal of the bond's Gram matrix G
+// index k times 2^(sign (s[k] - 1023)), at most 2^+-400, and op(B)'s times the inverse
+// (s null: as they are).  bond_scale: s from the diagonal of the bond's Gram matrix G
 // (n x n), rep times over; n and ldg from desc[0] and [5] where given (n then is
 // the capacity).
 struct Bond {

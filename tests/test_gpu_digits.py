@@ -329,3 +329,40 @@ def test_rounding_with_a_graded_gauge_gives_an_orthonormal_core(ttsn):
         assert r == 90 and bound < 1e-9
         assert float((A.T @ A - torch.eye(r, device=A.device, dtype=A.dtype)).abs().max()) <= bound
         assert float(torch.linalg.norm(tt.full().reshape(3000, -1) - X) / torch.linalg.norm(X)) <= 1e-6
+
+
+def test_full_tensor_with_an_index_that_one_core_does_not_have(ttsn):
+    """A row of zeros in one core against a column that is 2^40 above the other core's
+    columns: it adds nothing and must not set the scale of what does.  A term is off by
+    9.1 2^-58 2^(e_i + e_j) at most, the exponents those of entries scaled by m_k, the
+    largest of core 2's row k (a power of two at most 2 away, twice): under 2^-48 max_k(|a_ik|
+    m_k) max_k(|b_kj| / m_k)."""
+    rng = np.random.default_rng(11)
+    K = 90
+    A, B = 2.0 ** -40 * rng.standard_normal((3000, K)), rng.standard_normal((K, 2560))
+    A[:, 0], B[0] = rng.standard_normal(3000), 0.0
+    got = ttsn.TensorTrain([A[None], B[:, :, None]]).full().reshape(3000, 2560).cpu().numpy()
+    m = np.abs(B[1:]).max(1)
+    bound = K * 2.0 ** -48 * (np.abs(A[:, 1:]) * m).max(1)[:, None] * (np.abs(B[1:]) / m[:, None]).max(0)[None, :] \
+        + (K + 1) * np.finfo(float).eps * (np.abs(A) @ np.abs(B))
+    assert np.all(np.abs(got - A @ B) <= bound)
+
+
+def test_rounding_with_a_zero_column_gives_an_orthonormal_core(ttsn):
+    """A column of zeros (the emission column of a field without absorption) beside
+    columns of 2^-40: bounds as with the graded gauge."""
+    import torch
+
+    cores, _ = _gauged(np.random.default_rng(12), (3000, 64, 40), [90, 90], 0)
+    cores[0] *= 2.0 ** -40
+    cores[0][:, :, 0] = 0.0
+    tt = ttsn.TensorTrain(cores)
+    X = tt.full().reshape(3000, -1)
+    tt.round(eps=1e-6)
+    A = tt.cores()[0].reshape(3000, -1)
+    r = A.shape[1]
+    sv = torch.linalg.svdvals(X)
+    bound = 90 ** 2 * 2.0 ** -52 * float(sv[0] / sv[r - 1]) ** 2
+    assert r == 89 and bound < 1e-9
+    assert float((A.T @ A - torch.eye(r, device=A.device, dtype=A.dtype)).abs().max()) <= bound
+    assert float(torch.linalg.norm(tt.full().reshape(3000, -1) - X) / torch.linalg.norm(X)) <= 1e-6
