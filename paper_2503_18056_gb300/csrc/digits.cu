@@ -281,6 +281,11 @@ __device__ __forceinline__ unsigned char* tile_at(unsigned char* img, long rb, i
     return img + ((rb * nst + st) * S8 + s) * (long)DIG_BYTES;
 }
 
+// v times 2^s is at least 2^(e - 10)
+__device__ __forceinline__ bool is_large(double v, int s, int e) {
+    const int ex = (int)(mag(v) >> 52);
+    return ex != 0 && ex + s >= e - 10 + 1023;
+}
 // One operand (A's rows, or B's columns) of a product: rows x K.
 struct Side {
     const double* p;
@@ -288,7 +293,7 @@ struct Side {
     u64* mx;           // row maxima (where they are found ahead of the split)
     int* e;            // row exponents
     unsigned char* img;
-    int* large;  // a guarded call: each row's entries of at least 2^(e - 10)
+    int* large;  // a guarded product: each row's entries of at least 2^(e - 10)
     int* worst;  // and the most that a row falls short of K (split_rows_kernel; spread_kernel)
     int* eb;     // K > ONE_EXP_K: the words of a row's blocks (block_word), a block after the other
     long ebs;    // rows of eb
@@ -438,13 +443,17 @@ __global__ void __launch_bounds__(256) split_rows_kernel(Prod p, Side o, int* fl
         }
         const int e = SCALE ? split_exp(top, top == 0, flag) : split_exp(mx, flag);
         if (lane == 0 && r < rows) o.e[i0 + r] = e;
-        if (o.worst && mx != 0 && e != EXP_LOST) {
+        if (o.worst && r < rows) {
             int c = 0;
 #pragma unroll
             for (int t = 0; t < V; ++t)
-                c += ((int)(mag(v[t][0]) >> 52) >= e - 10 + 1023) + ((int)(mag(v[t][1]) >> 52) >= e - 10 + 1023);
-            c = K - __reduce_add_sync(0xffffffffu, c);
-            if (lane == 0 && c > *(volatile int*)o.worst) atomicMax(o.worst, c);
+                c += is_large(v[t][0], SCALE ? sc[SCALE ? t : 0].x : 0, e) + is_large(v[t][1], SCALE ? sc[SCALE ? t : 0].y : 0, e);
+            c = __reduce_add_sync(0xffffffffu, c);
+            const bool zero = SCALE ? top == 0 : mx == 0;
+            if (lane == 0) {
+                o.large[i0 + r] = zero ? K : c;
+                if (!zero && e != EXP_LOST && K - c > *(volatile int*)o.worst) atomicMax(o.worst, K - c);
+            }
         }
         const unsigned off = swz((int)(r & 63), 2 * (lane & 15));
 #pragma unroll
@@ -524,15 +533,14 @@ __global__ void __launch_bounds__(256) split_rows_long_kernel(Prod p, Side o, in
             if (k < Kc) v0 = A[r * ld + k];
             if (k + 1 < Kc) v1 = A[r * ld + k + 1];
         }
+        const int s0 = SCALE && k < Kc ? o.scale(p, p.k0 + k) : 0, s1 = SCALE && k + 1 < Kc ? o.scale(p, p.k0 + k + 1) : 0;
         if (o.large) {  // 16 lanes a row, whole warps (total is a multiple of 32)
-            const int lim = e - 10 + 1023;
-            const unsigned b0 = __ballot_sync(0xffffffffu, (int)(mag(v0) >> 52) >= lim);
-            const unsigned b1 = __ballot_sync(0xffffffffu, (int)(mag(v1) >> 52) >= lim);
+            const unsigned b0 = __ballot_sync(0xffffffffu, is_large(v0, s0, e));
+            const unsigned b1 = __ballot_sync(0xffffffffu, is_large(v1, s1, e));
             const unsigned half = threadIdx.x & 16 ? 0xffff0000u : 0xffffu;
             if (kw == 0 && r < rows) atomicAdd(o.large + i0 + r, __popc(b0 & half) + __popc(b1 & half));
         }
         unsigned w[S8];
-        const int s0 = SCALE && k < Kc ? o.scale(p, p.k0 + k) : 0, s1 = SCALE && k + 1 < Kc ? o.scale(p, p.k0 + k + 1) : 0;
         digits8x2(v0, v1, eb - s0, eb - s1, w);
         unsigned char* d = tile_at(o.img, r >> 6, nst, st, 0) + swz((int)(r & 63), 2 * kw);
 #pragma unroll
@@ -629,7 +637,8 @@ __global__ void __launch_bounds__(256, 4) split_strided_kernel(Prod p, Side o, i
             if (GUARD) {
                 int c = 0;
 #pragma unroll
-                for (int r = 0; r < 8; ++r) c += (int)((F[r] >> 52) & 0x7FF) >= e - 10 + 1023;
+                for (int r = 0; r < 8; ++r)
+                    c += is_large(__longlong_as_double((long long)F[r]), SCALE && k0 + r < Kc ? o.scale(p, p.k0 + k0 + r) : 0, e);
                 atomicAdd(&s_large[threadIdx.x & 31], c);
             }
 #pragma unroll
@@ -653,14 +662,21 @@ __global__ void __launch_bounds__(256, 4) split_strided_kernel(Prod p, Side o, i
     }
 }
 
-// *worst: the most indices of a nonzero row that are not large
-__global__ void __launch_bounds__(256) spread_kernel(long rows, int K, const int* __restrict__ large,
-                                                     const u64* __restrict__ mx, const int* __restrict__ e, int* worst) {
+// *worst: the most indices of a nonzero row that are not large; zero rows count as
+// large everywhere
+__global__ void __launch_bounds__(256) spread_kernel(Prod p, Side o) {
+    p.Mc = p.M;
+    if (!resolve(p) || (!o.strided && p.K <= ONE_EXP_K)) return;  // found by the split
+    const long rows = o.isB ? p.N : p.M;
     int w = 0;
-    for (long r = blockIdx.x * 256L + threadIdx.x; r < rows; r += gridDim.x * 256L)
-        if (mx[r] != 0 && e[r] != EXP_LOST) w = max(w, K - large[r]);
+    for (long r = blockIdx.x * 256L + threadIdx.x; r < rows; r += gridDim.x * 256L) {
+        if (o.mx[r] == 0)
+            o.large[r] = (int)p.K;
+        else if (o.e[r] != EXP_LOST)
+            w = max(w, (int)p.K - o.large[r]);
+    }
     w = __reduce_max_sync(0xffffffffu, w);
-    if ((threadIdx.x & 31) == 0 && w > *(volatile int*)worst) atomicMax(worst, w);
+    if ((threadIdx.x & 31) == 0 && w > *(volatile int*)o.worst) atomicMax(o.worst, w);
 }
 
 // ------------------------------------------------------------------ product
@@ -1063,11 +1079,12 @@ tt_status run(cudaStream_t s, bool ta, bool tb, long M, long N, long K, double a
     const int* ks = !scale ? nullptr : find ? kx : bond->s;
     const int sign = bond ? bond->sign : 0;
     int* ex = kx + (gram ? 0 : K);
-    int* large = guard ? ex + nrows : nullptr;
-    int* worst = guard ? flag + LOST_WORST : nullptr;
+    const bool count = guard || find;
+    int* large = count ? ex + nrows : nullptr;
+    int* worst = count ? flag + LOST_WORST : nullptr;
     int* eb = ex + 2 * nrows;  // behind the counts
     Side a{A, 0, ta ? 1 : 0, mx, ex, base + q.head + q.imgB, large, worst, eb, M, ks, sign};
-    Side b{B, 1, tb ? 0 : 1, mx + M, ex + M, base + q.head, guard ? large + M : nullptr, guard ? worst + 1 : nullptr,
+    Side b{B, 1, tb ? 0 : 1, mx + M, ex + M, base + q.head, count ? large + M : nullptr, count ? worst + 1 : nullptr,
            eb + (K + BLK_K - 1) / BLK_K * M, N, ks, sign};
     if (gram) {
         a.img = base + q.head;
@@ -1083,7 +1100,7 @@ tt_status run(cudaStream_t s, bool ta, bool tb, long M, long N, long K, double a
     // the flag and, where atomics find them, the maxima and counts start at zero
     const size_t maxima_bytes = a.strided || b.strided || K > ONE_EXP_K || find ? 8 * (size_t)nrows : 0;
     TT_CUDA_TRY(cudaMemsetAsync(flag, 0, 256 + maxima_bytes + (find ? 4 * (size_t)K : 0), s));
-    if (guard) TT_CUDA_TRY(cudaMemsetAsync(large, 0, 4 * (size_t)nrows, s));
+    if (count) TT_CUDA_TRY(cudaMemsetAsync(large, 0, 4 * (size_t)nrows, s));
     const bool fusable = K <= ONE_EXP_K;  // a captured step launches both forms when K may be longer
     auto maxima = [&](const Side& o) {
         const long rows = o.isB ? N : M;
@@ -1103,7 +1120,8 @@ tt_status run(cudaStream_t s, bool ta, bool tb, long M, long N, long K, double a
         if (o.strided) {
             const dim3 grid(blocks_for((rpad + 31) / 32, 4096), blocks_for(((long)nst * 2 + 7) / 8, 2048));
             note_launch();
-            (guard   ? split_strided_kernel<true, false>
+            (find    ? split_strided_kernel<true, true>
+             : guard ? split_strided_kernel<true, false>
              : scale ? split_strided_kernel<false, true>
                      : split_strided_kernel<false, false>)<<<grid, 256, 0, s>>>(p, o, flag);
             return;
@@ -1172,19 +1190,19 @@ tt_status run(cudaStream_t s, bool ta, bool tb, long M, long N, long K, double a
         note_launch();
         tc8_reduce_kernel<<<blocks_for((M * N + 255) / 256, 152L * 16), 256, 0, s>>>(p, planes, a.e, b.e, spc, alpha, C);
     }
-    if (guard) {
+    if (count) {
         auto spread = [&](const Side& o) {
             const long rows = o.isB ? N : M;
             if (!o.strided && fusable) return;  // found by the split
             note_launch();
-            spread_kernel<<<blocks_for((rows + 255) / 256, 152), 256, 0, s>>>(rows, (int)K, o.large, o.mx, o.e, o.worst);
+            spread_kernel<<<blocks_for((rows + 255) / 256, 152), 256, 0, s>>>(p, o);
         };
         spread(a);
         if (!gram) spread(b);
     }
     TT_CUDA_TRY(cudaGetLastError());
-    *lost = Lost{flag, a.e, b.e, guard ? 1 : 0, gram ? 1 : 0, reinterpret_cast<double*>(base + q.head), mx, a.eb, a.ebs,
-                 gram && !guard ? reinterpret_cast<float*>(ex + nrows) : nullptr};
+    *lost = Lost{flag, a.e, b.e, guard ? 1 : find ? 2 : 0, gram ? 1 : 0, reinterpret_cast<double*>(base + q.head), mx, a.eb, a.ebs,
+                 gram && !guard ? reinterpret_cast<float*>(ex + nrows) : nullptr, a.large, b.large};
     return TT_OK;
 }
 

@@ -236,6 +236,11 @@ prod_kernel(int M, int N, int K, double alpha, const double* __restrict__ A, lon
                 const unsigned a = __reduce_max_sync(0xffffffffu, lane < BT ? r : 0u);
                 const unsigned b = __reduce_max_sync(0xffffffffu, lane < BT ? 0u : r);
                 if (!(__uint_as_float(a) * __uint_as_float(b) > 1.0f)) continue;
+            } else if (lost.guard == 2) {  // rows that are lost are large nowhere
+                const int c = lane < BT ? lost.la[i] : lost.lb[i];
+                const int a = __reduce_min_sync(0xffffffffu, lane < BT ? c : K);
+                const int b = __reduce_min_sync(0xffffffffu, lane < BT ? K : c);
+                if (a + b >= K + K / 16) continue;
             } else if (!__any_sync(0xffffffffu, (lane < BT ? lost.a[i] : lost.b[i]) == EXP_LOST)) {
                 continue;
             }
@@ -535,7 +540,7 @@ void launch_one(cudaStream_t s, bool ordered, unsigned grid, const ProdArgs& a) 
 tt_status launch_prod(cudaStream_t s, bool ta, bool tb, bool ordered, long items, const ProdArgs& a) {
     // more CTAs than fit at once let the scheduler level uneven tiles; behind a
     // rounding's digit product they seldom have any (a library call may lose all)
-    const bool idle = a.lost.flag && !a.lost.guard && !a.desc;
+    const bool idle = a.lost.flag && a.lost.guard != 1 && !a.desc;
     const unsigned grid = (unsigned)std::max(1L, std::min(items, idle ? 152L * 8 : 152L * 64));
     note_launch();
     if (ta && tb)

@@ -196,7 +196,8 @@ size_t tc8_reserve_doubles(long M, long N, long K, bool gram);
 // entries and their blocks' words (gram_check_kernel): the exponent and, in the
 // low ten bits, the number of entries with digits.  rho: what gram_check_kernel
 // makes of them, an entry is lost where rho_i rho_j > 1 (not looked at in a guarded
-// product).
+// product).  guard: 1 a library call, 2 a handle's product at a scale that was found
+// from the operands; la, lb: the indices that each row is large at.
 constexpr int LOST_ALL = 0, LOST_ROWS = 1, LOST_WORST = 2;
 constexpr int EXP_LOST = 1 << 20;
 __host__ __device__ inline int block_exp(int word) { return word >> 10; }
@@ -210,16 +211,17 @@ struct Lost {
     const int* eb = nullptr;
     long ebs = 0;
     float* rho = nullptr;
+    const int *la = nullptr, *lb = nullptr;
 };
 #ifdef __CUDACC__
-// 2: everything is lost (of a guarded product also where two rows may have fewer
-// than K / 16 indices where both are large; the Gram has one operand), 1: some
-// rows, 0: nothing.
+// 2: everything is lost (of a library call also where two rows may have fewer than
+// K / 16 indices where both are large; the Gram has one operand), 1: some rows (of a
+// handle's product also the tiles with two such rows), 0: nothing.
 __device__ inline int tc8_lost(const Lost& l, int K) {
-    if (l.flag[LOST_ALL] ||
-        (l.guard && (long)l.flag[LOST_WORST] + l.flag[LOST_WORST + (l.gram ? 0 : 1)] > K - K / 16))
-        return 2;
-    return l.flag[LOST_ROWS] ? 1 : 0;
+    if (l.flag[LOST_ALL]) return 2;
+    const bool few = l.guard && (long)l.flag[LOST_WORST] + l.flag[LOST_WORST + (l.gram ? 0 : 1)] > K - K / 16;
+    if (few && l.guard == 1) return 2;
+    return few || l.flag[LOST_ROWS] ? 1 : 0;
 }
 #endif
 size_t tc8_head_doubles(long M, long N, long K, bool gram);

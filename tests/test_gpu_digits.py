@@ -366,3 +366,23 @@ def test_rounding_with_a_zero_column_gives_an_orthonormal_core(ttsn):
     assert r == 89 and bound < 1e-9
     assert float((A.T @ A - torch.eye(r, device=A.device, dtype=A.dtype)).abs().max()) <= bound
     assert float(torch.linalg.norm(tt.full().reshape(3000, -1) - X) / torch.linalg.norm(X)) <= 1e-6
+
+
+@pytest.mark.parametrize("M,K,N", [(3000, 90, 2560), (2560, 300, 300), (300, 2000, 300)])
+@pytest.mark.parametrize("which", [0, 1])
+def test_full_tensor_of_blocks_at_different_scales(ttsn, M, K, N, which):
+    """One core dense, the other of four blocks on their own indices, nine decades
+    apart: no scale of the index shows the small blocks' products to the dense core's
+    rows, so those are recomputed.  What is not has K / 18 indices at least where both
+    entries are within 2^-9 of the exponents, where a term is off by 9.1 2^-58: under
+    2^-30 of the sum |a||b|."""
+    rng = np.random.default_rng(K)
+    A, B = rng.standard_normal((M, K)), rng.standard_normal((K, N))
+    X = A if which else B
+    m, n = X.shape
+    keep = np.zeros((m, n))
+    for i in range(4):
+        keep[i * m // 4:(i + 1) * m // 4, i * n // 4:(i + 1) * n // 4] = 10.0 ** (-3 * i)
+    X *= keep
+    got = ttsn.TensorTrain([A[None], B[:, :, None]]).full().reshape(M, N).cpu().numpy()
+    assert np.all(np.abs(got - A @ B) <= (2.0 ** -30 + (K + 1) * np.finfo(float).eps) * (np.abs(A) @ np.abs(B)))
