@@ -203,9 +203,9 @@ __device__ __forceinline__ int split_stages_warp(long M, long N, long ntiles, in
     const int lim = split_limit(M, N, nst, unit), lane = threadIdx.x & 31;
     unsigned key = 0xffffffffu;
     for (int k = lane + 1; k <= lim; k += 32)
-        key = min(key, split_cost(k, ntiles, nst, unit) * 64u + (unsigned)(k - 1));
+        key = min(key, split_cost(k, ntiles, nst, unit) * 128u + (unsigned)(k - 1));
     key = __reduce_min_sync(0xffffffffu, key);
-    return stages_of_split((int)(key & 63u) + 1, nst, unit);
+    return stages_of_split((int)(key & 127u) + 1, nst, unit);
 }
 
 // ------------------------------------------------------------------ split
@@ -308,8 +308,8 @@ struct Side {
         return (sign ? (sign < 0) == (isB == 0) : (isB != 0) == (p.M > p.N)) ? -s : s;
     }
     template <bool SCALE>
-    __device__ __forceinline__ u64 mag_at(const Prod& p, const double* q, long k) const {
-        const u64 m = mag(*q);
+    __device__ __forceinline__ u64 mag_at(const Prod& p, double v, long k) const {
+        const u64 m = mag(v);
         const int ex = (int)(m >> 52);
         if (!SCALE || ex == 0 || ex == 0x7FF) return m;
         return (m & 0xFFFFFFFFFFFFFull) | (u64)min(max(ex + scale(p, k), 1), 0x7FF) << 52;
@@ -487,7 +487,7 @@ __global__ void __launch_bounds__(256) row_max_kernel(Prod p, Side o) {
         u64 m0 = 0, m1 = 0, m2 = 0, m3 = 0;
         int c = 0;
         auto see = [&](u64& m, long k) {
-            const u64 v = o.mag_at<SCALE>(p, row + k, k);
+            const u64 v = o.mag_at<SCALE>(p, row[k], k);
             m = umax(m, v);
             c += (v >> 52) != 0;
         };
@@ -554,16 +554,22 @@ __global__ void __launch_bounds__(256) split_rows_long_kernel(Prod p, Side o, in
 // stores 16 bytes a digit.  Bound by the latency of its loads: 8 rows fit 64
 // registers, four CTAs an SM (49,152 x 449: 156 us, 3.7 TB/s; with 16 rows a
 // thread, 128 registers and two CTAs 251 us, with 48 registers and spills 230).
+// Of up to MAX_WARPS warps: where there are fewer CTAs than fit at once, their time is
+// that of a warp's loads after one another, and 32 warps read a block of 512 rows in two
+// batches of eight loads each (3,000 x 100: 20.8 -> 10.8 us); more CTAs want eight warps
+// (500,000 x 449: 0.26 ms against 0.46 with 32).
+constexpr int MAX_WARPS = 32;
 template <bool SCALE>
-__global__ void __launch_bounds__(256) strided_max_kernel(Prod p, Side o) {
+__global__ void __launch_bounds__(32 * MAX_WARPS) strided_max_kernel(Prod p, Side o) {
     p.Mc = p.M;
     if (!resolve(p)) return;
     const long n = o.isB ? p.N : p.M, ld = o.isB ? p.ldb : p.lda;
     // a block of indices after the other, or one range a CTA
     const bool blocked = p.K > ONE_EXP_K;
     const long per = blocked ? BLK_K : (p.K + gridDim.y - 1) / gridDim.y;
-    __shared__ u64 part[8][32];
-    __shared__ int count[8][32];
+    const int W = blockDim.x >> 5;
+    __shared__ u64 part[MAX_WARPS][32];
+    __shared__ int count[MAX_WARPS][32];
     for (long jb = blockIdx.x * 32L; jb < n; jb += gridDim.x * 32L) {
         const long j = jb + (threadIdx.x & 31);
         u64 top = 0;
@@ -571,20 +577,27 @@ __global__ void __launch_bounds__(256) strided_max_kernel(Prod p, Side o) {
             const long k1 = min(p.K, (kb + 1) * per);
             u64 m0 = 0, m1 = 0, m2 = 0, m3 = 0;
             int c = 0;
-            auto see = [&](u64& m, long k) {
-                const u64 v = o.mag_at<SCALE>(p, o.p + k * ld + j, k);
+            auto see = [&](u64& m, double x, long k) {
+                const u64 v = o.mag_at<SCALE>(p, x, k);
                 m = umax(m, v);
                 c += (v >> 52) != 0;
             };
             if (j < n) {
                 long k = kb * per + (threadIdx.x >> 5);
-                for (; k + 24 < k1; k += 32) {
-                    see(m0, k);
-                    see(m1, k + 8);
-                    see(m2, k + 16);
-                    see(m3, k + 24);
+                for (; k + 7 * W < k1; k += 8 * W) {
+                    double x[8];
+#pragma unroll
+                    for (int t = 0; t < 8; ++t) x[t] = o.p[(k + W * t) * ld + j];
+#pragma unroll
+                    for (int t = 0; t < 8; t += 4) {
+                        see(m0, x[t], k + W * t);
+                        see(m1, x[t + 1], k + W * (t + 1));
+                        see(m2, x[t + 2], k + W * (t + 2));
+                        see(m3, x[t + 3], k + W * (t + 3));
+                    }
                 }
-                for (; k < k1; k += 8) see(m0, k);
+#pragma unroll 4
+                for (; k < k1; k += W) see(m0, o.p[k * ld + j], k);
             }
             __syncthreads();
             part[threadIdx.x >> 5][threadIdx.x & 31] = umax(umax(m0, m1), umax(m2, m3));
@@ -592,8 +605,8 @@ __global__ void __launch_bounds__(256) strided_max_kernel(Prod p, Side o) {
             __syncthreads();
             if (threadIdx.x < 32 && j < n) {
                 u64 m = part[0][threadIdx.x];
-#pragma unroll
-                for (int w = 1; w < 8; ++w) {
+#pragma unroll 8
+                for (int w = 1; w < W; ++w) {
                     m = umax(m, part[w][threadIdx.x]);
                     c += count[w][threadIdx.x];
                 }
@@ -1107,7 +1120,8 @@ tt_status run(cudaStream_t s, bool ta, bool tb, long M, long N, long K, double a
         if (o.strided) {
             note_launch();
             const dim3 grid(blocks_for((rows + 31) / 32, 4096), blocks_for(K / (fusable ? 256 : BLK_K), 512));
-            (scale ? strided_max_kernel<true> : strided_max_kernel<false>)<<<grid, 256, 0, s>>>(p, o);
+            const int threads = 32 * (grid.x * grid.y < 304 ? MAX_WARPS : 8);
+            (scale ? strided_max_kernel<true> : strided_max_kernel<false>)<<<grid, threads, 0, s>>>(p, o);
         } else if (!fusable) {
             note_launch();
             const unsigned grid = blocks_for((rows * ((K + BLK_K - 1) / BLK_K) + 7) / 8, 152L * 64);

@@ -60,12 +60,17 @@ TTSN_HD long tiles_of(long M, long N, int gram) {
 // blocks' sums, and with them the result's bits, do not depend on the chunks
 // (unit: stages that stay together).
 constexpr long PLANE_ELEMS = 1L << 23;
-constexpr int MAX_SPLITS = 64;
+// Whole blocks go badly into 64 parts: up to 80 of them (a Gram of 100,000 x 100, two
+// tiles: 66 splits of three blocks instead of 49 of four; of 30,000 x 60, one tile: 59 of
+// one block).
+constexpr int MAX_SPLITS = 64, MAX_BLOCK_SPLITS = 80;
 constexpr long CHUNK_MIN = 16384;  // no shorter contraction goes in chunks
 TTSN_HD int split_unit(long K) { return K > CHUNK_MIN ? T_BLK : 1; }
+TTSN_HD long most_splits(int nst, int unit) {
+    return unit > 1 ? least((nst + unit - 1) / unit, MAX_BLOCK_SPLITS) : least(nst / 4, MAX_SPLITS);
+}
 TTSN_HD int split_limit(long M, long N, int nst, int unit) {
-    long k = PLANE_ELEMS / (M * N);
-    k = least(k, least(nst / most(4, unit), MAX_SPLITS));
+    const long k = least(PLANE_ELEMS / (M * N), most_splits(nst, unit));
     return k < 1 ? 1 : (int)k;
 }
 TTSN_HD int stages_of_split(int k, int nst, int unit) { return (int)up((nst + k - 1) / k, unit); }
@@ -73,7 +78,7 @@ TTSN_HD unsigned split_cost(int k, long ntiles, int nst, int unit) {
     const int spc = stages_of_split(k, nst, unit), kk = (nst + spc - 1) / spc;
     const long waves = (ntiles * kk + 151) / 152;
     const long c = waves * (spc + 1) * 64 + kk;
-    return c > 0x03ffffffL ? 0x03ffffffu : (unsigned)c;
+    return c > 0x01ffffffL ? 0x01ffffffu : (unsigned)c;  // 25 bits (split_stages_warp)
 }
 TTSN_HD int split_stages(long M, long N, long ntiles, int nst, int unit) {
     const int lim = split_limit(M, N, nst, unit);
@@ -111,8 +116,8 @@ inline Plan make_plan(long M, long N, long K, bool gram, bool captured) {
     const bool sums = gram || p.Kc < K;  // planes although there is one split
     long elems = sums ? M * N : 0;
     if (captured) {
-        const long most_splits = least(nst / 4, MAX_SPLITS);
-        if (most_splits > 1) elems = most(elems, least(M * N * most_splits, PLANE_ELEMS));
+        const long splits = most(most_splits(nst, 1), K > CHUNK_MIN ? most_splits(nst, T_BLK) : 1);
+        if (splits > 1) elems = most(elems, least(M * N * splits, PLANE_ELEMS));
     } else {
         const int spc = split_stages(M, N, tiles_of(p.Mc, N, gram), nst, split_unit(K));
         if (spc < nst) elems = M * N * ((nst + spc - 1) / spc);
@@ -131,7 +136,7 @@ inline size_t reserve_bytes(long M, long N, long K, bool gram) {
     const long Np = up(N, gram ? T_M : RB), Kp = up(K, T_K), row = 2 * S8;
     const long imgB = least(Np * Kp, most(IMG_LIMIT / row, CHUNK_MIN * Np)) * row;
     const long imgA = gram ? 0 : least(up(M, T_M) * Kp, IMG_LIMIT / row) * row;
-    const long splits = least(stages(K) / 4, MAX_SPLITS);
+    const long splits = most(most_splits(stages(K), 1), K > CHUNK_MIN ? most_splits(stages(K), T_BLK) : 1);
     long elems = gram || K > CHUNK_MIN ? M * N : 0;
     if (splits > 1) elems = most(elems, least(M * N * splits, PLANE_ELEMS));
     return head_bytes(M, N, K, gram) + (size_t)(imgA + imgB + 16 * elems);
