@@ -83,8 +83,14 @@ TTSN_HD unsigned split_cost(int k, long ntiles, int nst, int unit) {
 TTSN_HD int split_stages(long M, long N, long ntiles, int nst, int unit) {
     const int lim = split_limit(M, N, nst, unit);
     int best = 1;
-    for (int k = 2; k <= lim; ++k)
-        if (split_cost(k, ntiles, nst, unit) < split_cost(best, ntiles, nst, unit)) best = k;
+    unsigned cost = split_cost(1, ntiles, nst, unit);
+    for (int k = 2; k <= lim; ++k) {
+        const unsigned c = split_cost(k, ntiles, nst, unit);
+        if (c < cost) {
+            cost = c;
+            best = k;
+        }
+    }
     return stages_of_split(best, nst, unit);
 }
 

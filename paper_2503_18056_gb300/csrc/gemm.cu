@@ -162,8 +162,14 @@ int prod_split(long M, long N, long K, int tri) {
     const long tiles = prod_tiles(M, N, tri);
     const int lim = prod_limit(tiles, K);
     int best = 1;
-    for (int k = 2; k <= lim; ++k)
-        if (prod_cost(tiles, K, k) < prod_cost(tiles, K, best)) best = k;
+    unsigned least = prod_cost(tiles, K, 1);
+    for (int k = 2; k <= lim; ++k) {
+        const unsigned c = prod_cost(tiles, K, k);
+        if (c < least) {
+            least = c;
+            best = k;
+        }
+    }
     return prod_final(K, best);
 }
 // Splits and indices per split of a rounding's product (ordered); tri: the Gram.
