@@ -48,7 +48,10 @@
 //   on D, but a power of two a row would see D on one side and 1 / D on the other.
 //   So they are formed at a scale of the index: the norms of A's columns where a
 //   rounding has their Gram matrix (Bond), else the smaller operand's entries
-//   (index_max_kernel).  A D of powers of two then changes no bit of tt_to_full.
+//   (index_max_kernel).  A D of powers of two then changes no bit of tt_to_full.  Where
+//   the scale is found so, it may still hide one operand's blocks from the other's
+//   rows: the entries above 2^-9 of a row's maximum are counted, and the 16 x 16 tiles
+//   with a row and a column that share fewer than K / 16 such indices are recomputed.
 //   What the smaller operand gives is not enough in a rounding: P_A's entries go like
 //   1 / sigma_j, and its largest ones would set the scale of A' columns to which they
 //   do not belong.
