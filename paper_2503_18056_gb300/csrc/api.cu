@@ -2751,8 +2751,9 @@ tt_status tt_to_full(tt_handle h, double* out_dev, size_t out_len) {
             outp = h->tmp[ti].p;
             ti ^= 1;
         }
+        const Bond entries{nullptr, 0, true};
         TT_TRY(dgemm_sk(s, false, false, (int)rows, (int)cols, h->r[k + 1], 1.0, h->core[k].p,
-                     h->r[k + 1], T, cols, outp, cols, h->partials, h->prod, false));
+                     h->r[k + 1], T, cols, outp, cols, h->partials, h->prod, false, &entries));
         T = outp;
         cols *= h->n[k];
     }

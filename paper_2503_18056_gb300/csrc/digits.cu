@@ -48,10 +48,11 @@
 //   on D, but a power of two a row would see D on one side and 1 / D on the other.
 //   So they are formed at a scale of the index: the norms of A's columns where a
 //   rounding has their Gram matrix (Bond), else the smaller operand's entries
-//   (index_max_kernel).  A D of powers of two then changes no bit of tt_to_full.  Where
-//   the scale is found so, it may still hide one operand's blocks from the other's
-//   rows: the entries above 2^-9 of a row's maximum are counted, and the 16 x 16 tiles
-//   with a row and a column that share fewer than K / 16 such indices are recomputed.
+//   (index_max_kernel).  A D of powers of two then changes no bit of tt_to_full.  Such
+//   a scale may still hide one operand's blocks from the other's rows; in tt_to_full,
+//   whose entries are the caller's, the entries above 2^-9 of a row's maximum are
+//   counted, and the 16 x 16 tiles with a row and a column that share fewer than K / 16
+//   such indices are recomputed.
 //   What the smaller operand gives is not enough in a rounding: P_A's entries go like
 //   1 / sigma_j, and its largest ones would set the scale of A' columns to which they
 //   do not belong.
@@ -1099,12 +1100,13 @@ tt_status run(cudaStream_t s, bool ta, bool tb, long M, long N, long K, double a
     int* flag = reinterpret_cast<int*>(base);
     u64* mx = reinterpret_cast<u64*>(base + 256);
     const long nrows = gram ? M : M + N;
-    const bool scale = !gram && !guard && !(bond && !bond->s), find = scale && !bond;
+    const bool entries = bond && bond->entries;
+    const bool scale = !gram && !guard && (!bond || bond->s || entries), find = scale && !(bond && bond->s);
     int* kx = reinterpret_cast<int*>(mx + nrows);  // of its own, found below
     const int* ks = !scale ? nullptr : find ? kx : bond->s;
     const int sign = bond ? bond->sign : 0;
     int* ex = kx + (gram ? 0 : K);
-    const bool count = guard || find;
+    const bool count = guard || entries;
     int* large = count ? ex + nrows : nullptr;
     int* worst = count ? flag + LOST_WORST : nullptr;
     int* eb = ex + 2 * nrows;  // behind the counts
@@ -1146,7 +1148,7 @@ tt_status run(cudaStream_t s, bool ta, bool tb, long M, long N, long K, double a
         if (o.strided) {
             const dim3 grid(blocks_for((rpad + 31) / 32, 4096), blocks_for(((long)nst * 2 + 7) / 8, 2048));
             note_launch();
-            (find    ? split_strided_kernel<true, true>
+            (entries ? split_strided_kernel<true, true>
              : guard ? split_strided_kernel<true, false>
              : scale ? split_strided_kernel<false, true>
                      : split_strided_kernel<false, false>)<<<grid, 256, 0, s>>>(p, o, flag);
@@ -1227,7 +1229,7 @@ tt_status run(cudaStream_t s, bool ta, bool tb, long M, long N, long K, double a
         if (!gram) spread(b);
     }
     TT_CUDA_TRY(cudaGetLastError());
-    *lost = Lost{flag, a.e, b.e, guard ? 1 : find ? 2 : 0, gram ? 1 : 0, reinterpret_cast<double*>(base + q.head), mx, a.eb, a.ebs,
+    *lost = Lost{flag, a.e, b.e, guard ? 1 : entries ? 2 : 0, gram ? 1 : 0, reinterpret_cast<double*>(base + q.head), mx, a.eb, a.ebs,
                  gram && !guard ? reinterpret_cast<float*>(ex + nrows) : nullptr, a.large, b.large};
     return TT_OK;
 }
