@@ -770,8 +770,8 @@ def run_batch(args, torch, ttsn):
 
 # ncu DRAM read + write bytes of one left Gram at the bench's rank cap (2,097,152
 # x 897), scaled by the rows from an ncu capture (dram__bytes_read and _write) of
-# the same kernels on a 500,000 x 897 operand: 28.64 GB.
-GRAM_LEFT_CAP_TRAFFIC = (19711065856 + 8932266496) * 2097152 / 500000
+# the same kernels on a 500,000 x 897 operand: 28.57 GB.
+GRAM_LEFT_CAP_TRAFFIC = (19836729344 + 8736779520) * 2097152 / 500000
 
 
 def roofline_of(prof, fp64_peak, peaks):

@@ -30,7 +30,7 @@
 // the sizes where it is used (tc8_wanted) have K >= 64.
 //
 // Measured (GB300, CUDA events, against the FP64 pipe's kernels): Gram of
-// 500,000 x 449 143 -> 5.95 ms (5.72 with one exponent a column), error against the
+// 500,000 x 449 143 -> 5.87 ms (5.67 with one exponent a column), error against the
 // exact product 1.3e-15 -> 1.2e-16 (2.4e-16); 200,000 x 577 times 577 x 96 22.4 ->
 // 1.8 ms, 8.0e-16 -> 5.5e-16.
 //
